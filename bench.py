@@ -739,7 +739,7 @@ def surrogate_leg(args, fdirw, torch, dev, stream, w, shape, D, c0, dt_macro, pr
         with torch.cuda.stream(stream):
             f = fdirw.FDiRW(shape, D, dt_macro, w.R, w.n_sub, prec, stream=stream)
             if mode == "fd":
-                f.kernels()                    # warm the autotuner outside the timed build
+                f.kernels()                    # warm up outside the timed build
                 stream.synchronize()
             e0.record(stream)
             acc = f.kernels() if mode == "fd" else net.build_kernels(f.ctx)
@@ -1057,7 +1057,7 @@ def main(argv=None):
     ap.add_argument("--ref-sample-1t", type=int, default=2048, help="sources of the single-thread oracle sample")
     ap.add_argument("--march-parts", type=int, default=0,
                     help="force a march thread mapping (1-3 threads per column, 4 = 2x2 TMEM blocks, 5 = TMEM "
-                         "lateral faces, 6 = source pairs in f32x2, 7 = column pairs with TMEM faces); 0 = autotune")
+                         "lateral faces, 6 = source pairs in f32x2, 7 = column pairs with TMEM faces); 0 = the fastest of the radius")
     ap.add_argument("--no-probe", action="store_true", help="skip the FP32 FMA and HBM read peak probes")
     ap.add_argument("--traffic", type=float, default=None,
                     help="DRAM bytes per march launch from an ncu capture of the current kernel")

@@ -99,10 +99,8 @@ typedef struct {
                              packed f32x2 arithmetic, lateral faces of both in Tensor Memory (R <= 8);
                              7 = one thread per pair of x-adjacent window columns with their lateral faces
                              and diagonals in Tensor Memory;
-                             window_R 9 and 10 take 4, 5 or 7 only (another request is autotuned between
-                             those three); 0 = autotune (each candidate timed once on the first build for a device, R
-                             and storage type, result cached for the process; that build synchronises the
-                             stream) */
+                             window_R 9 and 10 take 4, 5 or 7 only (another request is taken as 0);
+                             0 = the fastest one of the radius */
     int32_t  accum;       /* fdirw_accum; FDIRW_ACCUM_FP32 needs an FP32-march precision and an fdirw_create
                              or batch context (coarse-mesh contexts take FDIRW_ACCUM_FF only) */
 } fdirw_opts;
@@ -153,7 +151,7 @@ FDIRW_API int fdirw_stable_dt(const fdirw_grid* grid, const double* D_map, int32
  *   dt_macro   : macro step (>= 0, finite); dt_sub = dt_macro / n_sub
  *   window_R   : window radius, 0 <= R <= 10; <= 8 with FDIRW_FP64 (R = 0 gives the identity operator)
  *   n_sub      : explicit substeps per macro step, >= 0 (0 gives the identity operator)
- *   opts       : NULL for defaults (FDIRW_FP32, current device, default stream, no cap, autotune)
+ *   opts       : NULL for defaults (FDIRW_FP32, current device, default stream, no cap, fastest mapping)
  *   out        : receives the context (set to NULL on failure)
  * Computes the face conductances on the device and checks stability; the kernel cache is built
  * lazily (fdirw_kernels or the first fdirw_step).  Errors: FDIRW_ERR_ARG, FDIRW_ERR_UNSTABLE,

@@ -1,6 +1,6 @@
 """Builds libfdirw.so in-tree (``paper_2408_11376_gb300/_build/``) with nvcc for sm_103a only.
 
-The four translation units are compiled in parallel and linked with the static CUDA runtime, so the
+The translation units are compiled in parallel and linked with the static CUDA runtime, so the
 library depends only on the CUDA driver.  Rebuilds when a source or header is newer than the library.
 """
 from __future__ import annotations
@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libfdirw.so")
-SOURCES = ["api.cu", "setup.cu", "march.cu", "superpose.cu", "surrogate.cu", "noalloc.cu", "batch.cu", "coarse.cu", "flow.cu", "probe.cu"]
+SOURCES = ["api.cu", "setup.cu", "march.cu", "march_tm.cu", "superpose.cu", "surrogate.cu", "noalloc.cu", "batch.cu", "coarse.cu", "flow.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
               "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]

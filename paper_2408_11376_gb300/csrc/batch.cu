@@ -85,7 +85,6 @@ struct Batch {
     void* arena = nullptr;
     uint64_t arena_bytes = 0;
     int resident = -1;                           // chunk whose kernels the arena holds
-    int parts[kMaxR + 1] = {};                   // march mapping per radius (0 = not chosen yet)
     float2* chat = nullptr;
     cudaStream_t gs = nullptr;                   // capture stream
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -344,24 +343,6 @@ int ensure_arena(fdirw_ctx* c) {
     return FDIRW_OK;
 }
 
-// Chooses the march mapping of every radius present (timing candidates on the first chunk holding that
-// radius when autotuning); any kernels in the arena are invalid afterwards.
-int ensure_parts(fdirw_ctx* c) {
-    Batch& b = *c->batch;
-    bool tuned = false;
-    for (int r : b.radii) {
-        if (r == 0 || b.parts[r] != 0) continue;
-        for (const Chunk& ch : b.chunks) {
-            if (ch.seg_end[r] == ch.seg_begin[r]) continue;
-            FDIRW_CUDA(c, tune_march(march_args(c, ch, r), c->num_sms, c->parts_req, c->stream, &b.parts[r]));
-            tuned = true;
-            break;
-        }
-    }
-    if (tuned) b.resident = -1;
-    return FDIRW_OK;
-}
-
 // Timing events: inside a stream capture they must be external event nodes to be queryable after a
 // graph launch; outside a capture that flag is not accepted.
 cudaError_t record(cudaEvent_t ev, cudaStream_t st, bool captured) {
@@ -381,7 +362,7 @@ cudaError_t build_chunk(fdirw_ctx* c, int ci, cudaStream_t st, bool captured) {
         if (e != cudaSuccess) break;
         if (r == 0 || ch.seg_end[r] == ch.seg_begin[r]) continue;
         int used = 0;
-        e = launch_march(march_args(c, ch, r), c->num_sms, b.parts[r], st, &used);
+        e = launch_march(march_args(c, ch, r), c->num_sms, c->parts_req, st, &used);
         c->parts_used = used;
     }
     if (e == cudaSuccess) e = record(b.ev[4 * ci + 1], st, captured);
@@ -563,9 +544,8 @@ int batch_kernels(fdirw_ctx* c) {
     Batch& b = *c->batch;
     if (c->R == 0 || c->n_sub == 0) { c->kernels_ready = true; return FDIRW_OK; }
     if (b.chunks.size() != 1) return FDIRW_OK;        // built chunk by chunk inside fdirw_step
-    int rc = ensure_arena(c);
+    const int rc = ensure_arena(c);
     if (rc != FDIRW_OK) return rc;
-    if ((rc = ensure_parts(c)) != FDIRW_OK) return rc;
     FDIRW_CUDA(c, cudaEventRecord(b.fork, c->stream));
     FDIRW_CUDA(c, cudaStreamWaitEvent(b.gs, b.fork, 0));
     FDIRW_CUDA(c, build_chunk(c, 0, b.gs, false));
@@ -600,7 +580,6 @@ int batch_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps,
     } else {
         int rc = ensure_arena(c);
         if (rc != FDIRW_OK) return rc;
-        if ((rc = ensure_parts(c)) != FDIRW_OK) return rc;
         if ((rc = run_graph(c, src, dst, n_steps)) != FDIRW_OK) return rc;
         c->kernels_ready = b.chunks.size() == 1;
     }

@@ -77,14 +77,12 @@ struct MarchArgs {
 // Coarse-mesh march of the blocks a.list[src_begin..src_end): window radius R = window_R + (B - 1) / 2
 // (1..10), one source per CTA.
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st);
+// Mapping 4 of the FP32 march (2x2 column blocks, march_tm.cu), R in 1..10.
+cudaError_t launch_march_blocks(const MarchArgs& a, int num_sms, cudaStream_t st);
 // parts_req: FP32 march thread mapping (1..3 threads per window column, 4 = 2x2 column blocks with TMEM
-// faces, 5 = one column per thread with TMEM lateral faces), or 0 to autotune (timed once per device, R
-// and storage, then cached); parts_used receives the mapping launched.
+// coefficients, 5 = one column per thread with TMEM lateral faces, 6 = source pairs, 7 = column pairs), or 0 for
+// the fastest one of the radius; parts_used receives the mapping launched.
 cudaError_t launch_march(const MarchArgs& a, int num_sms, int parts_req, cudaStream_t st, int* parts_used);
-// The thread mapping launch_march would use for parts_req (timing the candidates on `a`'s sources when
-// autotuning and nothing is cached, which synchronises st and overwrites part of a.Q); launches nothing
-// else, so that the following launches can be captured into a graph.
-cudaError_t tune_march(const MarchArgs& a, int num_sms, int parts_req, cudaStream_t st, int* parts);
 
 // ---------------------------------------------------------------- superpose.cu
 // Padded layout of the scaled field chat = sigma * c: (nx+2R) x (ny+2R) x (nz+2R), zero halo.

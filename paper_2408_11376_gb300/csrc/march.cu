@@ -11,20 +11,14 @@
 //   - the FP64 path (the plain FP64 baseline) keeps u and the diagonal in registers and the face
 //     coefficients in shared memory (FP64 registers would not fit), same exchange scheme;
 //   - after the march each thread rounds its cells to the storage type, writes them into the
-//     destination-indexed cache Q[o][s + o] and sums the stored values in FP64; a fixed-order block
-//     reduction gives sigma_s = 1 / sum.
+//     destination-indexed cache Q[o][s + o] and sums the stored values (FP32 path: as 64-bit integers, FP64
+//     path: in FP64 in a fixed order); sigma_s = 1 / sum.
+// The mapping that runs unless a caller forces another one (2x2 column blocks) is in march_tm.cu.
 // Window cells outside the domain carry no coefficients, so they stay 0; faces leaving the window or
 // the domain have coefficient 0 (zero flux).  Bound: FP32 pipe + shared-memory bandwidth (FP32 path),
 // FP64 pipe (FP64 path).  HBM traffic is only the coefficient loads (L2-resident) and the cache writes.
 #include "fdirw_internal.h"
-
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
-#include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
+#include "march_common.cuh"
 
 namespace fdirw {
 
@@ -58,91 +52,13 @@ struct Map32 {
     static constexpr size_t SMEM = (size_t)((2 * BUF * 4 + 15) / 16) * 16 + (size_t)SPB * COLS * 8;
 };
 
-// Plane of the kernel cache for window cell (x, y, k) of a radius-R window: the cache is laid out for
-// radius a.Rq >= R (offset o = (x - R, y - R, k - R), plane (ox + Rq) + Wq ((oy + Rq) + Wq (oz + Rq))).
-__device__ __forceinline__ int64_t qplane(const MarchArgs& a, int R, int x, int y, int k) {
-    const int Wq = 2 * a.Rq + 1, d = a.Rq - R;
-    return (int64_t)(x + d) + (int64_t)Wq * ((y + d) + (int64_t)Wq * (k + d));
-}
-
-// Structure holding a source: its dimensions and first global cell (a batch concatenates structures;
-// a single grid is structure 0 with base 0).  s becomes the source's index within its structure.
-// qbase: first column of the structure in a destination-indexed cache (s_qbase, or base without it).
-struct SrcLoc {
-    int nx, ny, nz;
-    int64_t base, qbase;
-};
-__device__ __forceinline__ SrcLoc locate(const MarchArgs& a, bool ok, int64_t& s) {
-    SrcLoc L{a.g.nx, a.g.ny, a.g.nz, 0, 0};
-    if (ok && a.nstruct > 0) {
-        int lo = 0, hi = a.nstruct - 1;               // last structure whose first cell is <= s
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(a.s_base + mid) <= s) lo = mid; else hi = mid - 1;
-        }
-        const int4 d = __ldg(a.s_dims + lo);
-        const int64_t b = __ldg(a.s_base + lo);
-        L = SrcLoc{d.x, d.y, d.z, b, a.s_qbase ? __ldg(a.s_qbase + lo) : b};
-        s -= L.base;
-    }
-    return L;
-}
-
-// Column of the kernel cache for a stored value: the destination cell (destination-indexed layout) or
-// the source's position in the launch's source range (source-indexed layout of the radius buckets).
-__device__ __forceinline__ int64_t qcol(const MarchArgs& a, int64_t dest, int64_t pos) {
-    return a.src_major ? pos - a.src_begin : dest;
-}
-
-// Rounds v to the storage type, writes it to Q[idx] and returns the stored value widened to float
-// (exact for every storage type).  Q == nullptr: round only.
-__device__ __forceinline__ float put(void* Q, Store st, int64_t idx, float v) {
-    if (st == Store::F32) {
-        if (Q) reinterpret_cast<float*>(Q)[idx] = v;
-        return v;
-    } else if (st == Store::F16) {
-        const __half h = __float2half_rn(v);
-        if (Q) reinterpret_cast<__half*>(Q)[idx] = h;
-        return __half2float(h);
-    } else {
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        if (Q) reinterpret_cast<__nv_bfloat16*>(Q)[idx] = b;
-        return __bfloat162float(b);
-    }
-}
-
-// Stores the march's value for destination `dest` at `plane` (put), or, for a destination outside the
-// streamed slab, only rounds it to the storage type (sigma still sums it).
-__device__ __forceinline__ float store_q(const MarchArgs& a, int64_t plane, int64_t dest, int64_t pos, float v) {
-    if (a.dest_hi > a.dest_lo) {
-        if (dest < a.dest_lo || dest >= a.dest_hi) return put(nullptr, a.store, 0, v);
-        dest -= a.dest_lo;
-    }
-    return put(a.Q, a.store, plane * a.q_stride + qcol(a, dest, pos), v);
-}
-
-// sigma_s = 1 / (sum of the per-column FP64 partials of slot) for every slot of the batch, fixed order:
-// warp w takes slots w, w + nwarps, ...; lane l sums columns l, l + 32, ...; then a xor-butterfly.
-template <int COLS, int SPB>
-__device__ __forceinline__ void finish_sigma(const double* red, int64_t batch_first, int64_t src_end,
-                                             const int64_t* list, double* sigma) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int slot = warp; slot < SPB; slot += nwarps) {
-        double acc = 0.0;
-        for (int c = lane; c < COLS; c += 32) acc += red[slot * COLS + c];
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        const int64_t s = batch_first + slot;
-        if (lane == 0 && s < src_end) sigma[list ? list[s] : s] = acc > 0.0 ? 1.0 / acc : 0.0;
-    }
-}
-
 template <int R, int P>
 __global__ void __launch_bounds__(Map32<R, P>::THREADS, Map32<R, P>::MIN_BLOCKS) march_f32_kernel(MarchArgs a) {
     using M = Map32<R, P>;
     constexpr int W1 = M::W1, COLS = M::COLS, KS = M::KS, TPS = M::TPS, SPB = M::SPB, BUF = M::BUF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* xbuf = reinterpret_cast<float*>(smem_raw);                                  // [2][SPB*COLS][W1]
-    double* red = reinterpret_cast<double*>(smem_raw + ((2 * BUF * 4 + 15) / 16) * 16);  // [SPB*COLS]
+    int64_t* red = reinterpret_cast<int64_t*>(smem_raw + ((2 * BUF * 4 + 15) / 16) * 16);  // [SPB*COLS]
 
     const int t = threadIdx.x;
     const bool active = t < SPB * TPS;
@@ -264,9 +180,9 @@ __global__ void __launch_bounds__(Map32<R, P>::THREADS, Map32<R, P>::MIN_BLOCKS)
         }
         __syncthreads();
         for (int c = t; c < SPB * COLS; c += blockDim.x) {
-            double colsum = 0.0;
+            int64_t colsum = 0;
 #pragma unroll
-            for (int k = 0; k < W1; k++) colsum += (double)sbuf[c * W1 + k];
+            for (int k = 0; k < W1; k++) colsum += mass_fix(sbuf[c * W1 + k]);
             red[c] = colsum;
         }
         __syncthreads();
@@ -386,345 +302,6 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
 }
 
 // ---------------------------------------------------------------------------------------------------
-// 2x2-block mapping with TMEM-resident coefficients (mapping id 4).
-//
-// Each thread owns a 2x2 block of window columns (4*(2R+1) cells, u in registers), so the halo it
-// exchanges through shared memory per substep drops from 5 to 3 words per cell.  The 12 x/y face
-// coefficients of a block level (and the 4 diagonals, while they fit) no longer fit in registers; they
-// live in Tensor Memory, one TMEM lane per thread, and are streamed back level by level with
-// tcgen05.ld while the previous level computes (TMEM is read at ~2.5x the shared-memory rate on GB300).
-// The z faces and the remaining diagonals stay in registers.  The FP32 operations per cell and their
-// order are the same as in march_f32_kernel, so the results are bitwise identical.
-//
-// One CTA of 256 threads per SM (two threads per TMEM lane, 256 columns each; the CTA allocates all 512
-// columns once and frees them before it exits, and its shared-memory request keeps a second CTA off the
-// SM so an allocation never waits).
-// Where the stored values of one source of a CTA batch go (written by the source's first thread, read by
-// every thread of the CTA in the epilogue).
-struct SlotInfo {
-    int64_t qbase, pos, nxy;
-    int sx, sy, sz, nx, ny, nz, ok, pad;
-};
-
-template <int R>
-struct MapTm {
-    static constexpr int W1 = 2 * R + 1;
-    static constexpr int COLS = W1 * W1;
-    static constexpr int NB = R + 1;                      // blocks per window axis (last one half padding)
-    static constexpr int TPS = NB * NB;                   // threads per source
-    // R <= 8: 256 threads, two per TMEM lane (256 columns each); R = 9, 10: one source of 100 or 121
-    // threads per CTA, one per lane, so that every level's 16 words fit its 512 columns.
-    static constexpr int THREADS = TPS <= 81 ? 256 : 128;
-    static constexpr int TCOLS = THREADS == 256 ? 256 : 512;   // TMEM columns per thread
-    static constexpr int SPB = THREADS / TPS;
-    static constexpr int LEVEL = 4 * THREADS;             // floats per level: [sub-column][thread]
-    static constexpr int BUF = W1 * LEVEL;                // floats per exchange buffer
-    static constexpr int LA0 = (TCOLS - 12 * W1) / 4;
-    static constexpr int LA = LA0 < W1 ? LA0 : W1;        // levels whose diagonals live in TMEM
-    static constexpr int NR = W1 - LA;                    // levels whose diagonals live in registers
-    static constexpr size_t SMEM_USED = (size_t)2 * BUF * 4 + (size_t)SPB * COLS * 8 + (size_t)SPB * sizeof(SlotInfo);
-    static constexpr size_t SMEM = SMEM_USED > 120 * 1024 ? SMEM_USED : 120 * 1024;
-};
-
-__device__ __forceinline__ void tm_st16(uint32_t a, const uint32_t (&v)[16]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
-}
-__device__ __forceinline__ void tm_st8(uint32_t a, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-}
-__device__ __forceinline__ void tm_st4(uint32_t a, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
-                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
-}
-__device__ __forceinline__ void tm_ld16(uint32_t a, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(a));
-}
-__device__ __forceinline__ void tm_ld12(uint32_t a8, uint32_t a4, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(a8));
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]) : "r"(a4));
-}
-// Waits for every outstanding tcgen05.ld of the thread; the registers are in-out operands so that no
-// use of them is scheduled before the wait.
-__device__ __forceinline__ void tm_wait_ld(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :: "memory");
-}
-
-// TMEM word offsets of a block level: levels < LA hold 16 words [12 faces, 4 diagonals] at 16k; the
-// remaining levels hold their 12 faces as 8 words in region A and 4 words in region B (every access is
-// aligned to its width).
-template <int R>
-__device__ __forceinline__ void tm_level_offsets(int k, uint32_t& o16, uint32_t& o8, uint32_t& o4) {
-    using M = MapTm<R>;
-    o16 = (uint32_t)(16 * k);
-    o8 = (uint32_t)(16 * M::LA + 8 * (k - M::LA));
-    o4 = (uint32_t)(16 * M::LA + 8 * M::NR + 4 * (k - M::LA));
-}
-
-template <int R>
-__device__ __forceinline__ void tm_load_level(uint32_t tbase, int k, uint32_t (&r)[16]) {
-    uint32_t o16, o8, o4;
-    tm_level_offsets<R>(k, o16, o8, o4);
-    if (k < MapTm<R>::LA) tm_ld16(tbase + o16, r);
-    else tm_ld12(tbase + o8, tbase + o4, r);
-}
-
-template <int R>
-__global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArgs a) {
-    using M = MapTm<R>;
-    constexpr int W1 = M::W1, COLS = M::COLS, NB = M::NB, TPS = M::TPS, SPB = M::SPB;
-    constexpr int LEVEL = M::LEVEL, PLANE = M::THREADS, BUF = M::BUF, LA = M::LA, NR = M::NR;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* xbuf = reinterpret_cast<float*>(smem_raw);                         // [2][W1][4][256]
-    double* red = reinterpret_cast<double*>(smem_raw + (size_t)2 * BUF * 4);  // [SPB*COLS]
-    SlotInfo* sinfo = reinterpret_cast<SlotInfo*>(red + SPB * COLS);           // [SPB]
-    __shared__ uint32_t s_taddr;
-
-    const int t = threadIdx.x;
-    const int warp = t >> 5;
-    if (warp == 0) {
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_taddr);
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" :: "r"(dst) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t taddr = s_taddr;
-    const uint32_t tbase = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(256 * (warp >> 2));
-
-    const bool active = t < SPB * TPS;
-    const int slot = active ? t / TPS : 0;
-    const int b = active ? t - slot * TPS : 0;
-    const int bi = b % NB, bj = b / NB;
-    // Neighbour blocks; the own index at the window edge (the matching faces are 0) and for idle threads.
-    const int tl = (active && bi > 0) ? t - 1 : t;
-    const int tr = (active && bi < NB - 1) ? t + 1 : t;
-    const int tb = (active && bj > 0) ? t - NB : t;
-    const int tt = (active && bj < NB - 1) ? t + NB : t;
-    const int64_t nbatch = (a.src_end - a.src_begin + SPB - 1) / SPB;
-
-    for (int64_t bt = blockIdx.x; bt < nbatch; bt += gridDim.x) {
-        const int64_t first = a.src_begin + bt * SPB;
-        int64_t s = first + slot;
-        const bool src_ok = active && s < a.src_end;
-        if (src_ok && a.list) s = a.list[s];       // explicit source list (e.g. the surrogate's rejects)
-        const int64_t pos = first + slot;                     // position of the source in the launch range
-        const SrcLoc L = locate(a, src_ok, s);
-        const int nx = L.nx, ny = L.ny, nz = L.nz;
-        const int64_t nxy = (int64_t)nx * ny;
-        const float* ax = a.ax + L.base;   // coefficients of the source's structure
-        const float* ay = a.ay + L.base;
-        const float* az = a.az + L.base;
-        int sx = 0, sy = 0, sz = 0;
-        if (src_ok) {
-            sx = (int)(s % nx);
-            const int64_t r = s / nx;
-            sy = (int)(r % ny);
-            sz = (int)(r / ny);
-        }
-        // Window cell (x, y, k) -> global cell; validity; face coefficients (0 outside window/domain).
-        auto cell_ok = [&](int x, int y, int k) -> bool {
-            const int gx = sx - R + x, gy = sy - R + y, gz = sz - R + k;
-            return src_ok && x >= 0 && x < W1 && y >= 0 && y < W1 && k >= 0 && k < W1 &&
-                   gx >= 0 && gx < nx && gy >= 0 && gy < ny && gz >= 0 && gz < nz;
-        };
-        auto gidx = [&](int x, int y, int k) -> int64_t {
-            return (int64_t)(sx - R + x) + (int64_t)nx * (sy - R + y) + nxy * (sz - R + k);
-        };
-        auto xface = [&](int x, int y, int k) -> float {   // face between window x and x+1
-            return (x + 1 < W1 && cell_ok(x, y, k) && sx - R + x + 1 < nx) ? __ldg(ax + gidx(x, y, k)) : 0.f;
-        };
-        auto yface = [&](int x, int y, int k) -> float {
-            return (y + 1 < W1 && cell_ok(x, y, k) && sy - R + y + 1 < ny) ? __ldg(ay + gidx(x, y, k)) : 0.f;
-        };
-        auto zface = [&](int x, int y, int k) -> float {
-            return (k + 1 < W1 && cell_ok(x, y, k) && sz - R + k + 1 < nz) ? __ldg(az + gidx(x, y, k)) : 0.f;
-        };
-        if (active && b == 0)
-            sinfo[slot] = SlotInfo{L.qbase, pos, nxy, sx, sy, sz, nx, ny, nz, src_ok ? 1 : 0, 0};
-
-        // Registers: state u[sub][k], z faces cz[sub][k] (+z face of the cell), diagonals of the levels
-        // whose TMEM slot has no room for them.  Sub-column sc = sxb + 2*syb at window (2bi+sxb, 2bj+syb).
-        float u[4][W1], cz[4][W1], amr[NR > 0 ? NR : 1][4];
-#pragma unroll
-        for (int sc = 0; sc < 4; sc++) {
-            const int x = 2 * bi + (sc & 1), y = 2 * bj + (sc >> 1);
-#pragma unroll
-            for (int k = 0; k < W1; k++) {
-                cz[sc][k] = zface(x, y, k);
-                u[sc][k] = (src_ok && x == R && y == R && k == R) ? 1.f : 0.f;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < W1; k++) {
-            // faces of the level: rows (syb) for x, columns (sxb) for y
-            float f[16];
-            const int x0 = 2 * bi, y0 = 2 * bj;
-            f[0] = bi > 0 ? xface(x0 - 1, y0, k) : 0.f;       // L0
-            f[1] = xface(x0, y0, k);                           // I0
-            f[2] = xface(x0 + 1, y0, k);                       // R0
-            f[3] = bi > 0 ? xface(x0 - 1, y0 + 1, k) : 0.f;   // L1
-            f[4] = xface(x0, y0 + 1, k);                       // I1
-            f[5] = xface(x0 + 1, y0 + 1, k);                   // R1
-            f[6] = bj > 0 ? yface(x0, y0 - 1, k) : 0.f;       // B0
-            f[7] = yface(x0, y0, k);                           // J0
-            f[8] = yface(x0, y0 + 1, k);                       // T0
-            f[9] = bj > 0 ? yface(x0 + 1, y0 - 1, k) : 0.f;   // B1
-            f[10] = yface(x0 + 1, y0, k);                      // J1
-            f[11] = yface(x0 + 1, y0 + 1, k);                  // T1
-            // diagonals, same association as march_f32_kernel: -(((cxm+cxp)+(cym+cyp))+(czm+czp))
-            const float cxm[4] = {f[0], f[1], f[3], f[4]}, cxp[4] = {f[1], f[2], f[4], f[5]};
-            const float cym[4] = {f[6], f[9], f[7], f[10]}, cyp[4] = {f[7], f[10], f[8], f[11]};
-#pragma unroll
-            for (int sc = 0; sc < 4; sc++) {
-                const float zm = k > 0 ? cz[sc][k - 1] : 0.f;
-                f[12 + sc] = -(((cxm[sc] + cxp[sc]) + (cym[sc] + cyp[sc])) + (zm + cz[sc][k]));
-            }
-            uint32_t w[16];
-#pragma unroll
-            for (int q = 0; q < 16; q++) w[q] = __float_as_uint(f[q]);
-            uint32_t o16, o8, o4;
-            tm_level_offsets<R>(k, o16, o8, o4);
-            if (k < LA) {
-                tm_st16(tbase + o16, w);
-            } else {
-                tm_st8(tbase + o8, w);
-                tm_st4(tbase + o4, w + 8);
-#pragma unroll
-                for (int sc = 0; sc < 4; sc++) amr[(k - LA) < NR ? k - LA : 0][sc] = f[12 + sc];
-            }
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-
-        #pragma unroll(R <= 8 ? 2 : 1)   // two substeps per iteration: no register copies at the back edge
-        for (int it = 0; it < a.n_sub; it++) {
-            float* buf = xbuf + (it & 1) * BUF;
-            if (active) {
-#pragma unroll
-                for (int k = 0; k < W1; k++)
-#pragma unroll
-                    for (int sc = 0; sc < 4; sc++) buf[k * LEVEL + sc * PLANE + t] = u[sc][k];
-            }
-            __syncthreads();
-            // cb[k & 1]: coefficients of level k (ready); cb[(k + 1) & 1]: level k+1, loaded while level k
-            // computes (the loop is unrolled, so the two buffers are fixed registers and nothing is copied).
-            uint32_t cb[2][16];
-            tm_load_level<R>(tbase, 0, cb[0]);
-            tm_wait_ld(cb[0]);
-            float prev[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int k = 0; k < W1; k++) {
-                uint32_t (&cc)[16] = cb[k & 1];
-                uint32_t (&cn)[16] = cb[(k + 1) & 1];
-                if (k + 1 < W1) tm_load_level<R>(tbase, k + 1, cn);
-                const float* lv = buf + k * LEVEL;
-                const float l0 = lv[1 * PLANE + tl], l1 = lv[3 * PLANE + tl];
-                const float r0 = lv[0 * PLANE + tr], r1 = lv[2 * PLANE + tr];
-                const float b0 = lv[2 * PLANE + tb], b1 = lv[3 * PLANE + tb];
-                const float t0 = lv[0 * PLANE + tt], t1 = lv[1 * PLANE + tt];
-                float c[16];
-#pragma unroll
-                for (int q = 0; q < 16; q++) c[q] = __uint_as_float(cc[q]);
-                const float cxm[4] = {c[0], c[1], c[3], c[4]}, cxp[4] = {c[1], c[2], c[4], c[5]};
-                const float cym[4] = {c[6], c[9], c[7], c[10]}, cyp[4] = {c[7], c[10], c[8], c[11]};
-                const float uxm[4] = {l0, u[0][k], l1, u[2][k]}, uxp[4] = {u[1][k], r0, u[3][k], r1};
-                const float uym[4] = {b0, b1, u[0][k], u[1][k]}, uyp[4] = {u[2][k], u[3][k], t0, t1};
-                float nu[4];
-#pragma unroll
-                for (int sc = 0; sc < 4; sc++) {
-                    const float cur = u[sc][k];
-                    const float am = k < LA ? c[12 + sc] : amr[(k - LA) >= 0 ? k - LA : 0][sc];
-                    float v = am * cur;
-                    v = fmaf(cxm[sc], uxm[sc], v);
-                    v = fmaf(cxp[sc], uxp[sc], v);
-                    v = fmaf(cym[sc], uym[sc], v);
-                    v = fmaf(cyp[sc], uyp[sc], v);
-                    v = fmaf(k > 0 ? cz[sc][k > 0 ? k - 1 : 0] : 0.f, prev[sc], v);
-                    v = fmaf(cz[sc][k], k + 1 < W1 ? u[sc][k + 1 < W1 ? k + 1 : k] : 0.f, v);
-                    nu[sc] = __fadd_rn(cur, v);
-                }
-#pragma unroll
-                for (int sc = 0; sc < 4; sc++) { prev[sc] = u[sc][k]; u[sc][k] = nu[sc]; }
-                if (k + 1 < W1) tm_wait_ld(cn);
-            }
-        }
-
-        // Epilogue: round to the storage type, then per-column FP64 sums in k order (same order as
-        // march_f32_kernel) and the cache stores.
-        float* sbuf = xbuf + (a.n_sub & 1) * BUF;
-        if (active) {
-#pragma unroll
-            for (int sc = 0; sc < 4; sc++) {
-                const int x = 2 * bi + (sc & 1), y = 2 * bj + (sc >> 1);
-#pragma unroll
-                for (int k = 0; k < W1; k++) sbuf[k * LEVEL + sc * PLANE + t] = cell_ok(x, y, k) ? put(nullptr, a.store, 0, u[sc][k]) : 0.f;
-            }
-        }
-        __syncthreads();
-        // Stores with the batch's sources fastest: a cell's SPB sources have adjacent destinations in the
-        // same plane, so one warp store covers about 32 / SPB cells instead of 32 planes.  The values are
-        // already rounded, so storing rounds nothing further.
-        for (int w = t; w < SPB * W1 * W1 * W1; w += blockDim.x) {
-            const int sl = w % SPB, c3 = w / SPB;
-            const int x = c3 % W1, y = (c3 / W1) % W1, k = c3 / (W1 * W1);
-            const SlotInfo& si = sinfo[sl];
-            const int gx = si.sx - R + x, gy = si.sy - R + y, gz = si.sz - R + k;
-            if (!si.ok || gx < 0 || gx >= si.nx || gy < 0 || gy >= si.ny || gz < 0 || gz >= si.nz) continue;
-            const float v = sbuf[k * LEVEL + ((x & 1) + 2 * (y & 1)) * PLANE + sl * TPS + (x >> 1) + NB * (y >> 1)];
-            store_q(a, qplane(a, R, x, y, k), si.qbase + gx + (int64_t)si.nx * gy + si.nxy * gz, si.pos, v);
-        }
-        for (int c = t; c < SPB * COLS; c += blockDim.x) {
-            const int sl = c / COLS, cc = c - sl * COLS;
-            const int x = cc % W1, y = cc / W1;
-            const int tt2 = sl * TPS + (x >> 1) + NB * (y >> 1);
-            const int sc = (x & 1) + 2 * (y & 1);
-            double colsum = 0.0;
-#pragma unroll
-            for (int k = 0; k < W1; k++) colsum += (double)sbuf[k * LEVEL + sc * PLANE + tt2];
-            red[c] = colsum;
-        }
-        __syncthreads();
-        finish_sigma<COLS, SPB>(red, first, a.src_end, a.list, a.sigma);
-        __syncthreads();
-    }
-
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(taddr) : "memory");
-}
-
-template <int R>
-cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
-    using M = MapTm<R>;
-    static_assert(M::SPB >= 1, "a source must fit one CTA");
-    const int64_t nsrc = a.src_end - a.src_begin;
-    if (nsrc <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(march_tm_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::SMEM);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_tm_kernel<R>, M::THREADS, M::SMEM);
-    if (e != cudaSuccess) return e;
-    if (per_sm != 1) return cudaErrorInvalidConfiguration;   // TMEM allocation assumes one CTA per SM
-    const int64_t nbatch = (nsrc + M::SPB - 1) / M::SPB;
-    const int64_t grid = nbatch < (int64_t)num_sms ? nbatch : (int64_t)num_sms;
-    march_tm_kernel<R><<<(unsigned)grid, M::THREADS, M::SMEM, st>>>(a);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------------------
 // Column pairs with TMEM-resident faces and diagonals (mapping id 7; any R <= 10, made for R = 9, 10).
 //
 // Each thread owns two x-adjacent window columns (2 (2R+1) cells; the last pair of a window row is half
@@ -773,7 +350,7 @@ __global__ void __launch_bounds__(MapTmx<R>::THREADS, 1) march_tmx_kernel(MarchA
     constexpr int LEVEL = M::LEVEL, PLANE = M::THREADS, BUF = M::BUF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* xbuf = reinterpret_cast<float*>(smem_raw);                         // [2][W1][2][256]
-    double* red = reinterpret_cast<double*>(smem_raw + (size_t)2 * BUF * 4);  // [SPB*COLS]
+    int64_t* red = reinterpret_cast<int64_t*>(smem_raw + (size_t)2 * BUF * 4);  // [SPB*COLS]
     __shared__ uint32_t s_taddr;
 
     const int t = threadIdx.x;
@@ -940,9 +517,9 @@ __global__ void __launch_bounds__(MapTmx<R>::THREADS, 1) march_tmx_kernel(MarchA
             const int x = cc % W1, y = cc / W1;
             const int tt2 = sl * TPS + (x >> 1) + NBX * y;
             const int sc = x & 1;
-            double colsum = 0.0;
+            int64_t colsum = 0;
 #pragma unroll
-            for (int k = 0; k < W1; k++) colsum += (double)sbuf[k * LEVEL + sc * PLANE + tt2];
+            for (int k = 0; k < W1; k++) colsum += mass_fix(sbuf[k * LEVEL + sc * PLANE + tt2]);
             red[c] = colsum;
         }
         __syncthreads();
@@ -1063,7 +640,7 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
     constexpr int W1 = M::W1, COLS = M::COLS, NG = M::NG, BUF = M::BUF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* xbuf = reinterpret_cast<float*>(smem_raw);                                  // [2][COLS][W1]
-    double* red = reinterpret_cast<double*>(smem_raw + ((2 * BUF * 4 + 15) / 16) * 16);  // [COLS]
+    int64_t* red = reinterpret_cast<int64_t*>(smem_raw + ((2 * BUF * 4 + 15) / 16) * 16);  // [COLS]
     __shared__ uint32_t s_taddr;
 
     const int t = threadIdx.x, warp = t >> 5;
@@ -1230,7 +807,7 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
                 }
             }
             __syncthreads();
-            coarse_epilogue<R>(a, sbuf, red + COLS, first);
+            coarse_epilogue<R>(a, sbuf, reinterpret_cast<double*>(red + COLS), first);
         } else {
             if (active) {
 #pragma unroll
@@ -1246,9 +823,9 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
             }
             __syncthreads();
             for (int c = t; c < COLS; c += blockDim.x) {
-                double colsum = 0.0;
+                int64_t colsum = 0;
 #pragma unroll
-                for (int k = 0; k < W1; k++) colsum += (double)sbuf[c * W1 + k];
+                for (int k = 0; k < W1; k++) colsum += mass_fix(sbuf[c * W1 + k]);
                 red[c] = colsum;
             }
             __syncthreads();
@@ -1305,41 +882,13 @@ struct MapTmp {
     static_assert(R <= 8, "mapping 6 covers R <= 8");
 };
 
-__device__ __forceinline__ uint64_t f2pack(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ uint64_t u2pack(uint32_t lo, uint32_t hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ float f2lo(uint64_t v) { return __uint_as_float((uint32_t)(v & 0xffffffffull)); }
-__device__ __forceinline__ float f2hi(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 template <int R>
 __global__ void __launch_bounds__(MapTmp<R>::THREADS, 1) march_tmp_kernel(MarchArgs a) {
     using M = MapTmp<R>;
     constexpr int W1 = M::W1, COLS = M::COLS, NG = M::NG, BUF = M::BUF, PAIRS = M::PAIRS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t* xbuf = reinterpret_cast<uint64_t*>(smem_raw);                        // [2][PAIRS*COLS][W1]
-    double* red = reinterpret_cast<double*>(smem_raw + (size_t)2 * BUF * 8);      // [2*PAIRS][COLS]
+    int64_t* red = reinterpret_cast<int64_t*>(smem_raw + (size_t)2 * BUF * 8);      // [2*PAIRS][COLS]
     __shared__ uint32_t s_taddr;
 
     const int t = threadIdx.x, warp = t >> 5;
@@ -1494,12 +1043,12 @@ __global__ void __launch_bounds__(MapTmp<R>::THREADS, 1) march_tmp_kernel(MarchA
         __syncthreads();
         for (int c = t; c < PAIRS * COLS; c += blockDim.x) {
             const int pr = c / COLS, cl = c - pr * COLS;
-            double s0 = 0.0, s1 = 0.0;
+            int64_t s0 = 0, s1 = 0;
 #pragma unroll
             for (int k = 0; k < W1; k++) {
                 const uint64_t v = sbuf[c * W1 + k];
-                s0 += (double)f2lo(v);
-                s1 += (double)f2hi(v);
+                s0 += mass_fix(f2lo(v));
+                s1 += mass_fix(f2hi(v));
             }
             red[(2 * pr) * COLS + cl] = s0;
             red[(2 * pr + 1) * COLS + cl] = s1;
@@ -1555,7 +1104,7 @@ cudaError_t launch_f32_p(const MarchArgs& a, int P, int num_sms, cudaStream_t st
         case 1: return launch_f32<R, 1>(a, num_sms, st);
         case 2: return launch_f32<R, 2>(a, num_sms, st);
         case 3: return launch_f32<R, 3>(a, num_sms, st);
-        case 4: return launch_tm<R>(a, num_sms, st);
+        case 4: return launch_march_blocks(a, num_sms, st);
         case 5: return a.bx ? launch_tmc<R, false, true>(a, num_sms, st) : launch_tmc<R>(a, num_sms, st);
         case 6: return launch_tmp<R>(a, num_sms, st);
         case 7: return launch_tmx<R>(a, num_sms, st);
@@ -1605,82 +1154,32 @@ cudaError_t dispatch(const MarchArgs& a, int P, int num_sms, cudaStream_t st) {
         case 7: return launch_f32_p<7>(a, P, num_sms, st);
         case 8: return launch_f32_p<8>(a, P, num_sms, st);
         case 9: return P == 5 ? (a.bx ? launch_tmc<9, false, true>(a, num_sms, st) : launch_tmc<9>(a, num_sms, st))
-                       : P == 4 ? launch_tm<9>(a, num_sms, st) : P == 7 ? launch_tmx<9>(a, num_sms, st)
+                       : P == 4 ? launch_march_blocks(a, num_sms, st) : P == 7 ? launch_tmx<9>(a, num_sms, st)
                        : cudaErrorInvalidValue;
         case 10: return P == 5 ? (a.bx ? launch_tmc<10, false, true>(a, num_sms, st) : launch_tmc<10>(a, num_sms, st))
-                        : P == 4 ? launch_tm<10>(a, num_sms, st) : P == 7 ? launch_tmx<10>(a, num_sms, st)
+                        : P == 4 ? launch_march_blocks(a, num_sms, st) : P == 7 ? launch_tmx<10>(a, num_sms, st)
                         : cudaErrorInvalidValue;
         default: return cudaErrorInvalidValue;
     }
 }
 
-// Thread-mapping autotuner (P = threads per window column).  Each candidate is timed once on the
-// context stream over a sample of the real sources (the sample's results are identical whatever P is,
-// and the full launch overwrites them); the fastest is cached per (device, R, storage) for the process.
-std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int>, int> g_tune;
-
-int default_parts(int R) { return R > 8 ? 5 : R >= 4 ? 2 : 1; }
-
-cudaError_t tune_parts(const MarchArgs& a, int num_sms, cudaStream_t st, int* best) {
-    const int W1 = 2 * a.R + 1, cols = W1 * W1;
-    const int64_t per_wave = (int64_t)num_sms * ((512 / cols) > 0 ? 512 / cols : 1);
-    MarchArgs s = a;
-    s.src_end = a.src_begin + std::min<int64_t>(a.src_end - a.src_begin, 16 * per_wave);
-    MarchArgs warm = a;
-    warm.src_end = a.src_begin + std::min<int64_t>(a.src_end - a.src_begin, per_wave);
-    cudaEvent_t e0, e1;
-    cudaError_t e = cudaEventCreate(&e0);
-    if (e != cudaSuccess) return e;
-    e = cudaEventCreate(&e1);
-    if (e != cudaSuccess) { cudaEventDestroy(e0); return e; }
-    float best_ms = 1e30f;
-    *best = default_parts(a.R);
-    for (int P = 1; P <= 7 && e == cudaSuccess; P++) {
-        if (P <= 3 && P > W1) continue;
-        if (a.R > 8 && (P < 4 || P == 6)) continue; // mappings 4, 5 and 7 cover R = 9, 10
-        if (P == 5 && a.R < 6) continue;          // one CTA of < 6 warps per SM: never the fastest there
-        e = dispatch(warm, P, num_sms, st);
-        float ms = 1e30f;
-        for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {      // the faster of two timings
-            float t = 0.f;
-            e = cudaEventRecord(e0, st);
-            if (e == cudaSuccess) e = dispatch(s, P, num_sms, st);
-            if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-            if (e == cudaSuccess && t < ms) ms = t;
-        }
-        if (e == cudaSuccess && ms < best_ms) { best_ms = ms; *best = P; }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    return e;
-}
+// Thread mapping of an FP32 march when the caller does not force one.  Mapping 4 is the fastest at every radius
+// from 2 on (ms for 48^3 sources, BF16 kernels, 100 substeps, mappings 1-7; R = 9, 10 have 4, 5 and 7 only):
+//   R = 2: 1.52 3.77 2.16 1.00 9.27 1.23 1.34    R = 6: 61.5 30.8 31.9 12.4 27.5 18.7 25.5
+//   R = 3: 3.98 9.32 8.76 2.36 11.1 3.26 3.46    R = 8: 48.6 66.5 60.3 26.5 48.1 47.9 67.0
+//   R = 4: 17.4 19.1 21.2 4.42 15.3 6.92 7.47    R = 9: 48.6 (4) 54.6 (5) 74.7 (7)
+//   R = 5: 39.1 43.1 16.8 7.55 17.8 11.5 15.0    R = 10: 54.2 (4) 82.7 (5) 81.8 (7)
+// At R = 1 (27 cells a window) mapping 6 is: 0.42 0.47 0.52 0.36 6.96 0.33 0.39.
+int default_mapping(int R) { return R == 1 ? 6 : 4; }
 
 }  // namespace
 
-cudaError_t tune_march(const MarchArgs& a, int num_sms, int parts_req, cudaStream_t st, int* parts) {
-    if (a.store == Store::F64) { *parts = 1; return cudaSuccess; }
-    if (parts_req >= 1 && parts_req <= 7 && (a.R <= 8 || parts_req == 4 || parts_req == 5 || parts_req == 7)) {
-        *parts = parts_req;
-        return cudaSuccess;
-    }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, a.R, (int)a.store);
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune.find(key);
-        if (it != g_tune.end()) { *parts = it->second; return cudaSuccess; }
-    }
-    int P = 0;
-    cudaError_t e = tune_parts(a, num_sms, st, &P);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[key] = P;
-    *parts = P;
-    return cudaSuccess;
+int march_mapping(const MarchArgs& a, int parts_req) {
+    if (a.store == Store::F64) return 1;
+    if (a.bx) return 5;                           // direction-dependent coefficients: mapping 5 only
+    if (parts_req >= 1 && parts_req <= 7 && (a.R <= 8 || parts_req == 4 || parts_req == 5 || parts_req == 7))
+        return parts_req;
+    return default_mapping(a.R);
 }
 
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st) {
@@ -1700,31 +1199,7 @@ cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStre
 }
 
 cudaError_t launch_march(const MarchArgs& a, int num_sms, int parts_req, cudaStream_t st, int* parts_used) {
-    int P = 1;
-    if (a.bx && a.store != Store::F64) {          // direction-dependent coefficients: mapping 5 only
-        if (parts_used) *parts_used = 5;
-        return dispatch(a, 5, num_sms, st);
-    }
-    if (a.store != Store::F64) {
-        if (parts_req >= 1 && parts_req <= 7 && (a.R <= 8 || parts_req == 4 || parts_req == 5 || parts_req == 7)) {
-            P = parts_req;
-        } else {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            const auto key = std::make_tuple(dev, a.R, (int)a.store);
-            {
-                std::lock_guard<std::mutex> lk(g_tune_mu);
-                auto it = g_tune.find(key);
-                if (it != g_tune.end()) P = it->second; else P = 0;
-            }
-            if (P == 0) {
-                cudaError_t e = tune_parts(a, num_sms, st, &P);
-                if (e != cudaSuccess) return e;
-                std::lock_guard<std::mutex> lk(g_tune_mu);
-                g_tune[key] = P;
-            }
-        }
-    }
+    const int P = march_mapping(a, parts_req);
     if (parts_used) *parts_used = P;
     return dispatch(a, P, num_sms, st);
 }

@@ -1,0 +1,209 @@
+// Helpers shared by the march kernels: where a source lies, where its values go, the rounding to the
+// storage type, the kernel masses, Tensor Memory accesses and packed FP32 pairs.
+#pragma once
+
+#include "fdirw_internal.h"
+
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+namespace fdirw {
+
+namespace {
+
+// Plane of the kernel cache for window cell (x, y, k) of a radius-R window: the cache is laid out for
+// radius a.Rq >= R (offset o = (x - R, y - R, k - R), plane (ox + Rq) + Wq ((oy + Rq) + Wq (oz + Rq))).
+__device__ __forceinline__ int64_t qplane(const MarchArgs& a, int R, int x, int y, int k) {
+    const int Wq = 2 * a.Rq + 1, d = a.Rq - R;
+    return (int64_t)(x + d) + (int64_t)Wq * ((y + d) + (int64_t)Wq * (k + d));
+}
+
+// Structure holding a source: its dimensions and first global cell (a batch concatenates structures;
+// a single grid is structure 0 with base 0).  s becomes the source's index within its structure.
+// qbase: first column of the structure in a destination-indexed cache (s_qbase, or base without it).
+struct SrcLoc {
+    int nx, ny, nz;
+    int64_t base, qbase;
+};
+__device__ __forceinline__ SrcLoc locate(const MarchArgs& a, bool ok, int64_t& s) {
+    SrcLoc L{a.g.nx, a.g.ny, a.g.nz, 0, 0};
+    if (ok && a.nstruct > 0) {
+        int lo = 0, hi = a.nstruct - 1;               // last structure whose first cell is <= s
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(a.s_base + mid) <= s) lo = mid; else hi = mid - 1;
+        }
+        const int4 d = __ldg(a.s_dims + lo);
+        const int64_t b = __ldg(a.s_base + lo);
+        L = SrcLoc{d.x, d.y, d.z, b, a.s_qbase ? __ldg(a.s_qbase + lo) : b};
+        s -= L.base;
+    }
+    return L;
+}
+
+// Coordinates of cell s of a structure nx x ny x nz (32-bit division where it is enough).
+__device__ __forceinline__ void split_cell(int64_t s, int nx, int ny, int& x, int& y, int& z) {
+    if (s <= 0x7fffffff) {
+        const unsigned v = (unsigned)s, r = v / (unsigned)nx;
+        x = (int)(v - r * (unsigned)nx);
+        z = (int)(r / (unsigned)ny);
+        y = (int)(r - (unsigned)z * (unsigned)ny);
+    } else {
+        x = (int)(s % nx);
+        const int64_t r = s / nx;
+        y = (int)(r % ny);
+        z = (int)(r / ny);
+    }
+}
+
+// Column of the kernel cache for a stored value: the destination cell (destination-indexed layout) or
+// the source's position in the launch's source range (source-indexed layout of the radius buckets).
+__device__ __forceinline__ int64_t qcol(const MarchArgs& a, int64_t dest, int64_t pos) {
+    return a.src_major ? pos - a.src_begin : dest;
+}
+
+// Rounds v to the storage type, writes it to Q[idx] and returns the stored value widened to float
+// (exact for every storage type).  Q == nullptr: round only.
+__device__ __forceinline__ float put(void* Q, Store st, int64_t idx, float v) {
+    if (st == Store::F32) {
+        if (Q) reinterpret_cast<float*>(Q)[idx] = v;
+        return v;
+    } else if (st == Store::F16) {
+        const __half h = __float2half_rn(v);
+        if (Q) reinterpret_cast<__half*>(Q)[idx] = h;
+        return __half2float(h);
+    } else {
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        if (Q) reinterpret_cast<__nv_bfloat16*>(Q)[idx] = b;
+        return __bfloat162float(b);
+    }
+}
+
+// Stores the march's value for destination `dest` at `plane` (put), or, for a destination outside the
+// streamed slab, only rounds it to the storage type (sigma still sums it).
+__device__ __forceinline__ float store_q(const MarchArgs& a, int64_t plane, int64_t dest, int64_t pos, float v) {
+    if (a.dest_hi > a.dest_lo) {
+        if (dest < a.dest_lo || dest >= a.dest_hi) return put(nullptr, a.store, 0, v);
+        dest -= a.dest_lo;
+    }
+    return put(a.Q, a.store, plane * a.q_stride + qcol(a, dest, pos), v);
+}
+
+// Kernel masses of the FP32 march: every stored value as a multiple of 2^-60 (exact above 2^-36, rounded to
+// nearest below; a kernel's values are <= 1 and sum to about 1), summed as 64-bit integers.  The total is off
+// by at most W 2^-61 (2e-15 for 17^3 values; 7e-17 for random roundings, an FP64 sum's 1e-16), it does not
+// depend on the order of the sum, and it needs no FP64 instruction per value (1/73 of the FP32 rate here).
+__device__ __forceinline__ int64_t mass_fix(float v) { return __float2ll_rn(v * 0x1p60f); }
+// The same for a run of values without a conversion each (F2I runs at 1/8 of the FP32 rate): v + 6 leaves v's
+// multiples of 2^-21 in the mantissa bits (|v| < 2; a rounded substep can leave a value an ulp below 0 or above 1),
+// the exact rest + 1.5 2^-20 those of 2^-43, and the rest of that + 1.5 2^-37 those of 2^-60 (rounded to nearest,
+// ties as mass_fix).  Up to 500 values.
+struct MassSum {
+    uint32_t s1 = 0, s2 = 0, s3 = 0, n = 0;
+    __device__ __forceinline__ void add(float v) {
+        const float t1 = __fadd_rn(v, 6.f), r1 = __fsub_rn(v, __fsub_rn(t1, 6.f));
+        const float t2 = __fadd_rn(r1, 0x1.8p-20f), r2 = __fsub_rn(r1, __fsub_rn(t2, 0x1.8p-20f));
+        const float t3 = __fadd_rn(r2, 0x1.8p-37f);
+        s1 += __float_as_uint(t1);
+        s2 += __float_as_uint(t2);
+        s3 += __float_as_uint(t3);
+        n++;
+    }
+    __device__ __forceinline__ int64_t total() const {
+        return ((int64_t)(int32_t)(s1 - n * 0x40C00000u) << 39) + ((int64_t)(int32_t)(s2 - n * 0x35C00000u) << 17) +
+               (int64_t)(int32_t)(s3 - n * 0x2D400000u);
+    }
+};
+__device__ __forceinline__ double mass_of(int64_t m) { return (double)m * 0x1p-60; }
+__device__ __forceinline__ double mass_of(double m) { return m; }
+
+// sigma_s = 1 / (sum of the N partials of slot) for every slot of the batch (FP64 partials in a fixed order):
+// warp w takes slots w, w + nwarps, ...; lane l sums partials l, l + 32, ...; then a xor-butterfly.  Z sets of
+// partials lie ZSTRIDE apart.
+template <int N, int SPB, int Z = 1, int ZSTRIDE = 0, typename T>
+__device__ __forceinline__ void finish_sigma(const T* red, int64_t batch_first, int64_t src_end, const int64_t* list,
+                                             double* sigma) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    for (int slot = warp; slot < SPB; slot += nwarps) {
+        T acc = 0;
+        for (int z = 0; z < Z; z++)
+            for (int c = lane; c < N; c += 32) acc += red[z * ZSTRIDE + slot * N + c];
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        const int64_t s = batch_first + slot;
+        if (lane == 0 && s < src_end) sigma[list ? list[s] : s] = acc > 0 ? 1.0 / mass_of(acc) : 0.0;
+    }
+}
+
+__device__ __forceinline__ void tm_st16(uint32_t a, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+__device__ __forceinline__ void tm_st8(uint32_t a, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+__device__ __forceinline__ void tm_st4(uint32_t a, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
+                 :: "r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void tm_ld16(uint32_t a, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(a));
+}
+__device__ __forceinline__ void tm_ld4(uint32_t a, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+// 12 words: 8 at a8, 4 at a4.
+template <int N>
+__device__ __forceinline__ void tm_ld12(uint32_t a8, uint32_t a4, uint32_t (&r)[N]) {
+    static_assert(N >= 12, "room for 12 words");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(a8));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]) : "r"(a4));
+}
+// Waits for every outstanding tcgen05.ld of the thread; the registers are in-out operands so that no
+// use of them is scheduled before the wait.
+__device__ __forceinline__ void tm_wait_ld(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :: "memory");
+}
+
+__device__ __forceinline__ uint64_t f2pack(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ uint64_t u2pack(uint32_t lo, uint32_t hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ float f2lo(uint64_t v) { return __uint_as_float((uint32_t)(v & 0xffffffffull)); }
+__device__ __forceinline__ float f2hi(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+}  // namespace
+
+}  // namespace fdirw
