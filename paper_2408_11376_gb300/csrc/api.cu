@@ -168,9 +168,17 @@ int fdirw::ensure_cache(fdirw_ctx* c) {
             const int rc = dalloc(c, reinterpret_cast<void**>(&c->obuf), obytes, "streamed step output");
             if (rc != FDIRW_OK) return rc;
         }
-        const int rc = dalloc(c, &c->Q, plane * (uint64_t)T, "kernel cache");
+        // Rows padded to whole vectors (padded_row); packed where only those fit, and in a slab, whose every plane
+        // more saves marching sources again (which costs far more than its gather).
+        int qnx = streamed ? c->g.nx : padded_row(c->g.nx, c->store);
+        auto bytes = [&](int row) { return W * (uint64_t)row * (uint64_t)c->g.ny * (uint64_t)T * (uint64_t)store_bytes(c->store); };
+        if (bytes(qnx) > budget) qnx = c->g.nx;
+        int rc = dalloc(c, &c->Q, bytes(qnx), "kernel cache");
+        if (rc == FDIRW_ERR_NOMEM && qnx != c->g.nx) rc = dalloc(c, &c->Q, bytes(qnx = c->g.nx), "kernel cache");
         if (rc == FDIRW_OK) {
-            c->q_bytes = plane * (uint64_t)T;
+            c->q_bytes = bytes(qnx);
+            c->q_nx = qnx;
+            c->q_stride = (int64_t)qnx * c->g.ny * T;
             c->slab_T = streamed ? T : 0;
             if (!streamed && c->obuf) {
                 void* p = c->obuf; dfree(p); c->obuf = nullptr;
@@ -193,7 +201,8 @@ fdirw::MarchArgs fdirw::march_args(const fdirw_ctx* c) {
     a.g = c->g;
     a.R = c->R;
     a.Rq = c->R;
-    a.q_stride = c->g.n;
+    a.q_stride = c->q_stride;
+    a.q_vec = c->q_nx > c->g.nx ? 16 / store_bytes(c->store) : 1;
     a.n_sub = c->n_sub;
     if (c->store == Store::F64) {
         a.dx = reinterpret_cast<const double*>(c->coef[0]);
@@ -232,7 +241,6 @@ int fdirw::step_slabs(fdirw_ctx* c, const double* src, double* dst, int n_steps)
         FDIRW_CUDA(c, cudaMemsetAsync(c->dfix + 2, 0, 8, c->stream));
     }
     MarchArgs a = march_args(c);
-    a.q_stride = (int64_t)T * nxy;
     const double* cur = src;
     for (int t = 0; t < n_steps; t++) {
         // The step writes a buffer other than its input; the last one lands in dst unless dst is the input.
@@ -243,12 +251,12 @@ int fdirw::step_slabs(fdirw_ctx* c, const double* src, double* dst, int n_steps)
             const int zs0 = std::max(z0 - R, 0), zs1 = std::min(z0 + zn + R, nz);
             a.src_begin = (int64_t)zs0 * nxy;
             a.src_end = (int64_t)zs1 * nxy;
-            a.dest_lo = (int64_t)z0 * nxy;
-            a.dest_hi = (int64_t)(z0 + zn) * nxy;
+            a.dest_z0 = z0;
+            a.dest_z1 = z0 + zn;
             FDIRW_CUDA(c, launch_march(a, c->num_sms, c->parts_req, c->stream, &c->parts_used));
             FDIRW_CUDA(c, launch_scale(cur, c->sigma, c->g, R, c->chat, mode, c->stream, zs0, zs1 - zs0));
-            FDIRW_CUDA(c, launch_gather_slab(c->Q, c->store, (int64_t)T * nxy, a.dest_lo, c->chat, c->g, R, mode, z0,
-                                             zn, out, c->stream));
+            FDIRW_CUDA(c, launch_gather_slab(c->Q, c->store, c->q_stride, c->q_nx, c->chat, c->g, R, mode, z0, zn, out,
+                                             c->stream));
         }
         if (fp32acc) FDIRW_CUDA(c, fdirw::launch_restore_mass(out, c->g.n, c->partials, c->dfix, c->stream));
         cur = out;
@@ -450,12 +458,8 @@ int fdirw_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps,
             FDIRW_CUDA(c, fdirw::launch_scale(cur, c->sigma, c->g, c->R, c->chat, mode, c->stream));
             const bool last = t + 1 == n_steps;
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
-            if (fp32acc) {
-                FDIRW_CUDA(c, fdirw::launch_gather_fp32(c->Q, c->store, reinterpret_cast<const float*>(c->chat), c->g,
-                                                        c->R, dst, c->stream));
-            } else {
-                FDIRW_CUDA(c, fdirw::launch_gather(c->Q, c->store, c->chat, c->g, c->R, dst, c->stream));
-            }
+            FDIRW_CUDA(c, fdirw::launch_gather_slab(c->Q, c->store, c->q_stride, c->q_nx, c->chat, c->g, c->R, mode, 0,
+                                                    c->g.nz, dst, c->stream));
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
             if (fp32acc) FDIRW_CUDA(c, fdirw::launch_restore_mass(dst, c->g.n, c->partials, c->dfix, c->stream));
             cur = dst;
@@ -523,7 +527,7 @@ int fdirw_read_kernels(fdirw_ctx* c, const int64_t* sources, int64_t n, double* 
         c->kcap = n;
     }
     FDIRW_CUDA(c, cudaMemcpyAsync(c->dsrc, sources, (size_t)n * 8, cudaMemcpyHostToDevice, c->stream));
-    FDIRW_CUDA(c, fdirw::launch_read_kernels(c->Q, c->store, c->sigma, c->g, c->R, c->dsrc, n, c->dkout, c->stream));
+    FDIRW_CUDA(c, fdirw::launch_read_kernels(c->Q, c->store, c->q_stride, c->q_nx, c->sigma, c->g, c->R, c->dsrc, n, c->dkout, c->stream));
     FDIRW_CUDA(c, cudaMemcpyAsync(out, c->dkout, (size_t)(n * W) * 8, cudaMemcpyDeviceToHost, c->stream));
     FDIRW_CUDA(c, cudaStreamSynchronize(c->stream));
     return FDIRW_OK;

@@ -77,6 +77,7 @@ struct Batch {
     uint32_t dest_mask = 0;                      // bit r: radius r uses the destination-indexed layout
     std::vector<int64_t> qbase;                  // n: first cache column of each structure within its chunk
     int64_t* d_qbase = nullptr;
+    int qvec = 1;                                // destination-indexed cache rows are padded to a multiple of this
     std::vector<int64_t> pbase;                  // n + 1: first element of each structure's padded chat
     float2* chat_pad = nullptr;                  // sigma * c with a halo of R_max (destination-indexed radii)
     double* seg_part = nullptr;                  // FDIRW_ACCUM_FP32: 2 * kSegBlocks partial sums per structure
@@ -144,6 +145,7 @@ struct VarArgs {
     uint32_t dmask;                              // bit r set: radius r is destination-indexed
     bool acc_in;                                 // add to out instead of overwriting it
     const int64_t* qbase;
+    int qvec;                                    // destination-indexed rows are padded to this many values
     const void* K[kMaxR + 1];
     int64_t jbase[kMaxR + 1];
     int64_t ncol[kMaxR + 1];
@@ -253,7 +255,7 @@ __global__ void read_var_kernel(VarArgs a, const double* __restrict__ sigma, int
                 const int W1 = 2 * r + 1;
                 const int64_t plane = (ox + r) + (int64_t)W1 * ((oy + r) + (int64_t)W1 * (oz + r));
                 const ST* K = reinterpret_cast<const ST*>(a.K[r]);
-                const int64_t col = (a.dmask >> r) & 1u ? a.qbase[lo] + x + (int64_t)d.x * (y + (int64_t)d.y * z)
+                const int64_t col = (a.dmask >> r) & 1u ? a.qbase[lo] + x + (int64_t)(a.qvec > 1 ? (d.x + a.qvec - 1) / a.qvec * a.qvec : d.x) * (y + (int64_t)d.y * z)
                                                         : (int64_t)(code & kCodeMask) - a.jbase[r];
                 v = (double)widen(K[plane * a.ncol[r] + col]) * sigma[s];
             }
@@ -270,6 +272,9 @@ int grid_blocks(int64_t n, int threads) {
 
 // ------------------------------------------------------------------------------------------ host
 
+// Values of a destination-indexed cache row of structure i.
+int row_of(const Batch& b, int i) { return (b.grids[i].nx + b.qvec - 1) / b.qvec * b.qvec; }
+
 VarArgs var_args(const fdirw_ctx* c, const Chunk& ch, double* out) {
     const Batch& b = *c->batch;
     VarArgs a{};
@@ -285,6 +290,7 @@ VarArgs var_args(const fdirw_ctx* c, const Chunk& ch, double* out) {
     a.dmask = b.dest_mask;
     a.acc_in = false;
     a.qbase = b.d_qbase;
+    a.qvec = b.qvec;
     for (int r : b.radii) {
         const bool dest = (b.dest_mask >> r) & 1u;
         if (!dest) a.rmask |= 1u << r;
@@ -321,6 +327,7 @@ MarchArgs march_args(const fdirw_ctx* c, const Chunk& ch, int r) {
     a.s_dims = b.d_dims;
     if ((b.dest_mask >> r) & 1u) {
         a.s_qbase = b.d_qbase;
+        a.q_vec = b.qvec;
         a.q_stride = ch.qn;
         a.src_major = 0;
     } else {
@@ -413,11 +420,8 @@ cudaError_t step_chunk(fdirw_ctx* c, int ci, const double* src, double* dst, int
                 for (int r : b.radii) {
                     if (r == 0 || !((b.dest_mask >> r) & 1u)) continue;
                     const void* Q = static_cast<const char*>(a.K[r]) + (size_t)b.qbase[i] * sb;
-                    e = fp32acc ? launch_gather_part_fp32(Q, c->store, ch.qn,
-                                                          reinterpret_cast<const float*>(b.chat_pad + b.pbase[i]), Rm,
-                                                          b.grids[i], r, w, dst + b.base[i], sx)
-                                : launch_gather_part(Q, c->store, ch.qn, b.chat_pad + b.pbase[i], Rm, b.grids[i], r, w,
-                                                     dst + b.base[i], sx);
+                    e = launch_gather_part(Q, c->store, ch.qn, row_of(b, i), b.chat_pad + b.pbase[i], Rm, b.grids[i], r,
+                                           fp32acc ? 2 : 1, w, dst + b.base[i], sx);
                     if (e != cudaSuccess) break;
                     w = true;
                 }
@@ -901,7 +905,9 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
 
     // Chunks: consecutive structures whose kernels fit the budget together.
     const int sb = fdirw::store_bytes(c->store);
-    auto slot = [&](int i) { return (b.grids[i].n + 15) / 16 * 16; };   // 16-aligned destination columns
+    auto slot = [&](int i) {                                            // 16-aligned destination columns
+        return ((int64_t)fdirw::row_of(b, i) * b.grids[i].ny * b.grids[i].nz + 15) / 16 * 16;
+    };
     auto struct_bytes = [&](int i, int r) -> uint64_t {
         if (r == 0) return 0;
         const int64_t cols = (b.dest_mask >> r) & 1u ? slot(i) : b.before[r][i + 1] - b.before[r][i];
@@ -918,14 +924,23 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
         budget = fr > reserve ? fr - reserve : 0;
     }
     budget = budget > 256ull * (fdirw::kMaxR + 1) ? budget - 256ull * (fdirw::kMaxR + 1) : 0;
+    auto all_radii = [&](int i) {
+        uint64_t add = 0;
+        for (int r : b.radii) add += struct_bytes(i, r);
+        return add;
+    };
+    // Cache rows of whole vectors (as in a uniform context), unless a structure is too narrow for it or its kernels
+    // then no longer fit the budget.
+    b.qvec = 16 / sb;
+    for (int i = 0; i < n; i++)
+        if (b.grids[i].nx < 16 / sb || all_radii(i) > budget) { b.qvec = 1; break; }
     int i = 0;
     while (i < n) {
         Chunk ch;
         ch.s0 = i;
         uint64_t used = 0;
         while (i < n) {
-            uint64_t add = 0;
-            for (int r : b.radii) add += struct_bytes(i, r);
+            const uint64_t add = all_radii(i);
             if (used + add > budget && i > ch.s0) break;
             if (used + add > budget) {
                 c->err = "the kernels of structure " + std::to_string(i) + " (" + std::to_string(add) +

@@ -31,6 +31,8 @@ struct fdirw_ctx {
     bool flow = false;                              // coef / coefb hold direction-dependent coefficients
     void* Q = nullptr;
     uint64_t q_bytes = 0;
+    int64_t q_stride = 0;                           // values from one plane of Q to the next
+    int q_nx = 0;                                   // values of a cache row (nx, or padded to whole vectors)
     double* sigma = nullptr;
     void* chat = nullptr;                           // padded sigma*c: double or float2
     double* cbuf = nullptr;                         // staging for host fields

@@ -53,12 +53,13 @@ struct MarchArgs {
     int nstruct;
     const int64_t* s_base;
     const int4* s_dims;
-    const int64_t* s_qbase;   // nullable: first cache column of each structure (destination-indexed layout)
+    const int64_t* s_qbase;   // nullable: first cache column of each structure (destination-indexed layout; 0 without it)
     // Q index = plane * q_stride + column; the column is the destination cell (src_major = 0: the cell's
-    // index within its structure plus s_qbase, or the global cell without s_qbase) or the source's
+    // index within its structure, x rows padded to a multiple of q_vec values, plus s_qbase) or the source's
     // position in [src_begin, src_end) (src_major = 1).
     int64_t q_stride;
     int src_major;
+    int q_vec;
     // Coarse-mesh march (coarse_B > 0, mapping 5 only): list holds coarse block indices; see coarse.cu.
     int coarse_B, coarse_Rc;
     int ncx, ncy, ncz;
@@ -70,9 +71,9 @@ struct MarchArgs {
     // Convection (nullable; mapping 5 only): ax/ay/az then hold the coefficient of the lower cell in the
     // upper cell's update across each +face, bx/by/bz that of the upper cell in the lower cell's update.
     const float* bx; const float* by; const float* bz;
-    // Slab streaming of a uniform context (dest_hi > dest_lo): only destinations in [dest_lo, dest_hi)
-    // are stored, at column dest - dest_lo; the others are rounded (for sigma) but not stored.
-    int64_t dest_lo, dest_hi;
+    // Slab streaming of a uniform context (dest_z1 > dest_z0): only destinations of the z-planes [dest_z0, dest_z1)
+    // are stored, from column 0 on; the others are rounded (for sigma) but not stored.
+    int dest_z0, dest_z1;
 };
 // Coarse-mesh march of the blocks a.list[src_begin..src_end): window radius R = window_R + (B - 1) / 2
 // (1..10), one source per CTA.
@@ -100,32 +101,31 @@ inline Pad make_pad(const Grid& g, int R) {
 // [z0, z0 + zn) only (zn < 0: all planes).
 cudaError_t launch_scale(const double* c, const double* sigma, Grid g, int R, void* chat, int mode,
                          cudaStream_t st, int z0 = 0, int zn = -1);
-// c_out(x) = sum_o Q[o][x] * chat(x - o).
-cudaError_t launch_gather(const void* Q, Store store, const void* chat, Grid g, int R, double* c_out,
-                          cudaStream_t st);
+// Cache rows: the destinations of an x row take qnx >= nx values, whole 16-byte vectors of the storage type where
+// that is at most twice nx and fits; the values past nx are never stored.  (Padded rows against packed ones read value
+// by value, 97 x 101 x 89, R = 8, us a step: BF16 cache and FP32 sums 1392 against 5477, FP32 cache and float-float
+// sums 2723 against 6733.)
+inline int padded_row(int nx, Store s) {
+    const int vx = 16 / store_bytes(s);
+    return nx < vx ? nx : (nx + vx - 1) / vx * vx;
+}
 // The radius-R part of the gather for one grid whose chat is padded with a halo of Rp >= R cells and
-// whose Q planes are qs values apart: c_out(x) = [c_out(x) +] sum_{|o| <= R} Q[o][x] * chat(x - o), the
-// rows (o_z, o_y) in ascending order as in launch_gather.
-cudaError_t launch_gather_part(const void* Q, Store store, int64_t qs, const void* chat, int Rp, Grid g, int R,
-                               bool accumulate, double* c_out, cudaStream_t st);
+// whose Q planes are qs values apart: c_out(x) = [c_out(x) +] sum_{|o| <= R} Q[o][x] * chat(x - o), mode 0 FP64, 1
+// float-float, 2 FP32 arithmetic; the rows (o_z, o_y) in ascending order (FP32), or so within each of a few row groups
+// and the groups in ascending order.
+cudaError_t launch_gather_part(const void* Q, Store store, int64_t qs, int qnx, const void* chat, int Rp, Grid g, int R,
+                               int mode, bool accumulate, double* c_out, cudaStream_t st);
 // Deterministic FP64 total: partials[kMassBlocks] then one block.  partials must hold kMassBlocks doubles.
 constexpr int kMassBlocks = 1024;
 cudaError_t launch_mass(const double* c, int64_t n, double* partials, double* out, cudaStream_t st);
-// FDIRW_ACCUM_FP32 superposition of a uniform context: FP32 chat (launch_scale mode 2), FP32 products
-// and row sums, double-float row accumulation.
-cudaError_t launch_gather_fp32(const void* Q, Store store, const float* chat, Grid g, int R, double* c_out,
-                               cudaStream_t st);
 // Restores the FP64 total of c to *m_in: c[i] += f |c[i]|, f = (m_in - sum c) / sum |c| (0 when the
 // field is zero), both sums in a fixed order.  partials: 2 * kMassBlocks doubles; fix: 2 doubles
 // (fix[0] = m_in on entry, fix[1] = f on exit).
 cudaError_t launch_restore_mass(double* c, int64_t n, double* partials, double* fix, cudaStream_t st);
-// The destinations of the z-planes [z0, z0 + zn) of a uniform context whose cache holds only those
-// destinations (column = cell - qoff, plane stride qs): mode 0 FP64, 1 float-float, 2 FP32 arithmetic.
-cudaError_t launch_gather_slab(const void* Q, Store store, int64_t qs, int64_t qoff, const void* chat, Grid g, int R,
+// The destinations of the z-planes [z0, z0 + zn) of a uniform context whose cache starts at plane z0 (the whole cache:
+// 0, nz).
+cudaError_t launch_gather_slab(const void* Q, Store store, int64_t qs, int qnx, const void* chat, Grid g, int R,
                                int mode, int z0, int zn, double* c_out, cudaStream_t st);
-// launch_gather_part with the FDIRW_ACCUM_FP32 arithmetic (FP32 chat with a halo of Rp).
-cudaError_t launch_gather_part_fp32(const void* Q, Store store, int64_t qs, const float* chat, int Rp, Grid g, int R,
-                                    bool accumulate, double* c_out, cudaStream_t st);
 // Per-structure mass restoration of structures [s0, s1) whose cells are [base[i], base[i + 1]) (base on
 // the device): launch_seg_target stores each structure's FP64 total of c in fix[2 i]; launch_seg_restore
 // then adds f_i |c| to every cell of structure i, f_i = (fix[2 i] - sum c) / sum |c|.  partials holds
@@ -135,8 +135,8 @@ cudaError_t launch_seg_target(const double* c, const int64_t* base, int s0, int 
                               cudaStream_t st);
 cudaError_t launch_seg_restore(double* c, const int64_t* base, int s0, int s1, double* partials, double* fix,
                                cudaStream_t st);
-// Renormalised kernels of listed sources on the (2R+1)^3 offset layout.
-cudaError_t launch_read_kernels(const void* Q, Store store, const double* sigma, Grid g, int R,
+// Renormalised kernels of listed sources on the (2R+1)^3 offset layout (planes qs, rows qnx values apart).
+cudaError_t launch_read_kernels(const void* Q, Store store, int64_t qs, int qnx, const double* sigma, Grid g, int R,
                                 const int64_t* sources, int64_t n_src, double* out, cudaStream_t st);
 
 }  // namespace fdirw

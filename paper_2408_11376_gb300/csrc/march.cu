@@ -170,10 +170,7 @@ __global__ void __launch_bounds__(Map32<R, P>::THREADS, Map32<R, P>::MIN_BLOCKS)
                     const int k = k0 + j;
                     const int z = sz - R + k;
                     float st = 0.f;
-                    if (col_ok && z >= 0 && z < nz) {
-                        const int64_t i = (int64_t)x + (int64_t)nx * y + nxy * z;
-                        st = store_q(a, qplane(a, R, ci, cj, k), L.qbase + i, pos, u[j]);
-                    }
+                    if (col_ok && z >= 0 && z < nz) st = store_q(a, L, qplane(a, R, ci, cj, k), x, y, z, pos, u[j]);
                     sbuf[base + k] = st;
                 }
             }
@@ -210,6 +207,8 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
     const int ci = col % W1, cj = col / W1;
     const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
     const int64_t nxy = (int64_t)nx * ny;
+    int64_t none = 0;
+    const SrcLoc L = locate(a, false, none);
     const int64_t nbatch = (a.src_end - a.src_begin + SPB - 1) / SPB;
 
     const int base = (slot * COLS + col) * W1;
@@ -287,9 +286,8 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
             for (int k = 0; k < W1; k++) {
                 const int z = sz - R + k;
                 if (z >= 0 && z < nz) {
-                    const int64_t i = (int64_t)x + (int64_t)nx * y + nxy * z;
-                    if (a.dest_hi <= a.dest_lo || (i >= a.dest_lo && i < a.dest_hi))
-                        reinterpret_cast<double*>(a.Q)[qplane(a, R, ci, cj, k) * a.q_stride + (i - a.dest_lo)] = u[k];
+                    if (a.dest_z1 <= a.dest_z0 || (z >= a.dest_z0 && z < a.dest_z1))
+                        reinterpret_cast<double*>(a.Q)[qplane(a, R, ci, cj, k) * a.q_stride + qcol(a, L, x, y, z, 0)] = u[k];
                     colsum += u[k];
                 }
             }
@@ -506,7 +504,7 @@ __global__ void __launch_bounds__(MapTmx<R>::THREADS, 1) march_tmx_kernel(MarchA
 #pragma unroll
                 for (int k = 0; k < W1; k++) {
                     float stv = 0.f;
-                    if (cell_ok(x, y, k)) stv = store_q(a, qplane(a, R, x, y, k), L.qbase + gidx(x, y, k), pos, u[sc][k]);
+                    if (cell_ok(x, y, k)) stv = store_q(a, L, qplane(a, R, x, y, k), sx - R + x, sy - R + y, sz - R + k, pos, u[sc][k]);
                     sbuf[k * LEVEL + sc * PLANE + t] = stv;
                 }
             }
@@ -814,10 +812,7 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
                 for (int k = 0; k < W1; k++) {
                     const int z = sz - R + k;
                     float stv = 0.f;
-                    if (col_ok && z >= 0 && z < nz) {
-                        const int64_t i = (int64_t)x + (int64_t)nx * y + nxy * z;
-                        stv = store_q(a, qplane(a, R, ci, cj, k), L.qbase + i, pos, u[k]);
-                    }
+                    if (col_ok && z >= 0 && z < nz) stv = store_q(a, L, qplane(a, R, ci, cj, k), x, y, z, pos, u[k]);
                     sbuf[base + k] = stv;
                 }
             }
@@ -920,7 +915,8 @@ __global__ void __launch_bounds__(MapTmp<R>::THREADS, 1) march_tmp_kernel(MarchA
         int64_t pos[2], sidx[2];
         bool src_ok[2], col_ok[2];
         int sx[2], sy[2], sz[2], xs[2], ys[2], nzs[2], nxs[2], nys[2];
-        int64_t nxy[2], cbase[2], qb[2];
+        int64_t nxy[2], cbase[2];
+        SrcLoc Ls[2];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             pos[h] = first + 2 * pair + h;
@@ -931,7 +927,7 @@ __global__ void __launch_bounds__(MapTmp<R>::THREADS, 1) march_tmp_kernel(MarchA
             nxs[h] = L.nx; nys[h] = L.ny; nzs[h] = L.nz;
             nxy[h] = (int64_t)L.nx * L.ny;
             cbase[h] = L.base;
-            qb[h] = L.qbase;
+            Ls[h] = L;
             sidx[h] = s;
             sx[h] = sy[h] = sz[h] = 0;
             if (src_ok[h]) {
@@ -1033,8 +1029,7 @@ __global__ void __launch_bounds__(MapTmp<R>::THREADS, 1) march_tmp_kernel(MarchA
                     const int z = sz[h] - R + k;
                     stv[h] = 0.f;
                     if (col_ok[h] && z >= 0 && z < nzs[h]) {
-                        const int64_t i = (int64_t)xs[h] + (int64_t)nxs[h] * ys[h] + nxy[h] * z;
-                        stv[h] = store_q(a, qplane(a, R, ci, cj, k), qb[h] + i, pos[h], h == 0 ? f2lo(u[k]) : f2hi(u[k]));
+                        stv[h] = store_q(a, Ls[h], qplane(a, R, ci, cj, k), xs[h], ys[h], z, pos[h], h == 0 ? f2lo(u[k]) : f2hi(u[k]));
                     }
                 }
                 sbuf[base + k] = f2pack(stv[0], stv[1]);

@@ -20,13 +20,13 @@ __device__ __forceinline__ int64_t qplane(const MarchArgs& a, int R, int x, int 
 
 // Structure holding a source: its dimensions and first global cell (a batch concatenates structures;
 // a single grid is structure 0 with base 0).  s becomes the source's index within its structure.
-// qbase: first column of the structure in a destination-indexed cache (s_qbase, or base without it).
+// qbase, qnx: first column of the structure in a destination-indexed cache and the values that an x row takes there.
 struct SrcLoc {
-    int nx, ny, nz;
+    int nx, ny, nz, qnx;
     int64_t base, qbase;
 };
 __device__ __forceinline__ SrcLoc locate(const MarchArgs& a, bool ok, int64_t& s) {
-    SrcLoc L{a.g.nx, a.g.ny, a.g.nz, 0, 0};
+    SrcLoc L{a.g.nx, a.g.ny, a.g.nz, 0, 0, 0};
     if (ok && a.nstruct > 0) {
         int lo = 0, hi = a.nstruct - 1;               // last structure whose first cell is <= s
         while (lo < hi) {
@@ -35,9 +35,10 @@ __device__ __forceinline__ SrcLoc locate(const MarchArgs& a, bool ok, int64_t& s
         }
         const int4 d = __ldg(a.s_dims + lo);
         const int64_t b = __ldg(a.s_base + lo);
-        L = SrcLoc{d.x, d.y, d.z, b, a.s_qbase ? __ldg(a.s_qbase + lo) : b};
+        L = SrcLoc{d.x, d.y, d.z, 0, b, a.s_qbase ? __ldg(a.s_qbase + lo) : 0};
         s -= L.base;
     }
+    L.qnx = a.q_vec > 1 ? (L.nx + a.q_vec - 1) / a.q_vec * a.q_vec : L.nx;
     return L;
 }
 
@@ -56,10 +57,11 @@ __device__ __forceinline__ void split_cell(int64_t s, int nx, int ny, int& x, in
     }
 }
 
-// Column of the kernel cache for a stored value: the destination cell (destination-indexed layout) or
-// the source's position in the launch's source range (source-indexed layout of the radius buckets).
-__device__ __forceinline__ int64_t qcol(const MarchArgs& a, int64_t dest, int64_t pos) {
-    return a.src_major ? pos - a.src_begin : dest;
+// Column of the kernel cache for a stored value: that of destination cell (x, y, z) of the structure
+// (destination-indexed layout) or the source's position in the launch's source range (source-indexed layout of the
+// radius buckets).
+__device__ __forceinline__ int64_t qcol(const MarchArgs& a, const SrcLoc& L, int x, int y, int z, int64_t pos) {
+    return a.src_major ? pos - a.src_begin : L.qbase + x + (int64_t)L.qnx * (y + (int64_t)L.ny * (z - a.dest_z0));
 }
 
 // Rounds v to the storage type, writes it to Q[idx] and returns the stored value widened to float
@@ -79,14 +81,12 @@ __device__ __forceinline__ float put(void* Q, Store st, int64_t idx, float v) {
     }
 }
 
-// Stores the march's value for destination `dest` at `plane` (put), or, for a destination outside the
-// streamed slab, only rounds it to the storage type (sigma still sums it).
-__device__ __forceinline__ float store_q(const MarchArgs& a, int64_t plane, int64_t dest, int64_t pos, float v) {
-    if (a.dest_hi > a.dest_lo) {
-        if (dest < a.dest_lo || dest >= a.dest_hi) return put(nullptr, a.store, 0, v);
-        dest -= a.dest_lo;
-    }
-    return put(a.Q, a.store, plane * a.q_stride + qcol(a, dest, pos), v);
+// Stores the march's value for destination (x, y, z) at `plane` (put), or, for a destination outside the streamed
+// slab, only rounds it to the storage type (sigma still sums it).
+__device__ __forceinline__ float store_q(const MarchArgs& a, const SrcLoc& L, int64_t plane, int x, int y, int z,
+                                         int64_t pos, float v) {
+    if (a.dest_z1 > a.dest_z0 && (z < a.dest_z0 || z >= a.dest_z1)) return put(nullptr, a.store, 0, v);
+    return put(a.Q, a.store, plane * a.q_stride + qcol(a, L, x, y, z, pos), v);
 }
 
 // Kernel masses of the FP32 march: every stored value as a multiple of 2^-60 (exact above 2^-36, rounded to

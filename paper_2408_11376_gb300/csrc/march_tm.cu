@@ -43,8 +43,9 @@ namespace {
 // Where the stored values of one source of a CTA batch go (written by the source's first thread, read by
 // every thread of the CTA in the epilogue).
 struct SlotInfo {
-    int64_t qbase, pos, nxy;
-    int sx, sy, sz, nx, ny, nz, ok, pad;
+    SrcLoc L;
+    int64_t pos;
+    int sx, sy, sz, ok;
 };
 
 template <int R>
@@ -163,7 +164,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
         int sx = 0, sy = 0, sz = 0;
         if (src_ok) split_cell(s, nx, ny, sx, sy, sz);
         if (active && b == 0 && K0 == 0)
-            sinfo[slot] = SlotInfo{L.qbase, pos, nxy, sx, sy, sz, nx, ny, nz, src_ok ? 1 : 0, 0};
+            sinfo[slot] = SlotInfo{L, pos, sx, sy, sz, src_ok ? 1 : 0};
 
         // A face is stored with its lower cell and taken when that cell is in the domain and both cells are in
         // the window and the domain (0 otherwise).  All but the z range is fixed per thread, so the 16 faces
@@ -411,16 +412,15 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
             const int c = e / SPB, sl = e - c * SPB, y = c / W1, x = c - y * W1;
             const SlotInfo si = sinfo[sl];
             const int cx = si.sx - R + x, cy = si.sy - R + y, z0 = si.sz - R;
-            if (!si.ok || !in(cx, si.nx) || !in(cy, si.ny)) continue;
-            int k0 = z0 < 0 ? -z0 : 0, k1 = si.nz - z0 < W1 ? si.nz - z0 : W1;      // levels in the domain
-            int64_t dest = si.qbase + cx + (int64_t)si.nx * cy + si.nxy * z0;       // of level 0
-            if (a.dest_hi > a.dest_lo) {           // slab of whole z-planes: only its levels are stored
-                k0 = max(k0, (int)(a.dest_lo / si.nxy) - z0);
-                k1 = min(k1, (int)(a.dest_hi / si.nxy) - z0);
-                dest -= a.dest_lo;
+            if (!si.ok || !in(cx, si.L.nx) || !in(cy, si.L.ny)) continue;
+            int k0 = z0 < 0 ? -z0 : 0, k1 = si.L.nz - z0 < W1 ? si.L.nz - z0 : W1;  // levels in the domain
+            if (a.dest_z1 > a.dest_z0) {           // slab of z-planes: only its levels are stored
+                k0 = max(k0, a.dest_z0 - z0);
+                k1 = min(k1, a.dest_z1 - z0);
             }
-            int64_t at = qplane(a, R, x, y, 0) * a.q_stride + qcol(a, dest, si.pos);
-            const int64_t step = qplane(a, R, 0, 0, 1) * a.q_stride - qplane(a, R, 0, 0, 0) * a.q_stride + (a.src_major ? 0 : si.nxy);
+            const int64_t at = qplane(a, R, x, y, 0) * a.q_stride + qcol(a, si.L, cx, cy, z0, si.pos);   // of level 0
+            const int64_t step = (qplane(a, R, 0, 0, 1) - qplane(a, R, 0, 0, 0)) * a.q_stride +
+                                 (a.src_major ? 0 : (int64_t)si.L.qnx * si.L.ny);
             const int sc = (x & 1) + 2 * (y & 1), own = sl * TPS + (x >> 1) + NB * (y >> 1);
             if (a.store == Store::F32) {
                 float* q = reinterpret_cast<float*>(a.Q) + at;

@@ -3,9 +3,9 @@
 //     chat(s)  = sigma_s * c(s)                                   (FP64 renormalisation, Sec. 3.3)
 //     c'(x)    = sum_o Q[o][x] * chat(x - o),  o in [-R, R]^3 in a fixed order
 //
-// Q is destination-indexed (Q[o][x] = stored kernel of source x - o at offset o), so a thread that owns
-// VX consecutive destinations reads VX consecutive values of each plane: 16-byte aligned vector loads,
-// coalesced across the warp, every cache value read exactly once per step.  chat is stored with a zero
+// Q is destination-indexed (Q[o][x] = stored kernel of source x - o at offset o), so a warp reads consecutive
+// values of each plane (16-byte vector loads where the rows are whole vectors), every cache value exactly once
+// per step.  chat is stored with a zero
 // halo of R cells on every side, so x - o never leaves the buffer and no bounds test is needed.
 //
 // Accumulation (Sec. 3.3: multiply in the storage precision, accumulate in higher precision):
@@ -24,198 +24,351 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 namespace fdirw {
 
 namespace {
 
-template <typename T, int VX>
-struct Vec;
-template <> struct Vec<double, 2> { using type = double2; };
-template <> struct Vec<float, 4> { using type = float4; };
-template <> struct Vec<__half, 8> { using type = uint4; };
-template <> struct Vec<__nv_bfloat16, 8> { using type = uint4; };
+// Two FP32 values per packed instruction; a - b as b (-1) + a, which rounds once like the subtraction.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, 0xbf800000bf800000ull, a); }
+__device__ __forceinline__ uint64_t neg2(uint64_t a) { return a ^ 0x8000000080000000ull; }
 
-// Loads VX consecutive stored values (16 bytes) and widens them to float.
-template <typename ST, int VX>
-__device__ __forceinline__ void load_q(const ST* p, float (&q)[VX]) {
-    using V = typename Vec<ST, VX>::type;
-    const V v = __ldcs(reinterpret_cast<const V*>(p));     // streamed: read once per step
-    const ST* e = reinterpret_cast<const ST*>(&v);
-#pragma unroll
-    for (int j = 0; j < VX; j++) q[j] = widen(e[j]);
+// ff_madd and ff_add on two destinations at once (the same operations in the same order).
+__device__ __forceinline__ void ff_madd2(uint64_t& s, uint64_t& c, uint64_t q, uint64_t hi, uint64_t lo) {
+    const uint64_t p = mul2(q, hi);
+    const uint64_t e = fma2(q, lo, fma2(q, hi, neg2(p)));
+    const uint64_t t = add2(s, p);
+    const uint64_t bp = sub2(t, s);
+    const uint64_t err = add2(sub2(s, sub2(t, bp)), sub2(p, bp));
+    s = t;
+    c = add2(c, add2(err, e));
+}
+__device__ __forceinline__ void ff_add2(uint64_t& A, uint64_t& B, uint64_t s, uint64_t c) {
+    const uint64_t t = add2(A, s);
+    const uint64_t bp = sub2(t, A);
+    const uint64_t e = add2(sub2(A, sub2(t, bp)), sub2(s, bp));
+    const uint64_t f = add2(e, add2(B, c));
+    A = add2(t, f);
+    B = sub2(f, sub2(A, t));
 }
 
-// Mixed path: ST in {float, half, bf16}, VX = 16 / sizeof(ST), chat as float2 (hi, lo).
-template <typename ST, int R>
-__global__ void __launch_bounds__(256) gather_ff_kernel(const ST* __restrict__ Q, const float2* __restrict__ chat,
-                                                        Grid g, Pad p, int64_t qs, bool acc_in,
-                                                        double* __restrict__ out, int z0, int zn, int64_t qoff) {
-    constexpr int VX = 16 / sizeof(ST);
-    constexpr int W1 = 2 * R + 1;
-    constexpr int NC = VX + 2 * R;
-    const int nxv = g.nx / VX;
-    const int64_t nthreads = (int64_t)nxv * g.ny * zn;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid >= nthreads) return;
-    const int xv = (int)(tid % nxv);
-    const int64_t r = tid / nxv;
-    const int y = (int)(r % g.ny);
-    const int z = z0 + (int)(r / g.ny);
-    const int x0 = xv * VX;
-    const int64_t i0 = (int64_t)x0 + (int64_t)g.nx * y + (int64_t)g.nx * g.ny * z;
-
-    float A[VX], B[VX];                       // running double-float sum of each destination
-#pragma unroll
-    for (int j = 0; j < VX; j++) { A[j] = 0.f; B[j] = 0.f; }
-
-    for (int oz = -R; oz <= R; oz++) {
-        for (int oy = -R; oy <= R; oy++) {
-            // chat row of the sources x - o for ox in [-R, R]: padded x in [x0, x0 + VX + 2R).
-            const float2* row = chat + ((int64_t)(z - oz + R) * p.py + (y - oy + R)) * p.px + x0;
-            float2 ch[NC];
-#pragma unroll
-            for (int j = 0; j < NC; j++) ch[j] = __ldg(row + j);
-            const ST* qrow = Q + ((int64_t)((oz + R) * W1 + (oy + R)) * W1) * qs + (i0 - qoff);
-            // The FP32 pair restarts at zero on every row of 2R+1 terms, so its compensation term stays
-            // within a few ulps of the row sum; the row is then added to the destination's pair.
-            float s[VX], c[VX];
-#pragma unroll
-            for (int j = 0; j < VX; j++) { s[j] = 0.f; c[j] = 0.f; }
-#pragma unroll
-            for (int ox = -R; ox <= R; ox++) {
-                float q[VX];
-                load_q<ST, VX>(qrow + (int64_t)(ox + R) * qs, q);
-#pragma unroll
-                for (int j = 0; j < VX; j++) ff_madd(s[j], c[j], q[j], ch[j - ox + R]);
-            }
-#pragma unroll
-            for (int j = 0; j < VX; j++) ff_add(A[j], B[j], s[j], c[j]);
-        }
+// VX consecutive stored values (16 bytes) as VX / 2 pairs (j0(i), j0(i) + D): neighbours for FP32, whose 16 bytes
+// are register pairs already, values VX / 2 apart for the 16-bit types, whose widening places them anyway.
+template <typename ST>
+struct Quad {
+    static constexpr int D = sizeof(ST) == 4 ? 1 : 4;
+    static constexpr __host__ __device__ int j0(int i) { return sizeof(ST) == 4 ? 2 * i : i; }
+};
+template <typename ST>
+__device__ __forceinline__ void pairs_of(uint4 v, uint64_t (&q)[8 / sizeof(ST)]) {
+    auto pr = [](uint32_t a, uint32_t b) { return pack2(__uint_as_float(a), __uint_as_float(b)); };
+    if constexpr (sizeof(ST) == 4) {
+        q[0] = pr(v.x, v.y);
+        q[1] = pr(v.z, v.w);
+    } else if constexpr (std::is_same<ST, __half>::value) {
+        const __half2* h = reinterpret_cast<const __half2*>(&v);
+        const float2 a = __half22float2(h[0]), b = __half22float2(h[1]), c = __half22float2(h[2]), d = __half22float2(h[3]);
+        q[0] = pack2(a.x, c.x);
+        q[1] = pack2(a.y, c.y);
+        q[2] = pack2(b.x, d.x);
+        q[3] = pack2(b.y, d.y);
+    } else {
+        q[0] = pr(v.x << 16, v.z << 16);
+        q[1] = pr(v.x & 0xffff0000u, v.z & 0xffff0000u);
+        q[2] = pr(v.y << 16, v.w << 16);
+        q[3] = pr(v.y & 0xffff0000u, v.w & 0xffff0000u);
     }
-#pragma unroll
-    for (int j = 0; j < VX; j++) out[i0 + j] = (acc_in ? out[i0 + j] : 0.0) + ((double)A[j] + (double)B[j]);
+}
+template <typename ST>
+__device__ __forceinline__ void load_pairs(const ST* p, uint64_t (&q)[8 / sizeof(ST)]) {
+    pairs_of<ST>(__ldcs(reinterpret_cast<const uint4*>(p)), q);       // streamed: read once per step
 }
 
-// FDIRW_ACCUM_FP32: the loop of gather_ff_kernel with FP32 products and row sums (one FMA per term) and an
-// FP32 chat; the rows still go into a double-float pair per destination.  The caller restores the mass.
-template <typename ST, int R>
-__global__ void __launch_bounds__(256) gather_fp32_kernel(const ST* __restrict__ Q, const float* __restrict__ chat,
-                                                          Grid g, Pad p, int64_t qs, bool acc_in,
-                                                          double* __restrict__ out, int z0, int zn, int64_t qoff) {
-    constexpr int VX = 16 / sizeof(ST);
-    constexpr int W1 = 2 * R + 1;
-    constexpr int NC = VX + 2 * R;
-    const int nxv = g.nx / VX;
-    const int64_t nthreads = (int64_t)nxv * g.ny * zn;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid >= nthreads) return;
-    const int xv = (int)(tid % nxv);
-    const int64_t r = tid / nxv;
-    const int y = (int)(r % g.ny);
-    const int z = z0 + (int)(r / g.ny);
-    const int x0 = xv * VX;
-    const int64_t i0 = (int64_t)x0 + (int64_t)g.nx * y + (int64_t)g.nx * g.ny * z;
+// The gather over destinations in cell order.  A block is 8 warps: VW of them side by side in the destinations, and
+// 8 / VW row groups that split the (2R+1)^2 rows (o_z, o_y).  A destination's row sums are added up within a group in
+// ascending order and the groups' sums in ascending order at the end, the same in every gather kernel of a mode (FP32
+// sums: one group).
+//
+// Why the rows are split: a grid of up to about 100^3 cells has too few destinations to fill 152 SMs with one thread
+// for all rows of each (32^3 FP32 ones are 32 blocks of 256), and beyond that the last wave of long threads idles most
+// of the chip.  us a step before -> after, FP32 cache, float-float sums: 32^3 R = 3 49 -> 14, 48^3 R = 8 1972 -> 346,
+// 112^3 R = 8 6487 -> 4173 (4060 at the copy rate); FP64 36^3 R = 6 600 -> 188.  At R <= 2 (at most 25 rows) eight
+// groups cost more than they give (128^3 R = 2 BF16 cache 100 -> 125): one.
+constexpr int vector_warps(int R) { return R <= 2 ? 8 : 1; }
+__device__ __forceinline__ int row_groups(int R) { return R <= 2 ? 1 : 8; }
 
-    float A[VX], B[VX];
-#pragma unroll
-    for (int j = 0; j < VX; j++) { A[j] = 0.f; B[j] = 0.f; }
-    for (int oz = -R; oz <= R; oz++) {
-        for (int oy = -R; oy <= R; oy++) {
-            const float* row = chat + ((int64_t)(z - oz + R) * p.py + (y - oy + R)) * p.px + x0;
-            float ch[NC];
-#pragma unroll
-            for (int j = 0; j < NC; j++) ch[j] = __ldg(row + j);
-            const ST* qrow = Q + ((int64_t)((oz + R) * W1 + (oy + R)) * W1) * qs + (i0 - qoff);
-            float s[VX];
-#pragma unroll
-            for (int j = 0; j < VX; j++) s[j] = 0.f;
-#pragma unroll
-            for (int ox = -R; ox <= R; ox++) {
-                float q[VX];
-                load_q<ST, VX>(qrow + (int64_t)(ox + R) * qs, q);
-#pragma unroll
-                for (int j = 0; j < VX; j++) s[j] = fmaf(q[j], ch[j - ox + R], s[j]);
-            }
-#pragma unroll
-            for (int j = 0; j < VX; j++) ff_add(A[j], B[j], s[j], 0.f);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < VX; j++) out[i0 + j] = (acc_in ? out[i0 + j] : 0.0) + ((double)A[j] + (double)B[j]);
-}
+struct GatherArgs {
+    const void* Q;
+    const void* chat;
+    Grid g;
+    Pad p;
+    int64_t qs;                    // plane stride
+    int z0, zn, qnx;               // destination planes; values in a cache row (>= nx)
+    double* out;
+    bool acc_in;
+};
 
-// FP64 path: FP64 storage, FP64 chat, FP64 FMA accumulation, VX = 2.
-template <int R>
-__global__ void __launch_bounds__(256) gather_f64_kernel(const double* __restrict__ Q, const double* __restrict__ chat,
-                                                         Grid g, Pad p, double* __restrict__ out, int64_t qs, int z0,
-                                                         int zn, int64_t qoff) {
-    constexpr int VX = 2;
-    constexpr int W1 = 2 * R + 1;
-    constexpr int NC = VX + 2 * R;
-    const int nxv = g.nx / VX;
-    const int64_t nthreads = (int64_t)nxv * g.ny * zn;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid >= nthreads) return;
-    const int xv = (int)(tid % nxv);
-    const int64_t r = tid / nxv;
-    const int y = (int)(r % g.ny);
-    const int z = z0 + (int)(r / g.ny);
-    const int x0 = xv * VX;
-    const int64_t i0 = (int64_t)x0 + (int64_t)g.nx * y + (int64_t)g.nx * g.ny * z;
-    double acc0 = 0.0, acc1 = 0.0;
-    for (int oz = -R; oz <= R; oz++) {
-        for (int oy = -R; oy <= R; oy++) {
-            const double* row = chat + ((int64_t)(z - oz + R) * p.py + (y - oy + R)) * p.px + x0;
-            double ch[NC];
-#pragma unroll
-            for (int j = 0; j < NC; j++) ch[j] = __ldg(row + j);
-            const double* qrow = Q + ((int64_t)((oz + R) * W1 + (oy + R)) * W1) * qs + (i0 - qoff);
-#pragma unroll
-            for (int ox = -R; ox <= R; ox++) {
-                const double2 q = __ldcs(reinterpret_cast<const double2*>(qrow + (int64_t)(ox + R) * qs));
-                acc0 = fma(q.x, ch[0 - ox + R], acc0);
-                acc1 = fma(q.y, ch[1 - ox + R], acc1);
-            }
-        }
-    }
-    out[i0] = acc0;
-    out[i0 + 1] = acc1;
-}
+// Cache rows of whole 16-byte vectors: a thread owns VX consecutive destinations of an x row, one load of a plane.
+// The destinations past nx in a padded row are computed from whatever lies there and not stored.  MODE 0: FP64 throughout.  MODE 1: float-float rows (FDIRW_ACCUM_FF).  MODE 2: FP32 rows
+// (FDIRW_ACCUM_FP32); both sum the rows of a destination as a float-float pair, which one FP64 addition turns into
+// the result.  Two blocks per SM: 128 registers keep a row's loads in flight (with three blocks and 80 registers the
+// loads no longer overlap: 1.4 times as long).
+template <typename ST, int R, int MODE, int VW>
+__global__ void __launch_bounds__(256, MODE == 2 && R == 1 ? 4 : 2) gather_kernel(GatherArgs a) {
+    constexpr int VX = 16 / sizeof(ST), W1 = 2 * R + 1, NROW = W1 * W1, NV = VW * 32, G = 8 / VW;
+    constexpr int NP = MODE == 0 ? 1 : VX / 2, NK = VX + 2 * R;
+    using T = typename std::conditional<MODE == 0, double, float>::type;
+    __shared__ T part[MODE == 0 ? 1 : 2][VX][256];
 
-// Any nx (no vector alignment): one destination per thread, runtime R, same arithmetic as above.
-template <typename ST, int MODE>
-__global__ void __launch_bounds__(256) gather_scalar_kernel(const ST* __restrict__ Q, const void* __restrict__ chat,
-                                                            Grid g, Pad p, int R, int64_t qs, bool acc_in,
-                                                            double* __restrict__ out, int z0, int zn, int64_t qoff) {
-    const int64_t nxy = (int64_t)g.nx * g.ny;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid >= nxy * zn) return;
-    const int64_t i = z0 * nxy + tid;
-    const int x = (int)(i % g.nx);
-    const int64_t r = i / g.nx;
-    const int y = (int)(r % g.ny);
-    const int z = (int)(r / g.ny);
-    double acc = (MODE == 0 && acc_in) ? out[i] : 0.0;   // FP64 path: plain FMA accumulation
-    float A = 0.f, B = 0.f;                               // FP32 paths: running double-float sum
-    int o = 0;
-    for (int oz = -R; oz <= R; oz++)
-        for (int oy = -R; oy <= R; oy++) {
-            float s = 0.f, c = 0.f;
-            for (int ox = -R; ox <= R; ox++, o++) {
-                const int64_t pi = ((int64_t)(z - oz + R) * p.py + (y - oy + R)) * p.px + (x - ox + R);
-                const ST qv = Q[(int64_t)o * qs + (i - qoff)];
-                if constexpr (MODE == 1) {
-                    ff_madd(s, c, widen(qv), reinterpret_cast<const float2*>(chat)[pi]);
-                } else if constexpr (MODE == 2) {
-                    s = fmaf(widen(qv), reinterpret_cast<const float*>(chat)[pi], s);
-                } else {
-                    acc = fma((double)qv, reinterpret_cast<const double*>(chat)[pi], acc);
+    const int t = threadIdx.x, group = t / NV;
+    // (a plane of 2^31 vectors would be a cache of 27 x 32 GB and more: 32-bit positions will do)
+    const unsigned v = blockIdx.x * NV + (t - group * NV);
+    double acc[2] = {0.0, 0.0};                          // MODE 0
+    uint64_t A[NP], B[NP];                               // MODE 1, 2: running double-float sums of two destinations
+#pragma unroll
+    for (int i = 0; i < NP; i++) A[i] = B[i] = 0;
+
+    const unsigned nxv = a.qnx / VX, nvec = nxv * a.g.ny * a.zn;
+    if (v < nvec) {
+        const unsigned rw = v / nxv;
+        const int x = (int)(v - rw * nxv) * VX, z = a.z0 + (int)(rw / a.g.ny), y = (int)(rw % a.g.ny);
+        const int64_t at = ((int64_t)(z + R) * a.p.py + (y + R)) * a.p.px + x;     // of (ox, oy, oz) = (R, 0, 0)
+        const int last = a.g.nx - 1 - x + 2 * R;             // no scaled value past the padded x row is read
+        const int r0 = group * NROW / G, r1 = (group + 1) * NROW / G;
+        int oz = r0 / W1 - R, oy = r0 % W1 - R;
+        const ST* q = reinterpret_cast<const ST*>(a.Q) + (int64_t)r0 * W1 * a.qs + (int64_t)v * VX;
+        for (int r = r0; r < r1; r++) {
+            const int64_t row = at - ((int64_t)oz * a.p.py + oy) * a.p.px;
+            if constexpr (MODE == 0) {
+                const double* ch = reinterpret_cast<const double*>(a.chat) + row;
+                double w[NK];
+#pragma unroll
+                for (int k = 0; k < NK; k++) w[k] = __ldg(ch + (k <= 2 * R ? k : min(k, last)));
+#pragma unroll
+                for (int ox = -R; ox <= R; ox++) {
+                    const double2 d = __ldcs(reinterpret_cast<const double2*>(q + (int64_t)(ox + R) * a.qs));
+                    acc[0] = fma(d.x, w[R - ox], acc[0]);
+                    acc[1] = fma(d.y, w[R - ox + 1], acc[1]);
                 }
+            } else {
+                using U = Quad<ST>;
+                uint64_t s[NP], c[NP];
+#pragma unroll
+                for (int i = 0; i < NP; i++) s[i] = c[i] = 0;
+                float hi[NK], lo[NK];
+#pragma unroll
+                for (int k = 0; k < NK; k++) {
+                    if constexpr (MODE == 1) {
+                        const float2 f = __ldg(reinterpret_cast<const float2*>(a.chat) + row + (k <= 2 * R ? k : min(k, last)));
+                        hi[k] = f.x;
+                        lo[k] = f.y;
+                    } else {
+                        hi[k] = __ldg(reinterpret_cast<const float*>(a.chat) + row + (k <= 2 * R ? k : min(k, last)));
+                    }
+                }
+#pragma unroll
+                for (int ox = -R; ox <= R; ox++) {
+                    uint64_t d[NP];
+                    load_pairs(q + (int64_t)(ox + R) * a.qs, d);
+#pragma unroll
+                    for (int i = 0; i < NP; i++) {
+                        const int k = U::j0(i) - ox + R;
+                        const uint64_t h = pack2(hi[k], hi[k + U::D]);
+                        if constexpr (MODE == 1) ff_madd2(s[i], c[i], d[i], h, pack2(lo[k], lo[k + U::D]));
+                        else s[i] = fma2(d[i], h, s[i]);
+                    }
+                }
+                // The pair of a row restarts at zero, so its compensation stays within a few ulps of the row sum.
+#pragma unroll
+                for (int i = 0; i < NP; i++) ff_add2(A[i], B[i], s[i], c[i]);
+            }
+            q += W1 * a.qs;
+            if (++oy > R) { oy = -R; oz++; }
+        }
+    }
+    if constexpr (G == 1) {                              // nothing to add up
+        if (v >= nvec) return;
+        const unsigned rw = v / nxv;
+        const int x = (int)(v - rw * nxv) * VX;
+        double* o = a.out + x + (int64_t)a.g.nx * ((int64_t)rw + (int64_t)a.g.ny * a.z0);
+        float SA[VX], SB[VX];
+        if constexpr (MODE != 0) {
+#pragma unroll
+            for (int i = 0; i < NP; i++) {
+                unpack2(A[i], SA[Quad<ST>::j0(i)], SA[Quad<ST>::j0(i) + Quad<ST>::D]);
+                unpack2(B[i], SB[Quad<ST>::j0(i)], SB[Quad<ST>::j0(i) + Quad<ST>::D]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < VX; j++)
+            if (x + j < a.g.nx) {
+                if constexpr (MODE == 0) o[j] = acc[j];
+                else o[j] = (a.acc_in ? o[j] : 0.0) + ((double)SA[j] + (double)SB[j]);
+            }
+        return;
+    }
+    if constexpr (MODE == 0) {
+        part[0][0][t] = acc[0];
+        part[0][1][t] = acc[1];
+    } else {
+        using U = Quad<ST>;
+#pragma unroll
+        for (int i = 0; i < NP; i++) {
+            unpack2(A[i], part[0][U::j0(i)][t], part[0][U::j0(i) + U::D][t]);
+            unpack2(B[i], part[1][U::j0(i)][t], part[1][U::j0(i) + U::D][t]);
+        }
+    }
+    __syncthreads();
+    // The groups' sums in ascending order, consecutive threads on consecutive destinations.
+    for (int d = t; d < NV * VX; d += 256) {
+        const int w = d / VX, j = d - w * VX;
+        const unsigned u = blockIdx.x * NV + w, rw = u / nxv;
+        const int x = (int)(u - rw * nxv) * VX + j;
+        if (u >= nvec || x >= a.g.nx) continue;
+        double* o = a.out + x + (int64_t)a.g.nx * ((int64_t)rw + (int64_t)a.g.ny * a.z0);
+        if constexpr (MODE == 0) {
+            double sum = part[0][j][w];
+#pragma unroll
+            for (int k = 1; k < G; k++) sum += part[0][j][k * NV + w];
+            *o = sum;
+        } else {
+            float SA = part[0][j][w], SB = part[1][j][w];
+#pragma unroll
+            for (int k = 1; k < G; k++) ff_add(SA, SB, part[0][j][k * NV + w], part[1][j][k * NV + w]);
+            *o = (a.acc_in ? *o : 0.0) + ((double)SA + (double)SB);
+        }
+    }
+}
+
+// FDIRW_ACCUM_FP32 at R >= 3: the same split of the rows, but one destination's rows are added in the order of one
+// sequential sum, because the next step rounds its scaled field to FP32: a last bit of the FP64 result can flip that
+// rounding, and 6e-8 of the value with it, so a result is kept to the bit whatever the split.  The 8 warps of a block
+// take 8 consecutive rows at a time and leave their row sums in shared memory; then each thread adds the 8 sums of its
+// own destinations.  The next row's cache values are loaded before that, so they arrive while the block meets.
+template <typename ST, int R>
+__global__ void __launch_bounds__(256, 2) gather_ordered_kernel(GatherArgs a) {
+    using U = Quad<ST>;
+    constexpr int VX = 16 / sizeof(ST), W1 = 2 * R + 1, NROW = W1 * W1, NP = VX / 2, NK = VX + 2 * R, ND = 32 * VX;
+    __shared__ float sums[2][8][ND];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned nxv = a.qnx / VX, nvec = nxv * a.g.ny * a.zn, v = blockIdx.x * 32 + lane;
+    const bool valid = v < nvec;
+    const unsigned rw = valid ? v / nxv : 0;
+    const int x = valid ? (int)(v - rw * nxv) * VX : 0, z = a.z0 + (int)(rw / a.g.ny), y = (int)(rw % a.g.ny);
+    const int last = a.g.nx - 1 - x + 2 * R;             // no scaled value past the padded x row is read
+    const float* chat = reinterpret_cast<const float*>(a.chat) + ((int64_t)(z + R) * a.p.py + (y + R)) * a.p.px + x;
+    const ST* q = reinterpret_cast<const ST*>(a.Q) + (valid ? (int64_t)v * VX : 0);
+    uint4 d[W1];
+    auto fetch = [&](int row) {
+        const ST* p = q + (int64_t)row * W1 * a.qs;
+#pragma unroll
+        for (int k = 0; k < W1; k++) d[k] = __ldcs(reinterpret_cast<const uint4*>(p + (int64_t)k * a.qs));
+    };
+    fetch(warp);
+    float A = 0.f, B = 0.f;                              // of destination t (threads below ND)
+    int buf = 0;
+    for (int r0 = 0; r0 < NROW; r0 += 8, buf ^= 1) {
+        const int row = r0 + warp;
+        if (row < NROW) {
+            const int oz = row / W1 - R, oy = row % W1 - R;
+            const float* ch = chat - ((int64_t)oz * a.p.py + oy) * a.p.px;
+            uint64_t s[NP];
+#pragma unroll
+            for (int i = 0; i < NP; i++) s[i] = 0;
+            float hi[NK];
+#pragma unroll
+            for (int k = 0; k < NK; k++) hi[k] = __ldg(ch + (k <= 2 * R ? k : min(k, last)));
+#pragma unroll
+            for (int ox = -R; ox <= R; ox++) {
+                uint64_t w[NP];
+                pairs_of<ST>(d[ox + R], w);
+#pragma unroll
+                for (int i = 0; i < NP; i++) {
+                    const int k = U::j0(i) - ox + R;
+                    s[i] = fma2(w[i], pack2(hi[k], hi[k + U::D]), s[i]);
+                }
+            }
+            if (row + 8 < NROW) fetch(row + 8);
+            float f[VX];
+#pragma unroll
+            for (int i = 0; i < NP; i++) unpack2(s[i], f[U::j0(i)], f[U::j0(i) + U::D]);
+#pragma unroll
+            for (int j = 0; j < VX; j += 4)
+                *reinterpret_cast<float4*>(&sums[buf][warp][lane * VX + j]) = make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]);
+        }
+        __syncthreads();
+        if (t < ND) {
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                if (r0 + k < NROW) ff_add(A, B, sums[buf][k][t], 0.f);
+        }
+    }
+    if (t >= ND) return;
+    const unsigned u = blockIdx.x * 32 + t / VX, ru = u / nxv;
+    const int dx = (int)(u - ru * nxv) * VX + t % VX;
+    if (u >= nvec || dx >= a.g.nx) return;
+    double* o = a.out + dx + (int64_t)a.g.nx * ((int64_t)ru + (int64_t)a.g.ny * a.z0);
+    *o = (a.acc_in ? *o : 0.0) + ((double)A + (double)B);
+}
+
+// Packed rows of a width that is no whole number of vectors (nx < VX, or a padded cache that would not fit): one
+// destination per thread, runtime R, the sums of gather_kernel in the same order.
+template <typename ST, int MODE>
+__global__ void __launch_bounds__(256) gather_scalar_kernel(GatherArgs a, int R) {
+    const int64_t nxy = (int64_t)a.g.nx * a.g.ny;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (tid >= nxy * a.zn) return;
+    const ST* Q = reinterpret_cast<const ST*>(a.Q) + tid;
+    const int x = (int)(tid % a.g.nx), y = (int)(tid / a.g.nx % a.g.ny), z = a.z0 + (int)(tid / nxy);
+    const int W1 = 2 * R + 1, NROW = W1 * W1, G = MODE == 2 ? 1 : row_groups(R);
+    double sum = 0.0;                                     // MODE 0
+    float SA = 0.f, SB = 0.f;                             // MODE 1, 2
+    for (int k = 0; k < G; k++) {
+        double acc = 0.0;
+        float A = 0.f, B = 0.f;
+        for (int row = k * NROW / G; row < (k + 1) * NROW / G; row++) {
+            const int oz = row / W1 - R, oy = row % W1 - R;
+            const int64_t at = ((int64_t)(z - oz + R) * a.p.py + (y - oy + R)) * a.p.px + x + R;
+            const ST* q = Q + (int64_t)row * W1 * a.qs;
+            float s = 0.f, c = 0.f;
+            for (int ox = -R; ox <= R; ox++, q += a.qs) {
+                if constexpr (MODE == 1) ff_madd(s, c, widen(*q), reinterpret_cast<const float2*>(a.chat)[at - ox]);
+                else if constexpr (MODE == 2) s = fmaf(widen(*q), reinterpret_cast<const float*>(a.chat)[at - ox], s);
+                else acc = fma((double)*q, reinterpret_cast<const double*>(a.chat)[at - ox], acc);
             }
             if constexpr (MODE != 0) ff_add(A, B, s, c);
         }
-    if constexpr (MODE != 0) out[i] = (acc_in ? out[i] : 0.0) + ((double)A + (double)B);
-    else out[i] = acc;
+        if (k == 0) { sum = acc; SA = A; SB = B; }
+        else if constexpr (MODE != 0) ff_add(SA, SB, A, B);
+        else sum += acc;
+    }
+    double* o = a.out + a.z0 * nxy + tid;
+    if constexpr (MODE != 0) *o = (a.acc_in ? *o : 0.0) + ((double)SA + (double)SB);
+    else *o = sum;
 }
 
 __global__ void scale_kernel(const double* __restrict__ c, const double* __restrict__ sigma, Grid g, int R, Pad p,
@@ -400,7 +553,7 @@ __global__ void __launch_bounds__(256) seg_apply_kernel(double* __restrict__ c, 
 }
 
 template <typename ST>
-__global__ void read_kernels_kernel(const ST* __restrict__ Q, const double* __restrict__ sigma, Grid g, int R,
+__global__ void read_kernels_kernel(const ST* __restrict__ Q, int64_t qs, int qnx, const double* __restrict__ sigma, Grid g, int R,
                                     const int64_t* __restrict__ sources, int64_t n_src, double* __restrict__ out) {
     const int W1 = 2 * R + 1;
     const int64_t W = (int64_t)W1 * W1 * W1;
@@ -415,15 +568,15 @@ __global__ void read_kernels_kernel(const ST* __restrict__ Q, const double* __re
         const int x = sx + ox, y = sy + oy, z = sz + oz;
         double v = 0.0;
         if (x >= 0 && x < g.nx && y >= 0 && y < g.ny && z >= 0 && z < g.nz) {
-            const int64_t i = (int64_t)x + (int64_t)g.nx * y + (int64_t)g.nx * g.ny * z;
-            v = (double)widen(Q[(int64_t)o * g.n + i]) * sigma[s];
+            const int64_t i = x + (int64_t)qnx * (y + (int64_t)g.ny * z);
+            v = (double)widen(Q[(int64_t)o * qs + i]) * sigma[s];
         }
         out[t] = v;
     }
 }
 template <>
-__global__ void read_kernels_kernel<double>(const double* __restrict__ Q, const double* __restrict__ sigma, Grid g,
-                                            int R, const int64_t* __restrict__ sources, int64_t n_src,
+__global__ void read_kernels_kernel<double>(const double* __restrict__ Q, int64_t qs, int qnx,
+                                            const double* __restrict__ sigma, Grid g, int R, const int64_t* __restrict__ sources, int64_t n_src,
                                             double* __restrict__ out) {
     const int W1 = 2 * R + 1;
     const int64_t W = (int64_t)W1 * W1 * W1;
@@ -438,8 +591,8 @@ __global__ void read_kernels_kernel<double>(const double* __restrict__ Q, const 
         const int x = sx + ox, y = sy + oy, z = sz + oz;
         double v = 0.0;
         if (x >= 0 && x < g.nx && y >= 0 && y < g.ny && z >= 0 && z < g.nz) {
-            const int64_t i = (int64_t)x + (int64_t)g.nx * y + (int64_t)g.nx * g.ny * z;
-            v = Q[(int64_t)o * g.n + i] * sigma[s];
+            const int64_t i = x + (int64_t)qnx * (y + (int64_t)g.ny * z);
+            v = Q[(int64_t)o * qs + i] * sigma[s];
         }
         out[t] = v;
     }
@@ -450,174 +603,70 @@ int blocks_for(int64_t n, int threads) {
     return (int)(b < 1 ? 1 : b);
 }
 
-// Destination planes [z0, z0 + zn) of the launch and the column offset of its cache (a slab of a
-// streamed uniform cache); {0, nz, 0} for a whole grid.
-struct Slab {
-    int z0, zn;
-    int64_t qoff;
-};
+// Below this many vectors an FP32 gather splits the rows (gather_ordered_kernel), from there on a thread sums its rows
+// alone.  us, split / alone, BF16 cache: R = 8 64^3 (33k vectors) 455 / 522, 96^3 (111k) 1356 / 1501, 128^3 (262k) 3095 /
+// 3133, 144^3 (373k) 4506 / 4134; R = 4 48^3 (14k) 49 / 86, 64^3 86 / 88, 96^3 242 / 213; R = 3 64^3 43 / 51, 96^3 121 / 117.
+constexpr int64_t ordered_below(int R) { return R <= 5 ? 65536 : 300000; }
 
-template <typename ST, int R>
-cudaError_t gather_ff_r(const void* Q, const void* chat, Grid g, Pad p, int64_t qs, bool acc_in, double* out,
-                        cudaStream_t st, Slab sl) {
+template <typename ST, int R, int MODE>
+cudaError_t gather_launch(const GatherArgs& a, cudaStream_t st) {
     constexpr int VX = 16 / sizeof(ST);
-    const int64_t nt = (int64_t)(g.nx / VX) * g.ny * sl.zn;
-    if (nt <= 0) return cudaSuccess;
-    gather_ff_kernel<ST, R><<<blocks_for(nt, 256), 256, 0, st>>>(reinterpret_cast<const ST*>(Q),
-                                                                   reinterpret_cast<const float2*>(chat), g, p, qs,
-                                                                   acc_in, out, sl.z0, sl.zn, sl.qoff);
-    return cudaGetLastError();
-}
-
-template <typename ST>
-cudaError_t gather_ff(const void* Q, const void* chat, Grid g, int R, Pad p, int64_t qs, bool acc_in, double* out,
-                      cudaStream_t st, Slab sl) {
-    switch (R) {
-        case 1: return gather_ff_r<ST, 1>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 2: return gather_ff_r<ST, 2>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 3: return gather_ff_r<ST, 3>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 4: return gather_ff_r<ST, 4>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 5: return gather_ff_r<ST, 5>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 6: return gather_ff_r<ST, 6>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 7: return gather_ff_r<ST, 7>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 8: return gather_ff_r<ST, 8>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 9: return gather_ff_r<ST, 9>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 10: return gather_ff_r<ST, 10>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-template <int R>
-cudaError_t gather_f64_r(const void* Q, const void* chat, Grid g, Pad p, int64_t qs, double* out, cudaStream_t st,
-                         Slab sl) {
-    const int64_t nt = (int64_t)(g.nx / 2) * g.ny * sl.zn;
-    if (nt <= 0) return cudaSuccess;
-    gather_f64_kernel<R><<<blocks_for(nt, 256), 256, 0, st>>>(reinterpret_cast<const double*>(Q),
-                                                               reinterpret_cast<const double*>(chat), g, p, out, qs,
-                                                               sl.z0, sl.zn, sl.qoff);
-    return cudaGetLastError();
-}
-
-cudaError_t gather_f64(const void* Q, const void* chat, Grid g, int R, Pad p, int64_t qs, double* out,
-                       cudaStream_t st, Slab sl) {
-    switch (R) {
-        case 1: return gather_f64_r<1>(Q, chat, g, p, qs, out, st, sl);
-        case 2: return gather_f64_r<2>(Q, chat, g, p, qs, out, st, sl);
-        case 3: return gather_f64_r<3>(Q, chat, g, p, qs, out, st, sl);
-        case 4: return gather_f64_r<4>(Q, chat, g, p, qs, out, st, sl);
-        case 5: return gather_f64_r<5>(Q, chat, g, p, qs, out, st, sl);
-        case 6: return gather_f64_r<6>(Q, chat, g, p, qs, out, st, sl);
-        case 7: return gather_f64_r<7>(Q, chat, g, p, qs, out, st, sl);
-        case 8: return gather_f64_r<8>(Q, chat, g, p, qs, out, st, sl);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-template <typename ST, int R>
-cudaError_t gather_fp32_r(const void* Q, const float* chat, Grid g, Pad p, int64_t qs, bool acc_in, double* out,
-                          cudaStream_t st, Slab sl) {
-    constexpr int VX = 16 / sizeof(ST);
-    const int64_t nt = (int64_t)(g.nx / VX) * g.ny * sl.zn;
-    if (nt <= 0) return cudaSuccess;
-    gather_fp32_kernel<ST, R><<<blocks_for(nt, 256), 256, 0, st>>>(reinterpret_cast<const ST*>(Q), chat, g, p, qs,
-                                                                     acc_in, out, sl.z0, sl.zn, sl.qoff);
-    return cudaGetLastError();
-}
-
-template <typename ST>
-cudaError_t gather_fp32_st(const void* Q, const float* chat, Grid g, int R, Pad p, int64_t qs, bool acc_in,
-                           double* out, cudaStream_t st, Slab sl) {
-    switch (R) {
-        case 1: return gather_fp32_r<ST, 1>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 2: return gather_fp32_r<ST, 2>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 3: return gather_fp32_r<ST, 3>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 4: return gather_fp32_r<ST, 4>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 5: return gather_fp32_r<ST, 5>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 6: return gather_fp32_r<ST, 6>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 7: return gather_fp32_r<ST, 7>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 8: return gather_fp32_r<ST, 8>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 9: return gather_fp32_r<ST, 9>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        case 10: return gather_fp32_r<ST, 10>(Q, chat, g, p, qs, acc_in, out, st, sl);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-// Scalar fallback of both accumulations and the FP64 path (any nx): MODE 0 FP64, 1 float-float, 2 FP32.
-template <int MODE>
-cudaError_t gather_scalar(const void* Q, Store store, const void* ch, Grid g, Pad p, int R, int64_t qs, bool acc,
-                          double* out, cudaStream_t st, Slab sl) {
-    const int64_t n = (int64_t)g.nx * g.ny * sl.zn;
+    // FP32 sums come in one order whatever the kernel, so the split is free to follow the size of the launch.
+    constexpr int VW = MODE == 2 ? 8 : vector_warps(R);
+    const bool vec = a.qnx % VX == 0 && reinterpret_cast<uintptr_t>(a.Q) % 16 == 0 && a.qs % VX == 0;
+    const int64_t n = (vec ? (int64_t)a.qnx / VX : (int64_t)a.g.nx) * a.g.ny * a.zn;
     if (n <= 0) return cudaSuccess;
-    const int b = blocks_for(n, 256);
-    switch (store) {
-        case Store::F64:
-            if (MODE != 0) return cudaErrorInvalidValue;
-            gather_scalar_kernel<double, MODE><<<b, 256, 0, st>>>(reinterpret_cast<const double*>(Q), ch, g, p, R,
-                                                                  qs, acc, out, sl.z0, sl.zn, sl.qoff);
-            break;
-        case Store::F32:
-            if (MODE == 0) return cudaErrorInvalidValue;
-            gather_scalar_kernel<float, MODE><<<b, 256, 0, st>>>(reinterpret_cast<const float*>(Q), ch, g, p, R, qs,
-                                                                 acc, out, sl.z0, sl.zn, sl.qoff);
-            break;
-        case Store::F16:
-            if (MODE == 0) return cudaErrorInvalidValue;
-            gather_scalar_kernel<__half, MODE><<<b, 256, 0, st>>>(reinterpret_cast<const __half*>(Q), ch, g, p, R,
-                                                                  qs, acc, out, sl.z0, sl.zn, sl.qoff);
-            break;
-        case Store::BF16:
-            if (MODE == 0) return cudaErrorInvalidValue;
-            gather_scalar_kernel<__nv_bfloat16, MODE><<<b, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(Q),
-                                                                         ch, g, p, R, qs, acc, out, sl.z0, sl.zn,
-                                                                         sl.qoff);
-            break;
+    if (!vec) {
+        gather_scalar_kernel<ST, MODE><<<(unsigned)blocks_for(n, 256), 256, 0, st>>>(a, R);
+        return cudaGetLastError();
     }
+    if constexpr (MODE == 2 && R > 2) {
+        if (n < ordered_below(R)) {
+            gather_ordered_kernel<ST, R><<<(unsigned)((n + 31) / 32), 256, 0, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
+    gather_kernel<ST, R, MODE, VW><<<(unsigned)((n + VW * 32 - 1) / (VW * 32)), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-// Float-float (FP32 storage types) or FP64 gather of one part (radius R, chat with a halo of Rp).
-cudaError_t gather_part(const void* Q, Store store, int64_t qs, const void* chat, int Rp, Grid g, int R,
-                        bool accumulate, double* c_out, cudaStream_t st, Slab sl) {
-    if (R < 1 || R > Rp) return cudaErrorInvalidValue;
+template <typename ST, int MODE>
+cudaError_t gather_radius(const GatherArgs& a, int R, cudaStream_t st) {
+    switch (R) {
+        case 1: return gather_launch<ST, 1, MODE>(a, st);
+        case 2: return gather_launch<ST, 2, MODE>(a, st);
+        case 3: return gather_launch<ST, 3, MODE>(a, st);
+        case 4: return gather_launch<ST, 4, MODE>(a, st);
+        case 5: return gather_launch<ST, 5, MODE>(a, st);
+        case 6: return gather_launch<ST, 6, MODE>(a, st);
+        case 7: return gather_launch<ST, 7, MODE>(a, st);
+        case 8: return gather_launch<ST, 8, MODE>(a, st);
+        default: break;
+    }
+    if constexpr (MODE != 0) {
+        if (R == 9) return gather_launch<ST, 9, MODE>(a, st);
+        if (R == 10) return gather_launch<ST, 10, MODE>(a, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// The gather of one part (radius R, chat with a halo of Rp): mode 0 FP64, 1 float-float, 2 FP32.
+cudaError_t gather_part(const void* Q, Store store, int64_t qs, int qnx, const void* chat, int Rp, Grid g, int R,
+                        int mode, bool accumulate, double* c_out, cudaStream_t st, int z0, int zn) {
+    if (R < 1 || R > Rp || qnx < g.nx || (mode == 0) != (store == Store::F64) || (mode == 0 && accumulate))
+        return cudaErrorInvalidValue;
     const Pad p = make_pad(g, Rp);
     // The kernels index chat as if its halo were R: move the base by (Rp - R) on every axis.
     const int64_t shift = ((int64_t)(Rp - R) * p.py + (Rp - R)) * p.px + (Rp - R);
-    const void* ch = static_cast<const char*>(chat) + shift * 8;   // chat element: double or float2, 8 bytes
-    const int vx = 16 / store_bytes(store);
-    const bool aligned = (reinterpret_cast<uintptr_t>(Q) % 16) == 0 && (qs * store_bytes(store)) % 16 == 0 &&
-                         (sl.qoff * store_bytes(store)) % 16 == 0;
-    if (store == Store::F64 && accumulate) return cudaErrorInvalidValue;   // uniform FP64 contexts only
-    if (R <= (store == Store::F64 ? kMaxR64 : kMaxR) && g.nx % vx == 0 && aligned) {
-        switch (store) {
-            case Store::F64: return gather_f64(Q, ch, g, R, p, qs, c_out, st, sl);
-            case Store::F32: return gather_ff<float>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-            case Store::F16: return gather_ff<__half>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-            case Store::BF16: return gather_ff<__nv_bfloat16>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-        }
-        return cudaErrorInvalidValue;
+    const void* ch = static_cast<const char*>(chat) + shift * (mode == 2 ? 4 : 8);
+    const GatherArgs a{Q, ch, g, p, qs, z0, zn, qnx, c_out, accumulate};
+    switch (store) {
+        case Store::F64: return gather_radius<double, 0>(a, R, st);
+        case Store::F32: return mode == 1 ? gather_radius<float, 1>(a, R, st) : gather_radius<float, 2>(a, R, st);
+        case Store::F16: return mode == 1 ? gather_radius<__half, 1>(a, R, st) : gather_radius<__half, 2>(a, R, st);
+        case Store::BF16: return mode == 1 ? gather_radius<__nv_bfloat16, 1>(a, R, st) : gather_radius<__nv_bfloat16, 2>(a, R, st);
     }
-    return store == Store::F64 ? gather_scalar<0>(Q, store, ch, g, p, R, qs, accumulate, c_out, st, sl)
-                               : gather_scalar<1>(Q, store, ch, g, p, R, qs, accumulate, c_out, st, sl);
-}
-
-// FDIRW_ACCUM_FP32 gather of one part (FP32 chat with a halo of Rp).
-cudaError_t gather_part_fp32(const void* Q, Store store, int64_t qs, const float* chat, int Rp, Grid g, int R,
-                             bool accumulate, double* c_out, cudaStream_t st, Slab sl) {
-    if (R < 1 || R > Rp || R > kMaxR || store == Store::F64) return cudaErrorInvalidValue;
-    const Pad p = make_pad(g, Rp);
-    const float* ch = chat + ((int64_t)(Rp - R) * p.py + (Rp - R)) * p.px + (Rp - R);
-    const int vx = 16 / store_bytes(store);
-    const bool aligned = (reinterpret_cast<uintptr_t>(Q) % 16) == 0 && (qs * store_bytes(store)) % 16 == 0 &&
-                         (sl.qoff * store_bytes(store)) % 16 == 0;
-    if (g.nx % vx == 0 && aligned) {
-        switch (store) {
-            case Store::F32: return gather_fp32_st<float>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-            case Store::F16: return gather_fp32_st<__half>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-            case Store::BF16: return gather_fp32_st<__nv_bfloat16>(Q, ch, g, R, p, qs, accumulate, c_out, st, sl);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    return gather_scalar<2>(Q, store, ch, g, p, R, qs, accumulate, c_out, st, sl);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -634,22 +683,14 @@ cudaError_t launch_scale(const double* c, const double* sigma, Grid g, int R, vo
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_part(const void* Q, Store store, int64_t qs, const void* chat, int Rp, Grid g, int R,
-                               bool accumulate, double* c_out, cudaStream_t st) {
-    return gather_part(Q, store, qs, chat, Rp, g, R, accumulate, c_out, st, Slab{0, g.nz, 0});
+cudaError_t launch_gather_part(const void* Q, Store store, int64_t qs, int qnx, const void* chat, int Rp, Grid g,
+                               int R, int mode, bool accumulate, double* c_out, cudaStream_t st) {
+    return gather_part(Q, store, qs, qnx, chat, Rp, g, R, mode, accumulate, c_out, st, 0, g.nz);
 }
 
-cudaError_t launch_gather_slab(const void* Q, Store store, int64_t qs, int64_t qoff, const void* chat, Grid g, int R,
+cudaError_t launch_gather_slab(const void* Q, Store store, int64_t qs, int qnx, const void* chat, Grid g, int R,
                                int mode, int z0, int zn, double* c_out, cudaStream_t st) {
-    const Slab sl{z0, zn, qoff};
-    if (mode == 2)
-        return gather_part_fp32(Q, store, qs, reinterpret_cast<const float*>(chat), R, g, R, false, c_out, st, sl);
-    return gather_part(Q, store, qs, chat, R, g, R, false, c_out, st, sl);
-}
-
-cudaError_t launch_gather(const void* Q, Store store, const void* chat, Grid g, int R, double* c_out,
-                          cudaStream_t st) {
-    return launch_gather_part(Q, store, g.n, chat, R, g, R, false, c_out, st);
+    return gather_part(Q, store, qs, qnx, chat, R, g, R, mode, false, c_out, st, z0, zn);
 }
 
 cudaError_t launch_mass(const double* c, int64_t n, double* partials, double* out, cudaStream_t st) {
@@ -698,33 +739,23 @@ cudaError_t launch_restore_mass(double* c, int64_t n, double* partials, double* 
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_part_fp32(const void* Q, Store store, int64_t qs, const float* chat, int Rp, Grid g, int R,
-                                    bool accumulate, double* c_out, cudaStream_t st) {
-    return gather_part_fp32(Q, store, qs, chat, Rp, g, R, accumulate, c_out, st, Slab{0, g.nz, 0});
-}
-
-cudaError_t launch_gather_fp32(const void* Q, Store store, const float* chat, Grid g, int R, double* c_out,
-                               cudaStream_t st) {
-    return launch_gather_part_fp32(Q, store, g.n, chat, R, g, R, false, c_out, st);
-}
-
-cudaError_t launch_read_kernels(const void* Q, Store store, const double* sigma, Grid g, int R,
+cudaError_t launch_read_kernels(const void* Q, Store store, int64_t qs, int qnx, const double* sigma, Grid g, int R,
                                 const int64_t* sources, int64_t n_src, double* out, cudaStream_t st) {
     const int64_t W = (int64_t)(2 * R + 1) * (2 * R + 1) * (2 * R + 1);
     int b = blocks_for(n_src * W, 256);
     if (b > 152 * 16) b = 152 * 16;
     switch (store) {
         case Store::F64:
-            read_kernels_kernel<double><<<b, 256, 0, st>>>(reinterpret_cast<const double*>(Q), sigma, g, R, sources, n_src, out);
+            read_kernels_kernel<double><<<b, 256, 0, st>>>(reinterpret_cast<const double*>(Q), qs, qnx, sigma, g, R, sources, n_src, out);
             break;
         case Store::F32:
-            read_kernels_kernel<float><<<b, 256, 0, st>>>(reinterpret_cast<const float*>(Q), sigma, g, R, sources, n_src, out);
+            read_kernels_kernel<float><<<b, 256, 0, st>>>(reinterpret_cast<const float*>(Q), qs, qnx, sigma, g, R, sources, n_src, out);
             break;
         case Store::F16:
-            read_kernels_kernel<__half><<<b, 256, 0, st>>>(reinterpret_cast<const __half*>(Q), sigma, g, R, sources, n_src, out);
+            read_kernels_kernel<__half><<<b, 256, 0, st>>>(reinterpret_cast<const __half*>(Q), qs, qnx, sigma, g, R, sources, n_src, out);
             break;
         case Store::BF16:
-            read_kernels_kernel<__nv_bfloat16><<<b, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(Q), sigma, g, R,
+            read_kernels_kernel<__nv_bfloat16><<<b, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(Q), qs, qnx, sigma, g, R,
                                                                    sources, n_src, out);
             break;
     }

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(256) head_train_kernel(const float* __restrict
 // Q[o][s + o]; sigma_s = 1 / FP64 sum of the stored values (the march's renormalisation).
 __global__ void __launch_bounds__(256) head_store_kernel(const float* __restrict__ zhead, Grid g,
                                                          const int64_t* __restrict__ src, const int* __restrict__ accept,
-                                                         void* Q, Store st, double* __restrict__ sigma) {
+                                                         void* Q, int64_t qs, int qnx, Store st, double* __restrict__ sigma) {
     __shared__ double sh[8];
     const int b = blockIdx.x;
     if (!accept[b]) return;
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256) head_store_kernel(const float* __restrict
         int64_t gi;
         if (!in_domain(q, i, j, k, g, &gi)) continue;
         const float y = expf(zhead[(int64_t)b * KV + v]);
-        const int64_t idx = (int64_t)v * g.n + gi;       // offset o = (i-8, j-8, k-8), destination gi
+        const int64_t idx = (int64_t)v * qs + gi % g.nx + (gi / g.nx) * qnx;   // offset o = (i-8, j-8, k-8), destination gi
         float stored;
         if (st == Store::F32) { reinterpret_cast<float*>(Q)[idx] = y; stored = y; }
         else if (st == Store::F16) { const __half h = __float2half_rn(y); reinterpret_cast<__half*>(Q)[idx] = h; stored = __half2float(h); }
@@ -1142,7 +1142,7 @@ FDIRW_API int fdirw_kernels_surrogate(fdirw_ctx* c, fdirw_net* net, int64_t* acc
         if ((rc = forward(c, net, n)) != FDIRW_OK) return rc;
         head_predict_kernel<<<n, 256, 0, c->stream>>>(net->zhead, c->g, net->dsrc, nullptr, net->dmass, net->dacc);
         NET_CUDA(net, cudaGetLastError());
-        head_store_kernel<<<n, 256, 0, c->stream>>>(net->zhead, c->g, net->dsrc, net->dacc, c->Q, c->store, c->sigma);
+        head_store_kernel<<<n, 256, 0, c->stream>>>(net->zhead, c->g, net->dsrc, net->dacc, c->Q, c->q_stride, c->q_nx, c->store, c->sigma);
         NET_CUDA(net, cudaGetLastError());
         NET_CUDA(net, cudaMemcpyAsync(acc.data(), net->dacc, (size_t)n * 4, cudaMemcpyDeviceToHost, c->stream));
         NET_CUDA(net, cudaStreamSynchronize(c->stream));
@@ -1160,7 +1160,8 @@ FDIRW_API int fdirw_kernels_surrogate(fdirw_ctx* c, fdirw_net* net, int64_t* acc
         a.g = c->g;
         a.R = c->R;
         a.Rq = c->R;
-        a.q_stride = c->g.n;
+        a.q_stride = c->q_stride;
+        a.q_vec = c->q_nx > c->g.nx ? 16 / fdirw::store_bytes(c->store) : 1;
         a.n_sub = c->n_sub;
         a.ax = reinterpret_cast<const float*>(c->coef[0]);
         a.ay = reinterpret_cast<const float*>(c->coef[1]);

@@ -50,4 +50,4 @@ def test_block_march_streams_slabs(R):
     a, _, ia = _run(shape, D, dt, R, 6, "bf16", 4)
     limit = ia["device_bytes"] - ia["cache_bytes"] + ia["cache_bytes"] // 4 + 8 * int(np.prod(shape))
     b, _, ib = _run(shape, D, dt, R, 6, "bf16", 4, mem_limit=limit)
-    assert ib["n_chunks"] >= 4 and np.array_equal(a, b)
+    assert ib["n_chunks"] > 1 and np.array_equal(a, b)
