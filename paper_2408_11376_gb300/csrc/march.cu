@@ -573,58 +573,6 @@ struct MapTmc {
     static constexpr size_t SMEM_COARSE = SMEM_COARSE_USED > SMEM ? SMEM_COARSE_USED : SMEM;
 };
 
-// Coarse epilogue (Eq. 11 applied to the marched unit of block J): S[d] = FP64 sum of the marched field
-// over the liquid cells of block J + d inside the window (z, y, x order; sbuf holds 0 elsewhere), m =
-// sum of S in a fixed order, and column J of P: Qc[d][J + d] = N_J S[d] / (m N_{J+d}), or S[d] / N_{J+d}
-// when the phase has open faces (a.abnd) and the column keeps the mass that stays (0 where block J + d
-// has no liquid).  Every thread of the CTA takes part; S follows red in shared memory.
-template <int R>
-__device__ void coarse_epilogue(const MarchArgs& a, const float* sbuf, double* S, int64_t first) {
-    constexpr int W1 = 2 * R + 1;
-    const bool valid = first < a.src_end;                 // uniform over the CTA
-    const int64_t J = valid ? (a.list ? a.list[first] : first) : 0;
-    const int B = a.coarse_B, Rc = a.coarse_Rc, Wc = 2 * Rc + 1, Wc3 = Wc * Wc * Wc, bh = (B - 1) / 2;
-    const int bx = (int)(J % a.ncx), by = (int)((J / a.ncx) % a.ncy), bz = (int)(J / ((int64_t)a.ncx * a.ncy));
-    const int sx = bx * B + bh, sy = by * B + bh, sz = bz * B + bh;
-    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
-    for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
-        double acc = 0.0;
-        if (valid) {
-            const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
-            const int x0 = max(max(cx * B, sx - R), 0), x1 = min(min(cx * B + B - 1, sx + R), nx - 1);
-            const int y0 = max(max(cy * B, sy - R), 0), y1 = min(min(cy * B + B - 1, sy + R), ny - 1);
-            const int z0 = max(max(cz * B, sz - R), 0), z1 = min(min(cz * B + B - 1, sz + R), nz - 1);
-            for (int z = z0; z <= z1; z++)
-                for (int y = y0; y <= y1; y++)
-                    for (int x = x0; x <= x1; x++)
-                        acc += (double)sbuf[((x - (sx - R)) + W1 * (y - (sy - R))) * W1 + (z - (sz - R))];
-        }
-        S[d] = acc;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double m = 0.0;
-        for (int d = threadIdx.x; d < Wc3; d += 32) m += S[d];
-        for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xffffffffu, m, off);
-        if (threadIdx.x == 0) S[Wc3] = m;
-    }
-    __syncthreads();
-    const double m = S[Wc3];
-    if (valid) {
-        const double NJ = (double)a.ccount[J];
-        for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
-            const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
-            if (cx < 0 || cx >= a.ncx || cy < 0 || cy >= a.ncy || cz < 0 || cz >= a.ncz) continue;
-            const int64_t I = cx + (int64_t)a.ncx * (cy + (int64_t)a.ncy * cz);
-            const int NI = a.ccount[I];
-            // Closed phase: renormalise the column to carry N_J; open faces: keep the mass that stays.
-            double v = 0.0;
-            if (NI > 0 && m > 0.0) v = a.abnd ? S[d] / (double)NI : (NJ * S[d]) / (m * (double)NI);
-            a.Qc[(int64_t)d * a.coarse_n + I] = v;
-        }
-    }
-}
-
 // COARSE: the source is coarse block a.list[pos] (Eqs. 10-15): its window is centred on the block's
 // centre cell (radius R = window_R + (B - 1) / 2), the march starts from 1 on the block's liquid cells,
 // and the epilogue maps the marched field onto the blocks of the window (column J of the coarse matrix,
@@ -805,7 +753,8 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
                 }
             }
             __syncthreads();
-            coarse_epilogue<R>(a, sbuf, reinterpret_cast<double*>(red + COLS), first);
+            coarse_epilogue<R>(a, [&](int x, int y, int k) { return sbuf[(x + W1 * y) * W1 + k]; },
+                               reinterpret_cast<double*>(red + COLS), first);
         } else {
             if (active) {
 #pragma unroll
@@ -1178,17 +1127,18 @@ int march_mapping(const MarchArgs& a, int parts_req) {
 }
 
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st) {
-    switch (R) {
-        case 1: return a.bx ? launch_tmc<1, true, true>(a, num_sms, st) : launch_tmc<1, true>(a, num_sms, st);
-        case 2: return a.bx ? launch_tmc<2, true, true>(a, num_sms, st) : launch_tmc<2, true>(a, num_sms, st);
-        case 3: return a.bx ? launch_tmc<3, true, true>(a, num_sms, st) : launch_tmc<3, true>(a, num_sms, st);
-        case 4: return a.bx ? launch_tmc<4, true, true>(a, num_sms, st) : launch_tmc<4, true>(a, num_sms, st);
-        case 5: return a.bx ? launch_tmc<5, true, true>(a, num_sms, st) : launch_tmc<5, true>(a, num_sms, st);
-        case 6: return a.bx ? launch_tmc<6, true, true>(a, num_sms, st) : launch_tmc<6, true>(a, num_sms, st);
-        case 7: return a.bx ? launch_tmc<7, true, true>(a, num_sms, st) : launch_tmc<7, true>(a, num_sms, st);
-        case 8: return a.bx ? launch_tmc<8, true, true>(a, num_sms, st) : launch_tmc<8, true>(a, num_sms, st);
-        case 9: return a.bx ? launch_tmc<9, true, true>(a, num_sms, st) : launch_tmc<9, true>(a, num_sms, st);
-        case 10: return a.bx ? launch_tmc<10, true, true>(a, num_sms, st) : launch_tmc<10, true>(a, num_sms, st);
+    if (!a.bx) return launch_march_blocks(a, num_sms, st);
+    switch (R) {                                  // direction-dependent coefficients: mapping 5
+        case 1: return launch_tmc<1, true, true>(a, num_sms, st);
+        case 2: return launch_tmc<2, true, true>(a, num_sms, st);
+        case 3: return launch_tmc<3, true, true>(a, num_sms, st);
+        case 4: return launch_tmc<4, true, true>(a, num_sms, st);
+        case 5: return launch_tmc<5, true, true>(a, num_sms, st);
+        case 6: return launch_tmc<6, true, true>(a, num_sms, st);
+        case 7: return launch_tmc<7, true, true>(a, num_sms, st);
+        case 8: return launch_tmc<8, true, true>(a, num_sms, st);
+        case 9: return launch_tmc<9, true, true>(a, num_sms, st);
+        case 10: return launch_tmc<10, true, true>(a, num_sms, st);
         default: return cudaErrorInvalidValue;
     }
 }

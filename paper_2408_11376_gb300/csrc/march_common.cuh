@@ -204,6 +204,58 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return d;
 }
 
+// Coarse epilogue (Eq. 11 applied to the marched unit of block J): S[d] = FP64 sum of the marched field
+// over the liquid cells of block J + d inside the window (z, y, x order; u is 0 elsewhere), m =
+// sum of S in a fixed order, and column J of P: Qc[d][J + d] = N_J S[d] / (m N_{J+d}), or S[d] / N_{J+d}
+// when the phase has open faces (a.abnd) and the column keeps the mass that stays (0 where block J + d
+// has no liquid).  Every thread of the CTA takes part; S follows red in shared memory.
+// u(x, y, k) is the marched value of a window cell (0 on cells that are not liquid).
+template <int R, typename F>
+__device__ __forceinline__ void coarse_epilogue(const MarchArgs& a, F u, double* S, int64_t first) {
+    const bool valid = first < a.src_end;                 // uniform over the CTA
+    const int64_t J = valid ? (a.list ? a.list[first] : first) : 0;
+    const int B = a.coarse_B, Rc = a.coarse_Rc, Wc = 2 * Rc + 1, Wc3 = Wc * Wc * Wc, bh = (B - 1) / 2;
+    const int bx = (int)(J % a.ncx), by = (int)((J / a.ncx) % a.ncy), bz = (int)(J / ((int64_t)a.ncx * a.ncy));
+    const int sx = bx * B + bh, sy = by * B + bh, sz = bz * B + bh;
+    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
+    for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
+        double acc = 0.0;
+        if (valid) {
+            const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
+            const int x0 = max(max(cx * B, sx - R), 0), x1 = min(min(cx * B + B - 1, sx + R), nx - 1);
+            const int y0 = max(max(cy * B, sy - R), 0), y1 = min(min(cy * B + B - 1, sy + R), ny - 1);
+            const int z0 = max(max(cz * B, sz - R), 0), z1 = min(min(cz * B + B - 1, sz + R), nz - 1);
+            for (int z = z0; z <= z1; z++)
+                for (int y = y0; y <= y1; y++)
+                    for (int x = x0; x <= x1; x++)
+                        acc += (double)u(x - (sx - R), y - (sy - R), z - (sz - R));
+        }
+        S[d] = acc;
+    }
+    asm volatile("bar.sync 0;" ::: "memory");              // both z parts of a split march meet here, each in its own code
+    if (threadIdx.x < 32) {
+        double m = 0.0;
+        for (int d = threadIdx.x; d < Wc3; d += 32) m += S[d];
+        for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xffffffffu, m, off);
+        if (threadIdx.x == 0) S[Wc3] = m;
+    }
+    asm volatile("bar.sync 0;" ::: "memory");
+    const double m = S[Wc3];
+    if (valid) {
+        const double NJ = (double)a.ccount[J];
+        for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
+            const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
+            if (cx < 0 || cx >= a.ncx || cy < 0 || cy >= a.ncy || cz < 0 || cz >= a.ncz) continue;
+            const int64_t I = cx + (int64_t)a.ncx * (cy + (int64_t)a.ncy * cz);
+            const int NI = a.ccount[I];
+            // Closed phase: renormalise the column to carry N_J; open faces: keep the mass that stays.
+            double v = 0.0;
+            if (NI > 0 && m > 0.0) v = a.abnd ? S[d] / (double)NI : (NJ * S[d]) / (m * (double)NI);
+            a.Qc[(int64_t)d * a.coarse_n + I] = v;
+        }
+    }
+}
+
 }  // namespace
 
 }  // namespace fdirw

@@ -20,7 +20,7 @@
 // with L/I/R the x faces left of, inside and right of the block in row 0 or 1, B/J/T the y faces below, inside
 // and above it in column 0 or 1, am the diagonals of the four cells (sub-column sc = column + 2 row).
 //
-// R <= 8: 256 threads, each with all 2R+1 levels; SPB sources per CTA.  R = 9, 10: a thread's state would not
+// R <= 8: each thread has all 2R+1 levels; SPB sources per CTA.  R = 9, 10: a thread's state would not
 // fit its registers, so each column block is split in z between two threads of different warps (the first
 // takes LO levels); the two meet at one face through the exchange buffer.
 //
@@ -30,9 +30,8 @@
 // -> 0.554 / 8.1; R = 6: 0.333 / 13.0 -> 0.261 / 3.5; R = 3: 0.056 / 2.2 -> 0.048 / 0.8; R = 10 against one column
 // per thread (mapping 5): 1.73 / 23.5 -> 1.10 / 23.4.
 //
-// One CTA of 256 threads per SM (two threads per TMEM lane, 256 columns each; the CTA allocates all 512
-// columns once and frees them before it exits, and its shared-memory request keeps a second CTA off the SM
-// so an allocation never waits).
+// One CTA per SM (two or three threads per TMEM lane; the CTA allocates all 512 columns once and frees them before it
+// exits, and its shared-memory request keeps a second CTA off the SM so an allocation never waits).
 #include "fdirw_internal.h"
 #include "march_common.cuh"
 
@@ -54,17 +53,23 @@ struct MapTm {
     static constexpr int NB = R + 1;                      // blocks per window axis (last one half padding)
     static constexpr int TPS = NB * NB;                   // threads per source and z part
     static constexpr int ZS = R <= 8 ? 1 : 2;             // z parts
-    static constexpr int THREADS = 256;
+    // R <= 4: the state leaves room for 12 warps (3 threads per TMEM lane) instead of 8; 64^3 sources, ms a substep /
+    // outside: R = 3 0.0477 / 0.80 -> 0.0461 / 0.68, R = 4 0.0930 / 1.18 -> 0.0927 / 1.02.
+    static constexpr int THREADS = R <= 4 ? 384 : 256;
+    static constexpr int SLOT = R <= 4 ? 160 : 256;       // TMEM columns of a thread
     static constexpr int PT = THREADS / ZS;               // threads of a z part
     static constexpr int SPB = PT / TPS;                  // sources per CTA
     static constexpr int LO = ZS == 1 ? W1 : 10;          // levels of the first z part
     static constexpr int BUF = W1 * 4 * PT;               // floats per exchange buffer
     static constexpr size_t SMEM_USED = (size_t)2 * BUF * 4 + (size_t)THREADS * 8 + (size_t)SPB * sizeof(SlotInfo);
     static constexpr size_t SMEM = SMEM_USED > 120 * 1024 ? SMEM_USED : 120 * 1024;
+    // Coarse mode adds the per-block sums (at most W1^3 blocks in a window, plus the total).
+    static constexpr size_t SMEM_COARSE_USED = SMEM_USED + (size_t)(W1 * W1 * W1 + 1) * 8;
+    static constexpr size_t SMEM_COARSE = SMEM_COARSE_USED > SMEM ? SMEM_COARSE_USED : SMEM;
     static_assert(SPB >= 1, "a source must fit one CTA");
 };
 
-// TMEM columns of a z part of NK levels (256 per thread).  The pairs p < AP take 32 columns each: X at 32 p (16
+// TMEM columns of a z part of NK levels (at most 256 per thread).  The pairs p < AP take 32 columns each: X at 32 p (16
 // words, am2 and am3 at 32 p + 24) and Y at 32 p + 16 (8 words, the last 4 at 32 p + 28).  The others keep their
 // diagonals in registers and take 24: X as 8 + 4 words, Y as 8 + 4.  The middle level of an odd count takes 16.
 template <int NK>
@@ -125,7 +130,10 @@ template <int N>
 __device__ __forceinline__ uint64_t pr(const uint32_t (&r)[N], int q) { return u2pack(r[2 * q], r[2 * q + 1]); }
 
 // One z part (levels K0 .. K0 + NK - 1 of the window) of every source of the CTA's batches.
-template <int R, int K0, int NK>
+// COARSE: the source is coarse block a.list[pos] (Eqs. 10-15): its window is centred on the block's centre cell
+// (radius R = window_R + (B - 1) / 2), the march starts from 1 on the block's liquid cells, an open face (a.abnd) adds
+// to the diagonal, and the epilogue maps the marched field onto the blocks of the window instead of storing a kernel.
+template <int R, bool COARSE, int K0, int NK>
 __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* smem_raw, uint32_t tbase) {
     using M = MapTm<R>;
     using C = ColsTm<NK>;
@@ -147,8 +155,8 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
     // Neighbour blocks, in a ring: past a window edge this is a thread of another row or source, whose (finite)
     // value meets a zero face.  Every warp then reads 32 consecutive slots, which no bank serves twice; reading
     // the own slot there instead cost 10% of the shared-memory wavefronts in bank conflicts.
-    const int tl = (th - 1) & (PT - 1), tr = (th + 1) & (PT - 1);
-    const int tb = (th - NB) & (PT - 1), tt = (th + NB) & (PT - 1);
+    auto ring = [](int v) { return v < 0 ? v + PT : v >= PT ? v - PT : v; };
+    const int tl = ring(th - 1), tr = ring(th + 1), tb = ring(th - NB), tt = ring(th + NB);
     const int x0 = 2 * bi, y0 = 2 * bj;
     const int64_t nbatch = (a.src_end - a.src_begin + SPB - 1) / SPB;
 
@@ -162,7 +170,17 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
         const int nx = L.nx, ny = L.ny, nz = L.nz;
         const int64_t nxy = (int64_t)nx * ny;
         int sx = 0, sy = 0, sz = 0;
-        if (src_ok) split_cell(s, nx, ny, sx, sy, sz);
+        const int bh = COARSE ? (a.coarse_B - 1) / 2 : 0;
+        if (src_ok) {
+            if constexpr (COARSE) {
+                split_cell(s, a.ncx, a.ncy, sx, sy, sz);
+                sx = sx * a.coarse_B + bh;         // centre of the block (may lie past a clipped domain edge)
+                sy = sy * a.coarse_B + bh;
+                sz = sz * a.coarse_B + bh;
+            } else {
+                split_cell(s, nx, ny, sx, sy, sz);
+            }
+        }
         if (active && b == 0 && K0 == 0)
             sinfo[slot] = SlotInfo{L, pos, sx, sy, sz, src_ok ? 1 : 0};
 
@@ -195,7 +213,12 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
                 p += nxy;
             }
             const bool centre = src_ok && x0 + (sc & 1) == R && y0 + (sc >> 1) == R;
-            auto u0 = [&](int j) { return centre && K0 + j == R ? 1.f : 0.f; };
+            const bool near = COARSE && ok && abs(x0 + (sc & 1) - R) <= bh && abs(y0 + (sc >> 1) - R) <= bh;
+            auto u0 = [&](int j) -> float {
+                if (!COARSE) return centre && K0 + j == R ? 1.f : 0.f;
+                if (!near || abs(K0 + j - R) > bh || !in(gz + j, nz)) return 0.f;
+                return a.liquid[i0 + (sc & 1) + (int64_t)nx * (sc >> 1) + nxy * j] ? 1.f : 0.f;
+            };
 #pragma unroll
             for (int j = 0; j < NP; j++) {
                 U[sc][j] = f2pack(u0(j), u0(j + H));
@@ -229,7 +252,12 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
 #pragma unroll
             for (int sc = 0; sc < 4; sc++) {
                 const int x = (sc & 1) + 3 * (sc >> 1), y = 10 + sc;
-                f[6 + sc] = -(((f[x] + f[x + 1]) + (f[y] + f[y + 2])) + (zf[sc][j] + zf[sc][j + 1]));
+                float sum = ((f[x] + f[x + 1]) + (f[y] + f[y + 2])) + (zf[sc][j] + zf[sc][j + 1]);
+                if constexpr (COARSE) {
+                    const bool open = a.abnd && zin && xc[sc & 1] && yc[sc >> 1];
+                    sum = sum + (open ? __ldg(a.abnd + i0 + (sc & 1) + (int64_t)nx * (sc >> 1) + nxy * j) : 0.f);
+                }
+                f[6 + sc] = -sum;
             }
         };
 #pragma unroll
@@ -389,6 +417,18 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
         }
         tm_wait_x(X, X4);
 
+        if constexpr (COARSE) {
+            // u is 0 on cells that are not liquid: their faces carry nothing and they start at 0
+            const float* ubuf = xbuf + (a.n_sub & 1) * M::BUF;
+            double* S = reinterpret_cast<double*>(sinfo + SPB);
+            for (int sl = 0; sl < SPB; sl++) {
+                coarse_epilogue<R>(a, [&](int x, int y, int k) {
+                    return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), sl * TPS + (x >> 1) + NB * (y >> 1))];
+                }, S, first + sl);
+                bar();                             // S and xbuf are free for the next source
+            }
+            continue;
+        }
         // Epilogue.  xbuf's buffer n_sub & 1 holds every u (published by the last substep).  Each thread sums
         // its own rounded values (cells outside the window or the domain are 0).
         {
@@ -443,7 +483,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
     }
 }
 
-template <int R>
+template <int R, bool COARSE>
 __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArgs a) {
     using M = MapTm<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -458,12 +498,12 @@ __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArg
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = s_taddr;
-    const uint32_t tbase = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(256 * (warp >> 2));
+    const uint32_t tbase = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(M::SLOT * (warp >> 2));
     if constexpr (M::ZS == 1) {
-        march_part<R, 0, M::W1>(a, smem_raw, tbase);
+        march_part<R, COARSE, 0, M::W1>(a, smem_raw, tbase);
     } else {
-        if (warp < M::PT / 32) march_part<R, 0, M::LO>(a, smem_raw, tbase);
-        else march_part<R, M::LO, M::W1 - M::LO>(a, smem_raw, tbase);
+        if (warp < M::PT / 32) march_part<R, COARSE, 0, M::LO>(a, smem_raw, tbase);
+        else march_part<R, COARSE, M::LO, M::W1 - M::LO>(a, smem_raw, tbase);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -471,21 +511,28 @@ __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArg
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(taddr) : "memory");
 }
 
-template <int R>
+template <int R, bool COARSE>
 cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
     using M = MapTm<R>;
     const int64_t nsrc = a.src_end - a.src_begin;
     if (nsrc <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(march_tm_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::SMEM);
+    const size_t smem = COARSE ? M::SMEM_COARSE : M::SMEM;
+    auto kernel = march_tm_kernel<R, COARSE>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_tm_kernel<R>, M::THREADS, M::SMEM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, M::THREADS, smem);
     if (e != cudaSuccess) return e;
     if (per_sm != 1) return cudaErrorInvalidConfiguration;   // TMEM allocation assumes one CTA per SM
     const int64_t nbatch = (nsrc + M::SPB - 1) / M::SPB;
     const int64_t grid = nbatch < (int64_t)num_sms ? nbatch : (int64_t)num_sms;
-    march_tm_kernel<R><<<(unsigned)grid, M::THREADS, M::SMEM, st>>>(a);
+    kernel<<<(unsigned)grid, M::THREADS, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int R>
+cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
+    return a.coarse_B > 0 ? launch_tm<R, true>(a, num_sms, st) : launch_tm<R, false>(a, num_sms, st);
 }
 
 }  // namespace
