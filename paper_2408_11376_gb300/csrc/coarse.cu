@@ -48,6 +48,7 @@ struct Coarse {
     // Coupled macro step: FP64 solid-phase face conductances, a scratch field, phase-mass partials.
     double* gs = nullptr;                        // 3 N: +x/+y/+z solid-solid faces
     double* tmp = nullptr;                       // 2 N
+    double gs_max = 0.0;                         // largest per-cell sum of gs
     double* qpart = nullptr;                     // kMassBlocks
     double* qout = nullptr;                      // [Q_L, Q_S] per step, n_steps_cap * 2
     int64_t qcap = 0;
@@ -61,14 +62,39 @@ int grid_blocks(int64_t n, int threads) {
     return (int)(b < 1 ? 1 : b);
 }
 
+// Coordinates of cell i (32-bit division where it is enough: a 64-bit one per axis cost more than the rest of the
+// one-cell-per-thread kernels below).
+__device__ __forceinline__ void cell_of(int64_t i, const Grid& g, int& x, int& y, int& z) {
+    if (g.n <= 0x7fffffff) {
+        const unsigned v = (unsigned)i, r = v / (unsigned)g.nx, q = r / (unsigned)g.ny;
+        x = (int)(v - r * (unsigned)g.nx);
+        y = (int)(r - q * (unsigned)g.ny);
+        z = (int)q;
+    } else {
+        x = (int)(i % g.nx);
+        y = (int)(i / g.nx % g.ny);
+        z = (int)(i / ((int64_t)g.nx * g.ny));
+    }
+}
+
+// The largest of the warps' values (bits of non-negative doubles) into *max_bits, one atomic per warp (one per cell
+// serialised on the one address: 569 us for 96^3 cells, 136 so).
+__device__ __forceinline__ void max_bits_of(double v, unsigned long long* max_bits) {
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, b, off);
+        b = o > b ? o : b;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(max_bits, b);
+}
+
 // Zero the coefficient of every face with a non-liquid cell on either side.
 __global__ void mask_faces_kernel(Grid g, const uint8_t* __restrict__ liquid, float* __restrict__ ax,
                                   float* __restrict__ ay, float* __restrict__ az) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx);
-        const int y = (int)((i / g.nx) % g.ny);
-        const int z = (int)(i / nxy);
+        int x, y, z;
+        cell_of(i, g, x, y, z);
         const bool l = liquid[i] != 0;
         if (!l || x + 1 >= g.nx || !liquid[i + 1]) ax[i] = 0.f;
         if (!l || y + 1 >= g.ny || !liquid[i + g.nx]) ay[i] = 0.f;
@@ -90,19 +116,24 @@ __global__ void count_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, 
     }
 }
 
-// Eq. 13: C_I = (sum of c over the liquid cells of block I, z, y, x order) / N_I.
+// Eq. 13: C_I = (sum of c over the liquid cells of block I) / N_I.  One warp per block: lane l takes the block's cells
+// l, l + 32, ... in z, y, x order, then a xor-butterfly (one thread for a block's 125 cells left most of the GPU idle:
+// 96^3, B = 5, 27 -> 14 us).
 __global__ void map_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, int ncx, int ncy, int64_t nc,
                            const int32_t* __restrict__ count, const double* __restrict__ c, double* __restrict__ C) {
-    for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < nc; I += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t I = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); I < nc; I += step) {
         const int bx = (int)(I % ncx), by = (int)((I / ncx) % ncy), bz = (int)(I / ((int64_t)ncx * ncy));
         double s = 0.0;
-        for (int z = bz * B; z < min(bz * B + B, g.nz); z++)
-            for (int y = by * B; y < min(by * B + B, g.ny); y++)
-                for (int x = bx * B; x < min(bx * B + B, g.nx); x++) {
-                    const int64_t i = x + (int64_t)g.nx * (y + (int64_t)g.ny * z);
-                    if (liquid[i]) s += c[i];
-                }
-        C[I] = count[I] > 0 ? s / (double)count[I] : 0.0;
+        for (int e = lane; e < B * B * B; e += 32) {
+            const int x = bx * B + e % B, y = by * B + e / B % B, z = bz * B + e / (B * B);
+            if (x >= g.nx || y >= g.ny || z >= g.nz) continue;
+            const int64_t i = x + (int64_t)g.nx * (y + (int64_t)g.ny * z);
+            if (liquid[i]) s += c[i];
+        }
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) C[I] = count[I] > 0 ? s / (double)count[I] : 0.0;
     }
 }
 
@@ -112,8 +143,10 @@ __global__ void map_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, in
 __global__ void open_faces_kernel(Grid g, const double* __restrict__ D, const uint8_t* __restrict__ liquid,
                                   double lam, float* __restrict__ abnd, unsigned long long* __restrict__ max_bits) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
+    double most = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
+        int x, y, z;
+        cell_of(i, g, x, y, z);
         double gb = 0.0, sum = 0.0;
         if (liquid[i]) {
             const int faces = (x == 0) + (x == g.nx - 1) + (y == 0) + (y == g.ny - 1) + (z == 0) + (z == g.nz - 1);
@@ -131,45 +164,64 @@ __global__ void open_faces_kernel(Grid g, const double* __restrict__ D, const ui
             sum += gb;
         }
         abnd[i] = (float)(lam * gb);
-        atomicMax(max_bits, (unsigned long long)__double_as_longlong(sum));
+        most = fmax(most, sum);
     }
+    max_bits_of(most, max_bits);
 }
 
 // One explicit substep of the liquid phase over the whole grid with every far-field ghost at 1 (the
 // P_BC march): u' = u + (am u + sum c u_nb + abnd), am = -(sum of the cell's coefficients + abnd), in the
 // FP32 increment form and association of the windowed kernels.
-// With convection (bx != NULL) the inflow from the upper neighbour uses B and the diagonal sums the cell's
-// outflows (A of its +faces, B of its -faces), as the block-source march.
-__global__ void pbc_substep_kernel(Grid g, const float* __restrict__ ax, const float* __restrict__ ay,
-                                   const float* __restrict__ az, const float* __restrict__ bx,
-                                   const float* __restrict__ by, const float* __restrict__ bz,
-                                   const float* __restrict__ abnd, const float* __restrict__ u,
-                                   float* __restrict__ un) {
+// FLOW (convection): the inflow from the upper neighbour uses B and the diagonal sums the cell's outflows (A of its
+// +faces, B of its -faces), as the block-source march.
+// Bound: L2 (the six arrays fit it) and the launch.  A thread walks kPbcZ cells up a z column, the column's u and z faces
+// in registers; no index division (one cell per thread with 64-bit ones: 9.8 us a substep at 96^3, 5.4 so).
+constexpr int kPbcZ = 6;
+template <bool FLOW>
+__global__ void __launch_bounds__(256) pbc_substep_kernel(Grid g, const float* __restrict__ ax, const float* __restrict__ ay,
+                                                          const float* __restrict__ az, const float* __restrict__ bx,
+                                                          const float* __restrict__ by, const float* __restrict__ bz,
+                                                          const float* __restrict__ abnd, const float* __restrict__ u,
+                                                          float* __restrict__ un) {
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (x >= g.nx) return;
     const int64_t nxy = (int64_t)g.nx * g.ny;
-    const float* ux = bx ? bx : ax;                   // coefficient of the upper neighbour in this cell
-    const float* uy = bx ? by : ay;
-    const float* uz = bx ? bz : az;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
-        const float cxm = x > 0 ? ax[i - 1] : 0.f, cxp = x + 1 < g.nx ? ux[i] : 0.f;
-        const float cym = y > 0 ? ay[i - g.nx] : 0.f, cyp = y + 1 < g.ny ? uy[i] : 0.f;
-        const float czm = z > 0 ? az[i - nxy] : 0.f, czp = z + 1 < g.nz ? uz[i] : 0.f;
-        // outflows: the cell's own +faces (A) and the lower neighbours' B; equal to the inflows without flow
-        const float oxm = x > 0 ? ux[i - 1] : 0.f, oxp = x + 1 < g.nx ? ax[i] : 0.f;
-        const float oym = y > 0 ? uy[i - g.nx] : 0.f, oyp = y + 1 < g.ny ? ay[i] : 0.f;
-        const float ozm = z > 0 ? uz[i - nxy] : 0.f, ozp = z + 1 < g.nz ? az[i] : 0.f;
-        const float vb = abnd[i];
-        const float cur = u[i];
-        const float am = -((((oxm + oxp) + (oym + oyp)) + (ozm + ozp)) + vb);
-        float v = am * cur;
-        v = fmaf(cxm, x > 0 ? u[i - 1] : 0.f, v);
-        v = fmaf(cxp, x + 1 < g.nx ? u[i + 1] : 0.f, v);
-        v = fmaf(cym, y > 0 ? u[i - g.nx] : 0.f, v);
-        v = fmaf(cyp, y + 1 < g.ny ? u[i + g.nx] : 0.f, v);
-        v = fmaf(czm, z > 0 ? u[i - nxy] : 0.f, v);
-        v = fmaf(czp, z + 1 < g.nz ? u[i + nxy] : 0.f, v);
-        v = __fadd_rn(v, vb);                           // inflow from the ghosts at c_far = 1
-        un[i] = __fadd_rn(cur, v);
+    for (int64_t y = blockIdx.y * 8 + (threadIdx.x >> 5); y < g.ny; y += gridDim.y * 8)
+    for (int64_t z0 = blockIdx.z * kPbcZ; z0 < g.nz; z0 += gridDim.z * kPbcZ) {
+        int64_t i = x + (int64_t)g.nx * y + nxy * z0;
+        const float* ux = FLOW ? bx : ax;                 // coefficient of the upper neighbour in this cell
+        const float* uy = FLOW ? by : ay;
+        const float* uz = FLOW ? bz : az;
+        const bool xm = x > 0, xp = x + 1 < g.nx, ym = y > 0, yp = y + 1 < g.ny;
+        float czm = z0 > 0 ? az[i - nxy] : 0.f, ozm = FLOW && z0 > 0 ? uz[i - nxy] : czm;
+        float below = z0 > 0 ? u[i - nxy] : 0.f, cur = u[i];
+        const int64_t z1 = z0 + kPbcZ < g.nz ? z0 + kPbcZ : g.nz;
+        for (int64_t z = z0; z < z1; z++, i += nxy) {
+            const bool zp = z + 1 < g.nz;
+            const float above = zp ? u[i + nxy] : 0.f;
+            const float cxm = xm ? ax[i - 1] : 0.f, cxp = xp ? ux[i] : 0.f;
+            const float cym = ym ? ay[i - g.nx] : 0.f, cyp = yp ? uy[i] : 0.f;
+            const float czp = zp ? uz[i] : 0.f;
+            // outflows: the cell's own +faces (A) and the lower neighbours' B; equal to the inflows without flow
+            const float oxm = FLOW && xm ? ux[i - 1] : cxm, oxp = FLOW && xp ? ax[i] : cxp;
+            const float oym = FLOW && ym ? uy[i - g.nx] : cym, oyp = FLOW && yp ? ay[i] : cyp;
+            const float ozp = FLOW && zp ? az[i] : czp;
+            const float vb = abnd[i];
+            const float am = -((((oxm + oxp) + (oym + oyp)) + (ozm + ozp)) + vb);
+            float v = am * cur;
+            v = fmaf(cxm, xm ? u[i - 1] : 0.f, v);
+            v = fmaf(cxp, xp ? u[i + 1] : 0.f, v);
+            v = fmaf(cym, ym ? u[i - g.nx] : 0.f, v);
+            v = fmaf(cyp, yp ? u[i + g.nx] : 0.f, v);
+            v = fmaf(czm, below, v);
+            v = fmaf(czp, above, v);
+            v = __fadd_rn(v, vb);                           // inflow from the ghosts at c_far = 1
+            un[i] = __fadd_rn(cur, v);
+            below = cur;
+            cur = above;
+            czm = ozp;                                      // the face's A, into the cell above
+            ozm = czp;                                      // its B, out of it
+        }
     }
 }
 
@@ -181,29 +233,48 @@ __global__ void widen_kernel(const float* __restrict__ u, int64_t n, double* __r
 // Interface exchange of Eqs. 4-6 on every liquid/solid face, pre-step values, rate over dt; each cell adds
 // its faces' transfers in the order -z, -y, -x, +x, +y, +z (the order in which a raster sweep over the
 // lower cell of each face reaches them), f_L and f_S clamped at 0.  FP64 without contraction.
-__device__ __forceinline__ double exchange(const double* c, const uint8_t* liquid, int64_t a, int64_t b, double k,
-                                           double cS, double cL, double dt) {
-    // transfer from the liquid cell to the solid one across face (a, b); 0 unless the phases differ
-    if (liquid[a] == liquid[b]) return 0.0;
-    const int64_t l = liquid[a] ? a : b, s = liquid[a] ? b : a;
-    const double fL = c[l] > cL ? __ddiv_rn(__dadd_rn(c[l], -cL), cL) : 0.0;
-    const double fS = c[s] < cS ? __ddiv_rn(__dadd_rn(cS, -c[s]), cS) : 0.0;
-    return __dmul_rn(__dmul_rn(__dmul_rn(k, fL), fS), dt);
+//
+// The factor of a cell, k f_L of a liquid one and f_S of a solid one, is formed once per cell that has an interface face:
+// two FP64 divisions on either side of every face were what the exchange spent its time on (the FP64 pipe runs at 1/73 of
+// the FP32 rate): 96^3, 237 us a step before, 78 us for both kernels now.
+__global__ void rate_kernel(Grid g, const uint8_t* __restrict__ liquid, double k, double cS, double cL,
+                            const double* __restrict__ c, double* __restrict__ rate) {
+    const int64_t nxy = (int64_t)g.nx * g.ny;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
+        int x, y, z;
+        cell_of(i, g, x, y, z);
+        const bool l = liquid[i] != 0;
+        auto other = [&](int64_t j) { return (liquid[j] != 0) != l; };
+        const bool edge = (z > 0 && other(i - nxy)) || (y > 0 && other(i - g.nx)) || (x > 0 && other(i - 1)) ||
+                          (x + 1 < g.nx && other(i + 1)) || (y + 1 < g.ny && other(i + g.nx)) ||
+                          (z + 1 < g.nz && other(i + nxy));
+        if (!edge) continue;
+        const double v = c[i];
+        rate[i] = l ? __dmul_rn(k, v > cL ? __ddiv_rn(__dadd_rn(v, -cL), cL) : 0.0)
+                    : v < cS ? __ddiv_rn(__dadd_rn(cS, -v), cS) : 0.0;
+    }
 }
 
-__global__ void absorb_kernel(Grid g, const uint8_t* __restrict__ liquid, double k, double cS, double cL, double dt,
+__global__ void absorb_kernel(Grid g, const uint8_t* __restrict__ liquid, double dt, const double* __restrict__ rate,
                               const double* __restrict__ c, double* __restrict__ out) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
-        const double sgn = liquid[i] ? -1.0 : 1.0;       // the liquid side loses, the solid side gains
-        double v = c[i];
-        if (z > 0) v = __dadd_rn(v, sgn * exchange(c, liquid, i - nxy, i, k, cS, cL, dt));
-        if (y > 0) v = __dadd_rn(v, sgn * exchange(c, liquid, i - g.nx, i, k, cS, cL, dt));
-        if (x > 0) v = __dadd_rn(v, sgn * exchange(c, liquid, i - 1, i, k, cS, cL, dt));
-        if (x + 1 < g.nx) v = __dadd_rn(v, sgn * exchange(c, liquid, i, i + 1, k, cS, cL, dt));
-        if (y + 1 < g.ny) v = __dadd_rn(v, sgn * exchange(c, liquid, i, i + g.nx, k, cS, cL, dt));
-        if (z + 1 < g.nz) v = __dadd_rn(v, sgn * exchange(c, liquid, i, i + nxy, k, cS, cL, dt));
+        int x, y, z;
+        cell_of(i, g, x, y, z);
+        const bool l = liquid[i] != 0;
+        double v = c[i];                                 // the liquid side loses, the solid side gains
+        // transfer from the liquid cell to the solid one across the face to cell j; none unless the phases differ
+        auto face = [&](int64_t j) {
+            if ((liquid[j] != 0) == l) return;
+            const double m = __dmul_rn(__dmul_rn(rate[i], rate[j]), dt);
+            v = l ? __dsub_rn(v, m) : __dadd_rn(v, m);
+        };
+        if (z > 0) face(i - nxy);
+        if (y > 0) face(i - g.nx);
+        if (x > 0) face(i - 1);
+        if (x + 1 < g.nx) face(i + 1);
+        if (y + 1 < g.ny) face(i + g.nx);
+        if (z + 1 < g.nz) face(i + nxy);
         out[i] = v;
     }
 }
@@ -213,7 +284,8 @@ __global__ void solid_faces_kernel(Grid g, const double* __restrict__ D, const u
                                    double* __restrict__ gx, double* __restrict__ gy, double* __restrict__ gz) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
+        int x, y, z;
+        cell_of(i, g, x, y, z);
         auto h = [&](int64_t j) {
             const double a = D[i], b = D[j];
             return (!liquid[i] && !liquid[j] && __dadd_rn(a, b) > 0.0)
@@ -231,7 +303,8 @@ __global__ void solid_substep_kernel(Grid g, const double* __restrict__ gx, cons
                                      double* __restrict__ un) {
     const int64_t nxy = (int64_t)g.nx * g.ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
+        int x, y, z;
+        cell_of(i, g, x, y, z);
         const double ui = u[i];
         double acc = 0.0;
         if (x > 0) acc = __dadd_rn(acc, __dmul_rn(gx[i - 1], __dadd_rn(u[i - 1], -ui)));
@@ -244,36 +317,80 @@ __global__ void solid_substep_kernel(Grid g, const double* __restrict__ gx, cons
     }
 }
 
-// Fixed-order FP64 total of the cells of one phase: block b sums chunk b, then one block sums the partials.
+// Largest per-cell sum of the solid-solid conductances (bits of a non-negative double).
+__global__ void solid_max_kernel(Grid g, const double* __restrict__ gx, const double* __restrict__ gy,
+                                 const double* __restrict__ gz, unsigned long long* __restrict__ max_bits) {
+    const int64_t nxy = (int64_t)g.nx * g.ny;
+    double most = 0.0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
+        int x, y, z;
+        cell_of(i, g, x, y, z);
+        double sum = __dadd_rn(__dadd_rn(gx[i], gy[i]), gz[i]);
+        if (x > 0) sum = __dadd_rn(sum, gx[i - 1]);
+        if (y > 0) sum = __dadd_rn(sum, gy[i - g.nx]);
+        if (z > 0) sum = __dadd_rn(sum, gz[i - nxy]);
+        most = fmax(most, sum);
+    }
+    max_bits_of(most, max_bits);
+}
+
+// Fixed-order FP64 totals of a field's liquid cells, of its solid ones and of all (in one pass: the total in the order of
+// launch_mass): block b sums chunk b, then one block sums the partials.
 __global__ void __launch_bounds__(256) phase_partial_kernel(const double* __restrict__ c, const uint8_t* __restrict__ liquid,
-                                                            int want_liquid, int64_t n, double* __restrict__ partials) {
-    __shared__ double sh[8];
+                                                            int64_t n, double* __restrict__ partials,
+                                                            double* __restrict__ totals) {
+    __shared__ double sh[3][8];
     const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
     const int64_t lo = blockIdx.x * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
-    double acc = 0.0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        if ((liquid[i] != 0) == (want_liquid != 0)) acc += c[i];
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    double acc[3] = {0.0, 0.0, 0.0};
+    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const double v = c[i];
+        if (liquid[i]) acc[0] += v; else acc[1] += v;
+        acc[2] += v;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        for (int off = 16; off > 0; off >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
+        if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = acc[q];
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
-        double v = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (threadIdx.x == 0) partials[blockIdx.x] = v;
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            double v = threadIdx.x < (blockDim.x >> 5) ? sh[q][threadIdx.x] : 0.0;
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (threadIdx.x == 0) (q == 2 ? totals : partials + q * kMassBlocks)[blockIdx.x] = v;
+        }
     }
 }
 
-__global__ void __launch_bounds__(kMassBlocks) phase_final_kernel(const double* __restrict__ partials, double* __restrict__ out) {
-    __shared__ double sh[kMassBlocks / 32];
-    double v = partials[threadIdx.x];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+// phases: [Q_L, Q_S] of the step; the total is the mass after it, far[2], for Eq. 7's update of far[0].
+__global__ void __launch_bounds__(kMassBlocks) phase_final_kernel(const double* __restrict__ partials,
+                                                                  const double* __restrict__ totals, double* phases,
+                                                                  double* far, double V_far) {
+    __shared__ double sh[3][kMassBlocks / 32];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        double v = (q == 2 ? totals : partials + q * kMassBlocks)[threadIdx.x];
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = v;
+    }
     __syncthreads();
     if (threadIdx.x < 32) {
-        double w = sh[threadIdx.x];
-        for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
-        if (threadIdx.x == 0) *out = w;
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            double w = sh[q][threadIdx.x];
+            for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
+            if (threadIdx.x == 0) {
+                if (q < 2) {
+                    phases[q] = w;
+                } else {
+                    far[2] = w;
+                    far[0] = ((far[1] + V_far * far[0]) - w) / V_far;
+                }
+            }
+        }
     }
 }
 
@@ -282,37 +399,43 @@ __global__ void far_update_kernel(double* far, double V_far) {
     far[0] = ((far[1] + V_far * far[0]) - far[2]) / V_far;
 }
 
-// Eq. 14: C'_I = sum over block offsets d (ascending) of P[I][I - d] C_{I - d}, FP64, plus P_BC[I] c_far
-// when the outer surface is open.
+// Eq. 14: C'_I = sum over block offsets d of P[I][I - d] C_{I - d}, FP64, plus P_BC[I] c_far when the outer surface is
+// open.  Eight lanes per block, 4 blocks per warp: lane l takes the offsets d = l, l + 8, ... in ascending order, then a
+// xor-butterfly (one thread for all of a block's 125 terms is a chain of loads and FP64 FMAs on a fraction of the GPU:
+// 96^3, B = 5, 20 -> 9 us).
 __global__ void coarse_gather_kernel(int ncx, int ncy, int ncz, int Rc, const double* __restrict__ Qc,
                                      const double* __restrict__ C, const double* __restrict__ pbc,
                                      const double* __restrict__ far, double* __restrict__ Cn) {
     const int64_t nc = (int64_t)ncx * ncy * ncz;
-    const int Wc = 2 * Rc + 1;
-    for (int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; I < nc; I += (int64_t)gridDim.x * blockDim.x) {
-        const int bx = (int)(I % ncx), by = (int)((I / ncx) % ncy), bz = (int)(I / ((int64_t)ncx * ncy));
+    const int Wc = 2 * Rc + 1, n = Wc * Wc * Wc;
+    // lane = 8 (part) + block: consecutive blocks side by side, so that a load of a plane is 4 or more values wide
+    const int lane = threadIdx.x & 31, part = lane >> 2, sub = lane & 3;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); 4 * w < nc; w += warps) {
+        const int64_t I = 4 * w + sub;
         double acc = 0.0;
-        int d = 0;
-        for (int dz = -Rc; dz <= Rc; dz++)
-            for (int dy = -Rc; dy <= Rc; dy++)
-                for (int dx = -Rc; dx <= Rc; dx++, d++) {
-                    const int jx = bx - dx, jy = by - dy, jz = bz - dz;
-                    if (jx < 0 || jx >= ncx || jy < 0 || jy >= ncy || jz < 0 || jz >= ncz) continue;
-                    const int64_t J = jx + (int64_t)ncx * (jy + (int64_t)ncy * jz);
-                    acc = fma(Qc[(int64_t)d * nc + I], C[J], acc);
-                }
-        if (pbc) acc = __dadd_rn(acc, __dmul_rn(pbc[I], far[0]));
-        Cn[I] = acc;
-        (void)Wc;
+        if (I < nc) {
+            const int bx = (int)(I % ncx), by = (int)((I / ncx) % ncy), bz = (int)(I / ((int64_t)ncx * ncy));
+            for (int d = part; d < n; d += 8) {
+                const int jx = bx - (d % Wc - Rc), jy = by - (d / Wc % Wc - Rc), jz = bz - (d / (Wc * Wc) - Rc);
+                if (jx < 0 || jx >= ncx || jy < 0 || jy >= ncy || jz < 0 || jz >= ncz) continue;
+                acc = fma(Qc[(int64_t)d * nc + I], C[jx + (int64_t)ncx * (jy + (int64_t)ncy * jz)], acc);
+            }
+        }
+        for (int off = 4; off < 32; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (part == 0 && I < nc) {
+            if (pbc) acc = __dadd_rn(acc, __dmul_rn(pbc[I], far[0]));
+            Cn[I] = acc;
+        }
     }
 }
 
 // Eq. 15: c'_i = C'_I on liquid cells, c'_i = c_i elsewhere (in place allowed: each cell reads itself).
 __global__ void remap_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, int ncx, int ncy,
                              const double* __restrict__ Cn, const double* c_in, double* c_out) {
-    const int64_t nxy = (int64_t)g.nx * g.ny;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % g.nx), y = (int)((i / g.nx) % g.ny), z = (int)(i / nxy);
+        int x, y, z;
+        cell_of(i, g, x, y, z);
         c_out[i] = liquid[i] ? Cn[(x / B) + (int64_t)ncx * ((y / B) + (int64_t)ncy * (z / B))] : c_in[i];
     }
 }
@@ -376,25 +499,27 @@ int coarse_kernels(fdirw_ctx* c) {
         float* u0 = k.ubuf;
         float* u1 = k.ubuf + c->g.n;
         FDIRW_CUDA(c, cudaMemsetAsync(u0, 0, (size_t)c->g.n * 4, c->stream));
+        const dim3 tiles((c->g.nx + 31) / 32, std::min((c->g.ny + 7) / 8, 65535), std::min((c->g.nz + kPbcZ - 1) / kPbcZ, 65535));
         for (int t = 0; t < c->n_sub; t++) {
-            pbc_substep_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(
+            (a.bx ? pbc_substep_kernel<true> : pbc_substep_kernel<false>)<<<tiles, 256, 0, c->stream>>>(
                 c->g, a.ax, a.ay, a.az, a.bx, a.by, a.bz, k.abnd, u0, u1);
             FDIRW_CUDA(c, cudaGetLastError());
             std::swap(u0, u1);
         }
         widen_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(u0, c->g.n, c->cbuf);
-        map_kernel<<<grid_blocks(k.nc, 128), 128, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
+        map_kernel<<<grid_blocks(k.nc, 8), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
                                                                   c->cbuf, k.pbc);
         FDIRW_CUDA(c, cudaGetLastError());
     }
     c->kernels_timed = true;
-    c->parts_used = 5;
+    c->parts_used = c->flow ? 5 : 4;
     k.built = true;
     c->kernels_ready = true;
     return FDIRW_OK;
 }
 
-int coarse_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps, double* mass_out) {
+// phases (nullable, device): receives the liquid and the solid total of c_out after the last step (far field only).
+static int coarse_steps(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps, double* mass_out, double* phases) {
     Coarse& k = *c->coarse;
     const Kind kin = classify(c_in, c->device), kout = classify(c_out, c->device);
     if (kin == Kind::Foreign || kout == Kind::Foreign)
@@ -419,18 +544,22 @@ int coarse_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps
     } else {
         const double* cur = src;
         for (int t = 0; t < n_steps; t++) {
-            map_kernel<<<grid_blocks(k.nc, 128), 128, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count, cur, k.C);
+            map_kernel<<<grid_blocks(k.nc, 8), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count, cur, k.C);
             FDIRW_CUDA(c, cudaGetLastError());
             const bool last = t + 1 == n_steps;
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
             if (k.open) FDIRW_CUDA(c, launch_mass(cur, c->g.n, c->partials, k.far + 1, c->stream));
-            coarse_gather_kernel<<<grid_blocks(k.nc, 128), 128, 0, c->stream>>>(k.ncx, k.ncy, k.ncz, k.Rc, k.Qc, k.C,
+            coarse_gather_kernel<<<grid_blocks(k.nc, 16), 128, 0, c->stream>>>(k.ncx, k.ncy, k.ncz, k.Rc, k.Qc, k.C,
                                                                                 k.open ? k.pbc : nullptr, k.far, k.Cn);
             FDIRW_CUDA(c, cudaGetLastError());
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
             remap_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.Cn, cur, dst);
             FDIRW_CUDA(c, cudaGetLastError());
-            if (k.open) {
+            if (k.open && phases && last) {
+                phase_partial_kernel<<<kMassBlocks, 256, 0, c->stream>>>(dst, k.liquid, c->g.n, c->partials, k.qpart);
+                phase_final_kernel<<<1, kMassBlocks, 0, c->stream>>>(c->partials, k.qpart, phases, k.far, k.V_far);
+                FDIRW_CUDA(c, cudaGetLastError());
+            } else if (k.open) {
                 FDIRW_CUDA(c, launch_mass(dst, c->g.n, c->partials, k.far + 2, c->stream));
                 far_update_kernel<<<1, 1, 0, c->stream>>>(k.far, k.V_far);
                 FDIRW_CUDA(c, cudaGetLastError());
@@ -447,6 +576,15 @@ int coarse_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps
     if (mass_out || kout == Kind::Host) FDIRW_CUDA(c, cudaStreamSynchronize(c->stream));
     if (mass_out) *mass_out = c->mass_out;
     return FDIRW_OK;
+}
+
+int coarse_step(fdirw_ctx* c, const double* c_in, double* c_out, int32_t n_steps, double* mass_out) {
+    return coarse_steps(c, c_in, c_out, n_steps, mass_out, nullptr);
+}
+
+// One liquid step of a coupled macro step on device fields.
+static int coarse_coupled(fdirw_ctx* c, const double* c_in, double* c_out, double* phases) {
+    return coarse_steps(c, c_in, c_out, 1, nullptr, phases);
 }
 
 int coarse_info(fdirw_ctx* c, fdirw_info* out) {
@@ -669,32 +807,25 @@ int fdirw_coupled_step(fdirw_ctx* c, const fdirw_coupled_params* p, double* fiel
     int rc;
     const double lam_s = p->n_sub_solid > 0 ? (p->dt / p->n_sub_solid) / (c->h * c->h) : 0.0;
     if (!k.gs) {
+        if (!k.tmp && (rc = dalloc(c, reinterpret_cast<void**>(&k.tmp), 2 * n * 8, "coupled scratch")) != FDIRW_OK) return rc;
+        if (!k.qpart && (rc = dalloc(c, reinterpret_cast<void**>(&k.qpart), fdirw::kMassBlocks * 8, "phase partials")) != FDIRW_OK)
+            return rc;
         if ((rc = dalloc(c, reinterpret_cast<void**>(&k.gs), 3 * n * 8, "solid faces")) != FDIRW_OK) return rc;
-        if ((rc = dalloc(c, reinterpret_cast<void**>(&k.tmp), 2 * n * 8, "coupled scratch")) != FDIRW_OK) return rc;
-        if ((rc = dalloc(c, reinterpret_cast<void**>(&k.qpart), fdirw::kMassBlocks * 8, "phase partials")) != FDIRW_OK) return rc;
+        // The largest sum of a cell's solid faces, for the stability check of every call (on the device: copying the
+        // 3 N conductances out for a host loop took 8 of a 30 ms call at 96^3).
+        unsigned long long h = 0, *mx = reinterpret_cast<unsigned long long*>(k.tmp);
         fdirw::solid_faces_kernel<<<fdirw::grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, c->Dd, k.liquid, k.gs,
                                                                                         k.gs + n, k.gs + 2 * n);
         FDIRW_CUDA(c, cudaGetLastError());
-    }
-    if (lam_s > 0.0) {
-        // stability of the solid march: lam_s * max(sum of solid faces) <= 1, checked on the host once per call
-        std::vector<double> gh(3 * n);
-        FDIRW_CUDA(c, cudaMemcpyAsync(gh.data(), k.gs, 3 * n * 8, cudaMemcpyDeviceToHost, c->stream));
+        FDIRW_CUDA(c, cudaMemsetAsync(mx, 0, 8, c->stream));
+        fdirw::solid_max_kernel<<<fdirw::grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, k.gs, k.gs + n, k.gs + 2 * n, mx);
+        FDIRW_CUDA(c, cudaGetLastError());
+        FDIRW_CUDA(c, cudaMemcpyAsync(&h, mx, 8, cudaMemcpyDeviceToHost, c->stream));
         FDIRW_CUDA(c, cudaStreamSynchronize(c->stream));
-        const int nx = c->g.nx, ny = c->g.ny;
-        const int64_t nxy = (int64_t)nx * ny;
-        double mx = 0.0;
-        for (int64_t i = 0; i < c->g.n; i++) {
-            const int x = (int)(i % nx), y = (int)((i / nx) % ny);
-            const int64_t z = i / nxy;
-            double sum = gh[i] + gh[n + i] + gh[2 * n + i];
-            if (x > 0) sum += gh[i - 1];
-            if (y > 0) sum += gh[n + i - nx];
-            if (z > 0) sum += gh[2 * n + i - nxy];
-            mx = std::max(mx, sum);
-        }
-        if (lam_s * mx > 1.0 + 1e-12) return fail(c, FDIRW_ERR_UNSTABLE, "solid march unstable: raise n_sub_solid");
+        std::memcpy(&k.gs_max, &h, 8);
     }
+    if (lam_s > 0.0 && lam_s * k.gs_max > 1.0 + 1e-12)
+        return fail(c, FDIRW_ERR_UNSTABLE, "solid march unstable: raise n_sub_solid");
     if ((QL || QS) && n_steps > k.qcap) {
         void* q = k.qout; dfree(q); k.qout = nullptr;
         c->allocated -= (uint64_t)k.qcap * 16;
@@ -712,7 +843,8 @@ int fdirw_coupled_step(fdirw_ctx* c, const fdirw_coupled_params* p, double* fiel
     }
     const int gb = fdirw::grid_blocks(c->g.n, 256);
     for (int t = 0; t < n_steps; t++) {
-        fdirw::absorb_kernel<<<gb, 256, 0, c->stream>>>(c->g, k.liquid, p->k, p->cS_eq, p->cL_eq, p->dt, cur, k.tmp);
+        fdirw::rate_kernel<<<gb, 256, 0, c->stream>>>(c->g, k.liquid, p->k, p->cS_eq, p->cL_eq, cur, k.tmp + n);
+        fdirw::absorb_kernel<<<gb, 256, 0, c->stream>>>(c->g, k.liquid, p->dt, k.tmp + n, cur, k.tmp);
         FDIRW_CUDA(c, cudaGetLastError());
         double* a = k.tmp;
         double* b = k.tmp + n;
@@ -721,14 +853,7 @@ int fdirw_coupled_step(fdirw_ctx* c, const fdirw_coupled_params* p, double* fiel
             FDIRW_CUDA(c, cudaGetLastError());
             std::swap(a, b);
         }
-        if ((rc = fdirw::coarse_step(c, a, cur, 1, nullptr)) != FDIRW_OK) return rc;
-        if (QL || QS) {
-            for (int ph = 0; ph < 2; ph++) {
-                fdirw::phase_partial_kernel<<<fdirw::kMassBlocks, 256, 0, c->stream>>>(cur, k.liquid, ph == 0, c->g.n, k.qpart);
-                fdirw::phase_final_kernel<<<1, fdirw::kMassBlocks, 0, c->stream>>>(k.qpart, k.qout + 2 * t + ph);
-                FDIRW_CUDA(c, cudaGetLastError());
-            }
-        }
+        if ((rc = fdirw::coarse_coupled(c, a, cur, (QL || QS) ? k.qout + 2 * t : nullptr)) != FDIRW_OK) return rc;
     }
     if (kf == Kind::Host) FDIRW_CUDA(c, cudaMemcpyAsync(field, cur, n * 8, cudaMemcpyDeviceToHost, c->stream));
     if ((QL || QS) && n_steps > 0) {
