@@ -9,7 +9,8 @@
 //     the x/y neighbours are read from a double-buffered shared-memory copy of every column (one
 //     __syncthreads per substep);
 //   - the FP64 path (the plain FP64 baseline) keeps u and the diagonal in registers and the face
-//     coefficients in shared memory (FP64 registers would not fit), same exchange scheme;
+//     coefficients in shared memory (FP64 registers would not fit), same exchange scheme, on the part of the window
+//     that lies in the domain;
 //   - after the march each thread rounds its cells to the storage type, writes them into the
 //     destination-indexed cache Q[o][s + o] and sums the stored values (FP32 path: as 64-bit integers, FP64
 //     path: in FP64 in a fixed order); sigma_s = 1 / sum.
@@ -188,6 +189,12 @@ __global__ void __launch_bounds__(Map32<R, P>::THREADS, Map32<R, P>::MIN_BLOCKS)
     }
 }
 
+// The FP64 march.  Bound by the FP64 pipe (1/73 of the FP32 rate), so it computes no cell it need not: the threads of a
+// batch are dealt out over the window columns that lie in the domain (the first threads to the first source's columns, and
+// so on; warps past the last one idle), a column runs over its levels in the domain, and during the first substeps over
+// those the source has reached (a substep moves a value one cell: |dx| + |dy| + |dz| <= substeps; the rest is still 0).
+// The cells that are computed see the same operations in the same order.  36^3, R = 6, 120 substeps: 148 -> 114 ms; 20^3,
+// R = 8, 60 substeps: 31.0 -> 15.7 ms; 64^3, R = 6, 30 substeps: 217 -> 176 ms.
 template <int R>
 __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(MarchArgs a) {
     using S = Shape<R>;
@@ -199,100 +206,121 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
     double* fy = fx + BUF;                                 // +y
     double* fz = fy + BUF;                                 // +z
     double* red = fz + BUF;                                // [SPB*COLS]
+    // Window of each source of the batch within the domain: first window column and widths, levels [k0, k1), threads
+    // before it.
+    __shared__ int c0x[SPB], c0y[SPB], wx[SPB], wxy[SPB], k0s[SPB], k1s[SPB], src[SPB][3], before[SPB + 1];
 
     const int t = threadIdx.x;
-    const bool active = t < SPB * COLS;
-    const int slot = active ? t / COLS : 0;
-    const int col = active ? t - slot * COLS : 0;
-    const int ci = col % W1, cj = col / W1;
     const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
     const int64_t nxy = (int64_t)nx * ny;
     int64_t none = 0;
     const SrcLoc L = locate(a, false, none);
     const int64_t nbatch = (a.src_end - a.src_begin + SPB - 1) / SPB;
 
-    const int base = (slot * COLS + col) * W1;
-    const int xm = ci > 0 ? base - W1 : base;
-    const int xp = ci < 2 * R ? base + W1 : base;
-    const int ym = cj > 0 ? base - W1 * W1 : base;
-    const int yp = cj < 2 * R ? base + W1 * W1 : base;
+    // Columns outside the domain are not written: what lies there meets zero faces and has to be finite.
+    for (int i = t; i < 2 * BUF; i += blockDim.x) xbuf[i] = 0.0;
 
     for (int64_t b = blockIdx.x; b < nbatch; b += gridDim.x) {
         const int64_t first = a.src_begin + b * SPB;
-        int64_t s = first + slot;
-        const bool src_ok = active && s < a.src_end;
-        if (src_ok && a.list) s = a.list[s];       // explicit source list (e.g. the surrogate's rejects)
-        int sx = 0, sy = 0, sz = 0;
-        if (src_ok) {
-            sx = (int)(s % nx);
-            const int64_t r = s / nx;
-            sy = (int)(r % ny);
-            sz = (int)(r / ny);
+        if (t < SPB) {
+            int64_t s = first + t;
+            int n = 0;
+            if (s < a.src_end) {
+                if (a.list) s = a.list[s];         // explicit source list (e.g. the surrogate's rejects)
+                int sx, sy, sz;
+                split_cell(s, nx, ny, sx, sy, sz);
+                c0x[t] = max(R - sx, 0);
+                c0y[t] = max(R - sy, 0);
+                wx[t] = min(nx - 1 - sx, R) + R - c0x[t] + 1;
+                k0s[t] = max(R - sz, 0);
+                k1s[t] = min(nz - 1 - sz, R) + R + 1;
+                src[t][0] = sx; src[t][1] = sy; src[t][2] = sz;
+                n = wx[t] * (min(ny - 1 - sy, R) + R - c0y[t] + 1);
+            }
+            wxy[t] = n;
         }
-        const int x = sx - R + ci, y = sy - R + cj;
-        const bool col_ok = src_ok && x >= 0 && x < nx && y >= 0 && y < ny;
+        __syncthreads();
+        if (t <= SPB) {
+            int n = 0;
+#pragma unroll 8
+            for (int q = 0; q < t; q++) n += wxy[q];
+            before[t] = n;
+        }
+        for (int i = t; i < SPB * COLS; i += blockDim.x) red[i] = 0.0;
+        __syncthreads();
+        const bool own = t < before[SPB];
+        int slot = own ? t / COLS : 0;                           // no source has more than COLS columns
+        while (own && t >= before[slot + 1]) slot++;
+        const int c = own ? t - before[slot] : 0, w = own ? wx[slot] : 1;
+        const int cj = own ? c0y[slot] + c / w : 0, ci = own ? c0x[slot] + c % w : 0;
+        const int base = (slot * COLS + cj * W1 + ci) * W1;
+        const int sz = src[slot][2], x = src[slot][0] - R + ci, y = src[slot][1] - R + cj;
+        const int k0 = own ? k0s[slot] : 0, k1 = own ? k1s[slot] : 0;
+        const bool left = ci > 0 && x > 0, front = cj > 0 && y > 0;      // a lower neighbour in the window and the domain
+        const int xm = left ? base - W1 : base, xp = ci < 2 * R ? base + W1 : base;
+        const int ym = front ? base - W1 * W1 : base, yp = cj < 2 * R ? base + W1 * W1 : base;
 
         double u[W1];
 #pragma unroll
         for (int k = 0; k < W1; k++) {
-            const int z = sz - R + k;
-            const bool ok = col_ok && z >= 0 && z < nz;
-            double vxp = 0.0, vyp = 0.0, vz = 0.0;
-            if (ok) {
+            u[k] = own && ci == R && cj == R && k == R ? 1.0 : 0.0;
+            if (k >= k0 && k < k1) {
+                const int z = sz - R + k;
                 const int64_t i = (int64_t)x + (int64_t)nx * y + nxy * z;
-                if (ci < 2 * R && x + 1 < nx) vxp = __ldg(a.dx + i);
-                if (cj < 2 * R && y + 1 < ny) vyp = __ldg(a.dy + i);
-                if (k < 2 * R && z + 1 < nz) vz = __ldg(a.dz + i);
+                fx[base + k] = ci < 2 * R && x + 1 < nx ? __ldg(a.dx + i) : 0.0;
+                fy[base + k] = cj < 2 * R && y + 1 < ny ? __ldg(a.dy + i) : 0.0;
+                fz[base + k] = k < 2 * R && z + 1 < nz ? __ldg(a.dz + i) : 0.0;
             }
-            if (active) { fx[base + k] = vxp; fy[base + k] = vyp; fz[base + k] = vz; }
-            u[k] = (src_ok && ci == R && cj == R && k == R) ? 1.0 : 0.0;
         }
         __syncthreads();
         double a0[W1];
 #pragma unroll
         for (int k = 0; k < W1; k++) {
-            const double vxm = ci > 0 ? fx[xm + k] : 0.0;
-            const double vym = cj > 0 ? fy[ym + k] : 0.0;
-            const double vzm = k > 0 ? fz[base + k - 1] : 0.0;
-            a0[k] = 1.0 - (((vxm + fx[base + k]) + (vym + fy[base + k])) + (vzm + fz[base + k]));
+            a0[k] = 0.0;
+            if (k >= k0 && k < k1) {
+                const double vxm = left ? fx[xm + k] : 0.0;
+                const double vym = front ? fy[ym + k] : 0.0;
+                const double vzm = k > k0 ? fz[base + k - 1] : 0.0;
+                a0[k] = 1.0 - (((vxm + fx[base + k]) + (vym + fy[base + k])) + (vzm + fz[base + k]));
+            }
         }
 
+        const int lateral = abs(ci - R) + abs(cj - R);
         for (int it = 0; it < a.n_sub; it++) {
             double* buf = xbuf + (it & 1) * BUF;
-            if (active) {
 #pragma unroll
-                for (int k = 0; k < W1; k++) buf[base + k] = u[k];
-            }
+            for (int k = 0; k < W1; k++)
+                if (k >= k0 && k < k1) buf[base + k] = u[k];
             __syncthreads();
+            const int reach = it + 1 - lateral;                  // levels reached by the end of this substep
+            const int ka = max(k0, R - reach), kb = min(k1, R + reach + 1);
             double prev = 0.0;
 #pragma unroll
             for (int k = 0; k < W1; k++) {
+                if (k < ka || k >= kb) continue;
                 const double cur = u[k];
                 double v = a0[k] * cur;
-                if (ci > 0) v = fma(fx[xm + k], buf[xm + k], v);
+                if (left) v = fma(fx[xm + k], buf[xm + k], v);
                 v = fma(fx[base + k], buf[xp + k], v);
-                if (cj > 0) v = fma(fy[ym + k], buf[ym + k], v);
+                if (front) v = fma(fy[ym + k], buf[ym + k], v);
                 v = fma(fy[base + k], buf[yp + k], v);
-                if (k > 0) v = fma(fz[base + k - 1], prev, v);
-                if (k + 1 < W1) v = fma(fz[base + k], u[k + 1], v);
+                if (k > k0) v = fma(fz[base + k - 1], prev, v);
+                if (k + 1 < W1) v = fma(fz[base + k], u[k + 1 < W1 ? k + 1 : k], v);
                 prev = cur;
                 u[k] = v;
             }
         }
 
         double colsum = 0.0;
-        if (col_ok) {
 #pragma unroll
-            for (int k = 0; k < W1; k++) {
-                const int z = sz - R + k;
-                if (z >= 0 && z < nz) {
-                    if (a.dest_z1 <= a.dest_z0 || (z >= a.dest_z0 && z < a.dest_z1))
-                        reinterpret_cast<double*>(a.Q)[qplane(a, R, ci, cj, k) * a.q_stride + qcol(a, L, x, y, z, 0)] = u[k];
-                    colsum += u[k];
-                }
-            }
+        for (int k = 0; k < W1; k++) {
+            if (k < k0 || k >= k1) continue;
+            const int z = sz - R + k;
+            if (a.dest_z1 <= a.dest_z0 || (z >= a.dest_z0 && z < a.dest_z1))
+                reinterpret_cast<double*>(a.Q)[qplane(a, R, ci, cj, k) * a.q_stride + qcol(a, L, x, y, z, 0)] = u[k];
+            colsum += u[k];
         }
-        if (active) red[t] = colsum;
+        if (own) red[slot * COLS + cj * W1 + ci] = colsum;
         __syncthreads();
         finish_sigma<COLS, SPB>(red, first, a.src_end, a.list, a.sigma);
         __syncthreads();
