@@ -80,6 +80,8 @@ struct MarchArgs {
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st);
 // Mapping 4 of the FP32 march (2x2 column blocks, march_tm.cu), R in 1..10.
 cudaError_t launch_march_blocks(const MarchArgs& a, int num_sms, cudaStream_t st);
+// The march of sources with direction-dependent faces (a.bx; reported as mapping 5, march_flow.cu), R in 1..10.
+cudaError_t launch_march_flow(const MarchArgs& a, int num_sms, cudaStream_t st);
 // parts_req: FP32 march thread mapping (1..3 threads per window column, 4 = 2x2 column blocks with TMEM
 // coefficients, 5 = one column per thread with TMEM lateral faces, 6 = source pairs, 7 = column pairs), or 0 for
 // the fastest one of the radius; parts_used receives the mapping launched.

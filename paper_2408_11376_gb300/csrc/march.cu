@@ -1077,7 +1077,7 @@ cudaError_t launch_f32_p(const MarchArgs& a, int P, int num_sms, cudaStream_t st
         case 2: return launch_f32<R, 2>(a, num_sms, st);
         case 3: return launch_f32<R, 3>(a, num_sms, st);
         case 4: return launch_march_blocks(a, num_sms, st);
-        case 5: return a.bx ? launch_tmc<R, false, true>(a, num_sms, st) : launch_tmc<R>(a, num_sms, st);
+        case 5: return a.bx ? launch_march_flow(a, num_sms, st) : launch_tmc<R>(a, num_sms, st);
         case 6: return launch_tmp<R>(a, num_sms, st);
         case 7: return launch_tmx<R>(a, num_sms, st);
         default: return cudaErrorInvalidValue;
@@ -1125,10 +1125,10 @@ cudaError_t dispatch(const MarchArgs& a, int P, int num_sms, cudaStream_t st) {
         case 6: return launch_f32_p<6>(a, P, num_sms, st);
         case 7: return launch_f32_p<7>(a, P, num_sms, st);
         case 8: return launch_f32_p<8>(a, P, num_sms, st);
-        case 9: return P == 5 ? (a.bx ? launch_tmc<9, false, true>(a, num_sms, st) : launch_tmc<9>(a, num_sms, st))
+        case 9: return P == 5 ? (a.bx ? launch_march_flow(a, num_sms, st) : launch_tmc<9>(a, num_sms, st))
                        : P == 4 ? launch_march_blocks(a, num_sms, st) : P == 7 ? launch_tmx<9>(a, num_sms, st)
                        : cudaErrorInvalidValue;
-        case 10: return P == 5 ? (a.bx ? launch_tmc<10, false, true>(a, num_sms, st) : launch_tmc<10>(a, num_sms, st))
+        case 10: return P == 5 ? (a.bx ? launch_march_flow(a, num_sms, st) : launch_tmc<10>(a, num_sms, st))
                         : P == 4 ? launch_march_blocks(a, num_sms, st) : P == 7 ? launch_tmx<10>(a, num_sms, st)
                         : cudaErrorInvalidValue;
         default: return cudaErrorInvalidValue;

@@ -204,6 +204,51 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return d;
 }
 
+// Where the stored values of one source of a CTA batch go (written by the source's first thread, read by
+// every thread of the CTA in the epilogue).
+struct SlotInfo {
+    SrcLoc L;
+    int64_t pos;
+    int sx, sy, sz, ok;
+};
+
+// The cache stores of a CTA's batch, one window column of one source per thread and round, the batch's sources fastest:
+// they have adjacent destinations in a plane, so one warp store covers about 32 / SPB planes.  Along a column both
+// addresses advance by a constant (a plane of the cache and one of the grid).  u(x, y, k, slot): the marched value.
+template <int R, int SPB, int THREADS, typename F>
+__device__ __forceinline__ void store_columns(const MarchArgs& a, const SlotInfo* sinfo, F u) {
+    constexpr int W1 = 2 * R + 1;
+    for (int e = threadIdx.x; e < W1 * W1 * SPB; e += THREADS) {
+        const int c = e / SPB, sl = e - c * SPB, y = c / W1, x = c - y * W1;
+        const SlotInfo si = sinfo[sl];
+        const int cx = si.sx - R + x, cy = si.sy - R + y, z0 = si.sz - R;
+        if (!si.ok || cx < 0 || cx >= si.L.nx || cy < 0 || cy >= si.L.ny) continue;
+        int k0 = z0 < 0 ? -z0 : 0, k1 = si.L.nz - z0 < W1 ? si.L.nz - z0 : W1;      // levels in the domain
+        if (a.dest_z1 > a.dest_z0) {               // slab of z-planes: only its levels are stored
+            k0 = max(k0, a.dest_z0 - z0);
+            k1 = min(k1, a.dest_z1 - z0);
+        }
+        const int64_t at = qplane(a, R, x, y, 0) * a.q_stride + qcol(a, si.L, cx, cy, z0, si.pos);   // of level 0
+        const int64_t step = (qplane(a, R, 0, 0, 1) - qplane(a, R, 0, 0, 0)) * a.q_stride +
+                             (a.src_major ? 0 : (int64_t)si.L.qnx * si.L.ny);
+        if (a.store == Store::F32) {
+            float* q = reinterpret_cast<float*>(a.Q) + at;
+#pragma unroll
+            for (int k = 0; k < W1; k++, q += step)
+                if (k >= k0 && k < k1) *q = u(x, y, k, sl);
+        } else {
+            uint16_t* q = reinterpret_cast<uint16_t*>(a.Q) + at;
+            const bool half = a.store == Store::F16;
+#pragma unroll
+            for (int k = 0; k < W1; k++, q += step)
+                if (k >= k0 && k < k1) {
+                    const float v = u(x, y, k, sl);
+                    *q = half ? __half_as_ushort(__float2half_rn(v)) : __bfloat16_as_ushort(__float2bfloat16_rn(v));
+                }
+        }
+    }
+}
+
 // Coarse epilogue (Eq. 11 applied to the marched unit of block J): S[d] = FP64 sum of the marched field
 // over the liquid cells of block J + d inside the window (z, y, x order; u is 0 elsewhere), m =
 // sum of S in a fixed order, and column J of P: Qc[d][J + d] = N_J S[d] / (m N_{J+d}), or S[d] / N_{J+d}

@@ -39,14 +39,6 @@ namespace fdirw {
 
 namespace {
 
-// Where the stored values of one source of a CTA batch go (written by the source's first thread, read by
-// every thread of the CTA in the epilogue).
-struct SlotInfo {
-    SrcLoc L;
-    int64_t pos;
-    int sx, sy, sz, ok;
-};
-
 template <int R>
 struct MapTm {
     static constexpr int W1 = 2 * R + 1;
@@ -444,40 +436,10 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
             }
             red[(K0 > 0 ? PT : 0) + th] = m.total();
         }
-        // The cache stores, one window column of one source per thread and round, the batch's sources fastest:
-        // they have adjacent destinations in a plane, so one warp store covers about 32 / SPB planes.  Along a
-        // column both addresses advance by a constant (a plane of the cache and one of the grid).
         const float* ubuf = xbuf + (a.n_sub & 1) * M::BUF;
-        for (int e = t; e < W1 * W1 * SPB; e += M::THREADS) {
-            const int c = e / SPB, sl = e - c * SPB, y = c / W1, x = c - y * W1;
-            const SlotInfo si = sinfo[sl];
-            const int cx = si.sx - R + x, cy = si.sy - R + y, z0 = si.sz - R;
-            if (!si.ok || !in(cx, si.L.nx) || !in(cy, si.L.ny)) continue;
-            int k0 = z0 < 0 ? -z0 : 0, k1 = si.L.nz - z0 < W1 ? si.L.nz - z0 : W1;  // levels in the domain
-            if (a.dest_z1 > a.dest_z0) {           // slab of z-planes: only its levels are stored
-                k0 = max(k0, a.dest_z0 - z0);
-                k1 = min(k1, a.dest_z1 - z0);
-            }
-            const int64_t at = qplane(a, R, x, y, 0) * a.q_stride + qcol(a, si.L, cx, cy, z0, si.pos);   // of level 0
-            const int64_t step = (qplane(a, R, 0, 0, 1) - qplane(a, R, 0, 0, 0)) * a.q_stride +
-                                 (a.src_major ? 0 : (int64_t)si.L.qnx * si.L.ny);
-            const int sc = (x & 1) + 2 * (y & 1), own = sl * TPS + (x >> 1) + NB * (y >> 1);
-            if (a.store == Store::F32) {
-                float* q = reinterpret_cast<float*>(a.Q) + at;
-#pragma unroll
-                for (int k = 0; k < W1; k++, q += step)
-                    if (k >= k0 && k < k1) *q = ubuf[level_at<R>(k, sc, own)];
-            } else {
-                uint16_t* q = reinterpret_cast<uint16_t*>(a.Q) + at;
-                const bool half = a.store == Store::F16;
-#pragma unroll
-                for (int k = 0; k < W1; k++, q += step)
-                    if (k >= k0 && k < k1) {
-                        const float v = ubuf[level_at<R>(k, sc, own)];
-                        *q = half ? __half_as_ushort(__float2half_rn(v)) : __bfloat16_as_ushort(__float2bfloat16_rn(v));
-                    }
-            }
-        }
+        store_columns<R, SPB, M::THREADS>(a, sinfo, [&](int x, int y, int k, int sl) {
+            return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), sl * TPS + (x >> 1) + NB * (y >> 1))];
+        });
         bar();                                     // red is complete; sinfo and xbuf are free for the next batch
         finish_sigma<TPS, SPB, M::ZS, PT>(red, first, a.src_end, a.list, a.sigma);
     }
