@@ -9,7 +9,11 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <deque>
+#include <mutex>
 #include <string>
+#include <unordered_map>
+#include <vector>
 
 using fdirw::Grid;
 using fdirw::Store;
@@ -43,13 +47,109 @@ bool grid_ok(const fdirw_grid* g) {
            (double)g->nx * g->ny * g->nz < 9.0e15;
 }
 
+namespace {
+
+// Device blocks that contexts have freed, kept for the next ones: a small structure's run from create to destroy spent as
+// long in 15 cudaMalloc and 15 cudaFree calls (each free waits for the whole device) as in half of its kernels (32^3: 225
+// of 954 us).  Bounded: blocks up to 64 MB, 256 MB in all, the oldest given back to the driver beyond that, and all of
+// them when an allocation fails.  A block comes here only when no work uses it any more (its context's stream has been
+// waited for), so the next owner may use it on any stream.  Locked: contexts of several threads share it.
+class BlockPool {
+  public:
+    // An idle block of the device that holds `bytes` without wasting a quarter of them; nullptr: none.
+    void* take(int device, uint64_t bytes) {
+        if (bytes > kBlock) return nullptr;
+        std::lock_guard<std::mutex> lk(mu_);
+        auto best = idle_.end();
+        for (auto it = idle_.begin(); it != idle_.end(); ++it)
+            if (it->device == device && it->bytes >= bytes && it->bytes <= bytes + bytes / 4 + 512 &&
+                (best == idle_.end() || it->bytes < best->bytes))
+                best = it;
+        if (best == idle_.end()) return nullptr;
+        void* p = best->p;
+        live_[p] = *best;
+        idle_bytes_ -= best->bytes;
+        idle_.erase(best);
+        return p;
+    }
+    // A block fresh from the driver.
+    void hand_out(void* p, int device, uint64_t bytes) {
+        if (bytes > kBlock) return;
+        std::lock_guard<std::mutex> lk(mu_);
+        live_[p] = Block{p, bytes, device};
+    }
+    // Takes a block back; false: not one to keep.
+    bool keep(void* p) {
+        std::vector<void*> out;
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            auto it = live_.find(p);
+            if (it == live_.end()) return false;
+            idle_.push_back(it->second);
+            idle_bytes_ += it->second.bytes;
+            live_.erase(it);
+            while (idle_bytes_ > kTotal) {
+                out.push_back(idle_.front().p);
+                idle_bytes_ -= idle_.front().bytes;
+                idle_.pop_front();
+            }
+        }
+        for (void* q : out) cudaFree(q);
+        return true;
+    }
+    // Gives every idle block back; whether there were any.
+    bool trim() {
+        std::deque<Block> out;
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            out.swap(idle_);
+            idle_bytes_ = 0;
+        }
+        for (const Block& b : out) cudaFree(b.p);
+        return !out.empty();
+    }
+    uint64_t idle_on(int device) {
+        std::lock_guard<std::mutex> lk(mu_);
+        uint64_t n = 0;
+        for (const Block& b : idle_) if (b.device == device) n += b.bytes;
+        return n;
+    }
+
+  private:
+    static constexpr uint64_t kBlock = 64ull << 20, kTotal = 256ull << 20;
+    struct Block {
+        void* p;
+        uint64_t bytes;
+        int device;
+    };
+    std::mutex mu_;
+    std::unordered_map<void*, Block> live_;
+    std::deque<Block> idle_;                     // oldest first
+    uint64_t idle_bytes_ = 0;
+};
+
+BlockPool& pool() {
+    static BlockPool* p = new BlockPool();       // outlives every context (and the driver's own teardown)
+    return *p;
+}
+
+}  // namespace
+
 int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what) {
     *p = nullptr;
     if (bytes == 0) return FDIRW_OK;
     if (c->mem_limit && c->allocated + bytes > c->mem_limit)
         return fail(c, FDIRW_ERR_NOMEM, std::string("allocating ") + what + " (" + std::to_string(bytes) +
                                             " bytes) would exceed mem_limit " + std::to_string(c->mem_limit));
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = cudaSuccess;
+    if ((*p = pool().take(c->device, bytes)) == nullptr) {
+        e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation && pool().trim()) {
+            cudaGetLastError();
+            e = cudaMalloc(p, bytes);
+        }
+        if (e == cudaSuccess) pool().hand_out(*p, c->device, bytes);
+    }
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         *p = nullptr;
@@ -60,10 +160,16 @@ int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what) {
     return FDIRW_OK;
 }
 
+void drelease(void* p) {
+    if (p && !pool().keep(p)) cudaFree(p);
+}
+
 void dfree(void*& p) {
-    if (p) cudaFree(p);
+    drelease(p);
     p = nullptr;
 }
+
+uint64_t idle_device_bytes(int device) { return pool().idle_on(device); }
 
 }  // namespace host
 }  // namespace fdirw
@@ -94,9 +200,9 @@ int conductances(fdirw_ctx* c, const double* D, double* g3[3], double* max_sum) 
     if ((rc = dalloc(c, reinterpret_cast<void**>(&flags), 16, "flags")) != FDIRW_OK) return rc;
     const double* Dd = D;
     if (k == Kind::Host) {
-        if ((rc = dalloc(c, &dD, (uint64_t)g.n * 8, "D staging")) != FDIRW_OK) { cudaFree(flags); return rc; }
+        if ((rc = dalloc(c, &dD, (uint64_t)g.n * 8, "D staging")) != FDIRW_OK) { drelease(flags); return rc; }
         cudaError_t e = cudaMemcpyAsync(dD, D, (size_t)g.n * 8, cudaMemcpyHostToDevice, c->stream);
-        if (e != cudaSuccess) { cudaFree(dD); cudaFree(flags); return fail(c, FDIRW_ERR_CUDA, cuda_msg("copy D_map", e)); }
+        if (e != cudaSuccess) { drelease(dD); drelease(flags); return fail(c, FDIRW_ERR_CUDA, cuda_msg("copy D_map", e)); }
         Dd = reinterpret_cast<const double*>(dD);
     }
     unsigned long long h[2] = {0ull, 0ull};
@@ -104,8 +210,8 @@ int conductances(fdirw_ctx* c, const double* D, double* g3[3], double* max_sum) 
     if (e == cudaSuccess) e = fdirw::launch_conductance(Dd, g, g3[0], g3[1], g3[2], flags, flags + 1, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, flags, 16, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (dD) { cudaFree(dD); c->allocated -= (uint64_t)g.n * 8; }
-    cudaFree(flags);
+    if (dD) { drelease(dD); c->allocated -= (uint64_t)g.n * 8; }
+    drelease(flags);
     c->allocated -= 16;
     if (e != cudaSuccess) return fail(c, FDIRW_ERR_CUDA, cuda_msg("conductance kernel", e));
     if (h[1] != 0ull)
@@ -151,7 +257,7 @@ int fdirw::ensure_cache(fdirw_ctx* c) {
     size_t free_b = 0, total_b = 0;
     uint64_t budget = ~0ull;
     constexpr uint64_t kReserve = 1ull << 30;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) budget = free_b > kReserve ? free_b - kReserve : 0;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) budget = free_b + idle_device_bytes(c->device) > kReserve ? free_b + idle_device_bytes(c->device) - kReserve : 0;
     else cudaGetLastError();                                   // unknown: let the allocation decide
     if (c->mem_limit) budget = std::min<uint64_t>(budget, c->mem_limit > c->allocated ? c->mem_limit - c->allocated : 0);
     const uint64_t obytes = (uint64_t)c->g.n * 8;
@@ -287,7 +393,7 @@ int fdirw_stable_dt(const fdirw_grid* grid, const double* D_map, int32_t device,
     double* g3[3] = {nullptr, nullptr, nullptr};
     double m = 0.0;
     const int rc = conductances(&tmp, D_map, g3, &m);
-    for (auto& p : g3) if (p) cudaFree(p);
+    for (auto& p : g3) drelease(p);
     if (rc != FDIRW_OK) return fail(nullptr, rc, tmp.err);
     *dt_sub_max = m > 0.0 ? grid->h * grid->h / m : HUGE_VAL;
     return FDIRW_OK;
@@ -335,6 +441,7 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
 
     auto bail = [&](int rc) {
         std::string msg = c->err;
+        if (c->stream) cudaStreamSynchronize(c->stream); else cudaDeviceSynchronize();   // nothing uses what is released
         release(c);
         delete c;
         return fail(nullptr, rc, msg);
@@ -343,7 +450,7 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
     double* g3[3] = {nullptr, nullptr, nullptr};
     int rc = conductances(c, D_map, g3, &c->max_face_sum);
     if (rc != FDIRW_OK) {
-        for (auto& p : g3) if (p) cudaFree(p);
+        for (auto& p : g3) drelease(p);
         return bail(rc);
     }
     for (int a = 0; a < 3; a++) c->coef[a] = g3[a];
@@ -361,16 +468,26 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
             if (e != cudaSuccess) { c->err = cuda_msg("coefficient kernel", e); return bail(FDIRW_ERR_CUDA); }
         }
     } else {
+        void* f[3] = {nullptr, nullptr, nullptr};
+        cudaError_t e = cudaSuccess;
+        for (int a = 0; a < 3 && e == cudaSuccess; a++) {
+            if ((rc = dalloc(c, &f[a], n * 4, "coefficients")) != FDIRW_OK) {
+                for (void* p : f) drelease(p);
+                return bail(rc);
+            }
+            e = fdirw::launch_coef_f32(reinterpret_cast<double*>(c->coef[a]), c->lam, c->g.n, reinterpret_cast<float*>(f[a]),
+                                       c->stream);
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);      // the FP64 arrays are free again
+        if (e != cudaSuccess) {
+            for (void* p : f) drelease(p);
+            c->err = cuda_msg("coefficient kernel", e);
+            return bail(FDIRW_ERR_CUDA);
+        }
         for (int a = 0; a < 3; a++) {
-            void* f = nullptr;
-            if ((rc = dalloc(c, &f, n * 4, "coefficients")) != FDIRW_OK) return bail(rc);
-            cudaError_t e = fdirw::launch_coef_f32(reinterpret_cast<double*>(c->coef[a]), c->lam, c->g.n,
-                                                   reinterpret_cast<float*>(f), c->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-            if (e != cudaSuccess) { cudaFree(f); c->err = cuda_msg("coefficient kernel", e); return bail(FDIRW_ERR_CUDA); }
-            cudaFree(c->coef[a]);
+            drelease(c->coef[a]);
             c->allocated -= n * 8;
-            c->coef[a] = f;
+            c->coef[a] = f[a];
         }
     }
     const fdirw::Pad pad = fdirw::make_pad(c->g, c->R);
@@ -386,6 +503,7 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
     if ((rc = dalloc(c, reinterpret_cast<void**>(&c->dmass), 8, "mass")) != FDIRW_OK) return bail(rc);
     if ((rc = dalloc(c, reinterpret_cast<void**>(&c->dfix), 24, "mass restoration")) != FDIRW_OK) return bail(rc);
     cudaError_t e = cudaMemsetAsync(c->chat, 0, (size_t)pad.n * 8, c->stream);
+    if (e == cudaSuccess && c->accum == FDIRW_ACCUM_FP32) e = cudaMemsetAsync(c->dfix, 0, 24, c->stream);
     for (int i = 0; i < 4 && e == cudaSuccess; i++) e = cudaEventCreate(&c->ev[i]);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) { c->err = cuda_msg("context setup", e); return bail(FDIRW_ERR_CUDA); }

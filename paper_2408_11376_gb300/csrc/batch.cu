@@ -921,7 +921,8 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
         size_t fr = 0, tot = 0;
         if ((e = cudaMemGetInfo(&fr, &tot)) != cudaSuccess) return cuda_bail("cudaMemGetInfo", e);
         const uint64_t reserve = std::max<uint64_t>(1ull << 30, tot / 50);
-        budget = fr > reserve ? fr - reserve : 0;
+        const uint64_t free_b = fr + idle_device_bytes(c->device);
+        budget = free_b > reserve ? free_b - reserve : 0;
     }
     budget = budget > 256ull * (fdirw::kMaxR + 1) ? budget - 256ull * (fdirw::kMaxR + 1) : 0;
     auto all_radii = [&](int i) {

@@ -747,7 +747,7 @@ int fdirw_coarse_far_field(fdirw_ctx* c, double V_far, double c_far) {
         }
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h, mx, 8, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        cudaFree(mx);
+        drelease(mx);
         c->allocated -= 8;
         if (e != cudaSuccess) { cudaGetLastError(); return fail(c, FDIRW_ERR_CUDA, cuda_msg("open faces", e)); }
         double m;
@@ -886,7 +886,7 @@ int fdirw_read_coarse(fdirw_ctx* c, const int64_t* blocks, int64_t n, double* ou
     int rc = dalloc(c, reinterpret_cast<void**>(&db), (uint64_t)n * 8, "block list");
     if (rc != FDIRW_OK) return rc;
     rc = dalloc(c, reinterpret_cast<void**>(&dout), (uint64_t)(n * W3) * 8, "coarse readback");
-    if (rc != FDIRW_OK) { cudaFree(db); c->allocated -= (uint64_t)n * 8; return rc; }
+    if (rc != FDIRW_OK) { drelease(db); c->allocated -= (uint64_t)n * 8; return rc; }
     cudaError_t e = cudaMemcpyAsync(db, blocks, (size_t)n * 8, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) {
         fdirw::read_coarse_kernel<<<fdirw::grid_blocks(n * W3, 256), 256, 0, c->stream>>>(k.Qc, k.ncx, k.ncy, k.ncz, k.Rc,
@@ -895,8 +895,8 @@ int fdirw_read_coarse(fdirw_ctx* c, const int64_t* blocks, int64_t n, double* ou
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, (size_t)(n * W3) * 8, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(db);
-    cudaFree(dout);
+    drelease(db);
+    drelease(dout);
     c->allocated -= (uint64_t)n * 8 + (uint64_t)(n * W3) * 8;
     if (e != cudaSuccess) { cudaGetLastError(); return fail(c, FDIRW_ERR_CUDA, cuda_msg("read coarse matrix", e)); }
     return FDIRW_OK;

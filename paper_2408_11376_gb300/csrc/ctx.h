@@ -80,7 +80,11 @@ Kind classify(const void* p, int device);
 bool grid_ok(const fdirw_grid* g);
 // cudaMalloc that honours the context's mem_limit and keeps its byte count.
 int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what);
+// Frees a dalloc'ed block that no work uses any more (a pool of small ones keeps it for the next dalloc).
+void drelease(void* p);
 void dfree(void*& p);
+// Bytes of the pool's idle blocks on a device: free memory to a dalloc, though the driver counts them as used.
+uint64_t idle_device_bytes(int device);
 }  // namespace host
 
 #define FDIRW_CUDA(ctx, call)                                                                     \

@@ -102,7 +102,7 @@ int fdirw_set_velocity(fdirw_ctx* c, const double* w) {
     unsigned long long* mx = nullptr;
     if ((rc = dalloc(c, reinterpret_cast<void**>(&dw), 3 * n * 8, "velocity staging")) != FDIRW_OK) return rc;
     if ((rc = dalloc(c, reinterpret_cast<void**>(&mx), 8, "flags")) != FDIRW_OK) {
-        cudaFree(dw);
+        drelease(dw);
         c->allocated -= 3 * n * 8;
         return rc;
     }
@@ -110,7 +110,7 @@ int fdirw_set_velocity(fdirw_ctx* c, const double* w) {
     // separate allocations, so stage A and B in one block and copy them out.
     float* AB = nullptr;
     if ((rc = dalloc(c, reinterpret_cast<void**>(&AB), 6 * n * 4, "coefficient staging")) != FDIRW_OK) {
-        cudaFree(dw); cudaFree(mx);
+        drelease(dw); drelease(mx);
         c->allocated -= 3 * n * 8 + 8;
         return rc;
     }
@@ -149,9 +149,9 @@ int fdirw_set_velocity(fdirw_ctx* c, const double* w) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->coefb[a], AB + (3 + a) * n, n * 4, cudaMemcpyDeviceToDevice, c->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(dw);
-    cudaFree(mx);
-    cudaFree(AB);
+    drelease(dw);
+    drelease(mx);
+    drelease(AB);
     c->allocated -= 3 * n * 8 + 8 + 6 * n * 4;
     if (e != cudaSuccess) { cudaGetLastError(); return fail(c, FDIRW_ERR_CUDA, cuda_msg("velocity coefficients", e)); }
     if (!std::isfinite(m)) return fail(c, FDIRW_ERR_ARG, "w holds NaN or infinite values");
