@@ -55,15 +55,15 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return d;
 }
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, 0xbf800000bf800000ull, a); }
-__device__ __forceinline__ uint64_t neg2(uint64_t a) { return a ^ 0x8000000080000000ull; }
 
-// ff_madd and ff_add on two destinations at once (the same operations in the same order).
-__device__ __forceinline__ void ff_madd2(uint64_t& s, uint64_t& c, uint64_t q, uint64_t hi, uint64_t lo) {
-    const uint64_t p = mul2(q, hi);
-    const uint64_t e = fma2(q, lo, fma2(q, hi, neg2(p)));
-    const uint64_t t = add2(s, p);
+// ff_madd and ff_add on two destinations at once: the same operations in the same order, each rounding the same value up
+// to its sign (the product is formed as -p from nhi = -hi, so that nothing has to be negated per term).
+__device__ __forceinline__ void ff_madd2(uint64_t& s, uint64_t& c, uint64_t q, uint64_t hi, uint64_t nhi, uint64_t lo) {
+    const uint64_t np = mul2(q, nhi);
+    const uint64_t e = fma2(q, lo, fma2(q, hi, np));
+    const uint64_t t = sub2(s, np);
     const uint64_t bp = sub2(t, s);
-    const uint64_t err = add2(sub2(s, sub2(t, bp)), sub2(p, bp));
+    const uint64_t err = sub2(sub2(s, sub2(t, bp)), add2(np, bp));
     s = t;
     c = add2(c, add2(err, e));
 }
@@ -84,28 +84,49 @@ struct Quad {
     static constexpr __host__ __device__ int j0(int i) { return sizeof(ST) == 4 ? 2 * i : i; }
 };
 template <typename ST>
-__device__ __forceinline__ void pairs_of(uint4 v, uint64_t (&q)[8 / sizeof(ST)]) {
+__device__ __forceinline__ uint64_t pair_of(uint4 v, int i) {
     auto pr = [](uint32_t a, uint32_t b) { return pack2(__uint_as_float(a), __uint_as_float(b)); };
-    if constexpr (sizeof(ST) == 4) {
-        q[0] = pr(v.x, v.y);
-        q[1] = pr(v.z, v.w);
-    } else if constexpr (std::is_same<ST, __half>::value) {
-        const __half2* h = reinterpret_cast<const __half2*>(&v);
-        const float2 a = __half22float2(h[0]), b = __half22float2(h[1]), c = __half22float2(h[2]), d = __half22float2(h[3]);
-        q[0] = pack2(a.x, c.x);
-        q[1] = pack2(a.y, c.y);
-        q[2] = pack2(b.x, d.x);
-        q[3] = pack2(b.y, d.y);
+    if constexpr (sizeof(ST) == 4) return i ? pr(v.z, v.w) : pr(v.x, v.y);
+    const uint32_t a = i < 2 ? v.x : v.y, b = i < 2 ? v.z : v.w;
+    if constexpr (std::is_same<ST, __half>::value) {
+        const __half2 ha = *reinterpret_cast<const __half2*>(&a), hb = *reinterpret_cast<const __half2*>(&b);
+        return i & 1 ? pack2(__high2float(ha), __high2float(hb)) : pack2(__low2float(ha), __low2float(hb));
     } else {
-        q[0] = pr(v.x << 16, v.z << 16);
-        q[1] = pr(v.x & 0xffff0000u, v.z & 0xffff0000u);
-        q[2] = pr(v.y << 16, v.w << 16);
-        q[3] = pr(v.y & 0xffff0000u, v.w & 0xffff0000u);
+        return i & 1 ? pr(a & 0xffff0000u, b & 0xffff0000u) : pr(a << 16, b << 16);
     }
 }
-template <typename ST>
-__device__ __forceinline__ void load_pairs(const ST* p, uint64_t (&q)[8 / sizeof(ST)]) {
-    pairs_of<ST>(__ldcs(reinterpret_cast<const uint4*>(p)), q);       // streamed: read once per step
+
+// One row of VX destinations: s (and c, float-float) += q[o_x] chat(x - o_x), o_x ascending for every destination.  q: the
+// row's 2R+1 vectors; ch(k): its scaled values, k = x - o_x + R.  The loop goes over k, so that the pair of scaled values
+// at k (and its negative) is put together once for all destinations that it meets.  Float-float sums are bound by the
+// issue slots (11 packed operations of two cycles a pair of terms), and with the pairs made at every use 45% of the
+// instructions were moves and sign flips: us a step with BF16 storage before -> after, 192^3 R = 8 16680 -> 15790
+// (10230 at the copy rate), 64^3 R = 3 68 -> 63, 128^3 R = 2 205 -> 178; FP32 128^3 R = 1 61 -> 51.
+template <typename ST, int R, bool FF, typename F>
+__device__ __forceinline__ void row_sums(const uint4 (&q)[2 * R + 1], F ch, uint64_t (&s)[8 / sizeof(ST)],
+                                         uint64_t (&c)[8 / sizeof(ST)]) {
+    using U = Quad<ST>;
+    constexpr int NP = 8 / sizeof(ST), K1 = 2 * R + U::j0(NP - 1);
+    float2 v[K1 + U::D + 1];                              // (hi, lo); FP32: (value, -)
+#pragma unroll
+    for (int k = 0; k <= K1 + U::D; k++) v[k] = ch(k);
+#pragma unroll
+    for (int k = K1; k >= 0; k--) {
+        const uint64_t hi = pack2(v[k].x, v[k + U::D].x);
+        uint64_t nhi = 0, lo = 0;
+        if (FF) {
+            nhi = pack2(-v[k].x, -v[k + U::D].x);
+            lo = pack2(v[k].y, v[k + U::D].y);
+        }
+#pragma unroll
+        for (int i = 0; i < NP; i++) {
+            const int ox = U::j0(i) - k + R;
+            if (ox < -R || ox > R) continue;
+            const uint64_t w = pair_of<ST>(q[ox + R], i);
+            if constexpr (FF) ff_madd2(s[i], c[i], w, hi, nhi, lo);
+            else s[i] = fma2(w, hi, s[i]);
+        }
+    }
 }
 
 // The gather over destinations in cell order.  A block is 8 warps: VW of them side by side in the destinations, and
@@ -116,7 +137,7 @@ __device__ __forceinline__ void load_pairs(const ST* p, uint64_t (&q)[8 / sizeof
 // Why the rows are split: a grid of up to about 100^3 cells has too few destinations to fill 152 SMs with one thread
 // for all rows of each (32^3 FP32 ones are 32 blocks of 256), and beyond that the last wave of long threads idles most
 // of the chip.  us a step before -> after, FP32 cache, float-float sums: 32^3 R = 3 49 -> 14, 48^3 R = 8 1972 -> 346,
-// 112^3 R = 8 6487 -> 4173 (4060 at the copy rate); FP64 36^3 R = 6 600 -> 188.  At R <= 2 (at most 25 rows) eight
+// 112^3 R = 8 6487 -> 4110 (4060 at the copy rate); FP64 36^3 R = 6 600 -> 188.  At R <= 2 (at most 25 rows) eight
 // groups cost more than they give (128^3 R = 2 BF16 cache 100 -> 125): one.
 constexpr int vector_warps(int R) { return R <= 2 ? 8 : 1; }
 __device__ __forceinline__ int row_groups(int R) { return R <= 2 ? 1 : 8; }
@@ -133,9 +154,9 @@ struct GatherArgs {
 };
 
 // Cache rows of whole 16-byte vectors: a thread owns VX consecutive destinations of an x row, one load of a plane.
-// The destinations past nx in a padded row are computed from whatever lies there and not stored.  MODE 0: FP64 throughout.  MODE 1: float-float rows (FDIRW_ACCUM_FF).  MODE 2: FP32 rows
-// (FDIRW_ACCUM_FP32); both sum the rows of a destination as a float-float pair, which one FP64 addition turns into
-// the result.  Two blocks per SM: 128 registers keep a row's loads in flight (with three blocks and 80 registers the
+// The destinations past nx in a padded row are computed from whatever lies there and not stored.  MODE 0: FP64
+// throughout.  MODE 1: float-float rows (FDIRW_ACCUM_FF).  MODE 2: FP32 rows (FDIRW_ACCUM_FP32); both sum the rows of a
+// destination as a float-float pair, which one FP64 addition turns into the result.  Two blocks per SM: 128 registers keep a row's loads in flight (with three blocks and 80 registers the
 // loads no longer overlap: 1.4 times as long).
 template <typename ST, int R, int MODE, int VW>
 __global__ void __launch_bounds__(256, MODE == 2 && R == 1 ? 4 : 2) gather_kernel(GatherArgs a) {
@@ -175,33 +196,17 @@ __global__ void __launch_bounds__(256, MODE == 2 && R == 1 ? 4 : 2) gather_kerne
                     acc[1] = fma(d.y, w[R - ox + 1], acc[1]);
                 }
             } else {
-                using U = Quad<ST>;
                 uint64_t s[NP], c[NP];
 #pragma unroll
                 for (int i = 0; i < NP; i++) s[i] = c[i] = 0;
-                float hi[NK], lo[NK];
+                uint4 d[W1];                                 // streamed: read once per step
 #pragma unroll
-                for (int k = 0; k < NK; k++) {
-                    if constexpr (MODE == 1) {
-                        const float2 f = __ldg(reinterpret_cast<const float2*>(a.chat) + row + (k <= 2 * R ? k : min(k, last)));
-                        hi[k] = f.x;
-                        lo[k] = f.y;
-                    } else {
-                        hi[k] = __ldg(reinterpret_cast<const float*>(a.chat) + row + (k <= 2 * R ? k : min(k, last)));
-                    }
-                }
-#pragma unroll
-                for (int ox = -R; ox <= R; ox++) {
-                    uint64_t d[NP];
-                    load_pairs(q + (int64_t)(ox + R) * a.qs, d);
-#pragma unroll
-                    for (int i = 0; i < NP; i++) {
-                        const int k = U::j0(i) - ox + R;
-                        const uint64_t h = pack2(hi[k], hi[k + U::D]);
-                        if constexpr (MODE == 1) ff_madd2(s[i], c[i], d[i], h, pack2(lo[k], lo[k + U::D]));
-                        else s[i] = fma2(d[i], h, s[i]);
-                    }
-                }
+                for (int k = 0; k < W1; k++) d[k] = __ldcs(reinterpret_cast<const uint4*>(q + (int64_t)k * a.qs));
+                row_sums<ST, R, MODE == 1>(d, [&](int k) {
+                    const int64_t at_k = row + (k <= 2 * R ? k : min(k, last));
+                    if constexpr (MODE == 1) return __ldg(reinterpret_cast<const float2*>(a.chat) + at_k);
+                    else return make_float2(__ldg(reinterpret_cast<const float*>(a.chat) + at_k), 0.f);
+                }, s, c);
                 // The pair of a row restarts at zero, so its compensation stays within a few ulps of the row sum.
 #pragma unroll
                 for (int i = 0; i < NP; i++) ff_add2(A[i], B[i], s[i], c[i]);
@@ -272,7 +277,7 @@ __global__ void __launch_bounds__(256, MODE == 2 && R == 1 ? 4 : 2) gather_kerne
 template <typename ST, int R>
 __global__ void __launch_bounds__(256, 2) gather_ordered_kernel(GatherArgs a) {
     using U = Quad<ST>;
-    constexpr int VX = 16 / sizeof(ST), W1 = 2 * R + 1, NROW = W1 * W1, NP = VX / 2, NK = VX + 2 * R, ND = 32 * VX;
+    constexpr int VX = 16 / sizeof(ST), W1 = 2 * R + 1, NROW = W1 * W1, NP = VX / 2, ND = 32 * VX;
     __shared__ float sums[2][8][ND];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned nxv = a.qnx / VX, nvec = nxv * a.g.ny * a.zn, v = blockIdx.x * 32 + lane;
@@ -296,22 +301,10 @@ __global__ void __launch_bounds__(256, 2) gather_ordered_kernel(GatherArgs a) {
         if (row < NROW) {
             const int oz = row / W1 - R, oy = row % W1 - R;
             const float* ch = chat - ((int64_t)oz * a.p.py + oy) * a.p.px;
-            uint64_t s[NP];
+            uint64_t s[NP], c[NP];
 #pragma unroll
-            for (int i = 0; i < NP; i++) s[i] = 0;
-            float hi[NK];
-#pragma unroll
-            for (int k = 0; k < NK; k++) hi[k] = __ldg(ch + (k <= 2 * R ? k : min(k, last)));
-#pragma unroll
-            for (int ox = -R; ox <= R; ox++) {
-                uint64_t w[NP];
-                pairs_of<ST>(d[ox + R], w);
-#pragma unroll
-                for (int i = 0; i < NP; i++) {
-                    const int k = U::j0(i) - ox + R;
-                    s[i] = fma2(w[i], pack2(hi[k], hi[k + U::D]), s[i]);
-                }
-            }
+            for (int i = 0; i < NP; i++) s[i] = c[i] = 0;
+            row_sums<ST, R, false>(d, [&](int k) { return make_float2(__ldg(ch + (k <= 2 * R ? k : min(k, last))), 0.f); }, s, c);
             if (row + 8 < NROW) fetch(row + 8);
             float f[VX];
 #pragma unroll
