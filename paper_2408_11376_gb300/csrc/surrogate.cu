@@ -366,17 +366,38 @@ __global__ void __launch_bounds__(256) head_predict_kernel(const float* __restri
     }
 }
 
+// Adds up a block's sums in a fixed order (256 threads); the total is thread 0's.
+__device__ double block_sum(double acc) {
+    __shared__ double sh[8];
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    double w = 0.0;
+    if (threadIdx.x < 32) {
+        w = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+        for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
+    }
+    return w;
+}
+
 // Head for training: the generalised Kullback-Leibler divergence sum_v (y - k z + k ln k - k), y = exp(z),
 // over in-domain cells (0 ln 0 = 0) and its gradient y - k with respect to z (channel 0); the gradient
 // penalises predicted mass wherever the target kernel has less, which is what the mass gate checks.
+//   FP64 exponentials and logarithms bound it (2 FP64 FMAs a clock and SM; 154 us for 256 sources with both in one kernel
+// and one block a source).  A source's voxels go to HEAD_PARTS blocks, so that the last wave is short: 60 us.  k ln k,
+// which only the targets enter, is summed by target_term_kernel (82 us) on the side stream under the backward pass, one
+// block per SM.  Under the forward pass it cost more than it hid (the step took 1160 us: a kernel that is on an SM first
+// can hold up the convolution's 120 KB of shared memory).  Training step of 256 sources, with the weight gradients' sums
+// beside the convolutions: 1009 -> 898 us.
+constexpr int HEAD_PARTS = 10, HEAD_CHUNK = (KV + HEAD_PARTS - 1) / HEAD_PARTS, TERM_BLOCKS = 152;
+
 __global__ void __launch_bounds__(256) head_train_kernel(const float* __restrict__ zhead, Grid g,
                                                          const int64_t* __restrict__ src, const double* __restrict__ tgt,
                                                          __nv_bfloat16* __restrict__ grad, double* __restrict__ loss) {
-    __shared__ double sh[8];
-    const int b = blockIdx.x;
+    const int b = blockIdx.x, v1 = min(((int)blockIdx.y + 1) * HEAD_CHUNK, KV);
     const PatchPos q = pos_of(src[b], g);
     double acc = 0.0;
-    for (int v = threadIdx.x; v < KV; v += blockDim.x) {
+    for (int v = blockIdx.y * HEAD_CHUNK + threadIdx.x; v < v1; v += blockDim.x) {
         const int i = v % SP, j = (v / SP) % SP, k = v / (SP * SP);
         int64_t gi;
         const bool ind = in_domain(q, i, j, k, g, &gi);
@@ -385,19 +406,31 @@ __global__ void __launch_bounds__(256) head_train_kernel(const float* __restrict
             const double kk = tgt[(int64_t)b * KV + v];
             const double z = (double)zhead[(int64_t)b * KV + v];
             const double y = exp(z);
-            acc += y - kk * z + (kk > 0.0 ? kk * log(kk) : 0.0) - kk;
+            acc += y - kk * z - kk;
             gz = y - kk;
         }
         grad[(int64_t)b * PATCH + (int64_t)prow(i, j, k) * 8] = __float2bfloat16_rn((float)gz);
     }
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double w = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(0xffffffffu, w, off);
-        if (threadIdx.x == 0) loss[b] = w;
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) loss[b * HEAD_PARTS + blockIdx.y] = acc;
+}
+
+__global__ void __launch_bounds__(256) target_term_kernel(Grid g, const int64_t* __restrict__ src, int n,
+                                                          const double* __restrict__ tgt, double* __restrict__ loss) {
+    double acc = 0.0;
+    for (int item = blockIdx.x; item < n * HEAD_PARTS; item += gridDim.x) {
+        const int b = item / HEAD_PARTS, v0 = (item % HEAD_PARTS) * HEAD_CHUNK, v1 = min(v0 + HEAD_CHUNK, KV);
+        const PatchPos q = pos_of(src[b], g);
+        for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+            const int i = v % SP, j = (v / SP) % SP, k = v / (SP * SP);
+            int64_t gi;
+            if (!in_domain(q, i, j, k, g, &gi)) continue;
+            const double kk = tgt[(int64_t)b * KV + v];
+            if (kk > 0.0) acc += kk * log(kk);
+        }
     }
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) loss[blockIdx.x] = acc;
 }
 
 // Head for the kernel cache: accepted predictions are rounded to the storage type and written into
@@ -642,11 +675,14 @@ __global__ void __launch_bounds__(WG_THREADS) wgrad_kernel(const __grid_constant
 }
 
 // dW[tap][co][ci] = sum over the WG_PARTS partials in order; db[co] = the same sum of the ones slot (ci 0).
-__global__ void wgrad_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dW, float* __restrict__ db) {
+// A chain of loads (8 us, four times a step): it runs on the side stream beside the next layer's convolution.
+constexpr int WG_RED = 64;
+__global__ void __launch_bounds__(WG_RED) wgrad_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dW, float* __restrict__ db) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= TAPS * C * C + C) return;
     const int64_t idx = e < TAPS * C * C ? e : (int64_t)TAPS * C * C + (int64_t)(e - TAPS * C * C) * C;
     float s = 0.f;
+#pragma unroll 19                                          // the loads in flight together, the sum in order
     for (int p = 0; p < WG_PARTS; p++) s += partial[(int64_t)p * WG_SLOTS * C * C + idx];
     if (e < TAPS * C * C) dW[e] = s;
     else db[e - TAPS * C * C] = s;
@@ -729,6 +765,8 @@ struct fdirw_net {
     int* derr = nullptr;
     CUtensorMap tm_act[NL];        // weight-gradient views of act[l] and gbuf[i] (encoded with the buffers)
     CUtensorMap tm_grad[2];
+    cudaStream_t side = nullptr;   // training: what the tensor-core kernels leave SMs for (gradients())
+    cudaEvent_t fork[3] = {};      // [0], [1]: points of the context's stream (or back); [2]: of the side stream
     cudaEvent_t ev[2] = {};        // around the four convolutions of the last forward pass
     bool timed = false;
     uint64_t wait_ns = WAIT_NS;    // budget of each MMA wait (fdirw_net_test_wait)
@@ -816,7 +854,7 @@ int ensure_capacity(fdirw_net* net, int n) {
     NET_CUDA(net, cudaMalloc(&net->dkout, (size_t)cap * KV * 8));
     NET_CUDA(net, cudaMalloc(&net->dmass, (size_t)cap * 8));
     NET_CUDA(net, cudaMalloc(&net->dacc, (size_t)cap * 4));
-    NET_CUDA(net, cudaMalloc(&net->dloss, (size_t)cap * 8));
+    NET_CUDA(net, cudaMalloc(&net->dloss, ((size_t)cap * HEAD_PARTS + TERM_BLOCKS) * 8));
     if (const int rc = encode_maps(net, cap); rc != FDIRW_OK) return rc;
     net->cap = cap;
     return FDIRW_OK;
@@ -841,10 +879,14 @@ int launch_conv(fdirw_net* net, cudaStream_t st, int num_sms, const __nv_bfloat1
 int launch_wgrad(fdirw_net* net, cudaStream_t st, int l, int cur, int n, float* dW, float* db) {
     WgradArgs a{net->partial, n, net->derr, net->wait_ns, net->hold};
     NET_CUDA(net, cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM));
+    NET_CUDA(net, cudaStreamWaitEvent(st, net->fork[2], 0));       // the last layer's partials have been added up
     wgrad_kernel<<<WG_PARTS, WG_THREADS, WG_SMEM, st>>>(net->tm_act[l], net->tm_grad[cur], a);
     NET_CUDA(net, cudaGetLastError());
-    wgrad_reduce_kernel<<<(TAPS * C * C + C + 255) / 256, 256, 0, st>>>(net->partial, dW, db);
+    NET_CUDA(net, cudaEventRecord(net->fork[1], st));
+    NET_CUDA(net, cudaStreamWaitEvent(net->side, net->fork[1], 0));
+    wgrad_reduce_kernel<<<(TAPS * C * C + C + WG_RED - 1) / WG_RED, WG_RED, 0, net->side>>>(net->partial, dW, db);
     NET_CUDA(net, cudaGetLastError());
+    NET_CUDA(net, cudaEventRecord(net->fork[2], net->side));
     return FDIRW_OK;
 }
 
@@ -941,14 +983,38 @@ int gradients(fdirw_ctx* c, fdirw_net* net, const int64_t* sources, int64_t n, c
     int rc = upload_sources(c, net, sources, n);
     if (rc != FDIRW_OK) return rc;
     NET_CUDA(net, cudaMemcpyAsync(net->dtgt, targets, (size_t)n * KV * 8, cudaMemcpyDefault, c->stream));
+    // The side stream clears the head gradient under the forward pass, then sums the loss's target term and each layer's
+    // weight gradient partials under the backward pass.  It starts when the inputs are there.  However this function is
+    // left, the context's stream waits for it, so that nothing that uses or frees these buffers afterwards overtakes it.
+    cudaStream_t st = c->stream;
+    std::vector<double> lv((size_t)n * HEAD_PARTS + TERM_BLOCKS);
+    NET_CUDA(net, cudaEventRecord(net->fork[0], st));
+    NET_CUDA(net, cudaStreamWaitEvent(net->side, net->fork[0], 0));
+    struct Join {
+        fdirw_net* net;
+        cudaStream_t st;
+        bool done = false;
+        cudaError_t now() {
+            done = true;
+            const cudaError_t e = cudaEventRecord(net->fork[2], net->side);
+            return e != cudaSuccess ? e : cudaStreamWaitEvent(st, net->fork[2], 0);
+        }
+        ~Join() { if (!done) now(); }
+    } join{net, st};
+    NET_CUDA(net, cudaMemsetAsync(net->gbuf[0], 0, (size_t)n * PATCH * 2, net->side));
+    NET_CUDA(net, cudaEventRecord(net->fork[1], net->side));
     if ((rc = forward(c, net, (int)n)) != FDIRW_OK) return rc;
-    NET_CUDA(net, cudaMemsetAsync(net->gbuf[0], 0, (size_t)n * PATCH * 2, c->stream));
-    head_train_kernel<<<(int)n, 256, 0, c->stream>>>(net->zhead, c->g, net->dsrc, net->dtgt, net->gbuf[0], net->dloss);
+    NET_CUDA(net, cudaStreamWaitEvent(st, net->fork[1], 0));
+    head_train_kernel<<<dim3((unsigned)n, HEAD_PARTS), 256, 0, st>>>(net->zhead, c->g, net->dsrc, net->dtgt, net->gbuf[0], net->dloss);
+    NET_CUDA(net, cudaGetLastError());
+    NET_CUDA(net, cudaEventRecord(net->fork[1], st));
+    NET_CUDA(net, cudaStreamWaitEvent(net->side, net->fork[1], 0));
+    target_term_kernel<<<TERM_BLOCKS, 256, 0, net->side>>>(c->g, net->dsrc, (int)n, net->dtgt, net->dloss + n * HEAD_PARTS);
     NET_CUDA(net, cudaGetLastError());
     if ((rc = backward(c, net, (int)n, hook)) != FDIRW_OK) return rc;
-    std::vector<double> lv((size_t)n);
-    NET_CUDA(net, cudaMemcpyAsync(lv.data(), net->dloss, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream));
-    if ((rc = check_err(net, c->stream)) != FDIRW_OK) return rc;
+    NET_CUDA(net, join.now());
+    NET_CUDA(net, cudaMemcpyAsync(lv.data(), net->dloss, lv.size() * 8, cudaMemcpyDeviceToHost, st));
+    if ((rc = check_err(net, st)) != FDIRW_OK) return rc;
     double s = 0.0;
     for (double x : lv) s += x;
     if (loss_out) *loss_out = n > 0 ? s / (double)n : 0.0;
@@ -978,8 +1044,14 @@ FDIRW_API int fdirw_net_create(const float* params, int32_t device, fdirw_net** 
         cudaMalloc(&net->wf, (size_t)NL * WCAN * 2) != cudaSuccess || cudaMalloc(&net->wd, (size_t)NL * WCAN * 2) != cudaSuccess ||
         cudaMalloc(&net->partial, (size_t)WG_PARTS * WG_SLOTS * C * C * 4) != cudaSuccess ||
         cudaMalloc(&net->derr, 4) != cudaSuccess || cudaEventCreate(&net->ev[0]) != cudaSuccess ||
-        cudaEventCreate(&net->ev[1]) != cudaSuccess)
+        cudaEventCreate(&net->ev[1]) != cudaSuccess || cudaStreamCreateWithFlags(&net->side, cudaStreamNonBlocking) != cudaSuccess)
         return bail("allocating the network");
+    // Beside a tensor-core kernel: an SM keeps the shared memory that the next one needs (a kernel that leaves it to L1
+    // makes the next convolution wait until it has left the SM).
+    cudaFuncSetAttribute(target_term_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(wgrad_reduce_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    for (auto& e : net->fork)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return bail("allocating the network");
     if (cudaMemcpy(net->params, params, NPARAM * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(net->m, 0, NPARAM * 4) != cudaSuccess || cudaMemset(net->v, 0, NPARAM * 4) != cudaSuccess ||
         cudaMemset(net->derr, 0, 4) != cudaSuccess)
@@ -1006,6 +1078,8 @@ FDIRW_API void fdirw_net_destroy(fdirw_net* net) {
     cudaFree(net->zhead); cudaFree(net->dsrc); cudaFree(net->dtgt); cudaFree(net->dkout); cudaFree(net->dmass);
     cudaFree(net->dacc); cudaFree(net->dloss); cudaFree(net->partial); cudaFree(net->grads); cudaFree(net->derr);
     for (auto e : net->ev) if (e) cudaEventDestroy(e);
+    for (auto e : net->fork) if (e) cudaEventDestroy(e);
+    if (net->side) cudaStreamDestroy(net->side);
     delete net;
 }
 
