@@ -306,7 +306,7 @@ FDIRW_API int fdirw_coupled_step(fdirw_ctx* ctx, const fdirw_coupled_params* par
  * then carries, across each interior face, the diffusive flux lam g (u_lower - u_upper) plus the upwind
  * advective flux lam_a (w+ u_lower - w- u_upper), lam = dt_sub / h^2, lam_a = dt_sub / h, w+ = max(w, 0),
  * w- = max(-w, 0); window and domain edges stay closed.  The face coefficients are rounded once to FP32
- * and the march runs mapping 5 (direction-dependent faces); the superposition is unchanged.  On a
+ * and the march uses direction-dependent faces (reported as mapping 5); the superposition is unchanged.  On a
  * coarse-mesh context faces touching a non-liquid cell carry neither flux, the block-source march and
  * the P_BC march use the same faces, and the far field's open faces stay diffusive (open the far field
  * first: its stability check then includes the flow).  On a batch context w spans the concatenated cells

@@ -325,7 +325,7 @@ fdirw::MarchArgs fdirw::march_args(const fdirw_ctx* c) {
     a.src_begin = 0;
     a.src_end = c->g.n;
     a.list = nullptr;
-    if (c->flow) {                                    // convection: direction-dependent faces (mapping 5)
+    if (c->flow) {                                    // convection: direction-dependent faces (reported as mapping 5)
         a.bx = reinterpret_cast<const float*>(c->coefb[0]);
         a.by = reinterpret_cast<const float*>(c->coefb[1]);
         a.bz = reinterpret_cast<const float*>(c->coefb[2]);

@@ -314,7 +314,7 @@ MarchArgs march_args(const fdirw_ctx* c, const Chunk& ch, int r) {
     a.Q = static_cast<char*>(b.arena) + ch.k_off[r];
     a.store = c->store;
     a.sigma = c->sigma;
-    if (c->flow) {                                    // convection: direction-dependent faces (mapping 5)
+    if (c->flow) {                                    // convection: direction-dependent faces (reported as mapping 5)
         a.bx = reinterpret_cast<const float*>(c->coefb[0]);
         a.by = reinterpret_cast<const float*>(c->coefb[1]);
         a.bz = reinterpret_cast<const float*>(c->coefb[2]);

@@ -60,7 +60,7 @@ struct MarchArgs {
     int64_t q_stride;
     int src_major;
     int q_vec;
-    // Coarse-mesh march (coarse_B > 0, mapping 5 only): list holds coarse block indices; see coarse.cu.
+    // Coarse-mesh march (coarse_B > 0; launch_march_coarse): list holds coarse block indices; see coarse.cu.
     int coarse_B, coarse_Rc;
     int ncx, ncy, ncz;
     int64_t coarse_n;            // ncx * ncy * ncz
@@ -68,7 +68,7 @@ struct MarchArgs {
     const int32_t* ccount;       // coarse_n: liquid cells per block
     double* Qc;                  // (2 Rc + 1)^3 planes of coarse_n values, destination-indexed
     const float* abnd;           // nullable: lam * open-face conductance of each cell (far-field boundary)
-    // Convection (nullable; mapping 5 only): ax/ay/az then hold the coefficient of the lower cell in the
+    // Convection (nullable): ax/ay/az then hold the coefficient of the lower cell in the
     // upper cell's update across each +face, bx/by/bz that of the upper cell in the lower cell's update.
     const float* bx; const float* by; const float* bz;
     // Slab streaming of a uniform context (dest_z1 > dest_z0): only destinations of the z-planes [dest_z0, dest_z1)

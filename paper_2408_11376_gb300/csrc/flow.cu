@@ -3,7 +3,7 @@
 // cell i sends lam g + lam_a w+ of its value to the upper cell and receives lam g + lam_a w- of the
 // upper cell's, with lam = dt_sub / h^2 and lam_a = dt_sub / h.  The two coefficients replace the
 // symmetric lam g of the diffusion-only march: A (lower into upper) in the context's coefficient arrays,
-// B (upper into lower) in a second set, and the march runs mapping 5 with direction-dependent faces.
+// B (upper into lower) in a second set, and the march reads both (march_flow.cu, reported as mapping 5).
 // On a coarse-mesh context the liquid mask closes faces touching non-liquid cells for both fluxes, and
 // the block-source march and the P_BC march use the same coefficients; open faces stay diffusive.
 #include "fdirw.h"
