@@ -209,7 +209,8 @@ int conductances(fdirw_ctx* c, const double* D, double* g3[3], double* max_sum) 
     cudaError_t e = cudaMemsetAsync(flags, 0, 16, c->stream);
     if (e == cudaSuccess) e = fdirw::launch_conductance(Dd, g, g3[0], g3[1], g3[2], flags, flags + 1, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, flags, 16, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    const cudaError_t w = cudaStreamSynchronize(c->stream);      // also after a failure: the blocks go to other contexts
+    if (e == cudaSuccess) e = w;
     if (dD) { drelease(dD); c->allocated -= (uint64_t)g.n * 8; }
     drelease(flags);
     c->allocated -= 16;
@@ -478,7 +479,8 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
             e = fdirw::launch_coef_f32(reinterpret_cast<double*>(c->coef[a]), c->lam, c->g.n, reinterpret_cast<float*>(f[a]),
                                        c->stream);
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);      // the FP64 arrays are free again
+        const cudaError_t w = cudaStreamSynchronize(c->stream);      // also after a failure: the blocks go to other contexts
+        if (e == cudaSuccess) e = w;      // the FP64 arrays are free again
         if (e != cudaSuccess) {
             for (void* p : f) drelease(p);
             c->err = cuda_msg("coefficient kernel", e);

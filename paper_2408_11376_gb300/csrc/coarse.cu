@@ -746,7 +746,8 @@ int fdirw_coarse_far_field(fdirw_ctx* c, double V_far, double c_far) {
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h, mx, 8, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        const cudaError_t w = cudaStreamSynchronize(c->stream);      // also after a failure: the blocks go to other contexts
+        if (e == cudaSuccess) e = w;
         drelease(mx);
         c->allocated -= 8;
         if (e != cudaSuccess) { cudaGetLastError(); return fail(c, FDIRW_ERR_CUDA, cuda_msg("open faces", e)); }
@@ -894,7 +895,8 @@ int fdirw_read_coarse(fdirw_ctx* c, const int64_t* blocks, int64_t n, double* ou
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, (size_t)(n * W3) * 8, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    const cudaError_t w = cudaStreamSynchronize(c->stream);      // also after a failure: the blocks go to other contexts
+    if (e == cudaSuccess) e = w;
     drelease(db);
     drelease(dout);
     c->allocated -= (uint64_t)n * 8 + (uint64_t)(n * W3) * 8;
