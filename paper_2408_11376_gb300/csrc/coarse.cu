@@ -116,24 +116,36 @@ __global__ void count_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, 
     }
 }
 
-// Eq. 13: C_I = (sum of c over the liquid cells of block I) / N_I.  One warp per block: lane l takes the block's cells
-// l, l + 32, ... in z, y, x order, then a xor-butterfly (one thread for a block's 125 cells left most of the GPU idle:
-// 96^3, B = 5, 27 -> 14 us).
+// Eq. 13: C_I = (sum of c over the liquid cells of block I) / N_I.  Eight lanes per block, 4 blocks per warp: lane l takes
+// the block's (x, y) columns l, l + 8, ... and walks each in z, then a xor-butterfly.  One thread for a block's 125 cells
+// leaves most of a small grid's GPU idle; a whole warp spends the FP64 pipe (16 clocks an instruction and SM) on sums and
+// divisions of idle lanes.  B = 5, us at 96^3 / 192^3: one thread 27 / 48, a warp 14 / 80, eight lanes 11 / 34.
 __global__ void map_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, int ncx, int ncy, int64_t nc,
                            const int32_t* __restrict__ count, const double* __restrict__ c, double* __restrict__ C) {
-    const int lane = threadIdx.x & 31;
-    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t I = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); I < nc; I += step) {
-        const int bx = (int)(I % ncx), by = (int)((I / ncx) % ncy), bz = (int)(I / ((int64_t)ncx * ncy));
+    const int lane = threadIdx.x & 31, l = lane & 7;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), nxy = (int64_t)g.nx * g.ny;
+    Grid blocks = g;
+    blocks.nx = ncx;
+    blocks.ny = ncy;
+    blocks.n = nc;
+    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); 4 * w < nc; w += warps) {
+        const int64_t I = 4 * w + (lane >> 3);
         double s = 0.0;
-        for (int e = lane; e < B * B * B; e += 32) {
-            const int x = bx * B + e % B, y = by * B + e / B % B, z = bz * B + e / (B * B);
-            if (x >= g.nx || y >= g.ny || z >= g.nz) continue;
-            const int64_t i = x + (int64_t)g.nx * (y + (int64_t)g.ny * z);
-            if (liquid[i]) s += c[i];
+        if (I < nc) {
+            int bx, by, bz;
+            cell_of(I, blocks, bx, by, bz);
+            const int nz = min(B, g.nz - bz * B);
+            for (int e = l; e < B * B; e += 8) {
+                const int dy = e / B, x = bx * B + e - dy * B, y = by * B + dy;
+                if (x >= g.nx || y >= g.ny) continue;
+                const int64_t i = x + (int64_t)g.nx * y + nxy * ((int64_t)bz * B);
+#pragma unroll 5
+                for (int z = 0; z < nz; z++)
+                    if (liquid[i + z * nxy]) s += c[i + z * nxy];
+            }
         }
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        if (lane == 0) C[I] = count[I] > 0 ? s / (double)count[I] : 0.0;
+        for (int off = 1; off < 8; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (l == 0 && I < nc) C[I] = count[I] > 0 ? s / (double)count[I] : 0.0;
     }
 }
 
@@ -507,7 +519,7 @@ int coarse_kernels(fdirw_ctx* c) {
             std::swap(u0, u1);
         }
         widen_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(u0, c->g.n, c->cbuf);
-        map_kernel<<<grid_blocks(k.nc, 8), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
+        map_kernel<<<grid_blocks(k.nc, 32), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
                                                                   c->cbuf, k.pbc);
         FDIRW_CUDA(c, cudaGetLastError());
     }
@@ -544,7 +556,7 @@ static int coarse_steps(fdirw_ctx* c, const double* c_in, double* c_out, int32_t
     } else {
         const double* cur = src;
         for (int t = 0; t < n_steps; t++) {
-            map_kernel<<<grid_blocks(k.nc, 8), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count, cur, k.C);
+            map_kernel<<<grid_blocks(k.nc, 32), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count, cur, k.C);
             FDIRW_CUDA(c, cudaGetLastError());
             const bool last = t + 1 == n_steps;
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
