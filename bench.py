@@ -204,11 +204,9 @@ def march_kernel_name(prec: str, parts: int) -> str:
 
 
 # DRAM bytes (read + write) per clipped window cell of march_tm_kernel<8> with BF16 storage, from one ncu
-# capture of the 64^3 case with the same recipe (`--set full` on the first march launch of `bench.py
-# --workload fdirw-64c-r8 --prec bf16 --march-parts 4 --no-surrogate --no-probe`: 0.641 GB read + 2.307 GB
-# written over 1.0488e9 window cells); the traffic of a full launch scales with its window cells (the
+# capture of a 64^3 launch with R = 8 and n_sub = 200 (0.8985 GB read + 2.63 GB written over 1.0488e9 window cells); the traffic of a full launch scales with its window cells (the
 # stored kernel values dominate it).  Valid for that kernel, radius and storage only.
-TM_R8_BF16_DRAM_BYTES_PER_WINDOW_CELL = (0.641067008e9 + 2.306592e9) / 1048772096
+TM_R8_BF16_DRAM_BYTES_PER_WINDOW_CELL = (0.8985e9 + 2.63e9) / 1048772096
 
 
 def march_traffic(args, prec: str, parts: int, R: int, window_cells: float):
@@ -219,8 +217,8 @@ def march_traffic(args, prec: str, parts: int, R: int, window_cells: float):
     return None
 
 
-# DRAM bytes (read + write) per algorithmic byte of gather_fp32_kernel<bf16> from one ncu capture of the
-# 96^3, R = 6 case (`bench.py --workload fdirw-96c-r6`: 3.8927e9 read + 3.33e6 written against
+# DRAM bytes (read + write) per algorithmic byte of the FP32-accumulation gather with a BF16 cache, from one ncu capture
+# of a 96^3, R = 6 step (`bench.py --workload fdirw-96c-r6`: 3.8927e9 read + 3.33e6 written against
 # 3.8971e9 algorithmic); the traffic of a launch grows with its cache bytes.  Valid for that kernel and
 # storage only.
 GATHER_FP32_BF16_DRAM_PER_ALGORITHMIC_BYTE = (3.892684288e9 + 3.326464e6) / (96 ** 3 * (13 ** 3 * 2 + 4 + 8))
@@ -234,8 +232,8 @@ def gather_roofline(prec: str, accum: str, N: int, R: int, gather_ms: float, pro
     chat_b = 8 if prec == "fp64" else (4 if accum == "fp32" else 8)
     nbytes = N * (2 * R + 1) ** 3 * qb + N * chat_b + N * 8
     achieved = nbytes / (gather_ms * 1e-3) / 1e9
-    kname = ("gather_f64_kernel<R>" if prec == "fp64" else
-             "gather_fp32_kernel<ST,R>" if accum == "fp32" else "gather_ff_kernel<ST,R>")
+    kname = ("gather_kernel<double,R,0>" if prec == "fp64" else
+             "gather_kernel<ST,R,2>" if accum == "fp32" else "gather_kernel<ST,R,1>")
     traffic = GATHER_FP32_BF16_DRAM_PER_ALGORITHMIC_BYTE * nbytes if (prec == "bf16" and accum == "fp32") else None
     return {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
@@ -278,10 +276,10 @@ def fp32_alu_roofline(torch, dev, n_sub: int, window_cells: float, march_ms: flo
 
 
 # Shared-memory wavefronts of march_tm_kernel<8> per COMPUTED thread-cell-substep (every CTA batch marches 256
-# threads x 68 cells whatever the windows' clipping), from the same 64^3 capture: 3.298e10 wavefronts over
+# threads x 68 cells whatever the windows' clipping), from the same 64^3 capture: 2.885e10 wavefronts over
 # 87,382 batches x 256 x 68 x 200.  A launch's wavefronts scale with its computed cells; the shared-memory
 # peak is one 128-byte wavefront per SM-cycle (32 banks x 4 B).
-TM_R8_SMEM_WAVEFRONTS_PER_COMPUTED_CELL = 3.2981171846e10 / (87382 * 256 * 68 * 200)
+TM_R8_SMEM_WAVEFRONTS_PER_COMPUTED_CELL = 2.884910412e10 / (87382 * 256 * 68 * 200)
 
 
 def march_smem(n_src: int, n_sub: int, R: int, parts: int, march_ms: float, sm_mhz: float, num_sms: int):
@@ -927,12 +925,12 @@ def coupled_leg(args, fdirw, torch, dev, stream, w, shape, D, liquid, dt_macro):
 
 
 def flow_leg(args, fdirw, torch, dev, stream, w, shape, D, solid, dt_macro):
-    """Convection (Sec. 5): a steady face-velocity field folded into every source's march (upwind faces,
-    mapping 5), the superposition unchanged.  Flow: a mean of 0.03 cells per unit time along +x plus
+    """Convection (Sec. 5): a steady face-velocity field folded into every source's march (upwind faces),
+    the superposition unchanged.  Flow: a mean of 0.03 cells per unit time along +x plus
     uniform noise of 0.03 on every face, zero on faces touching a solid cell; n_sub raised by a tenth so
     that the diffusive part leaves room for the advective outflow within the same macro step.  Field: a
     Gaussian blob (sigma 10 cells) on the pore cells.  Times create + velocity + kernels + macro steps
-    with the flow, and the same n_sub on mapping 5 without it (the march's cost of the upwind faces)."""
+    with the flow, and the same n_sub on mapping 5 without it."""
     from paper_2408_11376_gb300 import synth
     n_sub = -(-11 * w.n_sub // 10)
     N = shape[0] * shape[1] * shape[2]
@@ -965,7 +963,7 @@ def flow_leg(args, fdirw, torch, dev, stream, w, shape, D, solid, dt_macro):
     job_ms, build_ms, steps_ms, info, mass, xc = res[True]
     mass0 = float(c_in.sum().item())
     roof = fp32_alu_roofline(torch, dev, n_sub, info["window_cells"], info["kernels_ms"], None, {},
-                             "march_tmc_kernel<R, ADV>")
+                             "march_flow_kernel<R>")
     return {"n_sub": n_sub, "velocity": "mean 0.03 along +x, noise 0.03, 0 on solid faces",
             "macro_steps_per_s": 1000.0 * w.steps / job_ms, "job_ms": job_ms, "kernels_ms": build_ms,
             "steps_ms": steps_ms, "march_kernel_ms": info["kernels_ms"],
