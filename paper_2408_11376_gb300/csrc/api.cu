@@ -473,6 +473,7 @@ int fdirw_create(const fdirw_grid* grid, const double* D_map, double dt_macro, i
         cudaError_t e = cudaSuccess;
         for (int a = 0; a < 3 && e == cudaSuccess; a++) {
             if ((rc = dalloc(c, &f[a], n * 4, "coefficients")) != FDIRW_OK) {
+                cudaStreamSynchronize(c->stream);            // the conversions queued so far write the blocks
                 for (void* p : f) drelease(p);
                 return bail(rc);
             }

@@ -1,0 +1,97 @@
+"""The library's host code on a stand-in for the CUDA runtime (fake_cudart.cpp): every call of a scenario is made to fail
+in turn.  Whatever fails, no device block may go back to the pool of idle blocks while work is queued that can still use it
+(another thread's context would get it), and what a failed call left half made is not taken for finished by the next."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2408_11376_gb300 import FDiRW, build, fdirw
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The library's objects linked with the stand-in, in the place of the library."""
+    if shutil.which("g++") is None:
+        pytest.skip("g++ not available")
+    build.build()
+    objs = [os.path.join(build.BUILD, s.replace(".cu", ".o")) for s in build.SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        build.build(force=True)
+    so = str(tmp_path_factory.mktemp("fake") / "libfdirw_fake.so")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CUDA_INCLUDE, "-o", so,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs], check=True)
+    saved = fdirw._lib
+    fdirw._lib = None
+    lib = fdirw.load(so)
+    lib.fake_calls.restype = lib.fake_violations.restype = lib.fake_launched.restype = ctypes.c_long
+    lib.fake_held.restype = ctypes.c_uint64
+    lib.fake_fail_at.argtypes = [ctypes.c_long]
+    lib.fake_scalar.argtypes = [ctypes.c_double]
+    lib.fake_free_bytes.argtypes = [ctypes.c_uint64]
+    yield lib
+    fdirw._lib = saved
+
+
+def _stream(lib):
+    s = ctypes.c_void_p()
+    assert lib.cudaStreamCreateWithFlags(ctypes.byref(s), 0) == 0
+    return s.value
+
+
+def _each_failure(lib, prepare, act, finish):
+    """act(state) with each of its runtime calls made to fail in turn, then finish(state); the calls that it made."""
+    k = 0
+    while True:
+        lib.fake_reset()
+        st = prepare()
+        lib.fake_fail_at(k)
+        try:
+            act(st)
+        except fdirw.FdirwError:
+            pass
+        n = lib.fake_calls()
+        lib.fake_fail_at(-1)
+        finish(st)
+        assert lib.fake_violations() == 0, f"call {k}: a block was given back under queued work"
+        k += 1
+        if k > n:
+            return n
+
+
+def _close(st):
+    for f in st:
+        f.close()
+
+
+# Sizes: the arrays that matter are above 64 MB, so that they go to cudaFree, where the stand-in looks, not to the pool.
+BIG = (256, 256, 257)
+
+
+def test_create(fake):
+    D = np.empty(int(np.prod(BIG)))
+    stream = _stream(fake)
+    for prec in ("fp32", "fp64"):
+        def act(st):
+            st.append(FDiRW(BIG, D, 0.1, 1, 1, prec, stream=stream))
+            st[0].kernels()
+            st[0].step(D, D, 1, want_mass=True)
+            st[0].read_kernels([0, 1])
+            st[0].read_kernels(range(9))
+        assert _each_failure(fake, list, act, _close) > 30
+
+
+@pytest.mark.parametrize("per_cell", range(8, 45, 4))
+def test_create_at_a_memory_limit(fake, per_cell):
+    D = np.empty(int(np.prod(BIG)))
+    fake.fake_reset()
+    with pytest.raises(fdirw.FdirwError) as e:
+        FDiRW(BIG, D, 0.1, 1, 1, stream=_stream(fake), mem_limit=per_cell * D.size + 64)
+    assert e.value.code == fdirw.FDIRW_ERR_NOMEM
+    assert fake.fake_violations() == 0
