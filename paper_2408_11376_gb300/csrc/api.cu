@@ -169,6 +169,16 @@ void dfree(void*& p) {
     p = nullptr;
 }
 
+void Scratch::release() {
+    if (blocks_.empty()) return;
+    cudaStreamSynchronize(c_->stream);
+    for (auto& b : blocks_) {
+        drelease(b.first);
+        c_->allocated -= b.second;
+    }
+    blocks_.clear();
+}
+
 uint64_t idle_device_bytes(int device) { return pool().idle_on(device); }
 
 }  // namespace host

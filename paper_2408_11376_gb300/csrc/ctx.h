@@ -3,6 +3,7 @@
 
 #include <cmath>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -83,6 +84,25 @@ int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what);
 // Frees a dalloc'ed block that no work uses any more (a pool of small ones keeps it for the next dalloc).
 void drelease(void* p);
 void dfree(void*& p);
+// Device blocks of one call.  However the call ends, they are given back only after the context's stream has finished.
+class Scratch {
+  public:
+    explicit Scratch(fdirw_ctx* c) : c_(c) {}
+    ~Scratch() { release(); }
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    template <typename T>
+    int get(T** p, uint64_t bytes, const char* what) {
+        const int rc = dalloc(c_, reinterpret_cast<void**>(p), bytes, what);
+        if (rc == FDIRW_OK) blocks_.push_back({*p, bytes});
+        return rc;
+    }
+    void release();
+
+  private:
+    fdirw_ctx* c_;
+    std::vector<std::pair<void*, uint64_t>> blocks_;
+};
 // Bytes of the pool's idle blocks on a device: free memory to a dalloc, though the driver counts them as used.
 uint64_t idle_device_bytes(int device);
 }  // namespace host

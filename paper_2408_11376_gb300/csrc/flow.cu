@@ -100,20 +100,13 @@ int fdirw_set_velocity(fdirw_ctx* c, const double* w) {
     }
     double* dw = nullptr;
     unsigned long long* mx = nullptr;
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&dw), 3 * n * 8, "velocity staging")) != FDIRW_OK) return rc;
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&mx), 8, "flags")) != FDIRW_OK) {
-        drelease(dw);
-        c->allocated -= 3 * n * 8;
-        return rc;
-    }
     // The coefficient arrays are contiguous per axis in this file's kernel; the context keeps three
     // separate allocations, so stage A and B in one block and copy them out.
     float* AB = nullptr;
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&AB), 6 * n * 4, "coefficient staging")) != FDIRW_OK) {
-        drelease(dw); drelease(mx);
-        c->allocated -= 3 * n * 8 + 8;
-        return rc;
-    }
+    Scratch tmp(c);
+    if ((rc = tmp.get(&dw, 3 * n * 8, "velocity staging")) != FDIRW_OK) return rc;
+    if ((rc = tmp.get(&mx, 8, "flags")) != FDIRW_OK) return rc;
+    if ((rc = tmp.get(&AB, 6 * n * 4, "coefficient staging")) != FDIRW_OK) return rc;
     unsigned long long h = 0;
     cudaError_t e = cudaMemcpyAsync(dw, w, 3 * n * 8, cudaMemcpyDefault, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(mx, 0, 8, c->stream);
@@ -149,10 +142,7 @@ int fdirw_set_velocity(fdirw_ctx* c, const double* w) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->coefb[a], AB + (3 + a) * n, n * 4, cudaMemcpyDeviceToDevice, c->stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    drelease(dw);
-    drelease(mx);
-    drelease(AB);
-    c->allocated -= 3 * n * 8 + 8 + 6 * n * 4;
+    tmp.release();
     if (e != cudaSuccess) { cudaGetLastError(); return fail(c, FDIRW_ERR_CUDA, cuda_msg("velocity coefficients", e)); }
     if (!std::isfinite(m)) return fail(c, FDIRW_ERR_ARG, "w holds NaN or infinite values");
     if (!stable) {

@@ -72,6 +72,7 @@ def _close(st):
 
 # Sizes: the arrays that matter are above 64 MB, so that they go to cudaFree, where the stand-in looks, not to the pool.
 BIG = (256, 256, 257)
+MID = (143, 143, 143)
 
 
 def test_create(fake):
@@ -95,3 +96,10 @@ def test_create_at_a_memory_limit(fake, per_cell):
         FDiRW(BIG, D, 0.1, 1, 1, stream=_stream(fake), mem_limit=per_cell * D.size + 64)
     assert e.value.code == fdirw.FDIRW_ERR_NOMEM
     assert fake.fake_violations() == 0
+
+
+def test_set_velocity(fake):
+    D = np.empty(int(np.prod(MID)))
+    w = np.empty(3 * D.size)
+    stream = _stream(fake)
+    assert _each_failure(fake, lambda: [FDiRW(MID, D, 0.1, 1, 1, stream=stream)], lambda st: st[0].set_velocity(w), _close) > 8
