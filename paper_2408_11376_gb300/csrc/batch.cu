@@ -741,8 +741,10 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
     b.Rmin = R_min;
     b.Rmax = R_max;
 
+    Scratch tmp(c);
     auto bail = [&](int rc) {
         std::string msg = c->err;
+        tmp.release();
         if (c->stream) cudaStreamSynchronize(c->stream); else cudaDeviceSynchronize();
         fdirw::batch_release(c);
         for (auto& p : c->coef) dfree(p);
@@ -796,14 +798,9 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
     double* g3 = nullptr;
     unsigned long long* flags = nullptr;
     int8_t* dR = nullptr;
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&g3), (uint64_t)maxn * 24, "conductance staging")) != FDIRW_OK) return bail(rc);
-    auto free_tmp = [&]() {
-        void* p = g3; if (p) { dfree(p); c->allocated -= (uint64_t)maxn * 24; } g3 = nullptr;
-        p = flags; if (p) { dfree(p); c->allocated -= 16; } flags = nullptr;
-        p = dR; if (p) { dfree(p); c->allocated -= N; } dR = nullptr;
-    };
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&flags), 16, "flags")) != FDIRW_OK) { free_tmp(); return bail(rc); }
-    if ((rc = dalloc(c, reinterpret_cast<void**>(&dR), N, "radius map")) != FDIRW_OK) { free_tmp(); return bail(rc); }
+    if ((rc = tmp.get(&g3, (uint64_t)maxn * 24, "conductance staging")) != FDIRW_OK) return bail(rc);
+    if ((rc = tmp.get(&flags, 16, "flags")) != FDIRW_OK) return bail(rc);
+    if ((rc = tmp.get(&dR, N, "radius map")) != FDIRW_OK) return bail(rc);
     double worst = 0.0;
     for (int i = 0; i < n && e == cudaSuccess; i++) {
         const fdirw::Grid& g = b.grids[i];
@@ -823,14 +820,12 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) break;
         if (h[1] != 0ull) {
-            free_tmp();
             c->err = "D map of structure " + std::to_string(i) + " holds NaN, infinite or negative values";
             return bail(FDIRW_ERR_ARG);
         }
         double m;
         std::memcpy(&m, &h[0], 8);
         if (b.lams[i] * m > 1.0 + 1e-12) {
-            free_tmp();
             char buf[256];
             std::snprintf(buf, sizeof buf, "unstable: structure %d has dt_sub*max(sum g)/h^2 = %.17g > 1", i, b.lams[i] * m);
             c->err = buf;
@@ -838,12 +833,12 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
         }
         if (b.lams[i] * m >= worst) { worst = b.lams[i] * m; c->max_face_sum = m; }
     }
-    if (e != cudaSuccess) { free_tmp(); return cuda_bail("batch setup", e); }
+    if (e != cudaSuccess) return cuda_bail("batch setup", e);
 
     // Buckets (host): code(s) = (R << 28) | position in the radius-R list, lists in global cell order.
     std::vector<int8_t> Rh(N);
     e = cudaMemcpy(Rh.data(), dR, N, cudaMemcpyDeviceToHost);
-    free_tmp();
+    tmp.release();
     if (e != cudaSuccess) return cuda_bail("copy radius map", e);
     std::vector<uint32_t> code(N);
     std::vector<int64_t> lists[fdirw::kMaxR + 1];

@@ -9,7 +9,7 @@ import subprocess
 import numpy as np
 import pytest
 
-from paper_2408_11376_gb300 import FDiRW, build, fdirw
+from paper_2408_11376_gb300 import FDiRW, FDiRWBatch, build, fdirw
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
@@ -83,8 +83,6 @@ def test_create(fake):
             st.append(FDiRW(BIG, D, 0.1, 1, 1, prec, stream=stream))
             st[0].kernels()
             st[0].step(D, D, 1, want_mass=True)
-            st[0].read_kernels([0, 1])
-            st[0].read_kernels(range(9))
         assert _each_failure(fake, list, act, _close) > 30
 
 
@@ -103,3 +101,18 @@ def test_set_velocity(fake):
     w = np.empty(3 * D.size)
     stream = _stream(fake)
     assert _each_failure(fake, lambda: [FDiRW(MID, D, 0.1, 1, 1, stream=stream)], lambda st: st[0].set_velocity(w), _close) > 8
+
+
+BATCH = [MID, (9, 8, 7)]
+
+
+def _batch(fake, stream):
+    fake.fake_fill(1)                                # the radius of every source
+    f = FDiRWBatch(BATCH, [np.empty(int(np.prod(s))) for s in BATCH], 0.1, 1, 1, 1, "bf16", stream=stream)
+    fake.fake_fill(0)
+    return f
+
+
+def test_batch_create(fake):
+    stream = _stream(fake)
+    assert _each_failure(fake, list, lambda st: st.append(_batch(fake, stream)), _close) > 30
