@@ -514,6 +514,9 @@ double window_cells_of(const Grid& g, const int8_t* R) {
 void release_batch(fdirw_ctx* c) {
     Batch* b = c->batch;
     if (!b) return;
+    // A call that failed can have left work on these streams that the context's stream does not wait for.
+    if (b->gs) cudaStreamSynchronize(b->gs);
+    for (auto s : b->aux) if (s) cudaStreamSynchronize(s);
     drop_graph(*b);
     void* p;
     p = b->d_base; dfree(p);

@@ -116,3 +116,13 @@ def _batch(fake, stream):
 def test_batch_create(fake):
     stream = _stream(fake)
     assert _each_failure(fake, list, lambda st: st.append(_batch(fake, stream)), _close) > 30
+
+
+def test_batch_work(fake):
+    stream = _stream(fake)
+    c = np.zeros(sum(int(np.prod(s)) for s in BATCH))
+
+    def work(st):
+        st[0].kernels()
+        st[0].step(c, c, 2)
+    assert _each_failure(fake, lambda: [_batch(fake, stream)], work, _close) > 30
