@@ -647,8 +647,8 @@ int fdirw_read_kernels(fdirw_ctx* c, const int64_t* sources, int64_t n, double* 
     DeviceGuard dg(c->device);
     const int64_t W = (int64_t)(2 * c->R + 1) * (2 * c->R + 1) * (2 * c->R + 1);
     if (n > c->kcap) {
-        void* p = c->dsrc; dfree(p); c->dsrc = nullptr;
-        p = c->dkout; dfree(p); c->dkout = nullptr;
+        retire(c, c->dsrc);
+        retire(c, c->dkout);
         c->allocated -= (uint64_t)c->kcap * (8 + 8 * W);
         c->kcap = 0;
         int rc = dalloc(c, reinterpret_cast<void**>(&c->dsrc), (uint64_t)n * 8, "source list");

@@ -615,8 +615,8 @@ int batch_read_kernels(fdirw_ctx* c, const int64_t* sources, int64_t n, double* 
     if (b.chunks.size() != 1 || b.resident != 0)
         return fail(c, FDIRW_ERR_STATE, "kernels of a batch are readable only when they all fit (one chunk) and are built");
     if (n > c->kcap) {
-        void* p = c->dsrc; dfree(p); c->dsrc = nullptr;
-        p = c->dkout; dfree(p); c->dkout = nullptr;
+        retire(c, c->dsrc);
+        retire(c, c->dkout);
         c->allocated -= (uint64_t)c->kcap * (8 + 8 * W);
         c->kcap = 0;
         int rc = dalloc(c, reinterpret_cast<void**>(&c->dsrc), (uint64_t)n * 8, "source list");

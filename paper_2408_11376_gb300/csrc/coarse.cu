@@ -840,7 +840,7 @@ int fdirw_coupled_step(fdirw_ctx* c, const fdirw_coupled_params* p, double* fiel
     if (lam_s > 0.0 && lam_s * k.gs_max > 1.0 + 1e-12)
         return fail(c, FDIRW_ERR_UNSTABLE, "solid march unstable: raise n_sub_solid");
     if ((QL || QS) && n_steps > k.qcap) {
-        void* q = k.qout; dfree(q); k.qout = nullptr;
+        retire(c, k.qout);
         c->allocated -= (uint64_t)k.qcap * 16;
         k.qcap = 0;
         if ((rc = dalloc(c, reinterpret_cast<void**>(&k.qout), (uint64_t)n_steps * 16, "phase masses")) != FDIRW_OK) return rc;

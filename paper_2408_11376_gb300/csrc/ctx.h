@@ -84,6 +84,14 @@ int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what);
 // Frees a dalloc'ed block that no work uses any more (a pool of small ones keeps it for the next dalloc).
 void drelease(void* p);
 void dfree(void*& p);
+// Gives a context's block back while the context goes on: after its stream, on which a call that failed can have left
+// work, has finished.
+template <typename T>
+void retire(fdirw_ctx* c, T*& p) {
+    if (p) cudaStreamSynchronize(c->stream);
+    drelease(p);
+    p = nullptr;
+}
 // Device blocks of one call.  However the call ends, they are given back only after the context's stream has finished.
 class Scratch {
   public:

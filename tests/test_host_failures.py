@@ -9,7 +9,7 @@ import subprocess
 import numpy as np
 import pytest
 
-from paper_2408_11376_gb300 import FDiRW, FDiRWBatch, build, fdirw
+from paper_2408_11376_gb300 import FDiRW, FDiRWBatch, FDiRWCoarse, build, fdirw
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
@@ -126,3 +126,36 @@ def test_batch_work(fake):
         st[0].kernels()
         st[0].step(c, c, 2)
     assert _each_failure(fake, lambda: [_batch(fake, stream)], work, _close) > 30
+
+
+def test_coarse(fake):
+    D = np.empty(int(np.prod(MID)))
+    stream = _stream(fake)
+
+    def act(st):
+        fake.fake_fill(1)                            # liquid cells of every block
+        st.append(FDiRWCoarse(MID, D, None, 3, 0.1, 1, 1, stream=stream))
+        st[0].far_field(10.0, 0.1)
+        st[0].coupled_step(D, 1, 1e-7, 1.0, 1e-5, 0.1, 1)
+        st[0].coupled_step(D, 3, 1e-7, 1.0, 1e-5, 0.1, 1)
+        st[0].read_coarse([0, 1])
+    assert _each_failure(fake, list, act, _close) > 40
+
+
+def test_read_back(fake):
+    """Read-back buffers that grow after a call that failed with its kernel queued."""
+    D = np.empty(int(np.prod(MID)))
+    stream = _stream(fake)
+
+    def prepare():
+        f = FDiRW(MID, D, 0.1, 1, 1, stream=stream)
+        f.kernels()
+        return [f]
+
+    def act(st):
+        st[0].read_kernels(np.zeros(330000, dtype=np.int64))
+
+    def grow(st):
+        st[0].read_kernels(np.zeros(330001, dtype=np.int64))
+        _close(st)
+    assert _each_failure(fake, prepare, act, grow) > 3
