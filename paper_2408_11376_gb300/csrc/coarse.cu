@@ -48,7 +48,8 @@ struct Coarse {
     // Coupled macro step: FP64 solid-phase face conductances, a scratch field, phase-mass partials.
     double* gs = nullptr;                        // 3 N: +x/+y/+z solid-solid faces
     double* tmp = nullptr;                       // 2 N
-    double gs_max = 0.0;                         // largest per-cell sum of gs
+    bool gs_ready = false;                       // gs has been computed
+    double gs_max = -1.0;                        // largest per-cell sum of gs; negative: not known yet
     double* qpart = nullptr;                     // kMassBlocks
     double* qout = nullptr;                      // [Q_L, Q_S] per step, n_steps_cap * 2
     int64_t qcap = 0;
@@ -819,17 +820,20 @@ int fdirw_coupled_step(fdirw_ctx* c, const fdirw_coupled_params* p, double* fiel
     const uint64_t n = (uint64_t)c->g.n;
     int rc;
     const double lam_s = p->n_sub_solid > 0 ? (p->dt / p->n_sub_solid) / (c->h * c->h) : 0.0;
-    if (!k.gs) {
+    if (!k.gs_ready) {
         if (!k.tmp && (rc = dalloc(c, reinterpret_cast<void**>(&k.tmp), 2 * n * 8, "coupled scratch")) != FDIRW_OK) return rc;
         if (!k.qpart && (rc = dalloc(c, reinterpret_cast<void**>(&k.qpart), fdirw::kMassBlocks * 8, "phase partials")) != FDIRW_OK)
             return rc;
-        if ((rc = dalloc(c, reinterpret_cast<void**>(&k.gs), 3 * n * 8, "solid faces")) != FDIRW_OK) return rc;
-        // The largest sum of a cell's solid faces, for the stability check of every call (on the device: copying the
-        // 3 N conductances out for a host loop took 8 of a 30 ms call at 96^3).
-        unsigned long long h = 0, *mx = reinterpret_cast<unsigned long long*>(k.tmp);
+        if (!k.gs && (rc = dalloc(c, reinterpret_cast<void**>(&k.gs), 3 * n * 8, "solid faces")) != FDIRW_OK) return rc;
         fdirw::solid_faces_kernel<<<fdirw::grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, c->Dd, k.liquid, k.gs,
                                                                                         k.gs + n, k.gs + 2 * n);
         FDIRW_CUDA(c, cudaGetLastError());
+        k.gs_ready = true;
+    }
+    if (lam_s > 0.0 && k.gs_max < 0.0) {
+        // The largest sum of a cell's solid faces, for the stability check of every call (on the device: copying the
+        // 3 N conductances out for a host loop took 8 of a 30 ms call at 96^3).
+        unsigned long long h = 0, *mx = reinterpret_cast<unsigned long long*>(k.tmp);
         FDIRW_CUDA(c, cudaMemsetAsync(mx, 0, 8, c->stream));
         fdirw::solid_max_kernel<<<fdirw::grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, k.gs, k.gs + n, k.gs + 2 * n, mx);
         FDIRW_CUDA(c, cudaGetLastError());

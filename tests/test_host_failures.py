@@ -159,3 +159,26 @@ def test_read_back(fake):
         st[0].read_kernels(np.zeros(330001, dtype=np.int64))
         _close(st)
     assert _each_failure(fake, prepare, act, grow) > 3
+
+
+def test_solid_stability_check_after_a_failed_call(fake):
+    """A call that failed while the solid faces were being made leaves no bound that the next one takes for checked."""
+    D = np.ones(12 * 11 * 10)
+    stream = _stream(fake)
+
+    def prepare():
+        f = FDiRWCoarse((12, 11, 10), D, None, 3, 0.1, 1, 1, stream=stream)
+        f.far_field(10.0, 0.1)
+        f.kernels()
+        fake.fake_scalar(1e6)                        # the largest sum of a cell's solid faces, as read from the device
+        return [f]
+
+    def act(st):
+        st[0].coupled_step(np.ones(D.size), 1, 1e-7, 1.0, 1e-5, 0.1, 1)
+
+    def again(st):
+        with pytest.raises(fdirw.FdirwError) as e:
+            act(st)
+        assert e.value.code == fdirw.FDIRW_ERR_UNSTABLE
+        _close(st)
+    assert _each_failure(fake, prepare, act, again) > 3
