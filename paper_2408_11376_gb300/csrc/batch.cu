@@ -29,6 +29,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 using namespace fdirw::host;
@@ -83,6 +84,7 @@ struct Batch {
     double* seg_part = nullptr;                  // FDIRW_ACCUM_FP32: 2 * kSegBlocks partial sums per structure
     double* seg_fix = nullptr;                   // FDIRW_ACCUM_FP32: [target total, factor] per structure
     std::vector<Chunk> chunks;
+    uint64_t budget = 0;                         // device bytes for the kernels of a chunk
     void* arena = nullptr;
     uint64_t arena_bytes = 0;
     int resident = -1;                           // chunk whose kernels the arena holds
@@ -273,7 +275,86 @@ int grid_blocks(int64_t n, int threads) {
 // ------------------------------------------------------------------------------------------ host
 
 // Values of a destination-indexed cache row of structure i.
-int row_of(const Batch& b, int i) { return (b.grids[i].nx + b.qvec - 1) / b.qvec * b.qvec; }
+int row_of(const Batch& b, int i, int qvec) { return (b.grids[i].nx + qvec - 1) / qvec * qvec; }
+int row_of(const Batch& b, int i) { return row_of(b, i, b.qvec); }
+
+// Chunks of consecutive structures whose kernels fit b.budget together, and each structure's first cache column, with
+// cache rows of a multiple of qvec values; too_large: a structure that does not fit alone (its bytes: need), or -1.
+struct Plan {
+    std::vector<Chunk> chunks;
+    std::vector<int64_t> qbase;
+    int too_large = -1;
+    uint64_t need = 0;
+    uint64_t arena() const {
+        uint64_t n = 0;
+        for (const Chunk& ch : chunks) n = std::max(n, ch.k_bytes);
+        return n;
+    }
+};
+Plan plan_chunks(const fdirw_ctx* c, int qvec) {
+    const Batch& b = *c->batch;
+    const int sb = store_bytes(c->store);
+    Plan p;
+    p.qbase.assign(b.n, 0);
+    auto slot = [&](int i) {                                            // 16-aligned destination columns
+        return ((int64_t)row_of(b, i, qvec) * b.grids[i].ny * b.grids[i].nz + 15) / 16 * 16;
+    };
+    auto kernel_bytes = [&](int i) {
+        uint64_t add = 0;
+        for (int r : b.radii) {
+            if (r == 0) continue;
+            const int64_t cols = (b.dest_mask >> r) & 1u ? slot(i) : b.before[r][i + 1] - b.before[r][i];
+            add += (uint64_t)cols * (uint64_t)wcells(r) * sb;
+        }
+        return add;
+    };
+    for (int i = 0; i < b.n;) {
+        Chunk ch;
+        ch.s0 = i;
+        uint64_t used = 0;
+        while (i < b.n) {
+            const uint64_t add = kernel_bytes(i);
+            if (used + add > b.budget) {
+                if (i > ch.s0) break;
+                p.too_large = i;
+                p.need = add;
+                return p;
+            }
+            used += add;
+            i++;
+        }
+        ch.s1 = i;
+        ch.c0 = b.base[ch.s0];
+        ch.c1 = b.base[ch.s1];
+        for (int k = ch.s0; k < ch.s1; k++) {
+            p.qbase[k] = ch.qn;
+            ch.qn += slot(k);
+        }
+        uint64_t off = 0;
+        for (int r : b.radii) {
+            ch.seg_begin[r] = b.before[r][ch.s0];
+            ch.seg_end[r] = b.before[r][ch.s1];
+            ch.k_off[r] = off;
+            const int64_t cols = (b.dest_mask >> r) & 1u ? ch.qn : ch.seg_end[r] - ch.seg_begin[r];
+            if (r > 0) off += align256((uint64_t)cols * wcells(r) * sb);
+        }
+        ch.k_bytes = off;
+        p.chunks.push_back(ch);
+    }
+    return p;
+}
+cudaError_t install_plan(fdirw_ctx* c, Plan&& p, int qvec) {
+    Batch& b = *c->batch;
+    std::swap(b.qbase, p.qbase);
+    const cudaError_t e = cudaMemcpyAsync(b.d_qbase, b.qbase.data(), (size_t)b.n * 8, cudaMemcpyHostToDevice, c->stream);
+    if (e != cudaSuccess) {
+        std::swap(b.qbase, p.qbase);
+        return e;
+    }
+    b.qvec = qvec;
+    b.chunks = std::move(p.chunks);
+    return cudaSuccess;
+}
 
 VarArgs var_args(const fdirw_ctx* c, const Chunk& ch, double* out) {
     const Batch& b = *c->batch;
@@ -343,7 +424,13 @@ int ensure_arena(fdirw_ctx* c) {
     uint64_t need = 0;
     for (const Chunk& ch : b.chunks) need = std::max(need, ch.k_bytes);
     if (need == 0) need = 256;
-    const int rc = dalloc(c, &b.arena, need, "kernel cache");
+    int rc = dalloc(c, &b.arena, need, "kernel cache");
+    if (rc == FDIRW_ERR_NOMEM && b.qvec > 1) {          // memory taken since: without the padding (as many chunks)
+        Plan packed = plan_chunks(c, 1);
+        need = std::max<uint64_t>(packed.arena(), 256);
+        FDIRW_CUDA(c, install_plan(c, std::move(packed), 1));
+        rc = dalloc(c, &b.arena, need, "kernel cache");
+    }
     if (rc != FDIRW_OK) return rc;
     b.arena_bytes = need;
     c->q_bytes = need;
@@ -901,75 +988,32 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
             return bail(rc);
     }
 
-    // Chunks: consecutive structures whose kernels fit the budget together.
-    const int sb = fdirw::store_bytes(c->store);
-    auto slot = [&](int i) {                                            // 16-aligned destination columns
-        return ((int64_t)fdirw::row_of(b, i) * b.grids[i].ny * b.grids[i].nz + 15) / 16 * 16;
-    };
-    auto struct_bytes = [&](int i, int r) -> uint64_t {
-        if (r == 0) return 0;
-        const int64_t cols = (b.dest_mask >> r) & 1u ? slot(i) : b.before[r][i + 1] - b.before[r][i];
-        return (uint64_t)cols * (uint64_t)fdirw::wcells(r) * sb;
-    };
-    b.qbase.assign(n, 0);
-    uint64_t budget;
     if (c->mem_limit) {
-        budget = c->mem_limit > c->allocated ? c->mem_limit - c->allocated : 0;
+        b.budget = c->mem_limit > c->allocated ? c->mem_limit - c->allocated : 0;
     } else {
         size_t fr = 0, tot = 0;
         if ((e = cudaMemGetInfo(&fr, &tot)) != cudaSuccess) return cuda_bail("cudaMemGetInfo", e);
         const uint64_t reserve = std::max<uint64_t>(1ull << 30, tot / 50);
         const uint64_t free_b = fr + idle_device_bytes(c->device);
-        budget = free_b > reserve ? free_b - reserve : 0;
+        b.budget = free_b > reserve ? free_b - reserve : 0;
     }
-    budget = budget > 256ull * (fdirw::kMaxR + 1) ? budget - 256ull * (fdirw::kMaxR + 1) : 0;
-    auto all_radii = [&](int i) {
-        uint64_t add = 0;
-        for (int r : b.radii) add += struct_bytes(i, r);
-        return add;
-    };
-    // Cache rows of whole vectors (as in a uniform context), unless a structure is too narrow for it or its kernels
-    // then no longer fit the budget.
-    b.qvec = 16 / sb;
-    for (int i = 0; i < n; i++)
-        if (b.grids[i].nx < 16 / sb || all_radii(i) > budget) { b.qvec = 1; break; }
-    int i = 0;
-    while (i < n) {
-        Chunk ch;
-        ch.s0 = i;
-        uint64_t used = 0;
-        while (i < n) {
-            const uint64_t add = all_radii(i);
-            if (used + add > budget && i > ch.s0) break;
-            if (used + add > budget) {
-                c->err = "the kernels of structure " + std::to_string(i) + " (" + std::to_string(add) +
-                         " bytes) do not fit the device memory budget (" + std::to_string(budget) + " bytes)";
-                return bail(FDIRW_ERR_NOMEM);
-            }
-            used += add;
-            i++;
-        }
-        ch.s1 = i;
-        ch.c0 = b.base[ch.s0];
-        ch.c1 = b.base[ch.s1];
-        ch.qn = 0;
-        for (int k = ch.s0; k < ch.s1; k++) {
-            b.qbase[k] = ch.qn;
-            ch.qn += slot(k);
-        }
-        uint64_t off = 0;
-        for (int r : b.radii) {
-            ch.seg_begin[r] = b.before[r][ch.s0];
-            ch.seg_end[r] = b.before[r][ch.s1];
-            ch.k_off[r] = off;
-            const int64_t cols = (b.dest_mask >> r) & 1u ? ch.qn : ch.seg_end[r] - ch.seg_begin[r];
-            if (r > 0) off += fdirw::align256((uint64_t)cols * fdirw::wcells(r) * sb);
-        }
-        ch.k_bytes = off;
-        b.chunks.push_back(ch);
+    b.budget = b.budget > 256ull * (fdirw::kMaxR + 1) ? b.budget - 256ull * (fdirw::kMaxR + 1) : 0;
+    fdirw::Plan plan = fdirw::plan_chunks(c, 1);
+    if (plan.too_large >= 0) {
+        c->err = "the kernels of structure " + std::to_string(plan.too_large) + " (" + std::to_string(plan.need) +
+                 " bytes) do not fit the device memory budget (" + std::to_string(b.budget) + " bytes)";
+        return bail(FDIRW_ERR_NOMEM);
     }
-    if ((e = cudaMemcpyAsync(b.d_qbase, b.qbase.data(), (size_t)n * 8, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess)
-        return cuda_bail("copy structure tables", e);
+    // Cache rows of whole vectors, as in a uniform context, unless a structure is narrower than one or the padding would
+    // split the batch: with a chunk more, every step marches all kernels again and none can be read back.
+    int qvec = 16 / fdirw::store_bytes(c->store);
+    for (const fdirw::Grid& g : b.grids) if (g.nx < qvec) { qvec = 1; break; }
+    if (qvec > 1) {
+        fdirw::Plan padded = fdirw::plan_chunks(c, qvec);
+        if (padded.too_large < 0 && padded.chunks.size() == plan.chunks.size()) plan = std::move(padded);
+        else qvec = 1;
+    }
+    if ((e = fdirw::install_plan(c, std::move(plan), qvec)) != cudaSuccess) return cuda_bail("copy structure tables", e);
     b.built.assign(b.chunks.size(), 0);
     b.stepped.assign(b.chunks.size(), 0);
     b.ev.assign(4 * b.chunks.size(), nullptr);

@@ -38,7 +38,8 @@ std::vector<std::string> launched;
 long calls = 0, fail_at = -1, violations = 0;
 std::uint64_t free_bytes = 1ull << 38;
 cudaError_t last = cudaSuccess;
-bool scalar_on = false, no_memory = false;
+bool scalar_on = false;
+long no_memory = 0, fail_n = 1l << 60;                       // allocations still to fail, those that fail together
 double scalar = 0.0;
 int fill = 0;
 struct Config {
@@ -102,10 +103,12 @@ void fake_reset() {
     calls = violations = 0;
     fail_at = -1;
     last = cudaSuccess;
-    scalar_on = no_memory = false;
+    scalar_on = false;
+    no_memory = 0;
     fill = 0;
 }
-void fake_fail_at(long k) { calls = 0; fail_at = k; no_memory = false; }
+// The k-th call from now fails; an allocation with the next n - 1 ones, or with all after it (n = 0).
+void fake_fail_at(long k, long n) { calls = 0; fail_at = k; no_memory = 0; fail_n = n ? n : 1l << 60; }
 long fake_calls() { return calls; }
 long fake_violations() { return violations; }
 void fake_scalar(double v) { scalar_on = true; scalar = v; }      // the value of every 8-byte copy to the host
@@ -123,9 +126,12 @@ long fake_launched(const char* part) {
 }
 
 // ---- memory
-cudaError_t cudaMalloc(void** p, size_t n) {                      // one that fails: so do all after it
-    no_memory = fails(cudaErrorMemoryAllocation) || no_memory;
-    if (no_memory) return last = cudaErrorMemoryAllocation;
+cudaError_t cudaMalloc(void** p, size_t n) {
+    if (fails(cudaErrorMemoryAllocation)) no_memory = fail_n;
+    if (no_memory > 0) {
+        no_memory--;
+        return last = cudaErrorMemoryAllocation;
+    }
     *p = std::malloc(n);
     if (n <= kSmall) std::memset(*p, 0xa5, n);
     blocks[*p] = n;

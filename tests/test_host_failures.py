@@ -1,6 +1,7 @@
 """The library's host code on a stand-in for the CUDA runtime (fake_cudart.cpp): every call of a scenario is made to fail
 in turn.  Whatever fails, no device block may go back to the pool of idle blocks while work is queued that can still use it
-(another thread's context would get it), and what a failed call left half made is not taken for finished by the next."""
+(another thread's context would get it), and what a failed call left half made is not taken for finished by the next.
+Then what contexts make of a memory limit and of an allocation that fails."""
 import ctypes
 import os
 import shutil
@@ -32,7 +33,7 @@ def fake(tmp_path_factory):
     lib = fdirw.load(so)
     lib.fake_calls.restype = lib.fake_violations.restype = lib.fake_launched.restype = ctypes.c_long
     lib.fake_held.restype = ctypes.c_uint64
-    lib.fake_fail_at.argtypes = [ctypes.c_long]
+    lib.fake_fail_at.argtypes = [ctypes.c_long, ctypes.c_long]
     lib.fake_scalar.argtypes = [ctypes.c_double]
     lib.fake_free_bytes.argtypes = [ctypes.c_uint64]
     yield lib
@@ -51,13 +52,13 @@ def _each_failure(lib, prepare, act, finish):
     while True:
         lib.fake_reset()
         st = prepare()
-        lib.fake_fail_at(k)
+        lib.fake_fail_at(k, 0)
         try:
             act(st)
         except fdirw.FdirwError:
             pass
         n = lib.fake_calls()
-        lib.fake_fail_at(-1)
+        lib.fake_fail_at(-1, 0)
         finish(st)
         assert lib.fake_violations() == 0, f"call {k}: a block was given back under queued work"
         k += 1
@@ -182,3 +183,41 @@ def test_solid_stability_check_after_a_failed_call(fake):
         assert e.value.code == fdirw.FDIRW_ERR_UNSTABLE
         _close(st)
     assert _each_failure(fake, prepare, act, again) > 3
+
+
+def _ragged_batch(fake, n, **kw):
+    fake.fake_fill(1)
+    f = FDiRWBatch([(17, 9, 9)] * n, [np.empty(1377)] * n, 0.1, 1, 1, 1, "bf16", stream=_stream(fake), **kw)
+    fake.fake_fill(0)
+    return f
+
+
+def _packed_bytes(n):
+    return 27 * 2 * 1392 * n                         # 1377 cells of a structure in slots of 16
+
+
+def test_batch_padding_does_not_split_it(fake):
+    """Cache rows of 17 values are padded to 24 where there is room, and never at the price of a chunk."""
+    fake.fake_reset()
+    n, c = 4, np.zeros(4 * 1377)
+    with _ragged_batch(fake, n) as f:
+        f.step(c, c)
+        i = f.info()
+        assert i["n_chunks"] == 1 and i["cache_bytes"] > _packed_bytes(n)
+        fixed = i["device_bytes"] - i["cache_bytes"]
+    for extra in (0, 256, _packed_bytes(n) // 8):
+        with _ragged_batch(fake, n, mem_limit=fixed + _packed_bytes(n) + 11 * 256 + extra) as f:
+            f.step(c, c)
+            i = f.info()
+            assert i["n_chunks"] == 1 and i["cache_bytes"] <= _packed_bytes(n) + 256
+
+
+def test_batch_drops_the_padding_when_its_allocation_fails(fake):
+    fake.fake_reset()
+    c = np.zeros(9 * 1377)
+    with _ragged_batch(fake, 9) as f:
+        fake.fake_fail_at(1, 2)                      # the arena (after the field's copy), also without idle blocks
+        f.step(c, c)
+        i = f.info()
+        assert i["n_chunks"] == 1 and i["cache_bytes"] <= _packed_bytes(9) + 256
+        f.read_kernels([0, 9 * 1377 - 1])
