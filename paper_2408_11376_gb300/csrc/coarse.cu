@@ -6,8 +6,8 @@
 //   P          column J: the remapped unit of block J (1 on its liquid cells, Eq. 12) marched n_sub
 //              explicit substeps on the block's window widened by R cells, then mapped (Eq. 11):
 //              P[I][J] = N_J S_I / (m N_I), S_I the marched mass on block I, m the total.  The march is
-//              mapping 4 in coarse mode (march_tm.cu), with convection one thread a column (march.cu); P is stored
-//              FP64, destination-indexed over the (2 Rc + 1)^3 block offsets, Rc = ceil(R / B)
+//              mapping 4 in coarse mode (march_tm.cu), with convection or one block per SM at most one thread a column
+//              (march.cu); P is stored FP64, destination-indexed over the (2 Rc + 1)^3 block offsets, Rc = ceil(R / B)
 //   step       mapping (Eq. 13): C_I = mean of c over the liquid cells of block I, FP64 in cell order;
 //              FDiRW calculation (Eq. 14): C'_I = sum_d P[I][I - d] C_{I - d}, FP64, d ascending;
 //              re-mapping (Eq. 15): c'_i = C'_I on every liquid cell of block I.
@@ -525,7 +525,7 @@ int coarse_kernels(fdirw_ctx* c) {
         FDIRW_CUDA(c, cudaGetLastError());
     }
     c->kernels_timed = true;
-    c->parts_used = c->flow ? 5 : 4;
+    c->parts_used = c->flow || k.nodes <= c->num_sms ? 5 : 4;
     k.built = true;
     c->kernels_ready = true;
     return FDIRW_OK;

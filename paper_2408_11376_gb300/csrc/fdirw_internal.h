@@ -74,9 +74,10 @@ struct MarchArgs {
     // Slab streaming of a uniform context (dest_z1 > dest_z0): only destinations of the z-planes [dest_z0, dest_z1)
     // are stored, from column 0 on; the others are rounded (for sigma) but not stored.
     int dest_z0, dest_z1;
+    int spb;                     // block march: sources that a CTA takes at a time (set by its launch)
 };
 // Coarse-mesh march of the blocks a.list[src_begin..src_end): window radius R = window_R + (B - 1) / 2
-// (1..10), one source per CTA.
+// (1..10).
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st);
 // Mapping 4 of the FP32 march (2x2 column blocks, march_tm.cu), R in 1..10.
 cudaError_t launch_march_blocks(const MarchArgs& a, int num_sms, cudaStream_t st);

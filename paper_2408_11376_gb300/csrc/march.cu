@@ -778,8 +778,8 @@ __global__ void __launch_bounds__(MapTmc<R>::THREADS, 1) march_tmc_kernel(MarchA
                 }
             }
             __syncthreads();
-            coarse_epilogue<R>(a, [&](int x, int y, int k) { return sbuf[(x + W1 * y) * W1 + k]; },
-                               reinterpret_cast<double*>(red + COLS), first);
+            coarse_epilogue<R>(a, [&](int x, int y, int k, int) { return sbuf[(x + W1 * y) * W1 + k]; },
+                               reinterpret_cast<double*>(red + COLS), first, 1);
         } else {
             if (active) {
 #pragma unroll
@@ -1132,14 +1132,15 @@ cudaError_t dispatch(const MarchArgs& a, int P, int num_sms, cudaStream_t st) {
     }
 }
 
-// Thread mapping of an FP32 march when the caller does not force one.  Mapping 4 is the fastest at every radius
-// from 2 on (ms for 48^3 sources, BF16 kernels, 100 substeps, mappings 1-7; R = 9, 10 have 4, 5 and 7 only):
+// Thread mapping of an FP32 march when the caller does not force one: 4, the fastest at every radius (ms for 48^3
+// sources, BF16 kernels, 100 substeps, mappings 1-7; R = 9, 10 have 4, 5 and 7 only):
 //   R = 2: 1.52 3.77 2.16 1.00 9.27 1.23 1.34    R = 6: 61.5 30.8 31.9 12.4 27.5 18.7 25.5
 //   R = 3: 3.98 9.32 8.76 2.36 11.1 3.26 3.46    R = 8: 48.6 66.5 60.3 26.5 48.1 47.9 67.0
 //   R = 4: 17.4 19.1 21.2 4.42 15.3 6.92 7.47    R = 9: 48.6 (4) 54.6 (5) 74.7 (7)
 //   R = 5: 39.1 43.1 16.8 7.55 17.8 11.5 15.0    R = 10: 54.2 (4) 82.7 (5) 81.8 (7)
-// At R = 1 (27 cells a window) mapping 6 is: 0.42 0.47 0.52 0.36 6.96 0.33 0.39.
-int default_mapping(int R) { return R == 1 ? 6 : 4; }
+// R = 1 (us, 60 substeps, mappings 1 2 3 4 6 7): 512 sources 28 21 18 17 33 23, 32768 92 99 107 82 84 101, 64^3 679 727 807
+// 508 546 682.
+constexpr int kDefaultMapping = 4;
 
 }  // namespace
 
@@ -1148,22 +1149,28 @@ int march_mapping(const MarchArgs& a, int parts_req) {
     if (a.bx) return 5;                           // direction-dependent coefficients: march_flow.cu
     if (parts_req >= 1 && parts_req <= 7 && (a.R <= 8 || parts_req == 4 || parts_req == 5 || parts_req == 7))
         return parts_req;
-    return default_mapping(a.R);
+    return kDefaultMapping;
 }
 
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st) {
-    if (!a.bx) return launch_march_blocks(a, num_sms, st);
-    switch (R) {                                  // direction-dependent coefficients
-        case 1: return launch_tmc<1, true>(a, num_sms, st);
-        case 2: return launch_tmc<2, true>(a, num_sms, st);
-        case 3: return launch_tmc<3, true>(a, num_sms, st);
-        case 4: return launch_tmc<4, true>(a, num_sms, st);
-        case 5: return launch_tmc<5, true>(a, num_sms, st);
-        case 6: return launch_tmc<6, true>(a, num_sms, st);
-        case 7: return launch_tmc<7, true>(a, num_sms, st);
-        case 8: return launch_tmc<8, true>(a, num_sms, st);
-        case 9: return launch_tmc<9, true>(a, num_sms, st);
-        case 10: return launch_tmc<10, true>(a, num_sms, st);
+    MarchArgs b = a;
+    if (!a.bx) {
+        if (a.src_end - a.src_begin > num_sms) return launch_march_blocks(a, num_sms, st);
+        // One block per SM at most: what counts is the latency of a substep, and a thread a column has the shorter one
+        // (15 x 14 x 13, B = 3, R = 2, 60 substeps: 31 us in 2x2 blocks, 21 so).  Both directions' faces are the same.
+        b.bx = a.ax; b.by = a.ay; b.bz = a.az;
+    }
+    switch (R) {                                  // one column per thread; direction-dependent coefficients
+        case 1: return launch_tmc<1, true>(b, num_sms, st);
+        case 2: return launch_tmc<2, true>(b, num_sms, st);
+        case 3: return launch_tmc<3, true>(b, num_sms, st);
+        case 4: return launch_tmc<4, true>(b, num_sms, st);
+        case 5: return launch_tmc<5, true>(b, num_sms, st);
+        case 6: return launch_tmc<6, true>(b, num_sms, st);
+        case 7: return launch_tmc<7, true>(b, num_sms, st);
+        case 8: return launch_tmc<8, true>(b, num_sms, st);
+        case 9: return launch_tmc<9, true>(b, num_sms, st);
+        case 10: return launch_tmc<10, true>(b, num_sms, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -249,55 +249,61 @@ __device__ __forceinline__ void store_columns(const MarchArgs& a, const SlotInfo
     }
 }
 
-// Coarse epilogue (Eq. 11 applied to the marched unit of block J): S[d] = FP64 sum of the marched field
-// over the liquid cells of block J + d inside the window (z, y, x order; u is 0 elsewhere), m =
+// Coarse epilogue (Eq. 11 applied to the marched units of the blocks list[first .. first + n)): S[d] = FP64 sum of the
+// marched field over the liquid cells of block J + d inside the window (z, y, x order; u is 0 elsewhere), m =
 // sum of S in a fixed order, and column J of P: Qc[d][J + d] = N_J S[d] / (m N_{J+d}), or S[d] / N_{J+d}
 // when the phase has open faces (a.abnd) and the column keeps the mass that stays (0 where block J + d
-// has no liquid).  Every thread of the CTA takes part; S follows red in shared memory.
-// u(x, y, k) is the marched value of a window cell (0 on cells that are not liquid).
+// has no liquid).  Every thread of the CTA takes part; S (W1^3 + 1 doubles) follows red in shared memory and holds as
+// many sources as fit, their sums side by side: one source after the other left most of the CTA waiting (30^3, B = 3,
+// R = 2, 24 sources a CTA, 3 substeps: 140 us a build, with fewer sources a CTA 19 now).
+// u(x, y, k, q) is the marched value of a window cell of source first + q (0 on cells that are not liquid).
 template <int R, typename F>
-__device__ __forceinline__ void coarse_epilogue(const MarchArgs& a, F u, double* S, int64_t first) {
-    const bool valid = first < a.src_end;                 // uniform over the CTA
-    const int64_t J = valid ? (a.list ? a.list[first] : first) : 0;
+__device__ __forceinline__ void coarse_epilogue(const MarchArgs& a, F u, double* S, int64_t first, int n) {
+    constexpr int W1 = 2 * R + 1;
     const int B = a.coarse_B, Rc = a.coarse_Rc, Wc = 2 * Rc + 1, Wc3 = Wc * Wc * Wc, bh = (B - 1) / 2;
-    const int bx = (int)(J % a.ncx), by = (int)((J / a.ncx) % a.ncy), bz = (int)(J / ((int64_t)a.ncx * a.ncy));
-    const int sx = bx * B + bh, sy = by * B + bh, sz = bz * B + bh;
-    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz;
-    for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
-        double acc = 0.0;
-        if (valid) {
+    const int nx = a.g.nx, ny = a.g.ny, nz = a.g.nz, cap = (W1 * W1 * W1 + 1) / (Wc3 + 1);
+    auto bar = [] { asm volatile("bar.sync 0;" ::: "memory"); };   // met by both z parts of a split march, each in its own code
+    for (int q0 = 0; q0 < n; q0 += cap) {
+        const int m = min(cap, n - q0);
+        // per threads a source; q >= m: no source's
+        const int per = blockDim.x / m, q = threadIdx.x / per;
+        const int64_t s = first + q0 + (q < m ? q : 0), J = a.list ? a.list[s] : s;
+        int bx, by, bz;
+        split_cell(J, a.ncx, a.ncy, bx, by, bz);
+        const int sx = bx * B + bh, sy = by * B + bh, sz = bz * B + bh;
+        for (int d = q < m ? threadIdx.x - q * per : Wc3; d < Wc3; d += per) {
             const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
             const int x0 = max(max(cx * B, sx - R), 0), x1 = min(min(cx * B + B - 1, sx + R), nx - 1);
             const int y0 = max(max(cy * B, sy - R), 0), y1 = min(min(cy * B + B - 1, sy + R), ny - 1);
             const int z0 = max(max(cz * B, sz - R), 0), z1 = min(min(cz * B + B - 1, sz + R), nz - 1);
+            double acc = 0.0;
             for (int z = z0; z <= z1; z++)
                 for (int y = y0; y <= y1; y++)
                     for (int x = x0; x <= x1; x++)
-                        acc += (double)u(x - (sx - R), y - (sy - R), z - (sz - R));
+                        acc += (double)u(x - (sx - R), y - (sy - R), z - (sz - R), q0 + q);
+            S[q * (Wc3 + 1) + d] = acc;
         }
-        S[d] = acc;
-    }
-    asm volatile("bar.sync 0;" ::: "memory");              // both z parts of a split march meet here, each in its own code
-    if (threadIdx.x < 32) {
-        double m = 0.0;
-        for (int d = threadIdx.x; d < Wc3; d += 32) m += S[d];
-        for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xffffffffu, m, off);
-        if (threadIdx.x == 0) S[Wc3] = m;
-    }
-    asm volatile("bar.sync 0;" ::: "memory");
-    const double m = S[Wc3];
-    if (valid) {
-        const double NJ = (double)a.ccount[J];
-        for (int d = threadIdx.x; d < Wc3; d += blockDim.x) {
+        bar();
+        for (int w = threadIdx.x >> 5; w < m; w += blockDim.x >> 5) {
+            double v = 0.0;
+            for (int d = threadIdx.x & 31; d < Wc3; d += 32) v += S[w * (Wc3 + 1) + d];
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if ((threadIdx.x & 31) == 0) S[w * (Wc3 + 1) + Wc3] = v;
+        }
+        bar();
+        const double mass = q < m ? S[q * (Wc3 + 1) + Wc3] : 0.0, NJ = (double)a.ccount[J];
+        for (int d = q < m ? threadIdx.x - q * per : Wc3; d < Wc3; d += per) {
             const int cx = bx + d % Wc - Rc, cy = by + (d / Wc) % Wc - Rc, cz = bz + d / (Wc * Wc) - Rc;
             if (cx < 0 || cx >= a.ncx || cy < 0 || cy >= a.ncy || cz < 0 || cz >= a.ncz) continue;
             const int64_t I = cx + (int64_t)a.ncx * (cy + (int64_t)a.ncy * cz);
             const int NI = a.ccount[I];
+            const double part = S[q * (Wc3 + 1) + d];
             // Closed phase: renormalise the column to carry N_J; open faces: keep the mass that stays.
             double v = 0.0;
-            if (NI > 0 && m > 0.0) v = a.abnd ? S[d] / (double)NI : (NJ * S[d]) / (m * (double)NI);
+            if (NI > 0 && mass > 0.0) v = a.abnd ? part / (double)NI : (NJ * part) / (mass * (double)NI);
             a.Qc[(int64_t)d * a.coarse_n + I] = v;
         }
+        bar();                                             // S is free again (and with the last one the marched values)
     }
 }
 

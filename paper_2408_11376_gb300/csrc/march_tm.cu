@@ -127,13 +127,14 @@ template <int N>
 __device__ __forceinline__ uint64_t pr(const uint32_t (&r)[N], int q) { return u2pack(r[2 * q], r[2 * q + 1]); }
 
 // One z part (levels K0 .. K0 + NK - 1 of the window) of every source of the CTA's batches.
+// SPREAD: a batch is a.spb sources, at most the SPB that fit (else SPB).
 // COARSE: the source is coarse block a.list[pos] (Eqs. 10-15): its window is centred on the block's centre cell
 // (radius R = window_R + (B - 1) / 2), the march starts from 1 on the block's liquid cells, an open face (a.abnd) adds
 // to the diagonal, and the epilogue maps the marched field onto the blocks of the window instead of storing a kernel.
 // G > 1 (one source at a time per CTA, R = 9, 10): the CTA marches G consecutive sources, keeps their rounded values in
 // shared memory and stores them together.  A plane gets G adjacent values then instead of one, and the stores, half of the
 // time outside the substeps, are as many sectors fewer (64^3 sources, R = 10, BF16, no substeps: 21.4 -> 15.3 ms; 100 substeps: 129 -> 122).
-template <int R, bool COARSE, int G, int K0, int NK>
+template <int R, bool COARSE, int G, bool SPREAD, int K0, int NK>
 __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* smem_raw, uint32_t tbase) {
     using M = MapTm<R>;
     using C = ColsTm<NK>;
@@ -151,7 +152,16 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
 
     const int t = threadIdx.x;
     const int th = M::ZS == 1 ? t : t & (PT - 1);
-    const bool active = th < SPB * TPS;
+    const int spb = SPREAD ? a.spb : SPB;          // sources that the CTA takes at a time
+    const bool active = th < spb * TPS;
+    // A warp without a source only meets the others at their barriers.  The zeros that its ring neighbours read stay.
+    const bool idle = SPREAD && (th & ~31) >= spb * TPS;
+    if (idle)
+        for (float* buf = xbuf; buf < xbuf + 2 * M::BUF; buf += M::BUF)
+            for (int sc = 0; sc < 4; sc++) {
+                for (int p = 0; p < R; p++) reinterpret_cast<uint64_t*>(buf)[pair_at<R>(p, sc, th)] = 0;
+                buf[mid_at<R>(sc, th)] = 0.f;
+            }
     const int slot = active ? th / TPS : 0;
     const int b = active ? th - slot * TPS : 0;
     const int bi = b % NB, bj = b / NB;
@@ -161,15 +171,20 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
     auto ring = [](int v) { return v < 0 ? v + PT : v >= PT ? v - PT : v; };
     const int tl = ring(th - 1), tr = ring(th + 1), tb = ring(th - NB), tt = ring(th + NB);
     const int x0 = 2 * bi, y0 = 2 * bj;
-    const int64_t nbatch = (a.src_end - a.src_begin + SPB * G - 1) / (SPB * G);
+    const int64_t nbatch = (a.src_end - a.src_begin + spb * G - 1) / (spb * G);
 
     for (int64_t bt = blockIdx.x; bt < nbatch; bt += gridDim.x) {
     if (G > 1 && K0 == 0 && t < G) sinfo[t].ok = 0;           // set by the sources that exist
     for (int g = 0; g < G; g++) {
-        const int64_t first = a.src_begin + bt * (SPB * G) + g;
+        const int64_t first = a.src_begin + bt * (spb * G) + g;
         if (G > 1 && first >= a.src_end) break;               // (uniform over the CTA)
+        const int64_t end = first + spb < a.src_end ? first + spb : a.src_end;
+        if (G == 1 && K0 == 0 && t < SPB && first + t >= end) sinfo[t].ok = 0;
+      if (idle) {
+        for (int it = 0; it <= a.n_sub; it++) bar();
+      } else {
         int64_t s = first + slot;
-        const bool src_ok = active && s < a.src_end;
+        const bool src_ok = active && s < end;
         if (src_ok && a.list) s = a.list[s];       // explicit source list (e.g. the surrogate's rejects)
         const int64_t pos = first + slot;          // position of the source in the launch range
         const SrcLoc L = locate(a, src_ok, s);
@@ -187,8 +202,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
                 split_cell(s, nx, ny, sx, sy, sz);
             }
         }
-        if (active && b == 0 && K0 == 0)
-            sinfo[G > 1 ? g : slot] = SlotInfo{L, pos, sx, sy, sz, src_ok ? 1 : 0};
+        if (src_ok && b == 0 && K0 == 0) sinfo[G > 1 ? g : slot] = SlotInfo{L, pos, sx, sy, sz, 1};
 
         // A face is stored with its lower cell and taken when that cell is in the domain and both cells are in
         // the window and the domain (0 otherwise).  All but the z range is fixed per thread, so the 16 faces
@@ -423,21 +437,8 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
         }
         tm_wait_x(X, X4);
 
-        if constexpr (COARSE) {
-            // u is 0 on cells that are not liquid: their faces carry nothing and they start at 0
-            const float* ubuf = xbuf + (a.n_sub & 1) * M::BUF;
-            double* S = reinterpret_cast<double*>(sinfo + SPB);
-            for (int sl = 0; sl < SPB; sl++) {
-                coarse_epilogue<R>(a, [&](int x, int y, int k) {
-                    return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), sl * TPS + (x >> 1) + NB * (y >> 1))];
-                }, S, first + sl);
-                bar();                             // S and xbuf are free for the next source
-            }
-            continue;
-        }
-        // Epilogue.  xbuf's buffer n_sub & 1 holds every u (published by the last substep).  Each thread sums
-        // its own rounded values (cells outside the window or the domain are 0).
-        {
+        if constexpr (!COARSE) {
+            // Each thread sums its own rounded values (cells outside the window or the domain are 0).
             MassSum m;
 #pragma unroll
             for (int sc = 0; sc < 4; sc++) {
@@ -450,34 +451,46 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
             }
             red[(K0 > 0 ? PT : 0) + th] = m.total();
         }
+        if constexpr (G > 1) {
+            if (active) {
+#pragma unroll
+                for (int sc = 0; sc < 4; sc++) {
+                    const int x = x0 + (sc & 1), y = y0 + (sc >> 1);
+                    if (x >= W1 || y >= W1) continue;
+                    Word* w = stage + G * (x + W1 * (y + W1 * K0)) + g;
+                    auto keep = [&](int j, float v) {
+                        if constexpr (G == 4)
+                            w[G * W1 * W1 * j] = a.store == Store::F16 ? __half_as_ushort(__float2half_rn(v))
+                                                                       : __bfloat16_as_ushort(__float2bfloat16_rn(v));
+                        else
+                            w[G * W1 * W1 * j] = v;
+                    };
+#pragma unroll
+                    for (int q = 0; q < NP; q++) {
+                        keep(q, f2lo(U[sc][q]));
+                        keep(q + H, f2hi(U[sc][q]));
+                    }
+                    if (MID) keep(NP, um[sc]);
+                }
+            }
+        }
+      }
+        // Epilogue.  xbuf's buffer n_sub & 1 holds every u (published by the last substep).
+        const float* ubuf = xbuf + (a.n_sub & 1) * M::BUF;
+        if constexpr (COARSE) {
+            // u is 0 on cells that are not liquid: their faces carry nothing and they start at 0
+            coarse_epilogue<R>(a, [&](int x, int y, int k, int q) {
+                return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), q * TPS + (x >> 1) + NB * (y >> 1))];
+            }, reinterpret_cast<double*>(sinfo + SPB), first, (int)(end - first));
+            continue;
+        }
         if constexpr (G == 1) {
-            const float* ubuf = xbuf + (a.n_sub & 1) * M::BUF;
             store_columns<R, SPB, M::THREADS>(a, sinfo, [&](int x, int y, int k, int sl) {
                 return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), sl * TPS + (x >> 1) + NB * (y >> 1))];
             });
-        } else if (active) {
-#pragma unroll
-            for (int sc = 0; sc < 4; sc++) {
-                const int x = x0 + (sc & 1), y = y0 + (sc >> 1);
-                if (x >= W1 || y >= W1) continue;
-                Word* w = stage + G * (x + W1 * (y + W1 * K0)) + g;
-                auto keep = [&](int j, float v) {
-                    if constexpr (G == 4)
-                        w[G * W1 * W1 * j] = a.store == Store::F16 ? __half_as_ushort(__float2half_rn(v))
-                                                                   : __bfloat16_as_ushort(__float2bfloat16_rn(v));
-                    else
-                        w[G * W1 * W1 * j] = v;
-                };
-#pragma unroll
-                for (int q = 0; q < NP; q++) {
-                    keep(q, f2lo(U[sc][q]));
-                    keep(q + H, f2hi(U[sc][q]));
-                }
-                if (MID) keep(NP, um[sc]);
-            }
         }
         bar();                                     // red (and stage) complete; xbuf is free for the next source
-        finish_sigma<TPS, SPB, M::ZS, PT>(red, first, a.src_end, a.list, a.sigma);
+        finish_sigma<TPS, SPB, M::ZS, PT>(red, first, end, a.list, a.sigma);
     }
     if constexpr (G > 1) {
         store_columns<R, G, M::THREADS>(a, sinfo, [&](int x, int y, int k, int sl) {
@@ -491,7 +504,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
     }
 }
 
-template <int R, bool COARSE, int G>
+template <int R, bool COARSE, int G, bool SPREAD>
 __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArgs a) {
     using M = MapTm<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -508,10 +521,10 @@ __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArg
     const uint32_t taddr = s_taddr;
     const uint32_t tbase = taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(M::SLOT * (warp >> 2));
     if constexpr (M::ZS == 1) {
-        march_part<R, COARSE, G, 0, M::W1>(a, smem_raw, tbase);
+        march_part<R, COARSE, G, SPREAD, 0, M::W1>(a, smem_raw, tbase);
     } else {
-        if (warp < M::PT / 32) march_part<R, COARSE, G, 0, M::LO>(a, smem_raw, tbase);
-        else march_part<R, COARSE, G, M::LO, M::W1 - M::LO>(a, smem_raw, tbase);
+        if (warp < M::PT / 32) march_part<R, COARSE, G, SPREAD, 0, M::LO>(a, smem_raw, tbase);
+        else march_part<R, COARSE, G, SPREAD, M::LO, M::W1 - M::LO>(a, smem_raw, tbase);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -519,37 +532,55 @@ __global__ void __launch_bounds__(MapTm<R>::THREADS, 1) march_tm_kernel(MarchArg
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(taddr) : "memory");
 }
 
-template <int R, bool COARSE, int G>
+// Sources of a CTA when a launch of nsrc is spread evenly over as many waves of CTAs as full ones (of spb) need.
+int even_spb(int64_t nsrc, int spb, int num_sms) {
+    const int64_t wave = (int64_t)num_sms * spb, ctas = (nsrc + wave - 1) / wave * num_sms;
+    return (int)((nsrc + ctas - 1) / ctas);
+}
+
+template <int R, bool COARSE, int G, bool SPREAD>
 cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
     using M = MapTm<R>;
     const int64_t nsrc = a.src_end - a.src_begin;
     if (nsrc <= 0) return cudaSuccess;
     const size_t smem = COARSE ? M::SMEM_COARSE : G > 1 ? M::SMEM_GROUP : M::SMEM;
-    auto kernel = march_tm_kernel<R, COARSE, G>;
+    auto kernel = march_tm_kernel<R, COARSE, G, SPREAD>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, M::THREADS, smem);
     if (e != cudaSuccess) return e;
     if (per_sm != 1) return cudaErrorInvalidConfiguration;   // TMEM allocation assumes one CTA per SM
-    const int64_t nbatch = (nsrc + M::SPB * G - 1) / (M::SPB * G);
+    MarchArgs b = a;
+    b.spb = SPREAD ? even_spb(nsrc, M::SPB, num_sms) : M::SPB;
+    const int64_t nbatch = (nsrc + b.spb * G - 1) / (b.spb * G);
     const int64_t grid = nbatch < (int64_t)num_sms ? nbatch : (int64_t)num_sms;
-    kernel<<<(unsigned)grid, M::THREADS, smem, st>>>(a);
+    kernel<<<(unsigned)grid, M::THREADS, smem, st>>>(b);
     return cudaGetLastError();
 }
 
 template <int R>
 cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
-    if (a.coarse_B > 0) return launch_tm<R, true, 1>(a, num_sms, st);
-    if constexpr (MapTm<R>::ZS > 1) {
+    using M = MapTm<R>;
+    const int64_t nsrc = a.src_end - a.src_begin;
+    // Coarse blocks are few: shares at every radius (us a build, 60 substeps, full CTAs -> shares: 30^3, B = 3, R = 2
+    // 175 -> 33; B = 5, R = 5 124 -> 62; 60 x 50 x 40, B = 5, R = 2 330 -> 79).
+    if (a.coarse_B > 0) return launch_tm<R, true, 1, (M::SPB > 1)>(a, num_sms, st);
+    if constexpr (M::ZS > 1) {
         // Groups where a last, partly filled wave of them costs less than a tenth; source-indexed columns are adjacent
         // whatever the order of the stores is, and gain the same.
-        const int64_t nsrc = a.src_end - a.src_begin;
         const int G = a.store == Store::F32 ? 2 : 4;
         if (nsrc >= (int64_t)num_sms * G * 10)
-            return G == 2 ? launch_tm<R, false, 2>(a, num_sms, st) : launch_tm<R, false, 4>(a, num_sms, st);
+            return G == 2 ? launch_tm<R, false, 2, false>(a, num_sms, st) : launch_tm<R, false, 4, false>(a, num_sms, st);
     }
-    return launch_tm<R, false, 1>(a, num_sms, st);
+    if constexpr (R <= 3) {
+        // A launch that does not fill every CTA: an even share each, warps without a source out of the march (us, 60
+        // substeps, BF16, full CTAs -> shares: 1000 sources R = 1 32 -> 18, R = 2 39 -> 23, R = 3 53 -> 27; 8000 sources
+        // R = 3 145 -> 141).  In a kernel of its own: the loop of full CTAs loses 3% to it.  From R = 4 on a CTA is full
+        // with 15 sources and less.
+        if (nsrc > 0 && even_spb(nsrc, M::SPB, num_sms) < M::SPB) return launch_tm<R, false, 1, true>(a, num_sms, st);
+    }
+    return launch_tm<R, false, 1, false>(a, num_sms, st);
 }
 
 }  // namespace
