@@ -8,8 +8,8 @@
 //              P[I][J] = N_J S_I / (m N_I), S_I the marched mass on block I, m the total.  The march is
 //              mapping 4 in coarse mode (march_tm.cu), with convection or one block per SM at most one thread a column
 //              (march.cu); P is stored FP64, destination-indexed over the (2 Rc + 1)^3 block offsets, Rc = ceil(R / B)
-//   step       mapping (Eq. 13): C_I = mean of c over the liquid cells of block I, FP64 in cell order;
-//              FDiRW calculation (Eq. 14): C'_I = sum_d P[I][I - d] C_{I - d}, FP64, d ascending;
+//   step       mapping (Eq. 13): C_I = mean of c over the liquid cells of block I, FP64 (map_kernel's order);
+//              FDiRW calculation (Eq. 14): C'_I = sum_d P[I][I - d] C_{I - d}, FP64 (coarse_gather_kernel's order);
 //              re-mapping (Eq. 15): c'_i = C'_I on every liquid cell of block I.
 #include "fdirw.h"
 #include "fdirw_internal.h"
@@ -117,35 +117,48 @@ __global__ void count_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, 
     }
 }
 
-// Eq. 13: C_I = (sum of c over the liquid cells of block I) / N_I.  Eight lanes per block, 4 blocks per warp: lane l takes
-// the block's (x, y) columns l, l + 8, ... and walks each in z, then a xor-butterfly.  One thread for a block's 125 cells
-// leaves most of a small grid's GPU idle; a whole warp spends the FP64 pipe (16 clocks an instruction and SM) on sums and
-// divisions of idle lanes.  B = 5, us at 96^3 / 192^3: one thread 27 / 48, a warp 14 / 80, eight lanes 11 / 34.
+// Eq. 13: C_I = (sum of c over the liquid cells of block I) / N_I.  LANES lanes per block, 32 / LANES blocks per warp:
+// lane l takes the block's (x, y) columns l, l + LANES, ... and walks each in z, then a xor-butterfly.  One thread for a
+// block's 125 cells leaves most of a small grid's GPU idle; a whole warp spends the FP64 pipe (16 clocks an instruction
+// and SM) on sums and divisions of idle lanes.  B = 5, us at 96^3 / 192^3: one thread 27 / 48, a warp 14 / 80, eight lanes
+// 11 / 34.
+template <int LANES>
 __global__ void map_kernel(Grid g, const uint8_t* __restrict__ liquid, int B, int ncx, int ncy, int64_t nc,
                            const int32_t* __restrict__ count, const double* __restrict__ c, double* __restrict__ C) {
-    const int lane = threadIdx.x & 31, l = lane & 7;
+    constexpr int NB = 32 / LANES;
+    const int lane = threadIdx.x & 31, l = lane % LANES;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5), nxy = (int64_t)g.nx * g.ny;
     Grid blocks = g;
     blocks.nx = ncx;
     blocks.ny = ncy;
     blocks.n = nc;
-    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); 4 * w < nc; w += warps) {
-        const int64_t I = 4 * w + (lane >> 3);
+    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); NB * w < nc; w += warps) {
+        const int64_t I = NB * w + lane / LANES;
         double s = 0.0;
         if (I < nc) {
             int bx, by, bz;
             cell_of(I, blocks, bx, by, bz);
-            const int nz = min(B, g.nz - bz * B);
-            for (int e = l; e < B * B; e += 8) {
-                const int dy = e / B, x = bx * B + e - dy * B, y = by * B + dy;
-                if (x >= g.nx || y >= g.ny) continue;
-                const int64_t i = x + (int64_t)g.nx * y + nxy * ((int64_t)bz * B);
+            if constexpr (LANES == 1) {
+                for (int z = bz * B; z < min(bz * B + B, g.nz); z++)
+                    for (int y = by * B; y < min(by * B + B, g.ny); y++)
+                        for (int x = bx * B; x < min(bx * B + B, g.nx); x++) {
+                            const int64_t i = x + (int64_t)g.nx * y + nxy * z;
+                            if (liquid[i]) s += c[i];
+                        }
+            } else {
+                const int nz = min(B, g.nz - bz * B);
+                for (int e = l; e < B * B; e += LANES) {
+                    const int dy = e / B, x = bx * B + e - dy * B, y = by * B + dy;
+                    if (x >= g.nx || y >= g.ny) continue;
+                    const int64_t i = x + (int64_t)g.nx * y + nxy * ((int64_t)bz * B);
 #pragma unroll 5
-                for (int z = 0; z < nz; z++)
-                    if (liquid[i + z * nxy]) s += c[i + z * nxy];
+                    for (int z = 0; z < nz; z++)
+                        if (liquid[i + z * nxy]) s += c[i + z * nxy];
+                }
             }
         }
-        for (int off = 1; off < 8; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+#pragma unroll
+        for (int off = 1; off < LANES; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
         if (l == 0 && I < nc) C[I] = count[I] > 0 ? s / (double)count[I] : 0.0;
     }
 }
@@ -413,29 +426,56 @@ __global__ void far_update_kernel(double* far, double V_far) {
 }
 
 // Eq. 14: C'_I = sum over block offsets d of P[I][I - d] C_{I - d}, FP64, plus P_BC[I] c_far when the outer surface is
-// open.  Eight lanes per block, 4 blocks per warp: lane l takes the offsets d = l, l + 8, ... in ascending order, then a
-// xor-butterfly (one thread for all of a block's 125 terms is a chain of loads and FP64 FMAs on a fraction of the GPU:
-// 96^3, B = 5, 20 -> 9 us).
-__global__ void coarse_gather_kernel(int ncx, int ncy, int ncz, int Rc, const double* __restrict__ Qc,
-                                     const double* __restrict__ C, const double* __restrict__ pbc,
-                                     const double* __restrict__ far, double* __restrict__ Cn) {
+// open.  PARTS = 8: a CTA takes 32 consecutive blocks, a lane each; warp w adds the offsets d = w, w + 8, ... in ascending
+// order, then the eight sums go pairwise.  PARTS = 1: one thread takes all offsets of a block in ascending order.  In both
+// a warp reads 32 consecutive values of a plane.
+template <int PARTS>
+__global__ void __launch_bounds__(PARTS == 1 ? 128 : 32 * PARTS) coarse_gather_kernel(int ncx, int ncy, int ncz, int Rc,
+                                                                                      const double* __restrict__ Qc,
+                                                                                      const double* __restrict__ C,
+                                                                                      const double* __restrict__ pbc,
+                                                                                      const double* __restrict__ far,
+                                                                                      double* __restrict__ Cn) {
+    constexpr int LANES = PARTS == 1 ? 128 : 32;
+    __shared__ double sums[PARTS][LANES];
     const int64_t nc = (int64_t)ncx * ncy * ncz;
-    const int Wc = 2 * Rc + 1, n = Wc * Wc * Wc;
-    // lane = 8 (part) + block: consecutive blocks side by side, so that a load of a plane is 4 or more values wide
-    const int lane = threadIdx.x & 31, part = lane >> 2, sub = lane & 3;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); 4 * w < nc; w += warps) {
-        const int64_t I = 4 * w + sub;
+    const int Wc = 2 * Rc + 1, n = Wc * Wc * Wc, lane = threadIdx.x % LANES, part = threadIdx.x / LANES;
+    const Grid blocks{ncx, ncy, ncz, nc};
+    for (int64_t I0 = (int64_t)blockIdx.x * LANES; I0 < nc; I0 += (int64_t)gridDim.x * LANES) {
+        const int64_t I = I0 + lane;
         double acc = 0.0;
         if (I < nc) {
-            const int bx = (int)(I % ncx), by = (int)((I / ncx) % ncy), bz = (int)(I / ((int64_t)ncx * ncy));
-            for (int d = part; d < n; d += 8) {
-                const int jx = bx - (d % Wc - Rc), jy = by - (d / Wc % Wc - Rc), jz = bz - (d / (Wc * Wc) - Rc);
-                if (jx < 0 || jx >= ncx || jy < 0 || jy >= ncy || jz < 0 || jz >= ncz) continue;
-                acc = fma(Qc[(int64_t)d * nc + I], C[jx + (int64_t)ncx * (jy + (int64_t)ncy * jz)], acc);
+            int bx, by, bz;
+            cell_of(I, blocks, bx, by, bz);
+            auto in = [](int v, int m) { return (unsigned)v < (unsigned)m; };
+            auto add = [&](int d, int jx, int jy, int jz) {
+                if (in(jx, ncx) && in(jy, ncy) && in(jz, ncz))
+                    acc = fma(Qc[(int64_t)d * nc + I], C[jx + (int64_t)ncx * (jy + (int64_t)ncy * jz)], acc);
+            };
+            if constexpr (PARTS == 1) {
+                int d = 0;
+                for (int dz = -Rc; dz <= Rc; dz++)
+                    for (int dy = -Rc; dy <= Rc; dy++)
+                        for (int dx = -Rc; dx <= Rc; dx++, d++) add(d, bx - dx, by - dy, bz - dz);
+            } else {
+                int dx = part % Wc, dy = part / Wc % Wc, dz = part / (Wc * Wc);      // offset d + Rc
+                for (int d = part; d < n; d += PARTS) {
+                    add(d, bx + Rc - dx, by + Rc - dy, bz + Rc - dz);
+                    for (dx += PARTS; dx >= Wc;) {
+                        dx -= Wc;
+                        if (++dy == Wc) { dy = 0; dz++; }
+                    }
+                }
             }
         }
-        for (int off = 4; off < 32; off <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if constexpr (PARTS > 1) {
+            sums[part][lane] = acc;
+            __syncthreads();
+            if (part == 0)
+                acc = ((sums[0][lane] + sums[1][lane]) + (sums[2][lane] + sums[3][lane])) +
+                      ((sums[4][lane] + sums[5][lane]) + (sums[6][lane] + sums[7][lane]));
+            __syncthreads();
+        }
         if (part == 0 && I < nc) {
             if (pbc) acc = __dadd_rn(acc, __dmul_rn(pbc[I], far[0]));
             Cn[I] = acc;
@@ -469,6 +509,35 @@ __global__ void read_coarse_kernel(const double* __restrict__ Qc, int ncx, int n
             v = Qc[(int64_t)d * nc + cx + (int64_t)ncx * (cy + (int64_t)ncy * cz)];
         out[t] = v;
     }
+}
+
+// Lanes per block: few blocks leave the GPU idle with one each; of many, lanes that share a block's sum cost FP64
+// instructions (16 clocks each on an SM) that add nothing.  us, 1 / 4 / 8 lanes: B = 5 96^3 (8000 blocks) 21 / 10 / 10,
+// 128^3 (18k) 27 / 12 / 14, 224^3 (91k) 33 / 42 / 51; B = 3 64^3 (11k) 10 / 8 / 8, 96^3 (33k) 10 / 10 / 12, 160^3 (157k)
+// 16 / 29 / 45; B = 1 96^3 33 / 119 / 244.
+cudaError_t launch_map(fdirw_ctx* c, const double* field, double* means) {
+    const Coarse& k = *c->coarse;
+    auto launch = [&](auto kernel, int lanes, int threads) {
+        kernel<<<grid_blocks(k.nc, threads / lanes), threads, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
+                                                                              field, means);
+        return cudaGetLastError();
+    };
+    if (k.B == 1 || k.nc > 40000) return launch(map_kernel<1>, 1, 128);
+    if (k.nc > 12000) return launch(map_kernel<4>, 4, 256);
+    return launch(map_kernel<8>, 8, 256);
+}
+
+// Eight threads per block where one each leaves the chain of a block's terms bare, that is with few blocks or many terms.
+// us, 1 / 8: Rc = 1 8000 blocks 8 / 6, 157k 13 / 21, 885k 72 / 113; Rc = 2 8000 23 / 8, 33k 23 / 14, 157k 53 / 59, 885k 279 /
+// 310; Rc = 3 8000 51 / 17, 80k 119 / 70, 262k 247 / 213, 885k 718 / 722.
+cudaError_t launch_coarse_gather(fdirw_ctx* c) {
+    const Coarse& k = *c->coarse;
+    const double* pbc = k.open ? k.pbc : nullptr;
+    if (k.nc <= 40000 || k.Rc >= 3)
+        coarse_gather_kernel<8><<<grid_blocks(k.nc, 32), 256, 0, c->stream>>>(k.ncx, k.ncy, k.ncz, k.Rc, k.Qc, k.C, pbc, k.far, k.Cn);
+    else
+        coarse_gather_kernel<1><<<grid_blocks(k.nc, 128), 128, 0, c->stream>>>(k.ncx, k.ncy, k.ncz, k.Rc, k.Qc, k.C, pbc, k.far, k.Cn);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -520,9 +589,7 @@ int coarse_kernels(fdirw_ctx* c) {
             std::swap(u0, u1);
         }
         widen_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(u0, c->g.n, c->cbuf);
-        map_kernel<<<grid_blocks(k.nc, 32), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count,
-                                                                  c->cbuf, k.pbc);
-        FDIRW_CUDA(c, cudaGetLastError());
+        FDIRW_CUDA(c, launch_map(c, c->cbuf, k.pbc));
     }
     c->kernels_timed = true;
     c->parts_used = c->flow || k.nodes <= c->num_sms ? 5 : 4;
@@ -557,14 +624,11 @@ static int coarse_steps(fdirw_ctx* c, const double* c_in, double* c_out, int32_t
     } else {
         const double* cur = src;
         for (int t = 0; t < n_steps; t++) {
-            map_kernel<<<grid_blocks(k.nc, 32), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.nc, k.count, cur, k.C);
-            FDIRW_CUDA(c, cudaGetLastError());
+            FDIRW_CUDA(c, launch_map(c, cur, k.C));
             const bool last = t + 1 == n_steps;
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[2], c->stream));
             if (k.open) FDIRW_CUDA(c, launch_mass(cur, c->g.n, c->partials, k.far + 1, c->stream));
-            coarse_gather_kernel<<<grid_blocks(k.nc, 16), 128, 0, c->stream>>>(k.ncx, k.ncy, k.ncz, k.Rc, k.Qc, k.C,
-                                                                                k.open ? k.pbc : nullptr, k.far, k.Cn);
-            FDIRW_CUDA(c, cudaGetLastError());
+            FDIRW_CUDA(c, launch_coarse_gather(c));
             if (last) FDIRW_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
             remap_kernel<<<grid_blocks(c->g.n, 256), 256, 0, c->stream>>>(c->g, k.liquid, k.B, k.ncx, k.ncy, k.Cn, cur, dst);
             FDIRW_CUDA(c, cudaGetLastError());
