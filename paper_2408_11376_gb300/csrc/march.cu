@@ -195,10 +195,13 @@ __global__ void __launch_bounds__(Map32<R, P>::THREADS, Map32<R, P>::MIN_BLOCKS)
 // those the source has reached (a substep moves a value one cell: |dx| + |dy| + |dz| <= substeps; the rest is still 0).
 // The cells that are computed see the same operations in the same order.  36^3, R = 6, 120 substeps: 148 -> 114 ms; 20^3,
 // R = 8, 60 substeps: 31.0 -> 15.7 ms; 64^3, R = 6, 30 substeps: 217 -> 176 ms.
+// ALL: a thread a column and every level of it, in the domain or not.  The three levels of R = 1 are not worth their
+// bounds (40 x 33 x 29, 60 substeps: 843 us with them, 790 without).
 template <int R>
 __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(MarchArgs a) {
     using S = Shape<R>;
     constexpr int W1 = S::W1, COLS = S::COLS, SPB = S::SPB64;
+    constexpr bool ALL = R == 1;
     constexpr int BUF = SPB * COLS * W1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* xbuf = reinterpret_cast<double*>(smem_raw);   // [2][BUF]
@@ -222,40 +225,64 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
 
     for (int64_t b = blockIdx.x; b < nbatch; b += gridDim.x) {
         const int64_t first = a.src_begin + b * SPB;
-        if (t < SPB) {
-            int64_t s = first + t;
-            int n = 0;
-            if (s < a.src_end) {
-                if (a.list) s = a.list[s];         // explicit source list (e.g. the surrogate's rejects)
-                int sx, sy, sz;
-                split_cell(s, nx, ny, sx, sy, sz);
-                c0x[t] = max(R - sx, 0);
-                c0y[t] = max(R - sy, 0);
-                wx[t] = min(nx - 1 - sx, R) + R - c0x[t] + 1;
-                k0s[t] = max(R - sz, 0);
-                k1s[t] = min(nz - 1 - sz, R) + R + 1;
-                src[t][0] = sx; src[t][1] = sy; src[t][2] = sz;
-                n = wx[t] * (min(ny - 1 - sy, R) + R - c0y[t] + 1);
+        bool own = false;
+        int slot = 0, ci = 0, cj = 0, sx = 0, sy = 0, sz = 0, d0 = 0, d1 = 0;    // [d0, d1): levels in the domain
+        if constexpr (ALL) {
+            if (t < SPB * COLS) {
+                slot = t / COLS;
+                cj = (t - slot * COLS) / W1;
+                ci = t - slot * COLS - cj * W1;
+                int64_t s = first + slot;
+                if (s < a.src_end) {
+                    if (a.list) s = a.list[s];
+                    split_cell(s, nx, ny, sx, sy, sz);
+                    own = (unsigned)(sx - R + ci) < (unsigned)nx && (unsigned)(sy - R + cj) < (unsigned)ny;
+                    d0 = own ? max(R - sz, 0) : 0;
+                    d1 = own ? min(nz - 1 - sz, R) + R + 1 : 0;
+                }
             }
-            wxy[t] = n;
-        }
-        __syncthreads();
-        if (t <= SPB) {
-            int n = 0;
+        } else {
+            if (t < SPB) {
+                int64_t s = first + t;
+                int n = 0;
+                if (s < a.src_end) {
+                    if (a.list) s = a.list[s];         // explicit source list (e.g. the surrogate's rejects)
+                    int sx, sy, sz;
+                    split_cell(s, nx, ny, sx, sy, sz);
+                    c0x[t] = max(R - sx, 0);
+                    c0y[t] = max(R - sy, 0);
+                    wx[t] = min(nx - 1 - sx, R) + R - c0x[t] + 1;
+                    k0s[t] = max(R - sz, 0);
+                    k1s[t] = min(nz - 1 - sz, R) + R + 1;
+                    src[t][0] = sx; src[t][1] = sy; src[t][2] = sz;
+                    n = wx[t] * (min(ny - 1 - sy, R) + R - c0y[t] + 1);
+                }
+                wxy[t] = n;
+            }
+            __syncthreads();
+            if (t <= SPB) {
+                int n = 0;
 #pragma unroll 8
-            for (int q = 0; q < t; q++) n += wxy[q];
-            before[t] = n;
+                for (int q = 0; q < t; q++) n += wxy[q];
+                before[t] = n;
+            }
+            for (int i = t; i < SPB * COLS; i += blockDim.x) red[i] = 0.0;
+            __syncthreads();
+            own = t < before[SPB];
+            slot = own ? t / COLS : 0;                           // no source has more than COLS columns
+            while (own && t >= before[slot + 1]) slot++;
+            const int c = own ? t - before[slot] : 0, w = own ? wx[slot] : 1;
+            cj = own ? c0y[slot] + c / w : 0;
+            ci = own ? c0x[slot] + c % w : 0;
+            sx = src[slot][0];
+            sy = src[slot][1];
+            sz = src[slot][2];
+            d0 = own ? k0s[slot] : 0;
+            d1 = own ? k1s[slot] : 0;
         }
-        for (int i = t; i < SPB * COLS; i += blockDim.x) red[i] = 0.0;
-        __syncthreads();
-        const bool own = t < before[SPB];
-        int slot = own ? t / COLS : 0;                           // no source has more than COLS columns
-        while (own && t >= before[slot + 1]) slot++;
-        const int c = own ? t - before[slot] : 0, w = own ? wx[slot] : 1;
-        const int cj = own ? c0y[slot] + c / w : 0, ci = own ? c0x[slot] + c % w : 0;
         const int base = (slot * COLS + cj * W1 + ci) * W1;
-        const int sz = src[slot][2], x = src[slot][0] - R + ci, y = src[slot][1] - R + cj;
-        const int k0 = own ? k0s[slot] : 0, k1 = own ? k1s[slot] : 0;
+        const int x = sx - R + ci, y = sy - R + cj;
+        const int k0 = ALL ? 0 : d0, k1 = ALL ? W1 : d1;                 // levels that are computed
         const bool left = ci > 0 && x > 0, front = cj > 0 && y > 0;      // a lower neighbour in the window and the domain
         const int xm = left ? base - W1 : base, xp = ci < 2 * R ? base + W1 : base;
         const int ym = front ? base - W1 * W1 : base, yp = cj < 2 * R ? base + W1 * W1 : base;
@@ -264,12 +291,13 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
 #pragma unroll
         for (int k = 0; k < W1; k++) {
             u[k] = own && ci == R && cj == R && k == R ? 1.0 : 0.0;
-            if (k >= k0 && k < k1) {
+            if (ALL ? own : k >= k0 && k < k1) {
                 const int z = sz - R + k;
                 const int64_t i = (int64_t)x + (int64_t)nx * y + nxy * z;
-                fx[base + k] = ci < 2 * R && x + 1 < nx ? __ldg(a.dx + i) : 0.0;
-                fy[base + k] = cj < 2 * R && y + 1 < ny ? __ldg(a.dy + i) : 0.0;
-                fz[base + k] = k < 2 * R && z + 1 < nz ? __ldg(a.dz + i) : 0.0;
+                const bool in = !ALL || (k >= d0 && k < d1);
+                fx[base + k] = in && ci < 2 * R && x + 1 < nx ? __ldg(a.dx + i) : 0.0;
+                fy[base + k] = in && cj < 2 * R && y + 1 < ny ? __ldg(a.dy + i) : 0.0;
+                fz[base + k] = in && k < 2 * R && z + 1 < nz ? __ldg(a.dz + i) : 0.0;
             }
         }
         __syncthreads();
@@ -288,12 +316,14 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
         const int lateral = abs(ci - R) + abs(cj - R);
         for (int it = 0; it < a.n_sub; it++) {
             double* buf = xbuf + (it & 1) * BUF;
+            if (!ALL || own)
 #pragma unroll
-            for (int k = 0; k < W1; k++)
-                if (k >= k0 && k < k1) buf[base + k] = u[k];
+                for (int k = 0; k < W1; k++)
+                    if (k >= k0 && k < k1) buf[base + k] = u[k];
             __syncthreads();
+            if (ALL && !own) continue;
             const int reach = it + 1 - lateral;                  // levels reached by the end of this substep
-            const int ka = max(k0, R - reach), kb = min(k1, R + reach + 1);
+            const int ka = ALL ? 0 : max(k0, R - reach), kb = ALL ? W1 : min(k1, R + reach + 1);
             double prev = 0.0;
 #pragma unroll
             for (int k = 0; k < W1; k++) {
@@ -314,13 +344,13 @@ __global__ void __launch_bounds__(Shape<R>::THREADS64, 1) march_f64_kernel(March
         double colsum = 0.0;
 #pragma unroll
         for (int k = 0; k < W1; k++) {
-            if (k < k0 || k >= k1) continue;
+            if (k < d0 || k >= d1) continue;
             const int z = sz - R + k;
             if (a.dest_z1 <= a.dest_z0 || (z >= a.dest_z0 && z < a.dest_z1))
                 reinterpret_cast<double*>(a.Q)[qplane(a, R, ci, cj, k) * a.q_stride + qcol(a, L, x, y, z, 0)] = u[k];
             colsum += u[k];
         }
-        if (own) red[slot * COLS + cj * W1 + ci] = colsum;
+        if (ALL ? t < SPB * COLS : own) red[slot * COLS + cj * W1 + ci] = own ? colsum : 0.0;
         __syncthreads();
         finish_sigma<COLS, SPB>(red, first, a.src_end, a.list, a.sigma);
         __syncthreads();

@@ -64,3 +64,27 @@ def test_coarse_matrix_equals_the_column_march(B, R, shape, open_surface):
             f.kernels()
             out.append(f.read_coarse(np.arange(nb)))
     assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("shape,n_sub", [((1, 1, 1), 2), ((1, 1, 5), 1), ((60, 1, 3), 9), ((2, 31, 2), 4), ((7, 9, 11), 30)])
+def test_fp64_march_of_radius_one(shape, n_sub):
+    """Every level of a column is computed there: kernels against the oracle, and the z-slabs of a streamed cache."""
+    import oracle
+    D = synth.random_diffusivity(shape, 60, 4.0)
+    lam = oracle.stable_dt_sub(shape, D)
+    lam = lam if np.isfinite(lam) else 1.0
+    src, c = np.arange(D.size), synth.random_field(D.size, 61)
+    out = []
+    with FDiRW(shape, D, n_sub * lam, 1, n_sub, "fp64") as f:
+        f.kernels()
+        ks = f.read_kernels(src).reshape(D.size, -1)
+        fixed = f.info()["device_bytes"] - f.info()["cache_bytes"] - D.size * (8 + 8 * 27)
+    ref = oracle.kernels(shape, D, lam, 1, n_sub, src)[0].reshape(D.size, -1)
+    assert (np.linalg.norm(ks - ref, axis=1) / np.linalg.norm(ref, axis=1)).max() <= 1e-13
+    # one z plane of the cache at a time, then all of it
+    for limit in ([fixed + 8 * D.size + 27 * 8 * shape[0] * shape[1]] if shape[2] > 1 else []) + [0]:
+        with FDiRW(shape, D, n_sub * lam, 1, n_sub, "fp64", mem_limit=limit) as f:
+            out.append(np.empty(D.size))
+            f.step(c, out[-1], 2)
+            assert f.info()["n_chunks"] == (shape[2] if limit else 1)
+    assert all(np.array_equal(out[-1], o) for o in out)
