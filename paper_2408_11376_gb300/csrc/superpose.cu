@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(256, 2) gather_ordered_kernel(GatherArgs a) {
     *o = (a.acc_in ? *o : 0.0) + ((double)A + (double)B);
 }
 
-// Packed rows of a width that is no whole number of vectors (nx < VX, or a padded cache that would not fit): one
+// Rows of a width that is no whole number of vectors (nx < VX, or a padded cache that would not fit), and R = 1: one
 // destination per thread, runtime R, the sums of gather_kernel in the same order.  Bound by the latency of its loads.  us a
 // step of a 7 x 40 x 40 box, BF16 cache, R = 8: float-float sums 1100 (without the unrolling by two 1716), FP32 sums 980
 // (1663 with the compiler's); R = 3 48 (55) and 34 (42).
@@ -337,12 +337,12 @@ __global__ void __launch_bounds__(256) gather_scalar_kernel(GatherArgs a, int R)
     const int64_t nxy = (int64_t)a.g.nx * a.g.ny;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (tid >= nxy * a.zn) return;
-    const ST* Q = reinterpret_cast<const ST*>(a.Q) + tid;
-    const int x = (int)(tid % a.g.nx), y = (int)(tid / a.g.nx % a.g.ny), z = a.z0 + (int)(tid / nxy);
+    const int64_t rw = tid / a.g.nx;
+    const int x = (int)(tid - rw * a.g.nx), y = (int)(rw % a.g.ny), z = a.z0 + (int)(rw / a.g.ny);
     const int W1 = 2 * R + 1, NROW = W1 * W1, G = MODE == 2 ? 1 : row_groups(R);
     double sum = 0.0;                                     // MODE 0
     float SA = 0.f, SB = 0.f;                             // MODE 1, 2
-    const ST* q = Q;
+    const ST* q = reinterpret_cast<const ST*>(a.Q) + rw * a.qnx + x;
     int row = 0, oz = -R, oy = -R;
     for (int k = 0; k < G; k++) {
         double acc = 0.0;
@@ -619,8 +619,11 @@ cudaError_t gather_launch(const GatherArgs& a, cudaStream_t st) {
     const bool vec = a.qnx % VX == 0 && reinterpret_cast<uintptr_t>(a.Q) % 16 == 0 && a.qs % VX == 0;
     const int64_t n = (vec ? (int64_t)a.qnx / VX : (int64_t)a.g.nx) * a.g.ny * a.zn;
     if (n <= 0) return cudaSuccess;
-    if (!vec) {
-        gather_scalar_kernel<ST, MODE><<<(unsigned)blocks_for(n, 256), 256, 0, st>>>(a, R);
+    // R = 1 has no rows to split (vector_warps): so few vectors of eight destinations leave the GPU to a handful of warps,
+    // and a thread a destination is faster (BF16 cache, float-float sums, us: 10 x 9 x 8 11.8 -> 9.9, 40^3 14.0 -> 9.8).
+    if (!vec || (R == 1 && MODE == 1 && sizeof(ST) == 2 && n <= 8000)) {
+        const int64_t cells = (int64_t)a.g.nx * a.g.ny * a.zn;
+        gather_scalar_kernel<ST, MODE><<<(unsigned)blocks_for(cells, 256), 256, 0, st>>>(a, R);
         return cudaGetLastError();
     }
     if constexpr (MODE == 2 && R > 2) {
