@@ -114,7 +114,9 @@ typedef struct {
     double   dt_sub;         /* dt_macro / n_sub */
     double   lam;            /* dt_sub / h^2 */
     double   max_face_sum;   /* max over cells of the sum of its face conductances */
-    uint64_t cache_bytes;    /* bytes of the kernel cache (N * (2R+1)^3 * storage size) */
+    uint64_t cache_bytes;    /* bytes of the kernel cache: N * (2R+1)^3 * storage size, its x rows padded to whole
+                                16-byte vectors where there is room for that (under a mem_limit: beside what later
+                                calls on the context can ask for); fewer when streamed */
     uint64_t device_bytes;   /* all device bytes held by the context */
     double   window_cells;   /* sum over sources of their clipped window sizes */
     float    kernels_ms;     /* device time of the last kernel-cache build (march kernel only) */

@@ -270,7 +270,8 @@ int fdirw::ensure_cache(fdirw_ctx* c) {
     constexpr uint64_t kReserve = 1ull << 30;
     if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) budget = free_b + idle_device_bytes(c->device) > kReserve ? free_b + idle_device_bytes(c->device) - kReserve : 0;
     else cudaGetLastError();                                   // unknown: let the allocation decide
-    if (c->mem_limit) budget = std::min<uint64_t>(budget, c->mem_limit > c->allocated ? c->mem_limit - c->allocated : 0);
+    const uint64_t cap = !c->mem_limit ? ~0ull : c->mem_limit > c->allocated ? c->mem_limit - c->allocated : 0;
+    budget = std::min(budget, cap);
     const uint64_t obytes = (uint64_t)c->g.n * 8;
     int T = c->g.nz;
     if (full > budget) {
@@ -285,11 +286,12 @@ int fdirw::ensure_cache(fdirw_ctx* c) {
             const int rc = dalloc(c, reinterpret_cast<void**>(&c->obuf), obytes, "streamed step output");
             if (rc != FDIRW_OK) return rc;
         }
-        // Rows padded to whole vectors (padded_row); packed where only those fit, and in a slab, whose every plane
-        // more saves marching sources again (which costs far more than its gather).
+        // Rows padded to whole vectors (padded_row); packed where only those fit, also with what later calls may ask of
+        // a mem_limit, and in a slab, whose every plane more saves marching sources again (which costs far more than its
+        // gather).
         int qnx = streamed ? c->g.nx : padded_row(c->g.nx, c->store);
         auto bytes = [&](int row) { return W * (uint64_t)row * (uint64_t)c->g.ny * (uint64_t)T * (uint64_t)store_bytes(c->store); };
-        if (bytes(qnx) > budget) qnx = c->g.nx;
+        if (bytes(qnx) > budget || (c->mem_limit && bytes(qnx) + later_bytes(c) > cap)) qnx = c->g.nx;
         int rc = dalloc(c, &c->Q, bytes(qnx), "kernel cache");
         if (rc == FDIRW_ERR_NOMEM && qnx != c->g.nx) rc = dalloc(c, &c->Q, bytes(qnx = c->g.nx), "kernel cache");
         if (rc == FDIRW_OK) {

@@ -1004,13 +1004,16 @@ int fdirw_create_batch(int32_t n, const fdirw_grid* grids, const double* const* 
                  " bytes) do not fit the device memory budget (" + std::to_string(b.budget) + " bytes)";
         return bail(FDIRW_ERR_NOMEM);
     }
-    // Cache rows of whole vectors, as in a uniform context, unless a structure is narrower than one or the padding would
-    // split the batch: with a chunk more, every step marches all kernels again and none can be read back.
+    // Cache rows of whole vectors, as in a uniform context, unless a structure is narrower than one, later calls may miss
+    // the bytes under a mem_limit, or the padding would split the batch: with a chunk more, every step marches all kernels
+    // again and none can be read back.
     int qvec = 16 / fdirw::store_bytes(c->store);
     for (const fdirw::Grid& g : b.grids) if (g.nx < qvec) { qvec = 1; break; }
     if (qvec > 1) {
         fdirw::Plan padded = fdirw::plan_chunks(c, qvec);
-        if (padded.too_large < 0 && padded.chunks.size() == plan.chunks.size()) plan = std::move(padded);
+        if (padded.too_large < 0 && padded.chunks.size() == plan.chunks.size() &&
+            (!c->mem_limit || padded.arena() + later_bytes(c) <= b.budget))
+            plan = std::move(padded);
         else qvec = 1;
     }
     if ((e = fdirw::install_plan(c, std::move(plan), qvec)) != cudaSuccess) return cuda_bail("copy structure tables", e);

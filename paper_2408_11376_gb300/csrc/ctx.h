@@ -111,6 +111,12 @@ class Scratch {
     fdirw_ctx* c_;
     std::vector<std::pair<void*, uint64_t>> blocks_;
 };
+// Bytes that later calls on a context can ask for beside its kernel cache: every kernel read back, a velocity field, the
+// surrogate's features.  Under a mem_limit the cache's rows are padded only where all of that still fits.
+inline uint64_t later_bytes(const fdirw_ctx* c) {
+    const uint64_t n = (uint64_t)c->g.n, W = (uint64_t)(2 * c->R + 1) * (2 * c->R + 1) * (2 * c->R + 1);
+    return n * (8 + 8 * W) + n * (3 * 4 + 3 * 8 + 6 * 4) + 8 + n * 2;
+}
 // Bytes of the pool's idle blocks on a device: free memory to a dalloc, though the driver counts them as used.
 uint64_t idle_device_bytes(int device);
 }  // namespace host

@@ -221,3 +221,35 @@ def test_batch_drops_the_padding_when_its_allocation_fails(fake):
         i = f.info()
         assert i["n_chunks"] == 1 and i["cache_bytes"] <= _packed_bytes(9) + 256
         f.read_kernels([0, 9 * 1377 - 1])
+
+
+def _limited(fake, make, cells, W):
+    """What a context of packed rows leaves for later calls at a memory limit, its padded one leaves as well."""
+    fake.fake_reset()
+    n_all, read = np.arange(cells), cells * (8 + 8 * W)
+    with make(0) as f:
+        f.kernels()
+        i = f.info()
+        padded, fixed = i["cache_bytes"], i["device_bytes"] - i["cache_bytes"]
+    with make(fixed + (1 << 30)) as f:               # room for everything
+        f.kernels()
+        assert f.info()["cache_bytes"] == padded
+    for later in (0, read, read // 2, 60 * cells + 8, read + 62 * cells):
+        with make(fixed + 27 * 2 * 17 * (cells // 17 + 15) + 11 * 256 + later) as f:
+            f.kernels()
+            assert f.info()["n_chunks"] == 1 and f.info()["cache_bytes"] < padded
+            if later >= read:
+                f.read_kernels(n_all)
+            elif later == read // 2:
+                f.read_kernels(n_all[:cells // 2])
+            elif later:
+                f.set_velocity(np.zeros(3 * cells))
+
+
+def test_padding_leaves_a_memory_limit_to_later_calls(fake):
+    D, stream = np.empty(17 * 81), _stream(fake)
+    _limited(fake, lambda limit: FDiRW((17, 9, 9), D, 0.1, 1, 1, "bf16", stream=stream, mem_limit=limit), D.size, 27)
+
+
+def test_batch_padding_leaves_a_memory_limit_to_later_calls(fake):
+    _limited(fake, lambda limit: _ragged_batch(fake, 4, mem_limit=limit), 4 * 1377, 27)
