@@ -195,8 +195,14 @@ FDIRW_API int fdirw_read_kernels(fdirw_ctx* ctx, const int64_t* sources, int64_t
 /* Snapshot of the context's configuration and last timings.  Synchronises on the timing events. */
 FDIRW_API int fdirw_get_info(fdirw_ctx* ctx, fdirw_info* out);
 
-/* Release all device memory held by the context.  NULL-safe. */
+/* Release all device memory held by the context.  NULL-safe.  Blocks of up to 64 MB stay with the library for the
+ * next contexts of the process, 256 MB of them at most, until an allocation of the library needs their memory or
+ * fdirw_release_idle gives them back. */
 FDIRW_API void fdirw_destroy(fdirw_ctx* ctx);
+
+/* Give the device memory that destroyed contexts have left with the library back to the driver, on every device;
+ * bytes (host pointer or NULL) receives how much that was.  Live contexts are not touched; any thread may call it. */
+FDIRW_API int fdirw_release_idle(uint64_t* bytes);
 
 /* Create one context for a batch of n independent structures whose sources use per-source window radii
  * (the paper has one domain and no window; Sec. 3.1 and Eq. 8 apply per structure).

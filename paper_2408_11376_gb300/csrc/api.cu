@@ -52,7 +52,7 @@ namespace {
 // Device blocks that contexts have freed, kept for the next ones: a small structure's run from create to destroy spent as
 // long in 15 cudaMalloc and 15 cudaFree calls (each free waits for the whole device) as in half of its kernels (32^3: 225
 // of 954 us).  Bounded: blocks up to 64 MB, 256 MB in all, the oldest given back to the driver beyond that, and all of
-// them when an allocation fails.  A block comes here only when no work uses it any more (its context's stream has been
+// them when an allocation of the library fails or a program asks for it (fdirw_release_idle).  A block comes here only when no work uses it any more (its context's stream has been
 // waited for), so the next owner may use it on any stream.  Locked: contexts of several threads share it.
 class BlockPool {
   public:
@@ -97,16 +97,18 @@ class BlockPool {
         for (void* q : out) cudaFree(q);
         return true;
     }
-    // Gives every idle block back; whether there were any.
-    bool trim() {
+    // Gives every idle block back; their bytes.
+    uint64_t trim() {
         std::deque<Block> out;
+        uint64_t bytes;
         {
             std::lock_guard<std::mutex> lk(mu_);
             out.swap(idle_);
+            bytes = idle_bytes_;
             idle_bytes_ = 0;
         }
         for (const Block& b : out) cudaFree(b.p);
-        return !out.empty();
+        return bytes;
     }
     uint64_t idle_on(int device) {
         std::lock_guard<std::mutex> lk(mu_);
@@ -135,6 +137,15 @@ BlockPool& pool() {
 
 }  // namespace
 
+cudaError_t device_malloc(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && pool().trim()) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what) {
     *p = nullptr;
     if (bytes == 0) return FDIRW_OK;
@@ -143,11 +154,7 @@ int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what) {
                                             " bytes) would exceed mem_limit " + std::to_string(c->mem_limit));
     cudaError_t e = cudaSuccess;
     if ((*p = pool().take(c->device, bytes)) == nullptr) {
-        e = cudaMalloc(p, bytes);
-        if (e == cudaErrorMemoryAllocation && pool().trim()) {
-            cudaGetLastError();
-            e = cudaMalloc(p, bytes);
-        }
+        e = device_malloc(p, bytes);
         if (e == cudaSuccess) pool().hand_out(*p, c->device, bytes);
     }
     if (e == cudaErrorMemoryAllocation) {
@@ -180,6 +187,7 @@ void Scratch::release() {
 }
 
 uint64_t idle_device_bytes(int device) { return pool().idle_on(device); }
+uint64_t release_idle() { return pool().trim(); }
 
 }  // namespace host
 }  // namespace fdirw
@@ -703,6 +711,12 @@ int fdirw_get_info(fdirw_ctx* c, fdirw_info* out) {
         FDIRW_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     out->n_chunks = c->slab_T ? (c->g.nz + c->slab_T - 1) / c->slab_T : 1;   // z-slabs of a streamed cache
+    return FDIRW_OK;
+}
+
+int fdirw_release_idle(uint64_t* bytes) {
+    const uint64_t n = release_idle();
+    if (bytes) *bytes = n;
     return FDIRW_OK;
 }
 

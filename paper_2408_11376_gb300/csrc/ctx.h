@@ -81,6 +81,10 @@ Kind classify(const void* p, int device);
 bool grid_ok(const fdirw_grid* g);
 // cudaMalloc that honours the context's mem_limit and keeps its byte count.
 int dalloc(fdirw_ctx* c, void** p, uint64_t bytes, const char* what);
+// cudaMalloc for everything that lives outside the pool: when memory is short, the pool's idle blocks go back first.
+cudaError_t device_malloc(void** p, size_t bytes);
+template <typename T>
+cudaError_t device_malloc(T** p, size_t bytes) { return device_malloc(reinterpret_cast<void**>(p), bytes); }
 // Frees a dalloc'ed block that no work uses any more (a pool of small ones keeps it for the next dalloc).
 void drelease(void* p);
 void dfree(void*& p);
@@ -119,6 +123,8 @@ inline uint64_t later_bytes(const fdirw_ctx* c) {
 }
 // Bytes of the pool's idle blocks on a device: free memory to a dalloc, though the driver counts them as used.
 uint64_t idle_device_bytes(int device);
+// Gives the pool's idle blocks back to the driver; their bytes.
+uint64_t release_idle();
 }  // namespace host
 
 #define FDIRW_CUDA(ctx, call)                                                                     \

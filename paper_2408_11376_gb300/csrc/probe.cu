@@ -2,6 +2,7 @@
 // (no counterpart in the paper): the FP32 FMA rate of a register-only loop, and the bandwidth of a
 // streaming read from HBM over a buffer larger than L2.  Neither touches a context.
 #include "fdirw_internal.h"
+#include "ctx.h"
 
 #include "fdirw.h"
 
@@ -59,8 +60,8 @@ extern "C" FDIRW_API int fdirw_probe_peaks(int32_t device, double* fp32_flops, d
     float* sink = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     std::string err;
-    cudaError_t e = cudaMalloc(&buf, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&sink, 16);
+    cudaError_t e = fdirw::host::device_malloc(&buf, bytes);
+    if (e == cudaSuccess) e = fdirw::host::device_malloc(&sink, 16);
     if (e == cudaSuccess) e = cudaMemset(buf, 0, bytes);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);

@@ -844,17 +844,17 @@ int ensure_capacity(fdirw_net* net, int n) {
     cudaFree(net->dmass); cudaFree(net->dacc); cudaFree(net->dloss);
     net->cap = 0;
     const size_t ab = (size_t)cap * PATCH * 2;
-    for (auto& p : net->act) NET_CUDA(net, cudaMalloc(&p, ab));
-    for (auto& p : net->gbuf) NET_CUDA(net, cudaMalloc(&p, ab));
+    for (auto& p : net->act) NET_CUDA(net, fdirw::host::device_malloc(&p, ab));
+    for (auto& p : net->gbuf) NET_CUDA(net, fdirw::host::device_malloc(&p, ab));
     for (auto& p : net->act) NET_CUDA(net, cudaMemset(p, 0, ab));       // halos stay zero from here on
     for (auto& p : net->gbuf) NET_CUDA(net, cudaMemset(p, 0, ab));
-    NET_CUDA(net, cudaMalloc(&net->zhead, (size_t)cap * KV * 4));
-    NET_CUDA(net, cudaMalloc(&net->dsrc, (size_t)cap * 8));
-    NET_CUDA(net, cudaMalloc(&net->dtgt, (size_t)cap * KV * 8));
-    NET_CUDA(net, cudaMalloc(&net->dkout, (size_t)cap * KV * 8));
-    NET_CUDA(net, cudaMalloc(&net->dmass, (size_t)cap * 8));
-    NET_CUDA(net, cudaMalloc(&net->dacc, (size_t)cap * 4));
-    NET_CUDA(net, cudaMalloc(&net->dloss, ((size_t)cap * HEAD_PARTS + TERM_BLOCKS) * 8));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->zhead, (size_t)cap * KV * 4));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dsrc, (size_t)cap * 8));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dtgt, (size_t)cap * KV * 8));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dkout, (size_t)cap * KV * 8));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dmass, (size_t)cap * 8));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dacc, (size_t)cap * 4));
+    NET_CUDA(net, fdirw::host::device_malloc(&net->dloss, ((size_t)cap * HEAD_PARTS + TERM_BLOCKS) * 8));
     if (const int rc = encode_maps(net, cap); rc != FDIRW_OK) return rc;
     net->cap = cap;
     return FDIRW_OK;
@@ -1039,11 +1039,11 @@ FDIRW_API int fdirw_net_create(const float* params, int32_t device, fdirw_net** 
         if (device >= 0) cudaSetDevice(prev);
         return nfail(nullptr, FDIRW_ERR_CUDA, msg);
     };
-    if (cudaMalloc(&net->params, NPARAM * 4) != cudaSuccess || cudaMalloc(&net->m, NPARAM * 4) != cudaSuccess ||
-        cudaMalloc(&net->v, NPARAM * 4) != cudaSuccess || cudaMalloc(&net->grads, NPARAM * 4) != cudaSuccess ||
-        cudaMalloc(&net->wf, (size_t)NL * WCAN * 2) != cudaSuccess || cudaMalloc(&net->wd, (size_t)NL * WCAN * 2) != cudaSuccess ||
-        cudaMalloc(&net->partial, (size_t)WG_PARTS * WG_SLOTS * C * C * 4) != cudaSuccess ||
-        cudaMalloc(&net->derr, 4) != cudaSuccess || cudaEventCreate(&net->ev[0]) != cudaSuccess ||
+    if (fdirw::host::device_malloc(&net->params, NPARAM * 4) != cudaSuccess || fdirw::host::device_malloc(&net->m, NPARAM * 4) != cudaSuccess ||
+        fdirw::host::device_malloc(&net->v, NPARAM * 4) != cudaSuccess || fdirw::host::device_malloc(&net->grads, NPARAM * 4) != cudaSuccess ||
+        fdirw::host::device_malloc(&net->wf, (size_t)NL * WCAN * 2) != cudaSuccess || fdirw::host::device_malloc(&net->wd, (size_t)NL * WCAN * 2) != cudaSuccess ||
+        fdirw::host::device_malloc(&net->partial, (size_t)WG_PARTS * WG_SLOTS * C * C * 4) != cudaSuccess ||
+        fdirw::host::device_malloc(&net->derr, 4) != cudaSuccess || cudaEventCreate(&net->ev[0]) != cudaSuccess ||
         cudaEventCreate(&net->ev[1]) != cudaSuccess || cudaStreamCreateWithFlags(&net->side, cudaStreamNonBlocking) != cudaSuccess)
         return bail("allocating the network");
     // Beside a tensor-core kernel: an SM keeps the shared memory that the next one needs (a kernel that leaves it to L1
@@ -1154,7 +1154,7 @@ FDIRW_API int fdirw_net_trace(fdirw_ctx* ctx, fdirw_net* net, const int64_t* sou
     cudaStream_t st = ctx->stream;
     const size_t vol = (size_t)n * C * KV;      // BF16 values of one traced volume set
     uint16_t* stage = nullptr;
-    if (acts_out || grads_out) NET_CUDA(net, cudaMalloc(&stage, vol * 2));
+    if (acts_out || grads_out) NET_CUDA(net, fdirw::host::device_malloc(&stage, vol * 2));
     const int ub = (int)std::min<int64_t>(((int64_t)vol + 255) / 256, 152 * 16);
     auto dump = [&](const __nv_bfloat16* src, uint16_t* dst) -> int {
         unpack_kernel<<<ub, 256, 0, st>>>(src, (int)n, stage);
@@ -1228,7 +1228,7 @@ FDIRW_API int fdirw_kernels_surrogate(fdirw_ctx* c, fdirw_net* net, int64_t* acc
     if ((rc = check_err(net, c->stream)) != FDIRW_OK) return rc;
     if (!rejected.empty()) {
         int64_t* dlist = nullptr;
-        NET_CUDA(net, cudaMalloc(&dlist, rejected.size() * 8));
+        NET_CUDA(net, fdirw::host::device_malloc(&dlist, rejected.size() * 8));
         cudaError_t e = cudaMemcpyAsync(dlist, rejected.data(), rejected.size() * 8, cudaMemcpyHostToDevice, c->stream);
         fdirw::MarchArgs a{};
         a.g = c->g;

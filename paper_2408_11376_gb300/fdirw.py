@@ -37,7 +37,7 @@ EXPORTED = ("fdirw_stable_dt", "fdirw_create", "fdirw_kernels", "fdirw_step", "f
             "fdirw_kernels_surrogate", "fdirw_create_batch", "fdirw_read_radius", "fdirw_create_coarse",
             "fdirw_read_coarse", "fdirw_coarse_far_field", "fdirw_coarse_get_far_field", "fdirw_read_coarse_pbc",
             "fdirw_coupled_step", "fdirw_set_velocity", "fdirw_net_trace", "fdirw_net_test_wait",
-            "fdirw_probe_peaks", "fdirw_net_timing")
+            "fdirw_probe_peaks", "fdirw_net_timing", "fdirw_release_idle")
 NET_NPARAM = 4 * 27 * 16 * 16 + 4 * 16
 NET_KV = 17 ** 3
 
@@ -122,6 +122,7 @@ def load(path: str | None = None):
         lib.fdirw_net_trace.argtypes = [vp, vp, vp, i64, vp, vp, vp, vp, vp, dp]
         lib.fdirw_net_test_wait.argtypes = [vp, ctypes.c_uint64, i32]
         lib.fdirw_probe_peaks.argtypes = [i32, dp, dp]
+        lib.fdirw_release_idle.argtypes = [vp]
         lib.fdirw_net_timing.argtypes = [vp, ctypes.POINTER(ctypes.c_float)]
         lib.fdirw_create_batch.argtypes = [i32, ctypes.POINTER(fdirw_grid), ctypes.POINTER(vp), ctypes.c_double, i32,
                                            i32, i32, ctypes.POINTER(fdirw_opts), ctypes.POINTER(vp)]
@@ -307,6 +308,13 @@ def fdirw_get_info(ctx: int) -> dict:
 def fdirw_destroy(ctx: int) -> None:
     if ctx:
         load().fdirw_destroy(ctypes.c_void_p(ctx))
+
+
+def fdirw_release_idle() -> int:
+    """Gives the device memory that destroyed contexts have left with the library back; returns its bytes."""
+    n = ctypes.c_uint64(0)
+    _check(load().fdirw_release_idle(ctypes.byref(n)))
+    return n.value
 
 
 def fdirw_probe_peaks(device: int = -1) -> dict:

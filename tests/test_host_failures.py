@@ -253,3 +253,36 @@ def test_padding_leaves_a_memory_limit_to_later_calls(fake):
 
 def test_batch_padding_leaves_a_memory_limit_to_later_calls(fake):
     _limited(fake, lambda limit: _ragged_batch(fake, 4, mem_limit=limit), 4 * 1377, 27)
+
+
+def test_idle_blocks_are_bounded_and_given_back(fake):
+    fake.fake_reset()
+    fdirw.fdirw_release_idle()
+    held = fake.fake_held()
+    D, stream = np.empty(160 ** 3), _stream(fake)    # arrays of 16 and 32 MB
+    live = [FDiRW((160,) * 3, D, 0.1, 0, 1, stream=stream) for _ in range(6)]
+    assert fake.fake_held() - held > 3 * (256 << 20)
+    _close(live)
+    idle = fake.fake_held() - held
+    assert 128 << 20 < idle <= 256 << 20
+    with FDiRW((160,) * 3, D, 0.1, 0, 1, stream=stream) as f:
+        assert fake.fake_held() - held <= idle + f.info()["device_bytes"] // 4      # the blocks are used again
+        assert fdirw.fdirw_release_idle() > 0
+        assert 0 <= fake.fake_held() - held - f.info()["device_bytes"] < 4096      # (a block can be some bytes larger)
+    fdirw.fdirw_release_idle()
+    assert fake.fake_held() == held and fdirw.fdirw_release_idle() == 0
+
+
+def test_network_takes_the_idle_blocks_memory(fake):
+    """Allocations outside the contexts find the memory that destroyed contexts left with the library."""
+    fake.fake_reset()
+    fdirw.fdirw_release_idle()
+    held, stream = fake.fake_held(), _stream(fake)
+    FDiRW((9, 9, 9), np.empty(729), 0.1, 1, 1, stream=stream).close()
+    assert fake.fake_held() > held
+    fake.fake_fail_at(2, 1)
+    net = fdirw.Net(np.zeros(fdirw.NET_NPARAM, dtype=np.float32))
+    fake.fake_fail_at(-1, 0)
+    idle = fdirw.fdirw_release_idle()
+    net.close()
+    assert idle == 0 and fake.fake_held() == held
