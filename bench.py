@@ -930,7 +930,7 @@ def flow_leg(args, fdirw, torch, dev, stream, w, shape, D, solid, dt_macro):
     uniform noise of 0.03 on every face, zero on faces touching a solid cell; n_sub raised by a tenth so
     that the diffusive part leaves room for the advective outflow within the same macro step.  Field: a
     Gaussian blob (sigma 10 cells) on the pore cells.  Times create + velocity + kernels + macro steps
-    with the flow, and the same n_sub on mapping 5 without it."""
+    with the flow, and the same n_sub without it (the diffusion march that a context without a velocity runs)."""
     from paper_2408_11376_gb300 import synth
     n_sub = -(-11 * w.n_sub // 10)
     N = shape[0] * shape[1] * shape[2]
@@ -946,8 +946,7 @@ def flow_leg(args, fdirw, torch, dev, stream, w, shape, D, solid, dt_macro):
         out = torch.empty_like(c_in)
         with torch.cuda.stream(stream):
             ev[0].record(stream)
-            ctx = fdirw.fdirw_create(shape, D, dt_macro, w.R, n_sub, args.prec, device=dev.index, stream=stream,
-                                     march_parts=5)
+            ctx = fdirw.fdirw_create(shape, D, dt_macro, w.R, n_sub, args.prec, device=dev.index, stream=stream)
             if flow:
                 fdirw.fdirw_set_velocity(ctx, vel, N)
             ev[1].record(stream)
@@ -967,7 +966,7 @@ def flow_leg(args, fdirw, torch, dev, stream, w, shape, D, solid, dt_macro):
     return {"n_sub": n_sub, "velocity": "mean 0.03 along +x, noise 0.03, 0 on solid faces",
             "macro_steps_per_s": 1000.0 * w.steps / job_ms, "job_ms": job_ms, "kernels_ms": build_ms,
             "steps_ms": steps_ms, "march_kernel_ms": info["kernels_ms"],
-            "march_kernel_ms_no_flow_same_mapping": res[False][3]["kernels_ms"],
+            "march_kernel_ms_no_flow": res[False][3]["kernels_ms"],
             "march_tflops": roof["achieved"], "march_frac_fp32": roof["frac"],
             "mass_rel_err": abs(mass - mass0) / mass0,
             "x_centroid_shift_vs_no_flow_cells": xc - res[False][5]}
