@@ -278,7 +278,7 @@ template <typename ST, int R>
 __global__ void __launch_bounds__(256, 2) gather_ordered_kernel(GatherArgs a) {
     using U = Quad<ST>;
     constexpr int VX = 16 / sizeof(ST), W1 = 2 * R + 1, NROW = W1 * W1, NP = VX / 2, ND = 32 * VX;
-    __shared__ float sums[2][8][ND];
+    __shared__ __align__(16) float sums[2][8][ND];      // stored 16 bytes at a time
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned nxv = a.qnx / VX, nvec = nxv * a.g.ny * a.zn, v = blockIdx.x * 32 + lane;
     const bool valid = v < nvec;
