@@ -178,13 +178,16 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
     for (int g = 0; g < G; g++) {
         const int64_t first = a.src_begin + bt * (spb * G) + g;
         if (G > 1 && first >= a.src_end) break;               // (uniform over the CTA)
-        const int64_t end = first + spb < a.src_end ? first + spb : a.src_end;
-        if (G == 1 && K0 == 0 && t < SPB && first + t >= end) sinfo[t].ok = 0;
+        auto end = [&]() -> int64_t {                         // of the sources that this batch may reach
+            if constexpr (SPREAD) return first + spb < a.src_end ? first + spb : a.src_end;
+            return a.src_end;
+        };
+        if (SPREAD && t >= spb && t < SPB) sinfo[t].ok = 0;
       if (idle) {
         for (int it = 0; it <= a.n_sub; it++) bar();
       } else {
         int64_t s = first + slot;
-        const bool src_ok = active && s < end;
+        const bool src_ok = active && s < end();
         if (src_ok && a.list) s = a.list[s];       // explicit source list (e.g. the surrogate's rejects)
         const int64_t pos = first + slot;          // position of the source in the launch range
         const SrcLoc L = locate(a, src_ok, s);
@@ -202,7 +205,8 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
                 split_cell(s, nx, ny, sx, sy, sz);
             }
         }
-        if (src_ok && b == 0 && K0 == 0) sinfo[G > 1 ? g : slot] = SlotInfo{L, pos, sx, sy, sz, 1};
+        if (active && b == 0 && K0 == 0)
+            sinfo[G > 1 ? g : slot] = SlotInfo{L, pos, sx, sy, sz, src_ok ? 1 : 0};
 
         // A face is stored with its lower cell and taken when that cell is in the domain and both cells are in
         // the window and the domain (0 otherwise).  All but the z range is fixed per thread, so the 16 faces
@@ -481,7 +485,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
             // u is 0 on cells that are not liquid: their faces carry nothing and they start at 0
             coarse_epilogue<R>(a, [&](int x, int y, int k, int q) {
                 return ubuf[level_at<R>(k, (x & 1) + 2 * (y & 1), q * TPS + (x >> 1) + NB * (y >> 1))];
-            }, reinterpret_cast<double*>(sinfo + SPB), first, (int)(end - first));
+            }, reinterpret_cast<double*>(sinfo + SPB), first, end() - first < spb ? (int)(end() - first) : spb);
             continue;
         }
         if constexpr (G == 1) {
@@ -490,7 +494,7 @@ __device__ __forceinline__ void march_part(const MarchArgs& a, unsigned char* sm
             });
         }
         bar();                                     // red (and stage) complete; xbuf is free for the next source
-        finish_sigma<TPS, SPB, M::ZS, PT>(red, first, end, a.list, a.sigma);
+        finish_sigma<TPS, SPB, M::ZS, PT>(red, first, end(), a.list, a.sigma);
     }
     if constexpr (G > 1) {
         store_columns<R, G, M::THREADS>(a, sinfo, [&](int x, int y, int k, int sl) {
