@@ -196,7 +196,7 @@ FDIRW_API int fdirw_read_kernels(fdirw_ctx* ctx, const int64_t* sources, int64_t
 FDIRW_API int fdirw_get_info(fdirw_ctx* ctx, fdirw_info* out);
 
 /* Release all device memory held by the context.  NULL-safe.  Blocks of up to 64 MB stay with the library for the
- * next contexts of the process, 256 MB of them at most, until an allocation of the library needs their memory or
+ * next contexts of the process, 256 MB and 512 blocks at most, until an allocation of the library needs their memory or
  * fdirw_release_idle gives them back. */
 FDIRW_API void fdirw_destroy(fdirw_ctx* ctx);
 

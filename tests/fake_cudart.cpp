@@ -119,6 +119,7 @@ uint64_t fake_held() {
     for (auto& b : blocks) n += b.second;
     return n;
 }
+long fake_blocks() { return (long)blocks.size(); }
 long fake_launched(const char* part) {
     long n = 0;
     for (auto& s : launched) n += s.find(part) != std::string::npos;

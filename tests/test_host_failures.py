@@ -31,7 +31,7 @@ def fake(tmp_path_factory):
     saved = fdirw._lib
     fdirw._lib = None
     lib = fdirw.load(so)
-    lib.fake_calls.restype = lib.fake_violations.restype = lib.fake_launched.restype = ctypes.c_long
+    lib.fake_calls.restype = lib.fake_violations.restype = lib.fake_launched.restype = lib.fake_blocks.restype = ctypes.c_long
     lib.fake_held.restype = ctypes.c_uint64
     lib.fake_fail_at.argtypes = [ctypes.c_long, ctypes.c_long]
     lib.fake_scalar.argtypes = [ctypes.c_double]
@@ -271,6 +271,17 @@ def test_idle_blocks_are_bounded_and_given_back(fake):
         assert 0 <= fake.fake_held() - held - f.info()["device_bytes"] < 4096      # (a block can be some bytes larger)
     fdirw.fdirw_release_idle()
     assert fake.fake_held() == held and fdirw.fdirw_release_idle() == 0
+
+
+def test_idle_blocks_are_bounded_in_number(fake):
+    """Many small contexts destroyed at once do not leave a list that every later allocation has to search."""
+    fake.fake_reset()
+    fdirw.fdirw_release_idle()
+    held, stream = fake.fake_blocks(), _stream(fake)
+    _close([FDiRW((9, 9, 9), np.empty(729), 0.1, 1, 1, stream=stream) for _ in range(100)])
+    assert 100 < fake.fake_blocks() - held <= 512
+    fdirw.fdirw_release_idle()
+    assert fake.fake_blocks() == held
 
 
 def test_network_takes_the_idle_blocks_memory(fake):
