@@ -28,7 +28,7 @@
 // the blocks included) are 25 of the 32 words a clock; the FP32 pipe is half busy.  64^3 sources, BF16 kernels, ms a
 // substep / ms outside the substeps (coefficients, sums, cache stores), scalar levels before: R = 8: 0.721 / 28.0
 // -> 0.554 / 8.1; R = 6: 0.333 / 13.0 -> 0.261 / 3.5; R = 3: 0.056 / 2.2 -> 0.048 / 0.8; R = 10 against one column
-// per thread (mapping 5): 1.73 / 23.5 -> 1.10 / 23.4.
+// per thread (mapping 5): 1.73 / 23.5 -> 1.10 / 15.3 (grouped stores; 23.4 without).
 //
 // One CTA per SM (two or three threads per TMEM lane; the CTA allocates all 512 columns once and frees them before it
 // exits, and its shared-memory request keeps a second CTA off the SM so an allocation never waits).
