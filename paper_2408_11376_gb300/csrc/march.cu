@@ -1162,7 +1162,7 @@ cudaError_t dispatch(const MarchArgs& a, int P, int num_sms, cudaStream_t st) {
     }
 }
 
-// Thread mapping of an FP32 march when the caller does not force one: 4, the fastest at every radius (ms for 48^3
+// Thread mapping of an FP32 march when the caller does not force one.  Mapping 4 is the fastest at every radius (ms for 48^3
 // sources, BF16 kernels, 100 substeps, mappings 1-7; R = 9, 10 have 4, 5 and 7 only):
 //   R = 2: 1.52 3.77 2.16 1.00 9.27 1.23 1.34    R = 6: 61.5 30.8 31.9 12.4 27.5 18.7 25.5
 //   R = 3: 3.98 9.32 8.76 2.36 11.1 3.26 3.46    R = 8: 48.6 66.5 60.3 26.5 48.1 47.9 67.0
@@ -1170,16 +1170,22 @@ cudaError_t dispatch(const MarchArgs& a, int P, int num_sms, cudaStream_t st) {
 //   R = 5: 39.1 43.1 16.8 7.55 17.8 11.5 15.0    R = 10: 54.2 (4) 82.7 (5) 81.8 (7)
 // R = 1 (us, 60 substeps, mappings 1 2 3 4 6 7): 512 sources 28 21 18 17 33 23, 32768 92 99 107 82 84 101, 64^3 679 727 807
 // 508 546 682.
-constexpr int kDefaultMapping = 4;
+// With one source per SM at most (two at R = 5-7) one thread a column has the shorter substep up to R = 8 (us, 60 substeps,
+// mappings 4 / 5: 152 sources R = 1 17 13, R = 3 25 16, R = 5 51 21, R = 8 72 45, R = 10 52 72; 216 sources R = 4 30 33, R = 5
+// 51 37, R = 7 64 58, R = 8 72 87).
+int default_mapping(const MarchArgs& a, int num_sms) {
+    const int64_t few = (int64_t)num_sms * (a.R >= 5 && a.R <= 7 ? 2 : 1);
+    return a.R <= 8 && a.src_end - a.src_begin <= few ? 5 : 4;
+}
 
 }  // namespace
 
-int march_mapping(const MarchArgs& a, int parts_req) {
+int march_mapping(const MarchArgs& a, int parts_req, int num_sms) {
     if (a.store == Store::F64) return 1;
     if (a.bx) return 5;                           // direction-dependent coefficients: march_flow.cu
     if (parts_req >= 1 && parts_req <= 7 && (a.R <= 8 || parts_req == 4 || parts_req == 5 || parts_req == 7))
         return parts_req;
-    return kDefaultMapping;
+    return default_mapping(a, num_sms);
 }
 
 cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStream_t st) {
@@ -1206,7 +1212,7 @@ cudaError_t launch_march_coarse(const MarchArgs& a, int R, int num_sms, cudaStre
 }
 
 cudaError_t launch_march(const MarchArgs& a, int num_sms, int parts_req, cudaStream_t st, int* parts_used) {
-    const int P = march_mapping(a, parts_req);
+    const int P = march_mapping(a, parts_req, num_sms);
     if (parts_used) *parts_used = P;
     return dispatch(a, P, num_sms, st);
 }

@@ -577,11 +577,11 @@ cudaError_t launch_tm(const MarchArgs& a, int num_sms, cudaStream_t st) {
         if (nsrc >= (int64_t)num_sms * G * 10)
             return G == 2 ? launch_tm<R, false, 2, false>(a, num_sms, st) : launch_tm<R, false, 4, false>(a, num_sms, st);
     }
-    if constexpr (R <= 3) {
+    if constexpr (R <= 4) {
         // A launch that does not fill every CTA: an even share each, warps without a source out of the march (us, 60
-        // substeps, BF16, full CTAs -> shares: 1000 sources R = 1 32 -> 18, R = 2 39 -> 23, R = 3 53 -> 27; 8000 sources
-        // R = 3 145 -> 141).  In a kernel of its own: the loop of full CTAs loses 3% to it.  From R = 4 on a CTA is full
-        // with 15 sources and less.
+        // substeps, BF16, full CTAs -> shares: 1000 sources R = 1 32 -> 18, R = 2 39 -> 23, R = 3 53 -> 27; 512 sources
+        // R = 4 63 -> 33; 8000 sources R = 3 145 -> 141).  In a kernel of its own: the loop of full CTAs loses 3% to it.
+        // From R = 5 on a CTA is full with 7 sources and less.
         if (nsrc > 0 && even_spb(nsrc, M::SPB, num_sms) < M::SPB) return launch_tm<R, false, 1, true>(a, num_sms, st);
     }
     return launch_tm<R, false, 1, false>(a, num_sms, st);

@@ -23,9 +23,9 @@ def _leave_values_in_shared_memory():
         f.kernels()
 
 
-@pytest.mark.parametrize("R", [1, 2, 3])
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 5, 7, 8])
 @pytest.mark.parametrize("shape", [(1, 1, 1), (19, 8, 1), (9, 17, 1), (7, 13, 11), (32, 19, 6), (41, 89, 1), (25, 20, 10),
-                                   (24, 19, 14), (32, 19, 24)])
+                                   (24, 19, 14), (32, 19, 24), (17, 18, 1), (5, 61, 1)])
 def test_small_launches_equal_the_column_march(R, shape):
     D = synth.random_diffusivity(shape, 20 + R, 5.0)
     dt = fdirw.fdirw_stable_dt(shape, D)
