@@ -631,7 +631,7 @@ struct MapTmc {
     static constexpr size_t SMEM_COARSE = SMEM_COARSE_USED > SMEM ? SMEM_COARSE_USED : SMEM;
 };
 
-// COARSE (coarse blocks with convection; without it they run in march_tm.cu): the source is coarse block a.list[pos]
+// COARSE (coarse blocks with convection, or one per SM at most; otherwise they run in march_tm.cu): the source is coarse block a.list[pos]
 // (Eqs. 10-15): its window is centred on the block's centre cell (radius R = window_R + (B - 1) / 2), the march starts
 // from 1 on the block's liquid cells, and the epilogue maps the marched field onto the blocks of the window (column J of
 // the coarse matrix, written destination-indexed) instead of storing a kernel.  The face coefficients differ by direction:

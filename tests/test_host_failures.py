@@ -13,7 +13,6 @@ import pytest
 from paper_2408_11376_gb300 import FDiRW, FDiRWBatch, FDiRWCoarse, build, fdirw
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
 
 
 @pytest.fixture(scope="module")
@@ -25,8 +24,9 @@ def fake(tmp_path_factory):
     objs = [os.path.join(build.BUILD, s.replace(".cu", ".o")) for s in build.SOURCES]
     if not all(os.path.exists(o) for o in objs):
         build.build(force=True)
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
     so = str(tmp_path_factory.mktemp("fake") / "libfdirw_fake.so")
-    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", CUDA_INCLUDE, "-o", so,
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", include, "-o", so,
                     os.path.join(HERE, "fake_cudart.cpp"), *objs], check=True)
     saved = fdirw._lib
     fdirw._lib = None
